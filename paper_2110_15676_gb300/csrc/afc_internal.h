@@ -34,12 +34,6 @@ int cuda_fail(cudaError_t e, const char* what);
     if (e__ != cudaSuccess) return afc::cuda_fail(e__, #call); \
   } while (0)
 
-// A CUDA-graph condition a kernel may set (use = false outside graphs).
-struct GraphCond {
-  bool use = false;
-  cudaGraphConditionalHandle h = 0;
-};
-
 // Offsets passed by value to kernels (constant bank, unrolled loops).
 struct Offsets {
   int K;          // number of offsets (odd)
@@ -207,8 +201,7 @@ int cn_linear_guess(afc_problem_s* p, const double* u_old, double* u);          
 // CN with the MC limiter (Sec. 2.2): Fold = F*(u_old), then res = b0 + (F*(u) + Fold)/2 - (M_L/dt + AA/2) u
 int mc_cn_old_flux(afc_problem_s* p, const double* u_old);
 int mc_cn_residual(afc_problem_s* p, const double* u, double* res, double* normsq_slot);
-// a = u - u_old, s = u + u_old after u += omega * delta (delta may be null)
-int cn_update(afc_problem_s* p, double omega, const double* delta, double* u, const double* u_old);
+int cn_update(afc_problem_s* p, const double* u, const double* u_old);                 // a = u - u_old, s = u + u_old
 int cn_limited_residual(afc_problem_s* p, const double* u_new, double dt, int limiter, int prelimit, double* res,
                         double* normsq_slot);                                      // needs cn_update first
 // MC
@@ -225,10 +218,10 @@ int mc_pair_residual(afc_problem_s* p, const double* u, int limiter, double* res
 
 // ---- reductions and BLAS-1 (krylov.cu) ----
 int dot_device(afc_problem_s* p, const double* x, const double* y, double* out_slot);
-// An update that the persistent BiCGStab applies to the solution x in its last pass,
-// unless the solve broke down: u += omega x, then a = u - uo and s = u + uo (the
-// damped CN correction and the node sums of the next flux pass, bit for bit what
-// cn_update computes).  u == nullptr: none.
+// An update that a persistent Krylov launch applies to its solution x in its last
+// pass, unless the solve broke down: u += omega x, and with `a` then a = u - uo and
+// s = u + uo (the damped correction and, for the CN scheme, the node sums of the next
+// flux pass).  u == nullptr: none.
 struct KrylovEpilogue {
   double omega = 0.0;
   double* u = nullptr;
@@ -237,12 +230,24 @@ struct KrylovEpilogue {
   double* s = nullptr;
   double* fp_sc = nullptr;   // graph form: the fixed-point scalars, where the solve counts itself
 };
-// *epi_done (if given) tells whether the solve applied *epi; when it did not, the
-// caller applies the update itself.
+// The updates of the fixed points: of a CN step, and of a stationary solve.
+inline KrylovEpilogue stationary_epilogue(afc_problem_s* p, const afc_opts* o) {
+  KrylovEpilogue e;
+  e.omega = o->omega;
+  e.u = p->u.p;
+  return e;
+}
+inline KrylovEpilogue step_epilogue(afc_problem_s* p, const afc_opts* o) {
+  KrylovEpilogue e = stationary_epilogue(p, o);
+  if (o->limiter == AFC_LIM_MC) return e;   // its fluxes need no node sums
+  e.uo = p->u0.p;
+  e.a = p->cn_a.p;
+  e.s = p->cn_s.p;
+  return e;
+}
 int krylov_solve(afc_problem_s* p, int system, const afc_opts* o, const double* rhs, double* x, int* its,
-                 double* res, const KrylovEpilogue* epi = nullptr, bool* epi_done = nullptr);
+                 double* res, const KrylovEpilogue* epi = nullptr);
 int dia_spmv(afc_problem_s* p, const double* A, const double* x, double* y);
-int axpy_device(afc_problem_s* p, double a, const double* x, double* y);   // y += a x
 int minmax_device(afc_problem_s* p, const double* x, double* mn, double* mx);
 void krylov_free(afc_problem_s* p);
 const void* krylov_key(afc_problem_s* p);   // changes when the solver workspace is reallocated

@@ -136,11 +136,10 @@ int finish_stats(afc_problem_s* p, afc_stats* st, int status) {
 
 // Damped fixed point of Sec. 4 in defect form: res = residual(u); stop if
 // ||res|| < sqrt(N) tol; solve B delta = res; u += omega delta.
-// With `epi`, a persistent BiCGStab applies the update in its last pass and update()
-// only runs where the solve did not.
-template <class Residual, class Update>
-int fixed_point(afc_problem_s* p, const afc_opts* o, int system, afc_stats* st, Residual residual, Update update,
-                const KrylovEpilogue* epi = nullptr) {
+// The persistent solve applies the update in its last pass (`epi`).
+template <class Residual>
+int fixed_point(afc_problem_s* p, const afc_opts* o, int system, afc_stats* st, Residual residual,
+                const KrylovEpilogue& epi) {
   const double thresh = std::sqrt((double)p->N) * o->fp_tol;
   int status = AFC_NOT_CONVERGED;
   for (int it = 0;; ++it) {
@@ -162,14 +161,12 @@ int fixed_point(afc_problem_s* p, const afc_opts* o, int system, afc_stats* st, 
     }
     int its = 0;
     double kres = 0;
-    bool applied = false;
-    e = krylov_solve(p, system, o, p->res.p, p->delta.p, &its, &kres, epi, &applied);
+    e = krylov_solve(p, system, o, p->res.p, p->delta.p, &its, &kres, &epi);
     if (e < 0) return e;
     if (st) {
       st->inner_its += its;
       st->outer_its += 1;
     }
-    if (!applied && (e = update())) return e;
   }
   return status;
 }
@@ -509,7 +506,7 @@ int step_impl(afc_problem p, const afc_opts* o, afc_stats* stt) {
     if ((st = mc_cn_old_flux(p, p->u0.p))) return st;
     st = fixed_point(
         p, o, 1, stt, [&]() { return mc_cn_residual(p, p->u.p, p->res.p, p->scal.p); },
-        [&]() { return axpy_device(p, o->omega, p->delta.p, p->u.p); });
+        step_epilogue(p, o));
     if (st < 0) return st;
     return finish_stats(p, stt, st);
   }
@@ -519,17 +516,11 @@ int step_impl(afc_problem p, const afc_opts* o, afc_stats* stt) {
     AFC_LAUNCH(p, "k_apply_dirichlet", k_apply_dirichlet<<<grid_for(N), kBlock, 0, s>>>(N, p->dir.p, p->udir.p, p->u.p));
     AFC_CUDA(cudaGetLastError());
   }
-  if ((st = cn_update(p, 0.0, nullptr, p->u.p, p->u0.p))) return st;
+  if ((st = cn_update(p, p->u.p, p->u0.p))) return st;
   const double dt = o->dt;
-  KrylovEpilogue epi;
-  epi.omega = o->omega;
-  epi.u = p->u.p;
-  epi.uo = p->u0.p;
-  epi.a = p->cn_a.p;
-  epi.s = p->cn_s.p;
   st = fixed_point(
       p, o, 1, stt, [&]() { return cn_limited_residual(p, p->u.p, dt, lim, o->prelimit, p->res.p, p->scal.p); },
-      [&]() { return cn_update(p, o->omega, p->delta.p, p->u.p, p->u0.p); }, &epi);
+      step_epilogue(p, o));
   if (st < 0) return st;
   return finish_stats(p, stt, st);
 }
@@ -555,7 +546,7 @@ int stationary_impl(afc_problem p, const afc_opts* o, afc_stats* stt) {
       p, o, 0, stt, [&]() {
         return mc_limited_residual(p, p->u.p, lim, p->res.p, p->scal.p, false, o->precision == AFC_MIXED);
       },
-      [&]() { return axpy_device(p, o->omega, p->delta.p, p->u.p); });
+      stationary_epilogue(p, o));
   if (st < 0) return st;
   return finish_stats(p, stt, st);
 }
@@ -633,7 +624,7 @@ int afc_cn_limited_sum(afc_problem p, double dt, int limiter, int prelimit, cons
   if ((st = to_device(p, p->ustage.p, u_new, p->N)) || (st = to_device(p, p->u0.p, u_old, p->N))) return st;
   if ((st = build_cn_system(p, dt))) return st;
   if ((st = cn_predictor(p, p->u0.p, dt))) return st;
-  if ((st = cn_update(p, 0.0, nullptr, p->ustage.p, p->u0.p))) return st;
+  if ((st = cn_update(p, p->ustage.p, p->u0.p))) return st;
   if ((st = cn_limited_residual(p, p->ustage.p, dt, limiter, prelimit, p->res.p, p->scal.p))) return st;
   if ((st = to_host(p, u_tilde, p->ut.p, p->N)) || (st = to_host(p, Rp, p->Rp.p, p->N)) ||
       (st = to_host(p, Rm, p->Rm.p, p->N)) || (st = to_host(p, Fstar, p->Fs.p, p->N)))

@@ -94,18 +94,13 @@ __global__ void k_bounds_of(int64_t N, Offsets of, const unsigned long long* __r
   Qm[i] = m * (from_key(kmin) - vi);
 }
 
-// Node sums of the CN flux: a = u - u_old, s = u + u_old; optionally first
-// u += omega * delta (the damped update of Sec. 4).
-__global__ void k_cn_update(int64_t N, double omega, const double* __restrict__ delta, double* __restrict__ u,
-                            const double* __restrict__ uo, double* __restrict__ a, double* __restrict__ s) {
+// Node sums of the CN flux: a = u - u_old, s = u + u_old (at the start of a step; each
+// solve renews them in its last pass).
+__global__ void k_cn_update(int64_t N, const double* __restrict__ u, const double* __restrict__ uo,
+                            double* __restrict__ a, double* __restrict__ s) {
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= N) return;
-  double ui = u[i];
-  if (delta) {
-    ui = ui + omega * delta[i];
-    u[i] = ui;
-  }
-  const double uoi = uo[i];
+  const double ui = u[i], uoi = uo[i];
   a[i] = ui - uoi;
   s[i] = ui + uoi;
 }
@@ -333,9 +328,9 @@ int cn_predictor(afc_problem_s* p, const double* u_old, double dt) {
   return AFC_OK;
 }
 
-int cn_update(afc_problem_s* p, double omega, const double* delta, double* u, const double* u_old) {
-  AFC_LAUNCH(p, "k_cn_update", k_cn_update<<<grid_for(p->N), kBlock, 0, p->stream>>>(p->N, omega, delta, u, u_old,
-                                                                                       p->cn_a.p, p->cn_s.p));
+int cn_update(afc_problem_s* p, const double* u, const double* u_old) {
+  AFC_LAUNCH(p, "k_cn_update",
+             k_cn_update<<<grid_for(p->N), kBlock, 0, p->stream>>>(p->N, u, u_old, p->cn_a.p, p->cn_s.p));
   AFC_CUDA(cudaGetLastError());
   return AFC_OK;
 }

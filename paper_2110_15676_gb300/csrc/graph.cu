@@ -28,7 +28,6 @@ __global__ void k_fp_init(double* sc, double thresh, int fixed, int maxit) {
   sc[F_THRESH] = thresh;
   sc[F_FIXED] = (double)fixed;
   sc[F_MAXIT] = (double)maxit;
-  sc[F_KBODY] = 0.0;
   sc[F_REVAL] = 0.0;
   sc[F_TIMEOUT] = 0.0;
 }
@@ -61,20 +60,6 @@ __global__ void k_fp_control(double* sc, const double* __restrict__ part, int np
   }
   cudaGraphSetConditional(h_loop, stop ? 0u : 1u);
   cudaGraphSetConditional(h_solve, stop ? 0u : 1u);
-}
-
-// After a linear solve: count it, its Krylov iterations and loop-body executions;
-// a solver breakdown ends the fixed point at the next control.
-__global__ void k_fp_after_solve(double* sc, const double* __restrict__ ksc, int gmres, int cycles_slot) {
-  if (threadIdx.x != 0) return;
-  sc[F_CORR] += 1.0;
-  sc[F_INNER] += ksc[kKrylovItsSlot];
-  sc[F_KBODY] += gmres ? ksc[cycles_slot] : ksc[kKrylovItsSlot];
-  if (ksc[kKrylovDoneSlot] == 2.0) sc[F_STATUS] = 2.0;
-  if (!gmres && ksc[kKrylovBarrierErrSlot] != 0.0) {
-    sc[F_STATUS] = 2.0;
-    sc[F_TIMEOUT] = 1.0;
-  }
 }
 
 __global__ void k_copy(int64_t n, const double* __restrict__ x, double* __restrict__ y) {
@@ -150,7 +135,7 @@ int enqueue_stats(afc_problem_s* p) {
 struct StepGraph {
   cudaGraphExec_t exec = nullptr;
   std::vector<unsigned char> key;
-  int64_t k_pro = 0, k_outer = 0, k_solve = 0, k_body = 0, k_epi = 0;
+  int64_t k_pro = 0, k_outer = 0, k_solve = 0, k_epi = 0;
   int kind = 0;   // 1 fixed point, 2 explicit SSP
 };
 
@@ -186,11 +171,11 @@ struct ProfOff {   // no event records inside captured graphs; captured launches
   }
 };
 
-// Build the fixed-point graph: prologue, while(outer){ residual; control; if(solve){ Krylov; update; count } },
-// epilogue.  `system` 1: CN step, 0: stationary.
-template <class Pro, class Res, class Upd>
-int build_fixed_point(afc_problem_s* p, const afc_opts* o, int system, Pro prologue, Res residual, Upd update,
-                      StepGraph& sg, const KrylovEpilogue* epi = nullptr) {
+// Build the fixed-point graph: prologue, while(outer){ residual; control; if(solve){ Krylov } }, epilogue.  The
+// persistent solve applies the update `epi` and counts itself in the fixed-point scalars.  `system` 1: CN step, 0: stationary.
+template <class Pro, class Res>
+int build_fixed_point(afc_problem_s* p, const afc_opts* o, int system, Pro prologue, Res residual, StepGraph& sg,
+                      KrylovEpilogue epi) {
   if (!p->cap_stream) AFC_CUDA(cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking));
   cudaStream_t cs = p->cap_stream;
   ProfOff po(p);
@@ -246,35 +231,13 @@ int build_fixed_point(afc_problem_s* p, const afc_opts* o, int system, Pro prolo
     cudaGraph_t sbody;
     cudaGraphNode_t ifnode;
     if ((st = add_conditional(body, bf, h_solve, cudaGraphCondTypeIf, &sbody, &ifnode))) break;
-    // Krylov solve (its while node counts separately), update and counters
     std::vector<cudaGraphNode_t> sf;
-    const int64_t l0 = p->launches;
-    bool applied = false;   // the persistent BiCGStab applies the update itself
-    // ... and then also counts the correction in the fixed-point scalars (no after-solve node)
-    KrylovEpilogue epc;
-    if (epi) {
-      epc = *epi;
-      epc.fp_sc = p->scal.p;
-    }
-    if ((st = krylov_graph(p, system, o, p->res.p, p->delta.p, cs, sbody, sf, epi ? &epc : nullptr, &applied)))
-      break;
-    const int64_t lk = p->launches - l0;
-    const int64_t body_k = o->ksp == AFC_KSP_GMRES ? 3 + 5 * (int64_t)o->gmres_restart : 5;
+    epi.fp_sc = p->scal.p;
     auto r3 = count([&]() -> int {
-      return capture_into(p, cs, sbody, sf, [&]() -> int {
-        if (applied) return AFC_OK;   // the fused solve updated u and counted the correction
-        int s = update();
-        if (s) return s;
-        AFC_LAUNCH(p, "k_fp_after_solve",
-                   k_fp_after_solve<<<1, 32, 0, p->stream>>>(p->scal.p, krylov_scalars(p),
-                                                             o->ksp == AFC_KSP_GMRES ? 1 : 0, krylov_cycles_slot()));
-        AFC_CUDA(cudaGetLastError());
-        return AFC_OK;
-      }, sf);
+      return krylov_graph(p, system, o, p->res.p, p->delta.p, cs, sbody, sf, &epi);
     });
     if ((st = r3.first)) break;
-    sg.k_body = body_k;
-    sg.k_solve = lk - body_k + r3.second;
+    sg.k_solve = r3.second;
     fr.assign(1, loop);
     auto r4 = count([&]() -> int { return capture_into(p, cs, g, fr, [&]() -> int { return enqueue_stats(p); }, fr); });
     if ((st = r4.first)) break;
@@ -293,8 +256,8 @@ int run_fixed_point_graph(afc_problem_s* p, StepGraph& sg, afc_stats* stt) {
   AFC_CUDA(cudaGraphLaunch(sg.exec, p->stream));
   AFC_CUDA(cudaStreamSynchronize(p->stream));
   const double* h = p->host_scal;
-  const int64_t reval = (int64_t)h[F_REVAL], corr = (int64_t)h[F_CORR], kbody = (int64_t)h[F_KBODY];
-  p->launches += sg.k_pro + reval * sg.k_outer + corr * sg.k_solve + kbody * sg.k_body + sg.k_epi;
+  const int64_t reval = (int64_t)h[F_REVAL], corr = (int64_t)h[F_CORR];
+  p->launches += sg.k_pro + reval * sg.k_outer + corr * sg.k_solve + sg.k_epi;
   int status = h[F_STATUS] == 1.0 ? AFC_OK : h[F_STATUS] == 2.0 ? AFC_E_NAN : AFC_NOT_CONVERGED;
   if (h[F_TIMEOUT] != 0.0) {
     // the barrier counter is inconsistent after blocks skipped barriers: clear it so
@@ -302,7 +265,7 @@ int run_fixed_point_graph(afc_problem_s* p, StepGraph& sg, afc_stats* stt) {
     const int rs = krylov_reset_barrier(p);
     if (rs) return rs;
     status = AFC_E_TIMEOUT;
-    set_error("a grid barrier of the persistent BiCGStab launch gave up waiting");
+    set_error("a grid barrier of the persistent Krylov launch gave up waiting");
   } else if (status == AFC_E_NAN) {
     set_error("non-finite nonlinear residual or Krylov breakdown");
   }
@@ -336,12 +299,7 @@ int cn_step_graph(afc_problem_s* p, const afc_opts* o, afc_stats* stt) {
     p->g_step = new StepGraph();
     const int lim = o->limiter;
     const double dt = o->dt;
-    KrylovEpilogue epi;
-    epi.omega = o->omega;
-    epi.u = p->u.p;
-    epi.uo = p->u0.p;
-    epi.a = p->cn_a.p;
-    epi.s = p->cn_s.p;
+    const KrylovEpilogue epi = step_epilogue(p, o);
     int st = build_fixed_point(
         p, o, 1,
         [&]() -> int {
@@ -360,16 +318,13 @@ int cn_step_graph(afc_problem_s* p, const afc_opts* o, afc_stats* stt) {
             AFC_LAUNCH(p, "k_apply_dirichlet",
                        k_apply_dirichlet_g<<<grid_for(N), kBlock, 0, p->stream>>>(N, p->dir.p, p->udir.p, p->u.p));
           }
-          return cn_update(p, 0.0, nullptr, p->u.p, p->u0.p);
+          return cn_update(p, p->u.p, p->u0.p);
         },
         [&]() -> int {
           if (lim == AFC_LIM_MC) return mc_cn_residual(p, p->u.p, p->res.p, nullptr);
           return cn_limited_residual(p, p->u.p, dt, lim, o->prelimit, p->res.p, nullptr);
         },
-        [&]() -> int {
-          if (lim == AFC_LIM_MC) return axpy_device(p, o->omega, p->delta.p, p->u.p);
-          return cn_update(p, o->omega, p->delta.p, p->u.p, p->u0.p);
-        }, *p->g_step, lim == AFC_LIM_MC ? nullptr : &epi);
+        *p->g_step, epi);
     if (st) {
       drop(p->g_step);
       return st;
@@ -396,7 +351,7 @@ int stationary_graph(afc_problem_s* p, const afc_opts* o, afc_stats* stt) {
         [&]() -> int {
           return mc_limited_residual(p, p->u.p, lim, p->res.p, nullptr, false, o->precision == AFC_MIXED);
         },
-        [&]() -> int { return axpy_device(p, o->omega, p->delta.p, p->u.p); }, *p->g_stat);
+        *p->g_stat, stationary_epilogue(p, o));
     if (st) {
       drop(p->g_stat);
       return st;

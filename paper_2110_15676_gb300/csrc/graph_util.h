@@ -52,29 +52,20 @@ inline int add_conditional(cudaGraph_t g, const std::vector<cudaGraphNode_t>& de
   return AFC_OK;
 }
 
-// Krylov solve of `system` appended to graph g after `frontier` (updated): the
-// solver's loop is a while node whose condition the iteration kernels keep.
+// Krylov solve of `system` appended to graph g after `frontier` (updated): one
+// persistent launch, which also applies and counts the update `epi`.
 int krylov_graph(afc_problem_s* p, int system, const afc_opts* o, const double* rhs, double* x, cudaStream_t cs,
-                 cudaGraph_t g, std::vector<cudaGraphNode_t>& frontier, const KrylovEpilogue* epi = nullptr,
-                 bool* epi_done = nullptr);
-
-// device address of the solver scalars (iteration count at slot kKrylovItsSlot)
-const double* krylov_scalars(afc_problem_s* p);
-constexpr int kKrylovItsSlot = 7;
-constexpr int kKrylovDoneSlot = 8;
-// 1 after a grid barrier of the persistent BiCGStab launch gave up waiting
-constexpr int kKrylovBarrierErrSlot = 19;
+                 cudaGraph_t g, std::vector<cudaGraphNode_t>& frontier, const KrylovEpilogue* epi);
 
 // fixed-point scalar slots (problem scalars p->scal)
 enum : int {
   F_NORMSQ = 0, F_CORR = 1, F_INNER = 2, F_RES0 = 3, F_RESF = 4, F_STATUS = 5, F_THRESH = 6, F_FIXED = 7,
-  F_MAXIT = 8, F_KBODY = 9, F_REVAL = 10, F_TIMEOUT = 11
+  F_MAXIT = 8, F_REVAL = 10, F_TIMEOUT = 11
 };
 // F_STATUS: 0 running, 1 converged / fixed count reached, 2 non-finite or a solver that
 // could not finish, 3 iteration limit; F_TIMEOUT: 1 after a grid barrier of the
-// persistent BiCGStab gave up waiting (F_STATUS is then 2)
-int krylov_cycles_slot();
-// Clear the grid barrier state of the persistent BiCGStab after a timeout (its
+// persistent solve gave up waiting (F_STATUS is then 2)
+// Clear the grid barrier state of the persistent solves after a timeout (its
 // counter is left inconsistent when blocks skip barriers); synchronises the stream.
 int krylov_reset_barrier(afc_problem_s* p);
 

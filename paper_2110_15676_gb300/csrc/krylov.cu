@@ -83,11 +83,6 @@ __global__ void k_dot(int64_t N, const double* __restrict__ x, const double* __r
   block_sum_to(v, part);
 }
 
-__global__ void k_axpy(int64_t N, double a, const double* __restrict__ x, double* __restrict__ y) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
-    y[i] = y[i] + a * x[i];
-}
-
 __global__ void k_minmax(int64_t N, const double* __restrict__ x, double* __restrict__ part) {
   double mn = INFINITY, mx = -INFINITY;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
@@ -153,12 +148,6 @@ int dot_device(afc_problem_s* p, const double* x, const double* y, double* out_s
   return AFC_OK;
 }
 
-int axpy_device(afc_problem_s* p, double a, const double* x, double* y) {
-  AFC_LAUNCH(p, "k_axpy", k_axpy<<<kRedBlocks, kBlock, 0, p->stream>>>(p->N, a, x, y));
-  AFC_CUDA(cudaGetLastError());
-  return AFC_OK;
-}
-
 int minmax_device(afc_problem_s* p, const double* x, double* mn, double* mx) {
   AFC_LAUNCH(p, "k_minmax", k_minmax<<<kRedBlocks, kBlock, 0, p->stream>>>(p->N, x, p->part.p));
   AFC_LAUNCH(p, "k_minmax_fin", k_minmax_fin<<<1, kBlock, 0, p->stream>>>(p->part.p, kRedBlocks, p->scal.p + 60));
@@ -183,18 +172,12 @@ constexpr int kMaxRestart = 32;   // GMRES(m), m <= 32: the Gram-Schmidt kernel 
 
 // device scalar slots
 enum : int {
-  S_RHO = 0, S_RHO_OLD, S_ALPHA, S_OMEGA, S_TOL, S_NRES, S_N0, S_ITS, S_DONE, S_MAXIT,
-  S_BETA, S_K_USED, S_INVH, S_CYCLE_DONE, S_FIRST, S_ATOL, S_RTOL, S_NO_REORTH,
-  S_CS = 20, S_SN = S_CS + kMaxRestart, S_G = S_SN + kMaxRestart, S_Y = S_G + kMaxRestart + 1,
-  S_H1 = S_Y + kMaxRestart, S_H2 = S_H1 + kMaxRestart + 1, S_HCOL = S_H2 + kMaxRestart + 1,
-  S_END = S_HCOL + (kMaxRestart + 1) * kMaxRestart
+  S_RHO = 0, S_RHO_OLD, S_ALPHA, S_OMEGA, S_TOL, S_NRES, S_N0, S_ITS, S_DONE, S_MAXIT, S_BETA, S_ATOL, S_RTOL,
+  S_CYCLES,   // GMRES restart cycles begun (true-residual evaluations)
+  S_BERR,     // persistent launches: a grid barrier gave up waiting
+  S_END
 };
 // S_DONE: 0 running, 1 converged, 2 breakdown / non-finite, 3 converged at s (x update pending), 4 maxit
-static_assert(S_ITS == kKrylovItsSlot && S_DONE == kKrylovDoneSlot, "slot numbers shared with graph.cu");
-constexpr int S_CYCLES = 18;   // GMRES restart cycles begun (true-residual evaluations)
-constexpr int S_BERR = 19;     // persistent BiCGStab: a grid barrier gave up waiting
-static_assert(S_CYCLES > S_NO_REORTH && S_BERR > S_CYCLES && S_BERR < S_CS, "slot range");
-static_assert(S_BERR == kKrylovBarrierErrSlot, "slot number shared with graph.cu");
 
 // A solver flag (a double slot holding 0 or a positive code) tested on its bit pattern:
 // a compare of doubles issues on GB300's FP64 pipe, where every warp instruction
@@ -211,10 +194,8 @@ struct KrylovWork {
   int pad = 0, m = 0, fp32 = -1;
   DBuf<char> vec;       // all vectors (with halos)
   DBuf<double> sc, part;
-  DBuf<unsigned int> counter;
   DBuf<unsigned int> barrier;   // GridBar of the persistent BiCGStab launch
-  int coop = -1;                // device supports cooperative launches (-1: not asked yet)
-  int nsm = 0;
+  int nsm = 0;                  // SMs of the device (0: not asked yet)
   double* hsc = nullptr;
   size_t vstride = 0;   // elements per vector incl. halo
 };
@@ -224,245 +205,6 @@ template struct DBuf<unsigned int>;
 template struct DBuf<uint16_t>;
 
 namespace {
-
-// ---- "last block" reductions ------------------------------------------------
-// A producer kernel writes one partial per block and counts finished blocks; the
-// block that finishes last sums all partials in block order (deterministic) and
-// updates the solver scalars.  Every block reads the scalars it needs before it
-// counts itself, and only the last block writes them, so no block of a kernel
-// sees a scalar that the same kernel changes.
-// Sum v over the block in a fixed order; every thread receives the total.
-__device__ __forceinline__ double block_allsum(double v) {
-  __shared__ double total;
-  if (blockDim.x > kBlock) {
-    __shared__ double sw[32];
-    v = warp_sum(v);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (lane == 0) sw[w] = v;
-    __syncthreads();
-    if (w == 0) {
-      const int nw = (blockDim.x + 31) >> 5;
-      double t = lane < nw ? sw[lane] : 0.0;
-      t = warp_sum(t);
-      if (lane == 0) total = t;
-    }
-  } else {
-    __shared__ double sh[kBlock];
-    sh[threadIdx.x] = v;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-      const double t = warp0_column_sum(sh);
-      if (threadIdx.x == 0) total = t;
-    }
-  }
-  __syncthreads();
-  const double r = total;
-  __syncthreads();
-  return r;
-}
-
-template <int NV>
-__device__ __forceinline__ bool last_block_sums(double (&v)[NV], double* part, int64_t pstride,
-                                                unsigned int* counter, double (&tot)[NV]) {
-  block_sums_to<NV>(v, part, pstride);
-  __shared__ bool am_last;
-  if (threadIdx.x == 0) {
-    __threadfence();
-    const unsigned int done = atomicAdd(counter, 1u);
-    am_last = done == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (!am_last) return false;
-  __threadfence();
-  const int n = gridDim.x;
-#pragma unroll
-  for (int q = 0; q < NV; ++q) {
-    // thread t adds partials t, t + blockDim.x, ... in turn, the loads eight at a time
-    double s = 0.0;
-    for (int b0 = threadIdx.x; b0 < n; b0 += 8 * blockDim.x) {
-      double x[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int b = b0 + u * blockDim.x;
-        x[u] = b < n ? __ldcg(part + q * pstride + b) : 0.0;
-      }
-#pragma unroll
-      for (int u = 0; u < 8; ++u) s += x[u];
-    }
-    tot[q] = block_allsum(s);
-  }
-  if (threadIdx.x == 0) *counter = 0u;
-  return true;
-}
-
-__device__ __forceinline__ bool stop_test(double nr, const double* sc) { return nr < sc[S_TOL]; }
-
-// ---- BiCGStab (van der Vorst 1992), Jacobi preconditioner on the directions ----
-template <class T>
-__global__ void k_bicg_init(int64_t N, const double* __restrict__ rhs, T* x, T* r, T* rh, T* p, T* v,
-                            double* __restrict__ part, unsigned int* counter, double* sc) {
-  T a0 = 0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
-    const T ri = (T)rhs[i];
-    x[i] = 0;
-    r[i] = ri;
-    rh[i] = ri;
-    p[i] = 0;
-    v[i] = 0;
-    a0 = fma(ri, ri, a0);
-  }
-  double acc[1] = {(double)a0};
-  double tot[1];
-  if (!last_block_sums<1>(acc, part, gridDim.x, counter, tot)) return;
-  if (threadIdx.x == 0) {
-    const double n0 = sqrt(tot[0]);
-    sc[S_N0] = n0;
-    sc[S_NRES] = n0;
-    sc[S_RHO] = tot[0];
-    sc[S_RHO_OLD] = 1.0;
-    sc[S_ALPHA] = 1.0;
-    sc[S_OMEGA] = 1.0;
-    sc[S_BETA] = (tot[0] / 1.0) * (1.0 / 1.0);
-    sc[S_TOL] = fmax(sc[S_ATOL], sc[S_RTOL] * n0);
-    sc[S_ITS] = 0.0;
-    sc[S_DONE] = !isfinite(n0) ? 2.0 : (n0 < sc[S_TOL] ? 1.0 : (sc[S_MAXIT] <= 0.0 ? 4.0 : 0.0));
-  }
-}
-
-// p = r + beta (p - omega v), phat = D^{-1} p
-template <class T>
-__global__ void k_bicg_p(int64_t N, const double* __restrict__ sc, const T* __restrict__ r, T* p,
-                         const T* __restrict__ v, const T* __restrict__ dinv, T* __restrict__ ph) {
-  if (flag_set(sc, S_DONE)) return;
-  const T beta = (T)sc[S_BETA];       // (rho / rho_old)(alpha / omega), formed once by the previous kernel
-  const T om = (T)sc[S_OMEGA];
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
-    const T pi = r[i] + beta * (p[i] - om * v[i]);
-    p[i] = pi;
-    ph[i] = dinv[i] * pi;
-  }
-}
-
-// v = B phat and (rhat, v); the last block sets alpha = rho / (rhat, v)
-template <int KT, class T>
-__global__ void k_bicg_spmv1(int64_t N, Offsets of, double* sc, const T* __restrict__ B, const T* __restrict__ x,
-                             T* __restrict__ y, const T* __restrict__ a, double* __restrict__ part,
-                             unsigned int* counter) {
-  if (flag_set(sc, S_DONE)) return;
-  const int K = KT > 0 ? KT : of.K;
-  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  double acc[1] = {0.0};
-  if (i < N) {
-    T s = 0;
-#pragma unroll
-    for (int k = 0; k < K; ++k) s = fma(B[k * N + i], x[i + of.o[k]], s);
-    y[i] = s;
-    acc[0] = (double)(a[i] * s);
-  }
-  double tot[1];
-  if (!last_block_sums<1>(acc, part, gridDim.x, counter, tot)) return;
-  if (threadIdx.x == 0) {
-    const double al = sc[S_RHO] / tot[0];
-    if (!isfinite(al) || tot[0] == 0.0) sc[S_DONE] = 2.0;
-    else sc[S_ALPHA] = al;
-  }
-}
-
-// s = r - alpha v, shat = D^{-1} s, ||s||; the last block tests convergence at s
-template <class T>
-__global__ void k_bicg_s(int64_t N, double* sc, const T* __restrict__ r, const T* __restrict__ v,
-                         const T* __restrict__ dinv, T* __restrict__ s, T* __restrict__ sh, double* __restrict__ part,
-                         unsigned int* counter) {
-  if (flag_set(sc, S_DONE)) return;
-  const T al = (T)sc[S_ALPHA];
-  T a0 = 0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
-    const T si = r[i] - al * v[i];
-    s[i] = si;
-    sh[i] = dinv[i] * si;
-    a0 = fma(si, si, a0);
-  }
-  double acc[1] = {(double)a0};
-  double tot[1];
-  if (!last_block_sums<1>(acc, part, gridDim.x, counter, tot)) return;
-  if (threadIdx.x == 0) {
-    const double ns = sqrt(tot[0]);
-    if (!isfinite(ns)) { sc[S_DONE] = 2.0; return; }
-    if (stop_test(ns, sc)) {
-      sc[S_NRES] = ns;
-      sc[S_ITS] += 1.0;
-      sc[S_DONE] = 3.0;     // converged at s: x += alpha phat in the next kernel
-    }
-  }
-}
-
-// t = B shat, (t, s), (t, t); the last block sets omega.  When the solve converged at
-// s, this kernel instead finishes x += alpha phat.
-template <int KT, class T>
-__global__ void k_bicg_spmv2(int64_t N, Offsets of, double* sc, const T* __restrict__ B, const T* __restrict__ sh,
-                             T* __restrict__ t, const T* __restrict__ s, T* __restrict__ x,
-                             const T* __restrict__ ph, double* __restrict__ part, unsigned int* counter) {
-  const double done = sc[S_DONE];
-  if (done != 0.0 && done != 3.0) return;
-  const int K = KT > 0 ? KT : of.K;
-  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  double acc[2] = {0.0, 0.0};
-  if (done == 3.0) {
-    if (i < N) x[i] = x[i] + (T)sc[S_ALPHA] * ph[i];
-  } else if (i < N) {
-    T v = 0;
-#pragma unroll
-    for (int k = 0; k < K; ++k) v = fma(B[k * N + i], sh[i + of.o[k]], v);
-    t[i] = v;
-    acc[0] = (double)(v * s[i]);
-    acc[1] = (double)(v * v);
-  }
-  double tot[2];
-  if (!last_block_sums<2>(acc, part, gridDim.x, counter, tot)) return;
-  if (threadIdx.x == 0) {
-    if (done == 3.0) { sc[S_DONE] = 1.0; return; }
-    const double om = tot[0] / tot[1];
-    if (!isfinite(om) || tot[1] == 0.0) sc[S_DONE] = 2.0;
-    else sc[S_OMEGA] = om;
-  }
-}
-
-// x += alpha phat + omega shat, r = s - omega t, ||r||, (rhat, r); the last block tests
-// convergence and rotates rho
-template <class T>
-__global__ void k_bicg_xr(int64_t N, double* sc, T* __restrict__ x, const T* __restrict__ ph,
-                          const T* __restrict__ sh, const T* __restrict__ s, const T* __restrict__ t,
-                          T* __restrict__ r, const T* __restrict__ rh, double* __restrict__ part,
-                          unsigned int* counter, GraphCond cond) {
-  if (flag_set(sc, S_DONE)) {
-    if (cond.use && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(cond.h, 0u);
-    return;
-  }
-  const T al = (T)sc[S_ALPHA], om = (T)sc[S_OMEGA];
-  T a0 = 0, a1 = 0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
-    x[i] = x[i] + al * ph[i] + om * sh[i];
-    const T ri = s[i] - om * t[i];
-    r[i] = ri;
-    a0 = fma(ri, ri, a0);
-    a1 = fma(rh[i], ri, a1);
-  }
-  double acc[2] = {(double)a0, (double)a1};
-  double tot[2];
-  if (!last_block_sums<2>(acc, part, gridDim.x, counter, tot)) return;
-  if (threadIdx.x == 0) {
-    const double nr = sqrt(tot[0]);
-    sc[S_NRES] = nr;
-    sc[S_RHO_OLD] = sc[S_RHO];
-    sc[S_RHO] = tot[1];
-    sc[S_BETA] = (sc[S_RHO] / sc[S_RHO_OLD]) * (sc[S_ALPHA] / sc[S_OMEGA]);
-    sc[S_ITS] += 1.0;
-    if (!isfinite(nr)) sc[S_DONE] = 2.0;
-    else if (stop_test(nr, sc)) sc[S_DONE] = 1.0;
-    else if (sc[S_ITS] >= sc[S_MAXIT]) sc[S_DONE] = 4.0;
-    if (cond.use) cudaGraphSetConditional(cond.h, sc[S_DONE] == 0.0 ? 1u : 0u);
-  }
-}
 
 // ---- BiCGStab as one persistent cooperative launch ----------------------------
 // The five phases of an iteration (p update, v = B phat, s update, t = B shat, x / r
@@ -544,6 +286,26 @@ __device__ __forceinline__ void grid_sums(double (&v)[NV], double* part, int& bu
                                           double (&tot)[NV], unsigned long long wait_ns) {
   const unsigned int old = grid_sums_begin<NV>(v, part, buf, bar);
   grid_sums_end<NV>(part, buf, bar, old, tot, wait_ns);
+}
+
+// The caller's update of a solve's last pass (KrylovEpilogue) at row i.
+__device__ __forceinline__ void krylov_update(const KrylovEpilogue& ep, int64_t i, double xi) {
+  const double ui = ep.u[i] + ep.omega * xi;
+  ep.u[i] = ui;
+  if (ep.a) {
+    const double uoi = ep.uo[i];
+    ep.a[i] = ui - uoi;
+    ep.s[i] = ui + uoi;
+  }
+}
+// The fixed-point loop's count of a correction (one thread of the solve's launch).
+__device__ __forceinline__ void krylov_count(const KrylovEpilogue& ep, int its, bool berr, bool broke) {
+  double* f = ep.fp_sc;
+  if (!f) return;
+  f[F_CORR] += 1.0;
+  f[F_INNER] += (double)its;
+  if (berr || broke) f[F_STATUS] = 2.0;
+  if (berr) f[F_TIMEOUT] = 1.0;
 }
 
 template <int KT, class T>
@@ -669,15 +431,10 @@ __global__ void __launch_bounds__(kFusedBlock, 1024 / kFusedBlock) k_bicg_fused(
     else if (its >= maxit) done = 4;
   }
   if (ep.u != nullptr && done != 2) {
-    const double om = ep.omega;
     for (int64_t i = i0; i < iend; i += stride) {
       const double xi = (double)x[i];
       xout[i] = xi;
-      const double ui = ep.u[i] + om * xi;
-      ep.u[i] = ui;
-      const double uoi = ep.uo[i];
-      ep.a[i] = ui - uoi;
-      ep.s[i] = ui + uoi;
+      krylov_update(ep, i, xi);
     }
   } else {
     for (int64_t i = i0; i < iend; i += stride) xout[i] = (double)x[i];
@@ -686,9 +443,6 @@ __global__ void __launch_bounds__(kFusedBlock, 1024 / kFusedBlock) k_bicg_fused(
     sc[S_ATOL] = atol;
     sc[S_RTOL] = rtol;
     sc[S_MAXIT] = (double)maxit;
-    sc[S_FIRST] = 1.0;
-    sc[S_K_USED] = 0.0;
-    sc[S_CYCLE_DONE] = 0.0;
     sc[S_TOL] = tol;
     sc[S_N0] = n0;
     sc[S_NRES] = nres;
@@ -698,339 +452,382 @@ __global__ void __launch_bounds__(kFusedBlock, 1024 / kFusedBlock) k_bicg_fused(
     sc[S_RHO] = rho;
     sc[S_DONE] = *berr ? 2.0 : (double)done;
     sc[S_BERR] = *berr ? 1.0 : 0.0;
-    if (ep.fp_sc) {   // the fixed-point loop's count of this correction (the after-solve node's work)
-      double* f = ep.fp_sc;
-      f[F_CORR] += 1.0;
-      f[F_INNER] += (double)its;
-      f[F_KBODY] += (double)its;
-      if (*berr || done == 2) f[F_STATUS] = 2.0;
-      if (*berr) f[F_TIMEOUT] = 1.0;
-    }
+    krylov_count(ep, its, *berr != 0, done == 2);
   }
-}
-
-// arm a solver loop: condition = (solver still running)
-__global__ void k_cond_running(const double* __restrict__ sc, GraphCond cond) {
-  if (threadIdx.x == 0 && cond.use) cudaGraphSetConditional(cond.h, sc[S_DONE] == 0.0 ? 1u : 0u);
-}
-
-template <class T>
-__global__ void k_to_double(int64_t N, const T* __restrict__ x, double* __restrict__ y) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
-    y[i] = (double)x[i];
 }
 
 // ---- GMRES(m), right Jacobi preconditioning, classical Gram-Schmidt with one
-// re-orthogonalisation pass ----
-
-// w = rhs - B x (x = 0 on the first cycle) and ||w||; the last block runs the stop test
-// on this true residual and starts a cycle: g = (beta, 0, ...), invh = 1 / beta
-template <int KT, class T>
-__global__ void k_gm_residual(int64_t N, Offsets of, double* sc, const T* __restrict__ B, const T* __restrict__ x,
-                              const double* __restrict__ rhs, T* __restrict__ w, double* __restrict__ part,
-                              unsigned int* counter) {
-  if (flag_set(sc, S_DONE)) return;
-  const int K = KT > 0 ? KT : of.K;
-  const bool first = flag_set(sc, S_FIRST);
-  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  double acc[1] = {0.0};
-  if (i < N) {
-    T s = 0;
-    if (!first) {
-#pragma unroll
-      for (int k = 0; k < K; ++k) s = fma(B[k * N + i], x[i + of.o[k]], s);
-    }
-    const T wi = (T)rhs[i] - s;
-    w[i] = wi;
-    acc[0] = (double)(wi * wi);
-  }
-  double tot[1];
-  if (!last_block_sums<1>(acc, part, gridDim.x, counter, tot)) return;
-  if (threadIdx.x == 0) {
-    const double beta = sqrt(tot[0]);
-    if (first) {
-      sc[S_N0] = beta;
-      sc[S_TOL] = fmax(sc[S_ATOL], sc[S_RTOL] * beta);
-      sc[S_ITS] = 0.0;
-      sc[S_FIRST] = 0.0;
-      sc[S_CYCLES] = 0.0;
-    }
-    sc[S_CYCLES] += 1.0;
-    sc[S_NRES] = beta;
-    sc[S_BETA] = beta;
-    sc[S_K_USED] = 0.0;
-    sc[S_CYCLE_DONE] = 0.0;
-    if (!isfinite(beta)) sc[S_DONE] = 2.0;
-    else if (stop_test(beta, sc)) sc[S_DONE] = 1.0;
-    else if (sc[S_ITS] >= sc[S_MAXIT]) sc[S_DONE] = 4.0;
-    for (int q = 0; q <= kMaxRestart; ++q) sc[S_G + q] = 0.0;
-    sc[S_G] = beta;
-    sc[S_INVH] = 1.0 / beta;
-  }
-}
-
-// v_k = w * invh; z = D^{-1} v_k
-template <class T>
-__global__ void k_gm_normalize(int64_t N, const double* __restrict__ sc, const T* __restrict__ w, T* __restrict__ vk,
-                               const T* __restrict__ dinv, T* __restrict__ z) {
-  if (flag_set(sc, S_DONE) || flag_set(sc, S_CYCLE_DONE)) return;
-  __shared__ T ihs;   // one conversion per block instead of one per thread
-  if (threadIdx.x == 0) ihs = (T)sc[S_INVH];
-  __syncthreads();
-  const T ih = ihs;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
-    const T vi = w[i] * ih;
-    vk[i] = vi;
-    z[i] = dinv[i] * vi;
-  }
-}
-
-template <int KT, class T>
-__global__ void k_gm_spmv(int64_t N, Offsets of, const double* __restrict__ sc, const T* __restrict__ B,
-                          const T* __restrict__ z, T* __restrict__ w) {
-  if (flag_set(sc, S_DONE) || flag_set(sc, S_CYCLE_DONE)) return;
-  const int K = KT > 0 ? KT : of.K;
-  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= N) return;
-  T s = 0;
-#pragma unroll
-  for (int k = 0; k < K; ++k) s = fma(B[k * N + i], z[i + of.o[k]], s);
-  w[i] = s;
-}
-
-// Gram-Schmidt pass: optionally w -= sum_q h[q] V_q (h at sc + hslot), then the dots
-// (w, V_q), q <= k (pass 1, 2) or ||w|| (pass 3).  The last block stores the dots at
-// sc + outslot (passes 1, 2) or completes Hessenberg column k (pass 3): H[0..k][k] =
-// h1 + h2, H[k+1][k] = ||w||, earlier Givens rotations, a new rotation, the residual
-// estimate |g[k+1]|, the end-of-cycle test and invh = 1 / ||w||.
-// A thread owns elements and holds all k + 1 running dots in registers (QMAX is the
-// compile-time bound on k + 1, the loops over q are unrolled and predicated), so each
-// element's k + 1 basis values are independent loads in flight together.
+// re-orthogonalisation pass, as one persistent cooperative launch ----------------
 //
-// Three launches per Arnoldi step: (1) h1 = V^T w and ||w||^2; (2) w -= V h1 and
-// h2 = V^T w (the re-orthogonalisation); (3) w -= V h2, ||w||, and the Hessenberg
-// column.  The last block of (1) applies the DGKS test: if ||w - V h1|| >= ||w|| / sqrt(2)
-// (with ||w - V h1||^2 = ||w||^2 - ||h1||^2 for orthonormal V) little of w lay in the
-// basis, the second projection would change nothing worth keeping, and (2) takes the
-// role of (3) directly (h2 = 0) while (3) does nothing.
-template <class T, int QMAX>
-__global__ void __launch_bounds__(256) k_gm_orth(int64_t N, double* sc, int k, int m, int hslot, int outslot,
-                                                 T* __restrict__ w, const T* __restrict__ V, size_t vstride,
-                                                 double* __restrict__ part, int64_t pstride, unsigned int* counter) {
-  if (flag_set(sc, S_DONE) || flag_set(sc, S_CYCLE_DONE)) return;
-  const bool first = hslot < 0;                               // launch (1)
-  const bool no_reorth = !first && flag_set(sc, S_NO_REORTH);
-  if (no_reorth && outslot < 0) return;                       // launch (3) has nothing to do
-  const bool want_norm = outslot < 0 || no_reorth;
-  if (want_norm && no_reorth) outslot = -1;
-  __shared__ T hs[QMAX];
-  for (int q = threadIdx.x; q < QMAX; q += blockDim.x) hs[q] = (hslot >= 0 && q <= k) ? (T)sc[hslot + q] : (T)0;
-  __syncthreads();
-  // running sums in the vector type (a thread sees a handful of elements); widened to
-  // double for the sums across warps and blocks
-  T acc[QMAX];
+// A whole solve (all restart cycles) is one launch.  With a launch per pass the solve
+// was bound by launches: five per Arnoldi step (7 to 21 us each on P1 49^3 to 129^3
+// for 1 to 10 us of traffic), and a captured cycle ran all m = 20 steps although the
+// stationary solves stop after 5 to 10 of them (the rest returned at once, but were
+// launched).  Here a step is two grid-wide sums (barriers), and a solve stops where it
+// stops.  Measured on one GB300, whole stationary MC solves (omega = 0.5, inner rtol 1e-2),
+// before and after: Q1 27x21x33 in double 301 -> 89 ms, P1 49^3 mixed 470 -> 153 ms, P1
+// 129^3 mixed 1.70 -> 1.40 s; the same iteration counts.
+//
+// Layout.  Block b owns the contiguous rows [N b / G, N (b + 1) / G) for every pass, so
+// everything but the product's gather of z is local to a block:
+//  * w (the new direction) stays in shared memory between the passes of a step (in
+//    global memory where a block's rows do not fit);
+//  * the basis vectors are stored unnormalised with their scale 1 / ||v_q|| beside them
+//    (in `scale`), so no pass only normalises; z = D^{-1} v_k is the one vector other
+//    blocks read, written by the pass that completes v_k;
+//  * the dots go eight basis vectors at a time: eight running sums and eight loads in
+//    flight per thread, w re-read from shared memory, each basis vector read once.
+// Scalars.  A double operation by all warps of an SM costs 16 cycles per warp on the
+// FP64 pipe, so the Hessenberg column, Givens rotations and tests run in one warp (or
+// one thread) of every block, redundantly and in the same order: every block obtains
+// the same bits and takes the same branches without another barrier.
+//
+// Per Arnoldi step k (V holds v_0 .. v_k):
+//  (1) w = B z / ||v_k||, h1 = V^T w, ||w||^2                       -> grid sums
+//      DGKS test: if ||w - V h1||^2 = ||w||^2 - ||h1||^2 >= ||w||^2 / 2 little of w lay in
+//      the basis and a second projection would change nothing worth keeping;
+//      otherwise w -= V h1, h2 = V^T w                               -> grid sums
+//  (2) v_{k+1} = w - V h, z = D^{-1} v_{k+1}, ||v_{k+1}||^2          -> grid sum
+//      Hessenberg column, rotations, |g[k+1]|, the end-of-cycle test.
+constexpr int kGmMaxBlock = 1024;
+constexpr int kGmQ = kMaxRestart + 2;      // sums of one grid-wide reduction: k + 1 dots and a norm
+constexpr size_t kGmSmemW = 160 * 1024;    // shared memory for a block's w (the rest stays L1)
+
+struct GmArgs {
+  int64_t N;
+  double* sc;
+  const double* rhs;
+  double* xout;
+  size_t vstride;
+  double* part;
+  GridBar* bar;
+  double atol, rtol;
+  int maxit, m, w_in_smem;
+  KrylovEpilogue ep;
+  unsigned long long wait_ns;
+};
+
+// Totals over a warp of eight values per lane in nine adds (a butterfly that halves the
+// values with the lanes: 4 + 2 + 1 adds exchange, 2 more finish) instead of forty; lane l
+// returns the total of value (l >> 2): bits 4, 3, 2 of the lane are bits 2, 1, 0 of the value.
+template <class T>
+__device__ __forceinline__ T warp_sum8(T (&v)[8]) {
+  const int lane = threadIdx.x & 31;
+  const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
+  T a[4];
 #pragma unroll
-  for (int q = 0; q < QMAX; ++q) acc[q] = (T)0;
-  T nrm = (T)0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
-    T v[QMAX];
-#pragma unroll
-    for (int q = 0; q < QMAX; ++q) v[q] = q <= k ? V[q * vstride + i] : (T)0;
-    T wi = w[i];
-    if (hslot >= 0) {
-#pragma unroll
-      for (int q = 0; q < QMAX; ++q) wi -= hs[q] * v[q];
-      w[i] = wi;
-    }
-    if (want_norm) {
-      nrm = fma(wi, wi, nrm);
-    } else {
-#pragma unroll
-      for (int q = 0; q < QMAX; ++q)
-        if (q <= k) acc[q] = fma(wi, v[q], acc[q]);
-      if (first) nrm = fma(wi, wi, nrm);
-    }
+  for (int j = 0; j < 4; ++j) {
+    const T send = b4 ? v[j] : v[j + 4], keep = b4 ? v[j + 4] : v[j];
+    a[j] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
   }
-  // sums: the k + 1 dots (and ||w||^2 as sum k + 1 in launch (1)), or the norm alone
-  const int nq = want_norm ? 1 : (first ? k + 2 : k + 1);
-  if (want_norm) {
-    const double t = block_allsum(to_dbl(nrm));
-    if (threadIdx.x == 0) part[blockIdx.x] = t;
-  } else {
-    // a block's warp sums meet in the vector type (for the single-precision instance: no
-    // FP64 instruction per warp and sum) and are widened once per block
-    __shared__ T red[kBlock / 32][QMAX + 1];
-    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  T c[2];
 #pragma unroll
-    for (int q = 0; q < QMAX; ++q) {
-      if (q > k) break;
-      const T t = warp_sum(acc[q]);
-      if (lane == 0) red[wp][q] = t;
+  for (int j = 0; j < 2; ++j) {
+    const T send = b3 ? a[j] : a[j + 2], keep = b3 ? a[j + 2] : a[j];
+    c[j] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
+  }
+  const T send = b2 ? c[0] : c[1], keep = b2 ? c[1] : c[0];
+  T t = keep + __shfl_xor_sync(0xffffffffu, send, 4);
+  t += __shfl_xor_sync(0xffffffffu, t, 2);
+  t += __shfl_xor_sync(0xffffffffu, t, 1);
+  return t;
+}
+
+// Scalars of a solve, one copy per block.  `red` holds the warps' sums, `tot` the grid's.
+template <class T>
+struct GmShared {
+  T red[kGmMaxBlock / 32][kGmQ + 6];   // rows padded to 8 x 5 values
+  T hs[kMaxRestart];                   // coefficients of the pass at hand, in the vector type
+  T invh;                              // 1 / ||v_k||
+  double tot[kGmQ];
+  double scale[kMaxRestart + 1];       // 1 / ||v_q||
+  double h1[kMaxRestart], h2[kMaxRestart];
+  double cs[kMaxRestart], sn[kMaxRestart], g[kMaxRestart + 1], y[kMaxRestart];
+  double H[kMaxRestart][kMaxRestart];  // H[row][col], upper triangle after the rotations
+  double nres, n0, tol;
+  int its, cycles, done, cycle_done, skip;
+};
+
+// Grid-wide totals of the block's nq sums (sh.red, one row per warp) in sh.tot.  Every
+// block adds the partials of all blocks in block order, so all obtain the same bits.
+// The partials alternate between two buffers, as in grid_sums_begin.  Ends with warp 0
+// holding the totals of the values it summed; the caller synchronises the block.
+template <class T>
+__device__ __forceinline__ void gm_grid_sums(GmShared<T>& sh, int nq, const GmArgs& a, int& buf) {
+  const int G = gridDim.x;
+  const int nwarp = blockDim.x >> 5, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double* pb = a.part + (size_t)buf * kGmQ * G;
+  buf ^= 1;
+  __syncthreads();   // sh.red is complete
+  if ((int)threadIdx.x < nq) {
+    T s0 = 0, s1 = 0, s2 = 0, s3 = 0;   // four chains: the adds of one are serial
+    int u = 0;
+    for (; u + 3 < nwarp; u += 4) {
+      s0 += sh.red[u][threadIdx.x];
+      s1 += sh.red[u + 1][threadIdx.x];
+      s2 += sh.red[u + 2][threadIdx.x];
+      s3 += sh.red[u + 3][threadIdx.x];
     }
-    if (first) {
-      const T t = warp_sum(nrm);
-      if (lane == 0) red[wp][k + 1] = t;
+    for (; u < nwarp; ++u) s0 += sh.red[u][threadIdx.x];
+    pb[(size_t)threadIdx.x * G + blockIdx.x] = to_dbl((s0 + s1) + (s2 + s3));
+  }
+  const unsigned int old = grid_arrive(a.bar);
+  grid_wait(a.bar, old, a.wait_ns);
+  for (int q = w; q < nq; q += nwarp) {
+    double t = 0.0;
+    for (int b0 = lane; b0 < G; b0 += 256) {
+      double x[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) x[u] = b0 + 32 * u < G ? __ldcg(pb + (size_t)q * G + b0 + 32 * u) : 0.0;
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (b0 - lane + 32 * u < G) t += x[u];
+    }
+    t = warp_sum(t);
+    if (lane == 0) sh.tot[q] = t;
+  }
+}
+
+// The warps' sums of one value per thread, as value q of sh.red.
+template <class T>
+__device__ __forceinline__ void gm_put(GmShared<T>& sh, T v, int q) {
+  v = warp_sum(v);
+  if ((threadIdx.x & 31) == 0) sh.red[threadIdx.x >> 5][q] = v;
+}
+
+// The warps' dots (w, v_q), q <= k, as values 0 .. k of sh.red.
+template <class T>
+__device__ __forceinline__ void gm_dots(GmShared<T>& sh, const T* w, const T* V, size_t vs, int64_t i0, int nrow,
+                                        int k) {
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  for (int q0 = 0; q0 <= k; q0 += 8) {
+    T acc[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) acc[j] = (T)0;
+    const T* Vq = V + (size_t)q0 * vs + i0;
+#pragma unroll 2
+    for (int r = threadIdx.x; r < nrow; r += blockDim.x) {
+      T v[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) v[j] = q0 + j <= k ? Vq[(size_t)j * vs + r] : (T)0;
+      const T wi = w[r];
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (q0 + j <= k) acc[j] = fma(wi, v[j], acc[j]);
+    }
+    const T t = warp_sum8(acc);
+    if ((lane & 3) == 0) sh.red[wp][q0 + (lane >> 2)] = t;
+  }
+}
+
+// w_r - sum_q hs[q] v_q[r], q <= k.
+template <class T>
+__device__ __forceinline__ T gm_project(const GmShared<T>& sh, T wi, const T* V, size_t vs, int64_t i, int k) {
+  for (int q0 = 0; q0 <= k; q0 += 8) {
+    T v[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] = q0 + j <= k ? V[(size_t)(q0 + j) * vs + i] : (T)0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      if (q0 + j <= k) wi -= sh.hs[q0 + j] * v[j];
+  }
+  return wi;
+}
+
+// Column k of the Hessenberg matrix (one thread): earlier rotations, a new one, the
+// residual estimate and the end-of-cycle test.
+template <class T>
+__device__ void gm_column(GmShared<T>& sh, int k, const GmArgs& a, bool berr) {
+  const double hk1 = sqrt(sh.tot[0]);
+  double c = sh.h1[0] + sh.h2[0];   // the column's running entry
+  for (int q = 0; q < k; ++q) {
+    const double b = sh.h1[q + 1] + sh.h2[q + 1];
+    sh.H[q][k] = sh.cs[q] * c + sh.sn[q] * b;
+    c = -sh.sn[q] * c + sh.cs[q] * b;
+  }
+  const double den = hypot(c, hk1);
+  sh.cs[k] = c / den;
+  sh.sn[k] = hk1 / den;
+  sh.H[k][k] = den;
+  const double gk = sh.g[k], gn = -sh.sn[k] * gk;
+  sh.g[k + 1] = gn;
+  sh.g[k] = sh.cs[k] * gk;
+  sh.its += 1;
+  sh.nres = fabs(gn);
+  sh.scale[k + 1] = 1.0 / hk1;
+  sh.invh = (T)sh.scale[k + 1];
+  if (!isfinite(den) || den == 0.0 || berr) sh.done = 2;
+  else if (fabs(gn) < sh.tol || sh.its >= a.maxit || k + 1 == a.m || hk1 == 0.0) sh.cycle_done = 1;
+}
+
+template <int KT, class T>
+__global__ void __launch_bounds__(kGmMaxBlock, 1) k_gm_fused(Offsets of, const T* __restrict__ B,
+                                                             const T* __restrict__ dinv, T* x, T* z, T* wg, T* V,
+                                                             GmArgs a) {
+  const int K = KT > 0 ? KT : of.K;
+  const int64_t N = a.N, G = gridDim.x;
+  const int64_t i0 = N * blockIdx.x / G;
+  const int nrow = (int)(N * (blockIdx.x + 1) / G - i0), nt = blockDim.x;
+  const size_t vs = a.vstride;
+  __shared__ GmShared<T> sh;
+  extern __shared__ char dyn[];
+  T* w = a.w_in_smem ? reinterpret_cast<T*>(dyn) : wg + i0;
+  volatile int* berr = &a.bar->err;
+  int buf = 0;
+  if (threadIdx.x == 0) {
+    sh.its = 0;
+    sh.cycles = 0;
+    sh.done = 0;
+  }
+  bool have_x = false;   // x = 0 until the first cycle's update
+  for (;;) {
+    // true residual v_0 = rhs - B x, z = D^{-1} v_0, ||v_0||
+    T nrm = 0;
+    for (int r = threadIdx.x; r < nrow; r += nt) {
+      const int64_t i = i0 + r;
+      T s = 0;
+      if (have_x) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) s = fma(B[k * N + i], x[i + of.o[k]], s);
+      }
+      const T wi = (T)a.rhs[i] - s;
+      V[i] = wi;
+      z[i] = dinv[i] * wi;
+      nrm = fma(wi, wi, nrm);
+    }
+    gm_put(sh, nrm, 0);
+    gm_grid_sums(sh, 1, a, buf);
+    if (threadIdx.x == 0) {
+      const double beta = sqrt(sh.tot[0]);
+      if (!have_x) {
+        sh.n0 = beta;
+        sh.tol = fmax(a.atol, a.rtol * beta);
+      }
+      sh.cycles += 1;
+      sh.nres = beta;
+      sh.cycle_done = 0;
+      if (!isfinite(beta) || *berr) sh.done = 2;
+      else if (beta < sh.tol) sh.done = 1;
+      else if (sh.its >= a.maxit) sh.done = 4;
+      sh.g[0] = beta;
+      sh.scale[0] = 1.0 / beta;
+      sh.invh = (T)sh.scale[0];
     }
     __syncthreads();
-    for (int q = threadIdx.x; q < nq; q += blockDim.x) {
-      T s = 0;
-      for (int u = 0; u < (int)(blockDim.x >> 5); ++u) s += red[u][q];
-      part[q * pstride + blockIdx.x] = to_dbl(s);
-    }
-  }
-  __threadfence();   // every thread that wrote a partial makes it visible before the count
-  __syncthreads();
-  __shared__ bool am_last;
-  if (threadIdx.x == 0) {
-    __threadfence();
-    am_last = atomicAdd(counter, 1u) == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (!am_last) return;
-  __threadfence();
-  // totals of the nq sums: warp q' takes q = q', q' + 8, ... (block order, fixed)
-  __shared__ double tot[QMAX + 1];
-  {
-    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-    // lane l adds partials l, l + 32, ... in turn, the loads eight at a time
-    const int n = gridDim.x;
-    for (int q = wp; q < nq; q += nwarp) {
-      double s = 0.0;
-      for (int b0 = lane; b0 < n; b0 += 256) {
-        double x[8];
+    if (sh.done != 0) break;
+    int ku = 0;   // columns of this cycle
+    for (int k = 0;; ++k) {
+      // (1) w = B z / ||v_k||, dots with v_0 .. v_k, ||w||^2
+      const T ih = sh.invh;
+      nrm = 0;
+      for (int r = threadIdx.x; r < nrow; r += nt) {
+        const int64_t i = i0 + r;
+        T s = 0;
 #pragma unroll
-        for (int u = 0; u < 8; ++u) x[u] = b0 + 32 * u < n ? __ldcg(part + q * pstride + b0 + 32 * u) : 0.0;
-#pragma unroll
-        for (int u = 0; u < 8; ++u) s += x[u];
+        for (int q = 0; q < K; ++q) s = fma(B[q * N + i], z[i + of.o[q]], s);
+        s *= ih;
+        w[r] = s;
+        nrm = fma(s, s, nrm);
       }
-      s = warp_sum(s);
-      if (lane == 0) tot[q] = s;
+      gm_dots(sh, w, V, vs, i0, nrow, k);
+      gm_put(sh, nrm, k + 1);
+      gm_grid_sums(sh, k + 2, a, buf);
+      __syncthreads();
+      if (threadIdx.x < 32) {
+        const int q = threadIdx.x;
+        double h = 0.0;
+        if (q <= k) {
+          h = sh.tot[q] * sh.scale[q];
+          sh.h1[q] = h;
+          sh.h2[q] = 0.0;
+          sh.hs[q] = (T)(h * sh.scale[q]);
+        }
+        const double proj = warp_sum(h * h);
+        const double ww = sh.tot[k + 1];
+        if (q == 0) sh.skip = ww - proj >= 0.5 * ww && ww > 0.0;
+      }
+      __syncthreads();
+      if (!sh.skip) {   // second projection: w -= V h1, h2 = V^T w
+        for (int r = threadIdx.x; r < nrow; r += nt) w[r] = gm_project(sh, w[r], V, vs, i0 + r, k);
+        gm_dots(sh, w, V, vs, i0, nrow, k);
+        gm_grid_sums(sh, k + 1, a, buf);
+        __syncthreads();
+        if ((int)threadIdx.x <= k) {
+          const double h = sh.tot[threadIdx.x] * sh.scale[threadIdx.x];
+          sh.h2[threadIdx.x] = h;
+          sh.hs[threadIdx.x] = (T)(h * sh.scale[threadIdx.x]);
+        }
+        __syncthreads();
+      }
+      // (2) v_{k+1} = w - V h, z = D^{-1} v_{k+1}, ||v_{k+1}||^2
+      nrm = 0;
+      T* vn = V + (size_t)(k + 1) * vs;
+#pragma unroll 2
+      for (int r = threadIdx.x; r < nrow; r += nt) {
+        const int64_t i = i0 + r;
+        const T wi = gm_project(sh, w[r], V, vs, i, k);
+        vn[i] = wi;
+        z[i] = dinv[i] * wi;
+        nrm = fma(wi, wi, nrm);
+      }
+      gm_put(sh, nrm, 0);
+      gm_grid_sums(sh, 1, a, buf);
+      if (threadIdx.x == 0) gm_column(sh, k, a, *berr != 0);
+      __syncthreads();
+      ku = k + 1;
+      if (sh.done != 0 || sh.cycle_done != 0) break;
     }
-  }
-  __syncthreads();
-  if (threadIdx.x != 0) return;
-  *counter = 0u;
-  if (!want_norm) {
-    for (int q = 0; q <= k; ++q) sc[outslot + q] = tot[q];
-    if (first) {   // DGKS test: re-orthogonalise only if ||w - V h1||^2 < ||w||^2 / 2
-      double proj = 0.0;
-      for (int q = 0; q <= k; ++q) proj += tot[q] * tot[q];
-      const double ww = tot[k + 1], rest = ww - proj;
-      const bool skip = rest >= 0.5 * ww && ww > 0.0;
-      sc[S_NO_REORTH] = skip ? 1.0 : 0.0;
-      if (skip)
-        for (int q = 0; q <= k; ++q) sc[S_H2 + q] = 0.0;
+    if (sh.done != 0) break;
+    // H y = g (columns from the last; lane c keeps g[c]), then x += D^{-1} sum_q y_q v_q / ||v_q||
+    if (threadIdx.x < 32) {
+      const int c = threadIdx.x;
+      double gc = c < ku ? sh.g[c] : 0.0;
+      const double inv = c < ku ? 1.0 / sh.H[c][c] : 0.0;
+      for (int q = ku - 1; q >= 0; --q) {
+        const double yq = __shfl_sync(0xffffffffu, gc * inv, q);
+        if (c == q) sh.y[q] = yq;
+        if (c < q) gc = fma(-sh.H[c][q], yq, gc);
+      }
+      __syncwarp();
+      if (c < ku) sh.hs[c] = (T)(sh.y[c] * sh.scale[c]);
     }
-    return;
-  }
-  const double hk1 = sqrt(tot[0]);
-  double* H = sc + S_HCOL;   // H[row * kMaxRestart + col]
-  for (int q = 0; q <= k; ++q) H[q * kMaxRestart + k] = sc[S_H1 + q] + sc[S_H2 + q];
-  H[(k + 1) * kMaxRestart + k] = hk1;
-  double* cs = sc + S_CS;
-  double* sn = sc + S_SN;
-  double* g = sc + S_G;
-  for (int q = 0; q < k; ++q) {
-    const double a = H[q * kMaxRestart + k], b = H[(q + 1) * kMaxRestart + k];
-    H[q * kMaxRestart + k] = cs[q] * a + sn[q] * b;
-    H[(q + 1) * kMaxRestart + k] = -sn[q] * a + cs[q] * b;
-  }
-  const double a = H[k * kMaxRestart + k], b = H[(k + 1) * kMaxRestart + k];
-  const double den = hypot(a, b);
-  cs[k] = a / den;
-  sn[k] = b / den;
-  H[k * kMaxRestart + k] = den;
-  H[(k + 1) * kMaxRestart + k] = 0.0;
-  g[k + 1] = -sn[k] * g[k];
-  g[k] = cs[k] * g[k];
-  sc[S_ITS] += 1.0;
-  sc[S_K_USED] = (double)(k + 1);
-  sc[S_NRES] = fabs(g[k + 1]);
-  sc[S_INVH] = 1.0 / hk1;
-  if (!isfinite(den) || den == 0.0) { sc[S_DONE] = 2.0; return; }
-  if (stop_test(fabs(g[k + 1]), sc) || sc[S_ITS] >= sc[S_MAXIT] || k + 1 == m || hk1 == 0.0) sc[S_CYCLE_DONE] = 1.0;
-}
-
-// Launch a Gram-Schmidt pass with the smallest register footprint that holds k + 1 dots,
-// on as many blocks as are resident at once (one wave), at most G.
-template <class T, int Q>
-int orth_grid(int G) {
-  static const int nb = [] {
-    int b = 0, dev = 0, nsm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_gm_orth<T, Q>, kBlock, 0) != cudaSuccess) {
-      cudaGetLastError();
-      b = 0;
+    __syncthreads();
+    for (int r = threadIdx.x; r < nrow; r += nt) {
+      const int64_t i = i0 + r;
+      T s = 0;
+      for (int q0 = 0; q0 < ku; q0 += 8) {
+        T v[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = q0 + j < ku ? V[(size_t)(q0 + j) * vs + i] : (T)0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          if (q0 + j < ku) s = fma(sh.hs[q0 + j], v[j], s);
+      }
+      const T d = dinv[i] * s;
+      x[i] = have_x ? x[i] + d : d;
     }
-    return b * nsm;
-  }();
-  return nb > 0 ? std::min(G, nb) : G;
-}
-
-template <class T>
-void orth_launch(afc_problem_s* p, int G, int64_t N, double* sc, int k, int m, int hslot, int outslot, T* w,
-                 const T* V, size_t vs, double* part, int64_t pst, unsigned int* cnt) {
-  cudaStream_t s = p->stream;
-#define AFC_ORTH(Q) AFC_LAUNCH(p, "k_gm_orth", k_gm_orth<T, Q><<<orth_grid<T, Q>(G), kBlock, 0, s>>>(N, sc, k, m, hslot, outslot, w, V, vs, part, pst, cnt))
-  if (k + 1 <= 4) AFC_ORTH(4);
-  else if (k + 1 <= 8) AFC_ORTH(8);
-  else if (k + 1 <= 12) AFC_ORTH(12);
-  else if (k + 1 <= 16) AFC_ORTH(16);
-  else if (k + 1 <= 20) AFC_ORTH(20);
-  else if (k + 1 <= 24) AFC_ORTH(24);
-  else AFC_ORTH(32);
-#undef AFC_ORTH
-}
-
-// back substitution H y = g for the k_used leading columns, then x += D^{-1} sum_q y_q V_q
-// (every block solves the small triangular system itself)
-template <class T>
-__global__ void k_gm_update(int64_t N, const double* __restrict__ sc, T* __restrict__ x, const T* __restrict__ V,
-                            size_t vstride, const T* __restrict__ dinv, GraphCond cond) {
-  // another restart cycle only while the solve is running (set before any early return)
-  if (cond.use && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(cond.h, sc[S_DONE] == 0.0 ? 1u : 0u);
-  if (sc[S_DONE] == 2.0) return;
-  const int ku = (int)sc[S_K_USED];
-  if (ku == 0) return;
-  __shared__ double ys[kMaxRestart];
-  __shared__ T yt[kMaxRestart];
-  // the leading ku x ku block of H and g, staged by the whole block (one round of loads
-  // instead of one dependent load per entry for the thread that solves)
-  __shared__ double hs[kMaxRestart * kMaxRestart];
-  __shared__ double gs[kMaxRestart];
-  for (int e = threadIdx.x; e < ku * ku; e += blockDim.x) {
-    const int q = e / ku, c = e - q * ku;
-    hs[q * kMaxRestart + c] = sc[S_HCOL + q * kMaxRestart + c];
+    have_x = true;
+    grid_barrier(a.bar, a.wait_ns);   // the next residual gathers x
   }
-  for (int q = threadIdx.x; q < ku; q += blockDim.x) gs[q] = sc[S_G + q];
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int q = ku - 1; q >= 0; --q) {
-      double s = gs[q];
-      for (int c = q + 1; c < ku; ++c) s -= hs[q * kMaxRestart + c] * ys[c];
-      ys[q] = s / hs[q * kMaxRestart + q];
-    }
-    for (int q = 0; q < ku; ++q) yt[q] = (T)ys[q];
+  // the solution, and the caller's update unless the solve broke down
+  const bool upd = a.ep.u != nullptr && sh.done != 2;
+  for (int r = threadIdx.x; r < nrow; r += nt) {
+    const int64_t i = i0 + r;
+    const double xi = have_x ? (double)x[i] : 0.0;
+    a.xout[i] = xi;
+    if (upd) krylov_update(a.ep, i, xi);
   }
-  __syncthreads();
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
-    T s = 0;
-    for (int q = 0; q < ku; ++q) s = fma(yt[q], V[q * vstride + i], s);
-    x[i] = x[i] + dinv[i] * s;
-  }
-}
-
-__global__ void k_solver_reset(double* sc, double atol, double rtol, int maxit) {
-  if (threadIdx.x == 0) {
-    sc[S_DONE] = 0.0;
-    sc[S_BERR] = 0.0;
-    sc[S_FIRST] = 1.0;
-    sc[S_K_USED] = 0.0;
-    sc[S_CYCLE_DONE] = 0.0;
-    sc[S_ATOL] = atol;
-    sc[S_RTOL] = rtol;
-    sc[S_MAXIT] = (double)maxit;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    double* sc = a.sc;
+    sc[S_N0] = sh.n0;
+    sc[S_TOL] = sh.tol;
+    sc[S_NRES] = sh.nres;
+    sc[S_BETA] = sh.nres;
+    sc[S_ITS] = (double)sh.its;
+    sc[S_CYCLES] = (double)sh.cycles;
+    sc[S_DONE] = *berr ? 2.0 : (double)sh.done;
+    sc[S_BERR] = *berr ? 1.0 : 0.0;
+    krylov_count(a.ep, sh.its, *berr != 0, sh.done == 2);
   }
 }
 
@@ -1041,7 +838,6 @@ void krylov_free(afc_problem_s* p) {
   p->kw->vec.free_();
   p->kw->sc.free_();
   p->kw->part.free_();
-  p->kw->counter.free_();
   if (p->kw->hsc) cudaFreeHost(p->kw->hsc);
   delete p->kw;
   p->kw = nullptr;
@@ -1069,7 +865,6 @@ int ensure_work(afc_problem_s* p, int nvec, bool fp32) {
   if (!w.sc.base) {
     int st = w.sc.alloc(S_END + 8);
     if (st) return st;
-    if ((st = w.counter.alloc(4))) return st;
     if ((st = w.barrier.alloc(4))) return st;
     if (cudaMallocHost((void**)&w.hsc, (S_END + 8) * sizeof(double)) != cudaSuccess) {
       set_error("cudaMallocHost failed");
@@ -1089,27 +884,29 @@ T* vec_at(KrylovWork& w, int q) {
   return reinterpret_cast<T*>(w.vec.base) + q * w.vstride + w.pad;
 }
 
-// The persistent BiCGStab launch on stream s (no synchronisation); *ok = false when
-// the device cannot run cooperative launches (the caller then takes the
-// kernel-per-phase path).
+// The device must run cooperative launches (GB300 does); its SM count, asked once.
+int coop_device(afc_problem_s* p) {
+  KrylovWork& w = *p->kw;
+  if (w.nsm > 0) return AFC_OK;
+  int c = 0;
+  AFC_CUDA(cudaDeviceGetAttribute(&c, cudaDevAttrCooperativeLaunch, p->device));
+  if (!c) { set_error("the Krylov solvers need a device with cooperative launches"); return AFC_E_CUDA; }
+  AFC_CUDA(cudaDeviceGetAttribute(&w.nsm, cudaDevAttrMultiProcessorCount, p->device));
+  return AFC_OK;
+}
+
+// The persistent BiCGStab launch on stream s (no synchronisation).
 template <class T>
 int bicg_fused_launch(afc_problem_s* p, cudaStream_t s, const T* B, const T* dinv, const afc_opts* o,
-                      const double* rhs, double* xout, bool* ok, const KrylovEpilogue* epi) {
+                      const double* rhs, double* xout, const KrylovEpilogue* epi) {
   KrylovWork& w = *p->kw;
-  if (w.coop < 0) {
-    int c = 0;
-    AFC_CUDA(cudaDeviceGetAttribute(&c, cudaDevAttrCooperativeLaunch, p->device));
-    AFC_CUDA(cudaDeviceGetAttribute(&w.nsm, cudaDevAttrMultiProcessorCount, p->device));
-    w.coop = c;
-  }
-  *ok = w.coop > 0;
-  if (!*ok) return AFC_OK;
+  int st = coop_device(p);
+  if (st) return st;
   const int64_t N = p->N;
   T *x = vec_at<T>(w, 0), *r = vec_at<T>(w, 1), *rh = vec_at<T>(w, 2), *pp = vec_at<T>(w, 3), *v = vec_at<T>(w, 4),
     *sv = vec_at<T>(w, 5), *t = vec_at<T>(w, 6), *ph = vec_at<T>(w, 7), *sh = vec_at<T>(w, 8);
   double* sc = w.sc.p;
   GridBar* bar = reinterpret_cast<GridBar*>(w.barrier.p);
-  int st = AFC_OK;
   with_K(p->K, [&](auto kc) {
     constexpr int KT = decltype(kc)::value;
     int nb = 0;
@@ -1139,126 +936,109 @@ int bicg_fused_launch(afc_problem_s* p, cudaStream_t s, const T* B, const T* din
   return st;
 }
 
-template <class T>
-int bicgstab_impl(afc_problem_s* p, const T* B, const T* dinv, const afc_opts* o, const double* rhs, double* xout,
-                  int* its, double* res, const KrylovEpilogue* epi, bool* epi_done) {
-  int st = ensure_work(p, 9, sizeof(T) == 4);
-  if (st) return st;
+// Host side of a persistent solve just launched: its scalars and status.
+int fused_result(afc_problem_s* p, const char* what, int* its, double* res) {
   KrylovWork& w = *p->kw;
-  const int64_t N = p->N;
   cudaStream_t s = p->stream;
-  T *x = vec_at<T>(w, 0), *r = vec_at<T>(w, 1), *rh = vec_at<T>(w, 2), *pp = vec_at<T>(w, 3), *v = vec_at<T>(w, 4),
-    *sv = vec_at<T>(w, 5), *t = vec_at<T>(w, 6), *ph = vec_at<T>(w, 7), *sh = vec_at<T>(w, 8);
-  double* sc = w.sc.p;
-  double* part = w.part.p;
-  unsigned int* cnt = w.counter.p;
-  const int G = kRedBlocks;
-  const int64_t gr = grid_for(N);
-  bool fused = false;
-  if ((st = bicg_fused_launch<T>(p, s, B, dinv, o, rhs, xout, &fused, epi))) return st;
-  if (epi_done) *epi_done = fused && epi != nullptr;
-  if (fused) {
-    AFC_CUDA(cudaMemcpyAsync(w.hsc, sc, (S_MAXIT + 1) * sizeof(double), cudaMemcpyDeviceToHost, s));
-    unsigned int* hbar = reinterpret_cast<unsigned int*>(w.hsc + S_END);
-    AFC_CUDA(cudaMemcpyAsync(hbar, w.barrier.p, 4 * sizeof(unsigned int), cudaMemcpyDeviceToHost, s));
-    AFC_CUDA(cudaStreamSynchronize(s));
-    if (its) *its = (int)w.hsc[S_ITS];
-    if (res) *res = w.hsc[S_NRES];
-    if (hbar[2] != 0u) {
-      AFC_CUDA(cudaMemsetAsync(w.barrier.p, 0, 4 * sizeof(unsigned int), s));
-      AFC_CUDA(cudaStreamSynchronize(s));
-      set_error("a grid barrier of the BiCGStab launch gave up waiting");
-      return AFC_E_TIMEOUT;
-    }
-    const double done = w.hsc[S_DONE];
-    if (done == 2.0) { set_error("BiCGStab breakdown or non-finite value"); return AFC_E_NAN; }
-    return done == 1.0 ? AFC_OK : AFC_NOT_CONVERGED;
-  }
-  AFC_LAUNCH(p, "k_solver_reset", k_solver_reset<<<1, 32, 0, s>>>(sc, o->ksp_atol, o->ksp_rtol, o->ksp_maxit));
-  AFC_LAUNCH(p, "k_bicg_init", k_bicg_init<T><<<G, kBlock, 0, s>>>(N, rhs, x, r, rh, pp, v, part, cnt, sc));
-  AFC_CUDA(cudaGetLastError());
-  int chunk = 2;
-  int launched = 0;
-  for (;;) {
-    AFC_CUDA(cudaMemcpyAsync(w.hsc, sc, (S_MAXIT + 1) * sizeof(double), cudaMemcpyDeviceToHost, s));
-    AFC_CUDA(cudaStreamSynchronize(s));
-    if (w.hsc[S_DONE] != 0.0 || launched >= o->ksp_maxit) break;
-    with_K(p->K, [&](auto kc) {
-      constexpr int KT = decltype(kc)::value;
-      for (int c = 0; c < chunk && launched < o->ksp_maxit; ++c, ++launched) {
-        AFC_LAUNCH(p, "k_bicg_p", k_bicg_p<T><<<G, kBlock, 0, s>>>(N, sc, r, pp, v, dinv, ph));
-        AFC_LAUNCH(p, "k_bicg_spmv1",
-                   k_bicg_spmv1<KT, T><<<gr, kBlock, 0, s>>>(N, p->offs, sc, B, ph, v, rh, part, cnt));
-        AFC_LAUNCH(p, "k_bicg_s", k_bicg_s<T><<<G, kBlock, 0, s>>>(N, sc, r, v, dinv, sv, sh, part, cnt));
-        AFC_LAUNCH(p, "k_bicg_spmv2",
-                   k_bicg_spmv2<KT, T><<<gr, kBlock, 0, s>>>(N, p->offs, sc, B, sh, t, sv, x, ph, part, cnt));
-        AFC_LAUNCH(p, "k_bicg_xr", k_bicg_xr<T><<<G, kBlock, 0, s>>>(N, sc, x, ph, sh, sv, t, r, rh, part, cnt,
-                                                                     GraphCond{}));
-      }
-    });
-    AFC_CUDA(cudaGetLastError());
-    chunk = std::min(chunk * 2, 16);
-  }
-  AFC_LAUNCH(p, "k_to_double", k_to_double<T><<<G, kBlock, 0, s>>>(N, x, xout));
-  AFC_CUDA(cudaGetLastError());
+  AFC_CUDA(cudaMemcpyAsync(w.hsc, w.sc.p, S_END * sizeof(double), cudaMemcpyDeviceToHost, s));
+  unsigned int* hbar = reinterpret_cast<unsigned int*>(w.hsc + S_END);
+  AFC_CUDA(cudaMemcpyAsync(hbar, w.barrier.p, 4 * sizeof(unsigned int), cudaMemcpyDeviceToHost, s));
+  AFC_CUDA(cudaStreamSynchronize(s));
   if (its) *its = (int)w.hsc[S_ITS];
   if (res) *res = w.hsc[S_NRES];
+  if (hbar[2] != 0u) {
+    const int st = krylov_reset_barrier(p);
+    if (st) return st;
+    set_error(std::string("a grid barrier of the ") + what + " launch gave up waiting");
+    return AFC_E_TIMEOUT;
+  }
   const double done = w.hsc[S_DONE];
-  if (done == 2.0) { set_error("BiCGStab breakdown or non-finite value"); return AFC_E_NAN; }
+  if (done == 2.0) { set_error(std::string(what) + " breakdown or non-finite value"); return AFC_E_NAN; }
   return done == 1.0 ? AFC_OK : AFC_NOT_CONVERGED;
 }
 
 template <class T>
-int gmres_impl(afc_problem_s* p, const T* B, const T* dinv, const afc_opts* o, const double* rhs, double* xout,
-               int* its, double* res) {
+int bicgstab_impl(afc_problem_s* p, const T* B, const T* dinv, const afc_opts* o, const double* rhs, double* xout,
+                  int* its, double* res, const KrylovEpilogue* epi) {
+  int st = ensure_work(p, 9, sizeof(T) == 4);
+  if (st) return st;
+  if ((st = bicg_fused_launch<T>(p, p->stream, B, dinv, o, rhs, xout, epi))) return st;
+  return fused_result(p, "BiCGStab", its, res);
+}
+
+// The persistent GMRES launch on stream s (no synchronisation).  One block per SM at
+// most, of as many warps as its rows fill (64 to 1024 threads): small systems spread
+// over all SMs with few warps each, because a block's FP64 sums cost 16 cycles per warp,
+// and leave room for the launches of other streams.
+template <class T>
+int gmres_fused_launch(afc_problem_s* p, cudaStream_t s, const T* B, const T* dinv, const afc_opts* o,
+                       const double* rhs, double* xout, const KrylovEpilogue* epi) {
+  KrylovWork& w = *p->kw;
+  int st = coop_device(p);
+  if (st) return st;
+  const int64_t N = p->N;
+  GmArgs a;
+  a.N = N;
+  a.sc = w.sc.p;
+  a.rhs = rhs;
+  a.xout = xout;
+  a.vstride = w.vstride;
+  a.part = w.part.p;
+  a.bar = reinterpret_cast<GridBar*>(w.barrier.p);
+  a.atol = o->ksp_atol;
+  a.rtol = o->ksp_rtol;
+  a.maxit = o->ksp_maxit;
+  a.m = o->gmres_restart;
+  if (epi) a.ep = *epi;
+  a.wait_ns = p->grid_wait_ns;
+  const int G = (int)std::max<int64_t>(1, std::min<int64_t>((N + 63) / 64, w.nsm));
+  const int64_t rows = (N + G - 1) / G;
+  const int block = (int)std::max<int64_t>(64, std::min<int64_t>(kGmMaxBlock, (rows + 31) / 32 * 32));
+  size_t smem = (size_t)rows * sizeof(T);
+  a.w_in_smem = smem <= kGmSmemW;
+  if (!a.w_in_smem) smem = 0;
+  with_K(p->K, [&](auto kc) {
+    constexpr int KT = decltype(kc)::value;
+    auto kern = k_gm_fused<KT, T>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGmSmemW);
+    int nb = 0;
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, block, smem);
+    if (e != cudaSuccess || nb < 1) {
+      st = cuda_fail(e != cudaSuccess ? e : cudaErrorInvalidConfiguration, "occupancy of k_gm_fused");
+      return;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)G);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaEvent_t ev = prof_start(p);
+    e = cudaLaunchKernelEx(&cfg, kern, p->offs, B, dinv, vec_at<T>(w, 0), vec_at<T>(w, 1), vec_at<T>(w, 2),
+                           vec_at<T>(w, 3), a);
+    prof_stop(p, "k_gm_fused", ev);
+    if (e != cudaSuccess) st = cuda_fail(e, "cudaLaunchKernelEx(k_gm_fused)");
+  });
+  return st;
+}
+
+int gmres_work(afc_problem_s* p, const afc_opts* o, bool fp32) {
   const int m = o->gmres_restart;
   if (m < 1 || m > kMaxRestart) { set_error("gmres_restart must be in 1..32"); return AFC_E_INVALID; }
-  // vectors: x, w, z, V_0..V_m
-  int st = ensure_work(p, 3 + m + 1, sizeof(T) == 4);
+  return ensure_work(p, 3 + m + 1, fp32);   // x, z, w, V_0 .. V_m
+}
+
+template <class T>
+int gmres_impl(afc_problem_s* p, const T* B, const T* dinv, const afc_opts* o, const double* rhs, double* xout,
+               int* its, double* res, const KrylovEpilogue* epi) {
+  int st = gmres_work(p, o, sizeof(T) == 4);
   if (st) return st;
-  KrylovWork& w = *p->kw;
-  const int64_t N = p->N;
-  cudaStream_t s = p->stream;
-  T *x = vec_at<T>(w, 0), *wv = vec_at<T>(w, 1), *z = vec_at<T>(w, 2), *V = vec_at<T>(w, 3);
-  const size_t vs = w.vstride;
-  double* sc = w.sc.p;
-  double* part = w.part.p;
-  unsigned int* cnt = w.counter.p;
-  const int G = kRedBlocks;
-  const int64_t gr = grid_for(N);
-  AFC_CUDA(cudaMemsetAsync(x - p->pad, 0, vs * sizeof(T), s));
-  AFC_LAUNCH(p, "k_solver_reset", k_solver_reset<<<1, 32, 0, s>>>(sc, o->ksp_atol, o->ksp_rtol, o->ksp_maxit));
-  for (;;) {
-    with_K(p->K, [&](auto kc) {
-      constexpr int KT = decltype(kc)::value;
-      AFC_LAUNCH(p, "k_gm_residual",
-                 k_gm_residual<KT, T><<<gr, kBlock, 0, s>>>(N, p->offs, sc, B, x, rhs, wv, part, cnt));
-    });
-    AFC_CUDA(cudaGetLastError());
-    AFC_CUDA(cudaMemcpyAsync(w.hsc, sc, S_CS * sizeof(double), cudaMemcpyDeviceToHost, s));
-    AFC_CUDA(cudaStreamSynchronize(s));
-    if (w.hsc[S_DONE] != 0.0) break;
-    AFC_LAUNCH(p, "k_gm_normalize", k_gm_normalize<T><<<G, kBlock, 0, s>>>(N, sc, wv, V, dinv, z));
-    for (int k = 0; k < m; ++k) {
-      with_K(p->K, [&](auto kc) {
-        constexpr int KT = decltype(kc)::value;
-        AFC_LAUNCH(p, "k_gm_spmv", k_gm_spmv<KT, T><<<gr, kBlock, 0, s>>>(N, p->offs, sc, B, z, wv));
-      });
-      orth_launch<T>(p, G, N, sc, k, m, -1, S_H1, wv, V, vs, part, G, cnt);
-      orth_launch<T>(p, G, N, sc, k, m, S_H1, S_H2, wv, V, vs, part, G, cnt);
-      orth_launch<T>(p, G, N, sc, k, m, S_H2, -1, wv, V, vs, part, G, cnt);
-      AFC_LAUNCH(p, "k_gm_normalize", k_gm_normalize<T><<<G, kBlock, 0, s>>>(N, sc, wv, V + (k + 1) * vs, dinv, z));
-    }
-    AFC_LAUNCH(p, "k_gm_update", k_gm_update<T><<<G, kBlock, 0, s>>>(N, sc, x, V, vs, dinv, GraphCond{}));
-    AFC_CUDA(cudaGetLastError());
-  }
-  AFC_LAUNCH(p, "k_to_double", k_to_double<T><<<G, kBlock, 0, s>>>(N, x, xout));
-  AFC_CUDA(cudaGetLastError());
-  if (its) *its = (int)w.hsc[S_ITS];
-  if (res) *res = w.hsc[S_NRES];
-  const double done = w.hsc[S_DONE];
-  if (done == 2.0) { set_error("GMRES breakdown or non-finite value"); return AFC_E_NAN; }
-  return done == 1.0 ? AFC_OK : AFC_NOT_CONVERGED;
+  if ((st = gmres_fused_launch<T>(p, p->stream, B, dinv, o, rhs, xout, epi))) return st;
+  return fused_result(p, "GMRES", its, res);
 }
 
 }  // namespace
@@ -1267,143 +1047,28 @@ namespace {
 
 template <class T>
 int bicgstab_graph(afc_problem_s* p, const T* B, const T* dinv, const afc_opts* o, const double* rhs, double* xout,
-                   cudaStream_t cs, cudaGraph_t g, std::vector<cudaGraphNode_t>& frontier,
-                   const KrylovEpilogue* epi, bool* epi_done) {
+                   cudaStream_t cs, cudaGraph_t g, std::vector<cudaGraphNode_t>& frontier, const KrylovEpilogue* epi) {
   int st = ensure_work(p, 9, sizeof(T) == 4);
   if (st) return st;
-  KrylovWork& w = *p->kw;
-  const int64_t N = p->N;
-  T *x = vec_at<T>(w, 0), *r = vec_at<T>(w, 1), *rh = vec_at<T>(w, 2), *pp = vec_at<T>(w, 3), *v = vec_at<T>(w, 4),
-    *sv = vec_at<T>(w, 5), *t = vec_at<T>(w, 6), *ph = vec_at<T>(w, 7), *sh = vec_at<T>(w, 8);
-  double* sc = w.sc.p;
-  double* part = w.part.p;
-  unsigned int* cnt = w.counter.p;
-  const int G = kRedBlocks;
-  const int64_t gr = grid_for(N);
-  if (w.coop < 0) {
-    int c = 0;
-    AFC_CUDA(cudaDeviceGetAttribute(&c, cudaDevAttrCooperativeLaunch, p->device));
-    AFC_CUDA(cudaDeviceGetAttribute(&w.nsm, cudaDevAttrMultiProcessorCount, p->device));
-    w.coop = c;
-  }
-  if (w.coop > 0) {   // the whole solve is one persistent launch: no loop node needed
-    if (epi_done) *epi_done = epi != nullptr;
-    return capture_into(p, cs, g, frontier, [&]() -> int {
-      bool ok = false;
-      int s2 = bicg_fused_launch<T>(p, p->stream, B, dinv, o, rhs, xout, &ok, epi);
-      if (s2) return s2;
-      AFC_CUDA(cudaGetLastError());
-      return AFC_OK;
-    }, frontier);
-  }
-  GraphCond cond;
-  cond.use = true;
-  AFC_CUDA(cudaGraphConditionalHandleCreate(&cond.h, g, 0, 0));
-  if ((st = capture_into(p, cs, g, frontier, [&]() -> int {
-         AFC_LAUNCH(p, "k_solver_reset",
-                    k_solver_reset<<<1, 32, 0, p->stream>>>(sc, o->ksp_atol, o->ksp_rtol, o->ksp_maxit));
-         AFC_LAUNCH(p, "k_bicg_init", k_bicg_init<T><<<G, kBlock, 0, p->stream>>>(N, rhs, x, r, rh, pp, v, part, cnt, sc));
-         AFC_LAUNCH(p, "k_cond_running", k_cond_running<<<1, 32, 0, p->stream>>>(sc, cond));
-         AFC_CUDA(cudaGetLastError());
-         return AFC_OK;
-       }, frontier)))
-    return st;
-  cudaGraph_t body;
-  cudaGraphNode_t loop;
-  if ((st = add_conditional(g, frontier, cond.h, cudaGraphCondTypeWhile, &body, &loop))) return st;
-  std::vector<cudaGraphNode_t> inner;
-  if ((st = capture_into(p, cs, body, {}, [&]() -> int {
-         with_K(p->K, [&](auto kc) {
-           constexpr int KT = decltype(kc)::value;
-           cudaStream_t s = p->stream;
-           AFC_LAUNCH(p, "k_bicg_p", k_bicg_p<T><<<G, kBlock, 0, s>>>(N, sc, r, pp, v, dinv, ph));
-           AFC_LAUNCH(p, "k_bicg_spmv1",
-                      k_bicg_spmv1<KT, T><<<gr, kBlock, 0, s>>>(N, p->offs, sc, B, ph, v, rh, part, cnt));
-           AFC_LAUNCH(p, "k_bicg_s", k_bicg_s<T><<<G, kBlock, 0, s>>>(N, sc, r, v, dinv, sv, sh, part, cnt));
-           AFC_LAUNCH(p, "k_bicg_spmv2",
-                      k_bicg_spmv2<KT, T><<<gr, kBlock, 0, s>>>(N, p->offs, sc, B, sh, t, sv, x, ph, part, cnt));
-           AFC_LAUNCH(p, "k_bicg_xr",
-                      k_bicg_xr<T><<<G, kBlock, 0, s>>>(N, sc, x, ph, sh, sv, t, r, rh, part, cnt, cond));
-         });
-         AFC_CUDA(cudaGetLastError());
-         return AFC_OK;
-       }, inner)))
-    return st;
-  frontier.assign(1, loop);
   return capture_into(p, cs, g, frontier, [&]() -> int {
-    AFC_LAUNCH(p, "k_to_double", k_to_double<T><<<G, kBlock, 0, p->stream>>>(N, x, xout));
-    AFC_CUDA(cudaGetLastError());
-    return AFC_OK;
+    return bicg_fused_launch<T>(p, p->stream, B, dinv, o, rhs, xout, epi);
   }, frontier);
 }
 
 template <class T>
 int gmres_graph(afc_problem_s* p, const T* B, const T* dinv, const afc_opts* o, const double* rhs, double* xout,
-                cudaStream_t cs, cudaGraph_t g, std::vector<cudaGraphNode_t>& frontier) {
-  const int m = o->gmres_restart;
-  if (m < 1 || m > kMaxRestart) { set_error("gmres_restart must be in 1..32"); return AFC_E_INVALID; }
-  int st = ensure_work(p, 3 + m + 1, sizeof(T) == 4);
+                cudaStream_t cs, cudaGraph_t g, std::vector<cudaGraphNode_t>& frontier, const KrylovEpilogue* epi) {
+  int st = gmres_work(p, o, sizeof(T) == 4);
   if (st) return st;
-  KrylovWork& w = *p->kw;
-  const int64_t N = p->N;
-  T *x = vec_at<T>(w, 0), *wv = vec_at<T>(w, 1), *z = vec_at<T>(w, 2), *V = vec_at<T>(w, 3);
-  const size_t vs = w.vstride;
-  double* sc = w.sc.p;
-  double* part = w.part.p;
-  unsigned int* cnt = w.counter.p;
-  const int G = kRedBlocks;
-  const int64_t gr = grid_for(N);
-  GraphCond cond;
-  cond.use = true;
-  AFC_CUDA(cudaGraphConditionalHandleCreate(&cond.h, g, 0, 0));
-  if ((st = capture_into(p, cs, g, frontier, [&]() -> int {
-         AFC_CUDA(cudaMemsetAsync(x - p->pad, 0, vs * sizeof(T), p->stream));
-         AFC_LAUNCH(p, "k_solver_reset",
-                    k_solver_reset<<<1, 32, 0, p->stream>>>(sc, o->ksp_atol, o->ksp_rtol, o->ksp_maxit));
-         AFC_LAUNCH(p, "k_cond_running", k_cond_running<<<1, 32, 0, p->stream>>>(sc, cond));
-         AFC_CUDA(cudaGetLastError());
-         return AFC_OK;
-       }, frontier)))
-    return st;
-  cudaGraph_t body;
-  cudaGraphNode_t loop;
-  if ((st = add_conditional(g, frontier, cond.h, cudaGraphCondTypeWhile, &body, &loop))) return st;
-  std::vector<cudaGraphNode_t> inner;
-  if ((st = capture_into(p, cs, body, {}, [&]() -> int {
-         cudaStream_t s = p->stream;
-         with_K(p->K, [&](auto kc) {
-           constexpr int KT = decltype(kc)::value;
-           AFC_LAUNCH(p, "k_gm_residual",
-                      k_gm_residual<KT, T><<<gr, kBlock, 0, s>>>(N, p->offs, sc, B, x, rhs, wv, part, cnt));
-           AFC_LAUNCH(p, "k_gm_normalize", k_gm_normalize<T><<<G, kBlock, 0, s>>>(N, sc, wv, V, dinv, z));
-           for (int k = 0; k < m; ++k) {
-             AFC_LAUNCH(p, "k_gm_spmv", k_gm_spmv<KT, T><<<gr, kBlock, 0, s>>>(N, p->offs, sc, B, z, wv));
-             orth_launch<T>(p, G, N, sc, k, m, -1, S_H1, wv, V, vs, part, G, cnt);
-             orth_launch<T>(p, G, N, sc, k, m, S_H1, S_H2, wv, V, vs, part, G, cnt);
-             orth_launch<T>(p, G, N, sc, k, m, S_H2, -1, wv, V, vs, part, G, cnt);
-             AFC_LAUNCH(p, "k_gm_normalize",
-                        k_gm_normalize<T><<<G, kBlock, 0, s>>>(N, sc, wv, V + (k + 1) * vs, dinv, z));
-           }
-           AFC_LAUNCH(p, "k_gm_update", k_gm_update<T><<<G, kBlock, 0, s>>>(N, sc, x, V, vs, dinv, cond));
-         });
-         AFC_CUDA(cudaGetLastError());
-         return AFC_OK;
-       }, inner)))
-    return st;
-  frontier.assign(1, loop);
   return capture_into(p, cs, g, frontier, [&]() -> int {
-    AFC_LAUNCH(p, "k_to_double", k_to_double<T><<<G, kBlock, 0, p->stream>>>(N, x, xout));
-    AFC_CUDA(cudaGetLastError());
-    return AFC_OK;
+    return gmres_fused_launch<T>(p, p->stream, B, dinv, o, rhs, xout, epi);
   }, frontier);
 }
 
 }  // namespace
 
 int krylov_graph(afc_problem_s* p, int system, const afc_opts* o, const double* rhs, double* x, cudaStream_t cs,
-                 cudaGraph_t g, std::vector<cudaGraphNode_t>& frontier, const KrylovEpilogue* epi,
-                 bool* epi_done) {
-  if (epi_done) *epi_done = false;
+                 cudaGraph_t g, std::vector<cudaGraphNode_t>& frontier, const KrylovEpilogue* epi) {
   const bool mixed = o->precision == AFC_MIXED;
   if (mixed && p->precision != AFC_MIXED) {
     set_error("mixed-precision solve needs afc_assemble(..., AFC_MIXED)");
@@ -1413,17 +1078,14 @@ int krylov_graph(afc_problem_s* p, int system, const afc_opts* o, const double* 
   if (mixed) {
     const float* B = system == 0 ? p->Bst32.p : p->Bcn32.p;
     const float* di = system == 0 ? p->dinv_st32.p : p->dinv_cn32.p;
-    return gm ? gmres_graph<float>(p, B, di, o, rhs, x, cs, g, frontier)
-              : bicgstab_graph<float>(p, B, di, o, rhs, x, cs, g, frontier, epi, epi_done);
+    return gm ? gmres_graph<float>(p, B, di, o, rhs, x, cs, g, frontier, epi)
+              : bicgstab_graph<float>(p, B, di, o, rhs, x, cs, g, frontier, epi);
   }
   const double* B = system == 0 ? p->Bst.p : p->Bcn.p;
   const double* di = system == 0 ? p->dinv_st.p : p->dinv_cn.p;
-  return gm ? gmres_graph<double>(p, B, di, o, rhs, x, cs, g, frontier)
-            : bicgstab_graph<double>(p, B, di, o, rhs, x, cs, g, frontier, epi, epi_done);
+  return gm ? gmres_graph<double>(p, B, di, o, rhs, x, cs, g, frontier, epi)
+            : bicgstab_graph<double>(p, B, di, o, rhs, x, cs, g, frontier, epi);
 }
-
-const double* krylov_scalars(afc_problem_s* p) { return p->kw ? p->kw->sc.p : nullptr; }
-int krylov_cycles_slot() { return S_CYCLES; }
 
 int krylov_reset_barrier(afc_problem_s* p) {
   if (!p->kw || !p->kw->barrier.p) return AFC_OK;
@@ -1434,8 +1096,7 @@ int krylov_reset_barrier(afc_problem_s* p) {
 const void* krylov_key(afc_problem_s* p) { return p->kw ? (const void*)p->kw->vec.base : nullptr; }
 
 int krylov_solve(afc_problem_s* p, int system, const afc_opts* o, const double* rhs, double* x, int* its,
-                 double* res, const KrylovEpilogue* epi, bool* epi_done) {
-  if (epi_done) *epi_done = false;
+                 double* res, const KrylovEpilogue* epi) {
   const bool mixed = o->precision == AFC_MIXED;
   if (mixed && p->precision != AFC_MIXED) {
     set_error("mixed-precision solve needs afc_assemble(..., AFC_MIXED)");
@@ -1446,13 +1107,13 @@ int krylov_solve(afc_problem_s* p, int system, const afc_opts* o, const double* 
   if (mixed) {
     const float* B = system == 0 ? p->Bst32.p : p->Bcn32.p;
     const float* di = system == 0 ? p->dinv_st32.p : p->dinv_cn32.p;
-    return gm ? gmres_impl<float>(p, B, di, o, rhs, x, its, res)
-              : bicgstab_impl<float>(p, B, di, o, rhs, x, its, res, epi, epi_done);
+    return gm ? gmres_impl<float>(p, B, di, o, rhs, x, its, res, epi)
+              : bicgstab_impl<float>(p, B, di, o, rhs, x, its, res, epi);
   }
   const double* B = system == 0 ? p->Bst.p : p->Bcn.p;
   const double* di = system == 0 ? p->dinv_st.p : p->dinv_cn.p;
-  return gm ? gmres_impl<double>(p, B, di, o, rhs, x, its, res)
-            : bicgstab_impl<double>(p, B, di, o, rhs, x, its, res, epi, epi_done);
+  return gm ? gmres_impl<double>(p, B, di, o, rhs, x, its, res, epi)
+            : bicgstab_impl<double>(p, B, di, o, rhs, x, its, res, epi);
 }
 
 }  // namespace afc

@@ -56,35 +56,39 @@ __device__ __forceinline__ unsigned int ld_acquire_gpu(const unsigned int* p) {
 
 // Arrive (after the block's threads have met): returns, in thread 0, the counter value
 // before this block's add.
+__device__ __forceinline__ unsigned int grid_arrive_thread(GridBar* gb) {   // the one thread of a block
+  const unsigned int add = blockIdx.x == 0 ? 0x80000000u - (gridDim.x - 1u) : 1u;
+  asm volatile("fence.acq_rel.gpu;" ::: "memory");
+  return atomicAdd(&gb->arrive, add);
+}
 __device__ __forceinline__ unsigned int grid_arrive(GridBar* gb) {
   __syncthreads();
-  unsigned int old = 0u;
-  if (threadIdx.x == 0) {
-    const unsigned int add = blockIdx.x == 0 ? 0x80000000u - (gridDim.x - 1u) : 1u;
-    asm volatile("fence.acq_rel.gpu;" ::: "memory");
-    old = atomicAdd(&gb->arrive, add);
-  }
-  return old;
+  return threadIdx.x == 0 ? grid_arrive_thread(gb) : 0u;
 }
 
-// Wait until every block has arrived (thread 0 passes what grid_arrive returned);
-// give up once limit_ns of the global timer have passed (limit 0: at the first poll
-// that finds the barrier still closed).
-__device__ __forceinline__ void grid_wait(GridBar* gb, unsigned int old,
-                                          unsigned long long limit_ns = kBarrierWaitNs) {
-  if (threadIdx.x == 0) {
-    volatile int* verr = &gb->err;
-    if (*verr == 0) {
-      const unsigned long long t0 = global_ns();
-      while (((old ^ ld_acquire_gpu(&gb->arrive)) & 0x80000000u) == 0u) {
-        if (*verr != 0) break;
-        if (global_ns() - t0 >= limit_ns) {
-          atomicExch(&gb->err, 1);
-          break;
-        }
-      }
+// One thread waits until every block has arrived (`old`: what its arrival found); gives up
+// once limit_ns of the global timer have passed (limit 0: at the first poll that finds
+// the barrier still closed), or when another block has.  The first polls look at the
+// counter alone: the error word and the global timer cost a trip each, so they are
+// read only on every 16th poll (a barrier opens within a few polls).
+__device__ __forceinline__ void grid_poll(GridBar* gb, unsigned int old, unsigned long long limit_ns) {
+  unsigned long long t0 = 0;
+  for (unsigned int n = 1; ((old ^ ld_acquire_gpu(&gb->arrive)) & 0x80000000u) == 0u; ++n) {
+    if ((n & 15u) != 0u && limit_ns != 0ull) continue;
+    if (*(volatile int*)&gb->err != 0) break;
+    const unsigned long long now = global_ns();
+    if (t0 == 0ull) t0 = now;
+    if (now - t0 >= limit_ns) {
+      atomicExch(&gb->err, 1);
+      break;
     }
   }
+}
+
+// The block waits (thread 0 passes what grid_arrive returned).
+__device__ __forceinline__ void grid_wait(GridBar* gb, unsigned int old,
+                                          unsigned long long limit_ns = kBarrierWaitNs) {
+  if (threadIdx.x == 0) grid_poll(gb, old, limit_ns);
   __syncthreads();
 }
 

@@ -22,6 +22,7 @@ int64_t grid_for(int64_t n, int block) { return (n + block - 1) / block; }
 
 template <class T>
 int DBuf<T>::alloc(int64_t n_, int64_t pad_) {
+  pad_ = (pad_ + 31) & ~(int64_t)31;   // the logical start stays on a 128-byte boundary
   if (base && n == n_ && pad == pad_) return AFC_OK;
   free_();
   size_t bytes = (size_t)(n_ + 2 * pad_) * sizeof(T);
@@ -194,7 +195,7 @@ struct KrylovWork {
   int pad = 0, m = 0, fp32 = -1;
   DBuf<char> vec;       // all vectors (with halos)
   DBuf<double> sc, part;
-  DBuf<unsigned int> barrier;   // GridBar of the persistent BiCGStab launch
+  DBuf<unsigned int> barrier;   // GridBar of the persistent launches
   int nsm = 0;                  // SMs of the device (0: not asked yet)
   double* hsc = nullptr;
   size_t vstride = 0;   // elements per vector incl. halo
@@ -465,33 +466,44 @@ __global__ void __launch_bounds__(kFusedBlock, 1024 / kFusedBlock) k_bicg_fused(
 // stationary solves stop after 5 to 10 of them (the rest returned at once, but were
 // launched).  Here a step is two grid-wide sums (barriers), and a solve stops where it
 // stops.  Measured on one GB300, whole stationary MC solves (omega = 0.5, inner rtol 1e-2),
-// before and after: Q1 27x21x33 in double 301 -> 89 ms, P1 49^3 mixed 470 -> 153 ms, P1
-// 129^3 mixed 1.70 -> 1.40 s; the same iteration counts.
+// against the launches per pass: Q1 27x21x33 in double 301 -> 63 ms, P1 49^3 mixed 470 ->
+// 111 ms, P1 129^3 mixed 1.70 -> 0.95 s; the same iteration counts.  Per Arnoldi step (P1 49^3 /
+// 129^3): product 1.7 / 25 us, dots 0.8 / 10, sums 2.9 / 5, second projection 3.7 / 20 (when
+// taken), completion 1.3 / 13, barrier 1.5 / 3.
 //
-// Layout.  Block b owns the contiguous rows [N b / G, N (b + 1) / G) for every pass, so
+// Layout.  Block b owns a contiguous range of rows (a multiple of 32) for every pass, so
 // everything but the product's gather of z is local to a block:
-//  * w (the new direction) stays in shared memory between the passes of a step (in
-//    global memory where a block's rows do not fit);
+//  * w (the new direction) stays in shared memory between the passes of a step, and so
+//    do the basis vectors where all m + 1 of a block fit (P1 65^3 in single precision);
+//    otherwise they are in global memory, read 16 bytes per load, four vectors at a
+//    time, each once per pass;
 //  * the basis vectors are stored unnormalised with their scale 1 / ||v_q|| beside them
 //    (in `scale`), so no pass only normalises; z = D^{-1} v_k is the one vector other
-//    blocks read, written by the pass that completes v_k;
-//  * the dots go eight basis vectors at a time: eight running sums and eight loads in
-//    flight per thread, w re-read from shared memory, each basis vector read once.
+//    blocks read, written by the pass that completes v_k.
 // Scalars.  A double operation by all warps of an SM costs 16 cycles per warp on the
-// FP64 pipe, so the Hessenberg column, Givens rotations and tests run in one warp (or
-// one thread) of every block, redundantly and in the same order: every block obtains
-// the same bits and takes the same branches without another barrier.
+// FP64 pipe, so the Hessenberg column, Givens rotations and tests run in one warp of
+// every block, redundantly and in the same order: every block obtains the same bits and
+// takes the same branches without another barrier.  That warp owns no rows: the column
+// of step k is rotated while the other warps project and then while they form the next
+// product, so the chain of dependent double operations (4 us a step when the block waited
+// for it) is hidden; the product that follows a cycle's last step is formed in vain.
 //
 // Per Arnoldi step k (V holds v_0 .. v_k):
-//  (1) w = B z / ||v_k||, h1 = V^T w, ||w||^2                       -> grid sums
+//  (1) w = B z, the dots of V and w, ||w||^2                          -> grid sums
 //      DGKS test: if ||w - V h1||^2 = ||w||^2 - ||h1||^2 >= ||w||^2 / 2 little of w lay in
 //      the basis and a second projection would change nothing worth keeping;
-//      otherwise w -= V h1, h2 = V^T w                               -> grid sums
-//  (2) v_{k+1} = w - V h, z = D^{-1} v_{k+1}, ||v_{k+1}||^2          -> grid sum
+//      otherwise w -= V h1, h2 = V^T w, ||w||^2                      -> grid sums
+//  (2) v_{k+1} = w - V h, z = D^{-1} v_{k+1}, ||v_{k+1}||^2          -> grid sum (or barrier)
 //      Hessenberg column, rotations, |g[k+1]|, the end-of-cycle test.
-constexpr int kGmMaxBlock = 1024;
-constexpr int kGmQ = kMaxRestart + 2;      // sums of one grid-wide reduction: k + 1 dots and a norm
-constexpr size_t kGmSmemW = 160 * 1024;    // shared memory for a block's w (the rest stays L1)
+// Threads of a block, at most: with the basis in shared memory (few rows: 96 registers keep
+// more of a row's loads in flight), and in global memory (64 registers).
+constexpr int kGmBlockS = 544, kGmBlock = 1024;
+constexpr int kGmMinCompute = 224;         // threads with rows: few-row blocks still need warps that poll
+constexpr int kGmUnit = 32;                // rows of a block come in multiples of this
+constexpr int kGmQ = kMaxRestart + 2;      // values of one exchange: k + 1 dots and a norm
+// Shared memory for w and V: what is left of 228 KB stays L1, where the product's gather
+// of z lives (three bands of a block's rows: ~90 KB suffice up to the sizes that fit).
+constexpr size_t kGmSmem = 160 * 1024;
 
 struct GmArgs {
   int64_t N;
@@ -499,93 +511,145 @@ struct GmArgs {
   const double* rhs;
   double* xout;
   size_t vstride;
-  double* part;
   GridBar* bar;
+  double* part;
   double atol, rtol;
-  int maxit, m, w_in_smem;
+  int maxit, m, compute, rows;
+  bool w_in_smem;
   KrylovEpilogue ep;
   unsigned long long wait_ns;
 };
 
-// Totals over a warp of eight values per lane in nine adds (a butterfly that halves the
-// values with the lanes: 4 + 2 + 1 adds exchange, 2 more finish) instead of forty; lane l
-// returns the total of value (l >> 2): bits 4, 3, 2 of the lane are bits 2, 1, 0 of the value.
+// 16 bytes of a vector.
 template <class T>
-__device__ __forceinline__ T warp_sum8(T (&v)[8]) {
+struct alignas(16) Pack {
+  static constexpr int W = 16 / sizeof(T);
+  T e[W];
+};
+
+// Totals over a warp of four values per lane in six adds (a butterfly that halves the values
+// with the lanes, then sums) instead of twenty; lane l returns the total of value l >> 3
+// (bits 4 and 3 of the lane are bits 1 and 0 of the value).
+template <class T>
+__device__ __forceinline__ T warp_sum4(const T (&v)[4]) {
   const int lane = threadIdx.x & 31;
-  const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
-  T a[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const T send = b4 ? v[j] : v[j + 4], keep = b4 ? v[j + 4] : v[j];
-    a[j] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-  }
-  T c[2];
+  const bool b4 = lane & 16, b3 = lane & 8;
+  T a[2];
 #pragma unroll
   for (int j = 0; j < 2; ++j) {
-    const T send = b3 ? a[j] : a[j + 2], keep = b3 ? a[j + 2] : a[j];
-    c[j] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
+    const T send = b4 ? v[j] : v[j + 2], keep = b4 ? v[j + 2] : v[j];
+    a[j] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
   }
-  const T send = b2 ? c[0] : c[1], keep = b2 ? c[1] : c[0];
-  T t = keep + __shfl_xor_sync(0xffffffffu, send, 4);
-  t += __shfl_xor_sync(0xffffffffu, t, 2);
-  t += __shfl_xor_sync(0xffffffffu, t, 1);
+  const T send = b3 ? a[0] : a[1], keep = b3 ? a[1] : a[0];
+  T t = keep + __shfl_xor_sync(0xffffffffu, send, 8);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
   return t;
 }
 
-// Scalars of a solve, one copy per block.  `red` holds the warps' sums, `tot` the grid's.
+// Scalars of a solve, one copy per block.
 template <class T>
 struct GmShared {
-  T red[kGmMaxBlock / 32][kGmQ + 6];   // rows padded to 8 x 5 values
-  T hs[kMaxRestart];                   // coefficients of the pass at hand, in the vector type
-  T invh;                              // 1 / ||v_k||
-  double tot[kGmQ];
+  T red[kGmBlock / 32][kGmQ + 3];   // the warps' sums (rows padded against bank conflicts)
+  T hs[kMaxRestart];                   // coefficients of the projection at hand, in the vector type
+  T ih;                                // factor of w in the projection
+  double tot[kGmQ];                    // totals of the last exchange
+  double nrm2;                         // ||v_{k+1}||^2
   double scale[kMaxRestart + 1];       // 1 / ||v_q||
   double h1[kMaxRestart], h2[kMaxRestart];
   double cs[kMaxRestart], sn[kMaxRestart], g[kMaxRestart + 1], y[kMaxRestart];
   double H[kMaxRestart][kMaxRestart];  // H[row][col], upper triangle after the rotations
+  double run;                          // running entry of the column being rotated
   double nres, n0, tol;
   int its, cycles, done, cycle_done, skip;
 };
 
-// Grid-wide totals of the block's nq sums (sh.red, one row per warp) in sh.tot.  Every
-// block adds the partials of all blocks in block order, so all obtain the same bits.
-// The partials alternate between two buffers, as in grid_sums_begin.  Ends with warp 0
-// holding the totals of the values it summed; the caller synchronises the block.
-template <class T>
-__device__ __forceinline__ void gm_grid_sums(GmShared<T>& sh, int nq, const GmArgs& a, int& buf) {
-  const int G = gridDim.x;
-  const int nwarp = blockDim.x >> 5, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  double* pb = a.part + (size_t)buf * kGmQ * G;
+// The total over a warp of one partial of G per slot, p[0 .. G), in a fixed order.
+__device__ __forceinline__ double gm_total(const double* p, int G) {
+  const int lane = threadIdx.x & 31;
+  double x[5];   // G <= 160
+#pragma unroll
+  for (int u = 0; u < 5; ++u) x[u] = lane + 32 * u < G ? __ldcg(p + lane + 32 * u) : 0.0;
+  const double t = ((x[0] + x[1]) + (x[2] + x[3])) + x[4];
+  return warp_sum(t);
+}
+// Single-precision partials in 64-bit fixed point scaled to the largest (its mantissa at
+// bits 30 .. 53, so 160 blocks cannot overflow), one rounding at the end: no less exact than
+// a sum in double, and on the integer pipe (eight double adds by each of a dozen warps at
+// once held the FP64 pipe for most of a microsecond).  Inf and NaN come out as NaN.
+__device__ __forceinline__ double gm_total(const float* p, int G) {
+  const int lane = threadIdx.x & 31;
+  unsigned x[5];   // G <= 160
+  unsigned e = 0;
+#pragma unroll
+  for (int u = 0; u < 5; ++u) {
+    x[u] = lane + 32 * u < G ? __float_as_uint(__ldcg(p + lane + 32 * u)) : 0u;
+    e = max(e, (x[u] >> 23) & 0xffu);
+  }
+  e = __reduce_max_sync(0xffffffffu, e);
+  if (e == 0xffu) return __longlong_as_double(0x7ff8000000000000ll);
+  e = max(e, 1u);
+  long long t = 0;
+#pragma unroll
+  for (int u = 0; u < 5; ++u) {
+    const unsigned xe = (x[u] >> 23) & 0xffu, m = (x[u] & 0x7fffffu) | (xe ? 0x800000u : 0u);
+    const unsigned sh = min(e - max(xe, 1u), 63u);
+    const long long v = (long long)(((unsigned long long)m << 30) >> sh);
+    t += (x[u] >> 31) ? -v : v;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  const double d = (double)t;   // t * 2^(e - 127 - 23 - 30): the exponent moves exactly
+  return t == 0 ? 0.0 : __longlong_as_double(__double_as_longlong(d) + ((long long)((int)e - 180) << 52));
+}
+
+// A grid-wide sum of nq values and a barrier: the warps' sums in sh.red (rows 0 .. nw - 1)
+// are added and stored by warp 0, whose first lane arrives and polls; then warp q adds all
+// blocks' partials of value q into sh.tot (the same bits in every block), and `take()` runs
+// in warp 0 (with nq <= 1 before the block meets again, in the same warp).  Memory: the
+// block's threads meet, so that lane's fence releases what they wrote; it polls with acquire
+// loads, and the block meets again before anyone uses what `take` stored or what other
+// blocks wrote.  The partials alternate between two buffers (a block can run at most one
+// sum ahead of another).
+template <class T, class F>
+__device__ __forceinline__ void gm_exchange(GmShared<T>& sh, int nq, int nw, const GmArgs& a, int& buf, F&& take) {
+  const int G = gridDim.x, lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  T* pb = reinterpret_cast<T*>(a.part) + (size_t)buf * kGmQ * G;
   buf ^= 1;
   __syncthreads();   // sh.red is complete
-  if ((int)threadIdx.x < nq) {
-    T s0 = 0, s1 = 0, s2 = 0, s3 = 0;   // four chains: the adds of one are serial
-    int u = 0;
-    for (; u + 3 < nwarp; u += 4) {
-      s0 += sh.red[u][threadIdx.x];
-      s1 += sh.red[u + 1][threadIdx.x];
-      s2 += sh.red[u + 2][threadIdx.x];
-      s3 += sh.red[u + 3][threadIdx.x];
+  if (wp == 0) {
+#pragma unroll 1
+    for (int q = lane; q < nq; q += 32) {
+      T s0 = 0, s1 = 0, s2 = 0, s3 = 0;   // four chains: the adds of one are serial
+      int u = 0;
+#pragma unroll 1
+      for (; u + 3 < nw; u += 4) {
+        s0 += sh.red[u][q];
+        s1 += sh.red[u + 1][q];
+        s2 += sh.red[u + 2][q];
+        s3 += sh.red[u + 3][q];
+      }
+      for (; u < nw; ++u) s0 += sh.red[u][q];
+      pb[(size_t)q * G + blockIdx.x] = (s0 + s1) + (s2 + s3);
     }
-    for (; u < nwarp; ++u) s0 += sh.red[u][threadIdx.x];
-    pb[(size_t)threadIdx.x * G + blockIdx.x] = to_dbl((s0 + s1) + (s2 + s3));
+    __syncwarp();
+    if (lane == 0) grid_poll(a.bar, grid_arrive_thread(a.bar), a.wait_ns);
+    __syncwarp();
   }
-  const unsigned int old = grid_arrive(a.bar);
-  grid_wait(a.bar, old, a.wait_ns);
-  for (int q = w; q < nq; q += nwarp) {
-    double t = 0.0;
-    for (int b0 = lane; b0 < G; b0 += 256) {
-      double x[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) x[u] = b0 + 32 * u < G ? __ldcg(pb + (size_t)q * G + b0 + 32 * u) : 0.0;
-#pragma unroll
-      for (int u = 0; u < 8; ++u)
-        if (b0 - lane + 32 * u < G) t += x[u];
+  if (nq > 1) __syncthreads();
+  if (nq > 1 || wp == 0) {
+#pragma unroll 1
+    for (int q = wp; q < nq; q += blockDim.x >> 5) {
+      const double t = gm_total(pb + (size_t)q * G, G);
+      if (lane == 0) sh.tot[q] = t;
     }
-    t = warp_sum(t);
-    if (lane == 0) sh.tot[q] = t;
   }
+  if (nq > 1) __syncthreads();
+  if (wp == 0) {
+    __syncwarp();
+    take();
+  }
+  __syncthreads();
 }
 
 // The warps' sums of one value per thread, as value q of sh.red.
@@ -595,86 +659,224 @@ __device__ __forceinline__ void gm_put(GmShared<T>& sh, T v, int q) {
   if ((threadIdx.x & 31) == 0) sh.red[threadIdx.x >> 5][q] = v;
 }
 
-// The warps' dots (w, v_q), q <= k, as values 0 .. k of sh.red.
-template <class T>
-__device__ __forceinline__ void gm_dots(GmShared<T>& sh, const T* w, const T* V, size_t vs, int64_t i0, int nrow,
-                                        int k) {
-  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-  for (int q0 = 0; q0 <= k; q0 += 8) {
-    T acc[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) acc[j] = (T)0;
-    const T* Vq = V + (size_t)q0 * vs + i0;
-#pragma unroll 2
-    for (int r = threadIdx.x; r < nrow; r += blockDim.x) {
-      T v[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) v[j] = q0 + j <= k ? Vq[(size_t)j * vs + r] : (T)0;
-      const T wi = w[r];
-#pragma unroll
-      for (int j = 0; j < 8; ++j)
-        if (q0 + j <= k) acc[j] = fma(wi, v[j], acc[j]);
-    }
-    const T t = warp_sum8(acc);
-    if ((lane & 3) == 0) sh.red[wp][q0 + (lane >> 2)] = t;
-  }
+// Run f(NQ as a constant, q) over q = 0 .. n - 1 in steps of four and a rest of one to three:
+// loops over the basis without a predicate per vector (which cost the registers that hold
+// the loads in flight).
+template <class F>
+__device__ __forceinline__ void by_fours(int n, F&& f) {
+  int q = 0;
+#pragma unroll 1
+  for (; q + 4 <= n; q += 4) f(std::integral_constant<int, 4>{}, q);
+  if (n - q == 3) f(std::integral_constant<int, 3>{}, q);
+  else if (n - q == 2) f(std::integral_constant<int, 2>{}, q);
+  else if (n - q == 1) f(std::integral_constant<int, 1>{}, q);
 }
 
-// w_r - sum_q hs[q] v_q[r], q <= k.
+// The warps' dots (w, v_q), q <= k, as values 0 .. k of sh.red, and (w, w) as value k + 1.
+// ng: groups of 16 bytes in a block's rows; nw: warps that hold any.
 template <class T>
-__device__ __forceinline__ T gm_project(const GmShared<T>& sh, T wi, const T* V, size_t vs, int64_t i, int k) {
-  for (int q0 = 0; q0 <= k; q0 += 8) {
-    T v[8];
+__device__ __forceinline__ void gm_dots(GmShared<T>& sh, const T* w, const T* V, size_t vs, int ng, int nw, int nt,
+                                        int k) {
+  constexpr int W = Pack<T>::W;
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  if (wp >= nw) return;
+  by_fours(k + 1, [&](auto nq, int q0) {
+    constexpr int NQ = decltype(nq)::value;
+    T acc[4] = {0, 0, 0, 0};
+    const T* Vq = V + (size_t)q0 * vs;
+#pragma unroll 1
+    for (int g = threadIdx.x; g < ng; g += nt) {
+      const Pack<T> wi = *reinterpret_cast<const Pack<T>*>(w + g * W);
+      Pack<T> v[NQ];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) v[j] = q0 + j <= k ? V[(size_t)(q0 + j) * vs + i] : (T)0;
+      for (int j = 0; j < NQ; ++j) v[j] = *reinterpret_cast<const Pack<T>*>(Vq + j * vs + g * W);
 #pragma unroll
-    for (int j = 0; j < 8; ++j)
-      if (q0 + j <= k) wi -= sh.hs[q0 + j] * v[j];
+      for (int j = 0; j < NQ; ++j)
+#pragma unroll
+        for (int e = 0; e < W; ++e) acc[j] = fma(wi.e[e], v[j].e[e], acc[j]);
+    }
+    const T t = warp_sum4(acc);
+    if ((lane & 7) == 0 && (lane >> 3) < NQ) sh.red[wp][q0 + (lane >> 3)] = t;
+  });
+  T nrm = 0;
+#pragma unroll 1
+  for (int g = threadIdx.x; g < ng; g += nt) {
+    const Pack<T> wi = *reinterpret_cast<const Pack<T>*>(w + g * W);
+#pragma unroll
+    for (int e = 0; e < W; ++e) nrm = fma(wi.e[e], wi.e[e], nrm);
   }
+  gm_put(sh, nrm, k + 1);
+}
+
+// ih w - sum_q hs[q] v_q (q <= k) of group g.
+template <class T>
+__device__ __forceinline__ Pack<T> gm_project(const GmShared<T>& sh, T ih, const T* w, const T* V, size_t vs, int g,
+                                              int k) {
+  constexpr int W = Pack<T>::W;
+  Pack<T> wi = *reinterpret_cast<const Pack<T>*>(w + g * W);
+#pragma unroll
+  for (int e = 0; e < W; ++e) wi.e[e] *= ih;
+  by_fours(k + 1, [&](auto nq, int q0) {
+    constexpr int NQ = decltype(nq)::value;
+    Pack<T> v[NQ];
+#pragma unroll
+    for (int j = 0; j < NQ; ++j) v[j] = *reinterpret_cast<const Pack<T>*>(V + (size_t)(q0 + j) * vs + g * W);
+#pragma unroll
+    for (int j = 0; j < NQ; ++j)
+#pragma unroll
+      for (int e = 0; e < W; ++e) wi.e[e] -= sh.hs[q0 + j] * v[j].e[e];
+  });
   return wi;
 }
 
-// Column k of the Hessenberg matrix (one thread): earlier rotations, a new one, the
-// residual estimate and the end-of-cycle test.
+// The passes over a block's rows.
+// w = ih w - V h.
 template <class T>
-__device__ void gm_column(GmShared<T>& sh, int k, const GmArgs& a, bool berr) {
-  const double hk1 = sqrt(sh.tot[0]);
-  double c = sh.h1[0] + sh.h2[0];   // the column's running entry
-  for (int q = 0; q < k; ++q) {
-    const double b = sh.h1[q + 1] + sh.h2[q + 1];
-    sh.H[q][k] = sh.cs[q] * c + sh.sn[q] * b;
-    c = -sh.sn[q] * c + sh.cs[q] * b;
+__device__ __forceinline__ void gm_reproject(const GmShared<T>& sh, T* w, const T* V, size_t vs, int ng, int nt, int k) {
+  const T ih = sh.ih;
+#pragma unroll 1
+  for (int g = threadIdx.x; g < ng; g += nt)
+    *reinterpret_cast<Pack<T>*>(w + g * Pack<T>::W) = gm_project(sh, ih, w, V, vs, g, k);
+}
+// v_{k+1} = ih w - V h, z = D^{-1} v_{k+1} at the block's rows, and with `norm` the warps' sums
+// of ||v_{k+1}||^2.
+template <class T>
+__device__ __forceinline__ void gm_complete(GmShared<T>& sh, const T* w, T* V, size_t vs, int ng, int nt, int k,
+                                         const T* __restrict__ dinv, T* z, int nrow, bool norm) {
+  constexpr int W = Pack<T>::W;
+  const T ih = sh.ih;
+  T* vn = V + (size_t)(k + 1) * vs;
+  T nrm = 0;
+#pragma unroll 1
+  for (int g = threadIdx.x; g < ng; g += nt) {
+    const Pack<T> v = gm_project(sh, ih, w, V, vs, g, k);
+    *reinterpret_cast<Pack<T>*>(vn + g * W) = v;
+#pragma unroll
+    for (int e = 0; e < W; ++e) {
+      const int r = g * W + e;
+      if (r < nrow) z[r] = dinv[r] * v.e[e];
+      nrm = fma(v.e[e], v.e[e], nrm);
+    }
   }
-  const double den = hypot(c, hk1);
-  sh.cs[k] = c / den;
-  sh.sn[k] = hk1 / den;
+  if (norm) gm_put(sh, nrm, 0);
+}
+// x (+)= D^{-1} sum_q hs[q] v_q, q < ku (sh.ih = 0 and hs negated: the projection's form).
+template <class T>
+__device__ __forceinline__ void gm_update(const GmShared<T>& sh, const T* w, const T* V, size_t vs, int ng, int nt, int ku,
+                                       const T* __restrict__ dinv, T* x, int nrow, bool have_x) {
+  constexpr int W = Pack<T>::W;
+#pragma unroll 1
+  for (int g = threadIdx.x; g < ng; g += nt) {
+    const Pack<T> s = gm_project(sh, (T)0, w, V, vs, g, ku - 1);
+#pragma unroll
+    for (int e = 0; e < W; ++e) {
+      const int r = g * W + e;
+      if (r < nrow) {
+        const T d = dinv[r] * s.e[e];
+        x[r] = have_x ? x[r] + d : d;
+      }
+    }
+  }
+}
+
+// Column k of the Hessenberg matrix, in the scalar warp: the earlier rotations (while the
+// other warps complete v_{k+1}).  The running entry c <- -sn_q c + cs_q b_q is one dependent
+// multiply-add per rotation; lane q forms the products and its entry of the column.
+template <class T>
+__device__ __forceinline__ void gm_rotate(GmShared<T>& sh, int k, bool twice) {
+  const int q = threadIdx.x & 31;
+  double cb = 0.0, sb = 0.0, cs = 0.0, sn = 0.0, mine = 0.0;
+  if (q < k) {
+    const double b = sh.h1[q + 1] + sh.h2[q + 1];
+    cs = sh.cs[q];
+    sn = sh.sn[q];
+    cb = cs * b;
+    sb = sn * b;
+  }
+  double c = sh.h1[0] + sh.h2[0];
+#pragma unroll 1
+  for (int r = 0; r < k; ++r) {
+    if (q == r) mine = c;
+    c = fma(-__shfl_sync(0xffffffffu, sn, r), c, __shfl_sync(0xffffffffu, cb, r));
+  }
+  if (q < k) sh.H[q][k] = fma(cs, mine, sb);
+  if (q == 0) sh.run = c;
+  // after a second projection w was almost orthogonal: ||w - V h2||^2 = ||w||^2 - ||h2||^2 loses
+  // nothing, and the norm needs no sum of its own
+  if (twice) {
+    const double h = q <= k ? sh.h2[q] : 0.0, p = warp_sum(h * h);
+    if (q == 0) sh.nrm2 = fmax(sh.nrm2 - p, 0.0);
+  }
+}
+// ... then, from ||v_{k+1}||^2, the new rotation, the residual estimate and the
+// end-of-cycle test (while they form the next product).
+template <class T>
+__device__ __forceinline__ void gm_column(GmShared<T>& sh, int k, const GmArgs& a, bool berr) {
+  const double n2 = sh.nrm2, c = sh.run, den2 = fma(c, c, n2);
+  const double inv = rsqrt(n2), hk1 = n2 > 0.0 ? n2 * inv : sqrt(n2);
+  const double rden = rsqrt(den2), den = den2 > 0.0 ? den2 * rden : sqrt(den2);
+  const double sk = hk1 * rden, ck = c * rden;
+  sh.cs[k] = ck;
+  sh.sn[k] = sk;
   sh.H[k][k] = den;
-  const double gk = sh.g[k], gn = -sh.sn[k] * gk;
+  const double gk = sh.g[k], gn = -sk * gk;
   sh.g[k + 1] = gn;
-  sh.g[k] = sh.cs[k] * gk;
+  sh.g[k] = ck * gk;
   sh.its += 1;
   sh.nres = fabs(gn);
-  sh.scale[k + 1] = 1.0 / hk1;
-  sh.invh = (T)sh.scale[k + 1];
+  sh.scale[k + 1] = inv;
   if (!isfinite(den) || den == 0.0 || berr) sh.done = 2;
   else if (fabs(gn) < sh.tol || sh.its >= a.maxit || k + 1 == a.m || hk1 == 0.0) sh.cycle_done = 1;
 }
 
-template <int KT, class T>
-__global__ void __launch_bounds__(kGmMaxBlock, 1) k_gm_fused(Offsets of, const T* __restrict__ B,
-                                                             const T* __restrict__ dinv, T* x, T* z, T* wg, T* V,
-                                                             GmArgs a) {
+// w = B z over a block's rows (B, z, w at the block's first row).  The row's addresses are
+// formed inside the loop, from a stride and a base the compiler cannot see through: hoisted
+// out of it they took 4 K registers, and the row's 2 K loads went out a few at a time.
+// STREAM: the matrix goes past L2 (evict first), which the basis vectors then keep (P1 129^3 in
+// single precision: product 26.8 -> 24.9 us, dots 13.9 -> 10.4 us).
+template <int KT, bool STREAM, class T>
+__device__ __forceinline__ void gm_product(const Offsets& of, int64_t N, const T* __restrict__ B, const T* z, T* w,
+                                           int nrow, int nt) {
   const int K = KT > 0 ? KT : of.K;
-  const int64_t N = a.N, G = gridDim.x;
-  const int64_t i0 = N * blockIdx.x / G;
-  const int nrow = (int)(N * (blockIdx.x + 1) / G - i0), nt = blockDim.x;
-  const size_t vs = a.vstride;
+#pragma unroll 1
+  for (int r = threadIdx.x; r < nrow; r += nt) {
+    int64_t n = N;
+    const T* zr = z + r;
+    asm volatile("" : "+l"(n), "+l"(zr));
+    const T* br = B + r;
+    T s = 0;
+#pragma unroll
+    for (int q = 0; q < K; ++q) s = fma(STREAM ? __ldcs(br + q * n) : br[q * n], zr[of.o[q]], s);
+    w[r] = s;
+  }
+}
+
+// VS: the basis in shared memory.
+template <int KT, class T, bool VS>
+__global__ void __launch_bounds__(VS ? kGmBlockS : kGmBlock, 1) k_gm_fused(Offsets of, const T* __restrict__ B,
+                                                             const T* __restrict__ dinv, T* x, T* z, T* wg, T* Vg,
+                                                             GmArgs a) {
+  constexpr int W = Pack<T>::W;
+  const int64_t N = a.N;
+  const int64_t units = (N + kGmUnit - 1) / kGmUnit;
+  const int64_t i0 = units * blockIdx.x / gridDim.x * kGmUnit;
+  const int64_t i1 = units * (blockIdx.x + 1) / gridDim.x * kGmUnit;
+  const int nrow = (int)((i1 < N ? i1 : N) - i0);
+  const int nt = a.compute;                       // threads with rows; the last warp has the scalars
+  const bool rows_warp = (int)threadIdx.x < nt, scalar = (int)threadIdx.x == nt;   // scalar: its first lane
+  const int ng = (nrow + W - 1) / W;              // 16-byte groups; the last one may reach past N
+  const int nw = min(nt, (ng + 31) / 32 * 32) / 32;   // warps that hold any
   __shared__ GmShared<T> sh;
-  extern __shared__ char dyn[];
-  T* w = a.w_in_smem ? reinterpret_cast<T*>(dyn) : wg + i0;
+  extern __shared__ __align__(16) char dyn[];
+  // w (and V) of this block: in shared memory, or at its rows in global memory.  The tail of
+  // the last group is zero and stays so (w, V and B z are 0 there).
+  T* const w = VS || a.w_in_smem ? reinterpret_cast<T*>(dyn) : wg + i0;
+  T* const V = VS ? reinterpret_cast<T*>(dyn) + a.rows : Vg + i0;
+  const size_t vs = VS ? (size_t)a.rows : a.vstride;
+  for (int r = nrow + threadIdx.x; r < ng * W; r += blockDim.x) w[r] = (T)0;
   volatile int* berr = &a.bar->err;
   int buf = 0;
-  if (threadIdx.x == 0) {
+  if (scalar) {
     sh.its = 0;
     sh.cycles = 0;
     sh.done = 0;
@@ -682,22 +884,29 @@ __global__ void __launch_bounds__(kGmMaxBlock, 1) k_gm_fused(Offsets of, const T
   bool have_x = false;   // x = 0 until the first cycle's update
   for (;;) {
     // true residual v_0 = rhs - B x, z = D^{-1} v_0, ||v_0||
-    T nrm = 0;
-    for (int r = threadIdx.x; r < nrow; r += nt) {
-      const int64_t i = i0 + r;
-      T s = 0;
-      if (have_x) {
+    if (have_x && rows_warp) gm_product<KT, !VS>(of, N, B + i0, x + i0, w, nrow, nt);
+    __syncthreads();
+    if (rows_warp) {
+      T nrm = 0;
+#pragma unroll 1
+      for (int g = threadIdx.x; g < ng; g += nt) {
+        Pack<T> v;
 #pragma unroll
-        for (int k = 0; k < K; ++k) s = fma(B[k * N + i], x[i + of.o[k]], s);
+        for (int e = 0; e < W; ++e) {
+          const int r = g * W + e;
+          v.e[e] = (T)0;
+          if (r < nrow) {
+            v.e[e] = have_x ? (T)a.rhs[i0 + r] - w[r] : (T)a.rhs[i0 + r];
+            z[i0 + r] = dinv[i0 + r] * v.e[e];
+          }
+          nrm = fma(v.e[e], v.e[e], nrm);
+        }
+        *reinterpret_cast<Pack<T>*>(V + g * W) = v;
       }
-      const T wi = (T)a.rhs[i] - s;
-      V[i] = wi;
-      z[i] = dinv[i] * wi;
-      nrm = fma(wi, wi, nrm);
+      gm_put(sh, nrm, 0);
     }
-    gm_put(sh, nrm, 0);
-    gm_grid_sums(sh, 1, a, buf);
-    if (threadIdx.x == 0) {
+    gm_exchange(sh, 1, nw, a, buf, [&]() {
+      if (threadIdx.x != 0) return;
       const double beta = sqrt(sh.tot[0]);
       if (!have_x) {
         sh.n0 = beta;
@@ -711,71 +920,66 @@ __global__ void __launch_bounds__(kGmMaxBlock, 1) k_gm_fused(Offsets of, const T
       else if (sh.its >= a.maxit) sh.done = 4;
       sh.g[0] = beta;
       sh.scale[0] = 1.0 / beta;
-      sh.invh = (T)sh.scale[0];
-    }
-    __syncthreads();
+    });
     if (sh.done != 0) break;
     int ku = 0;   // columns of this cycle
     for (int k = 0;; ++k) {
-      // (1) w = B z / ||v_k||, dots with v_0 .. v_k, ||w||^2
-      const T ih = sh.invh;
-      nrm = 0;
-      for (int r = threadIdx.x; r < nrow; r += nt) {
-        const int64_t i = i0 + r;
-        T s = 0;
-#pragma unroll
-        for (int q = 0; q < K; ++q) s = fma(B[q * N + i], z[i + of.o[q]], s);
-        s *= ih;
-        w[r] = s;
-        nrm = fma(s, s, nrm);
+      // (1) w = B z and its dots; meanwhile the scalar warp ends column k - 1
+      if (rows_warp) {
+        gm_product<KT, !VS>(of, N, B + i0, z + i0, w, nrow, nt);
+      } else if (scalar && k > 0) {
+        gm_column(sh, k - 1, a, *berr != 0);
       }
-      gm_dots(sh, w, V, vs, i0, nrow, k);
-      gm_put(sh, nrm, k + 1);
-      gm_grid_sums(sh, k + 2, a, buf);
       __syncthreads();
-      if (threadIdx.x < 32) {
+      ku = k;
+      if (sh.done != 0 || (k > 0 && sh.cycle_done != 0)) break;
+      gm_dots(sh, w, V, vs, ng, nw, nt, k);
+      // h1 and the projection's coefficients: w stands for w / ||v_k||, v_q for v_q / ||v_q||
+      gm_exchange(sh, k + 2, nw, a, buf, [&]() {
         const int q = threadIdx.x;
+        const double sk = sh.scale[k], ww = sh.tot[k + 1] * (sk * sk);
         double h = 0.0;
         if (q <= k) {
-          h = sh.tot[q] * sh.scale[q];
+          const double sq = sh.scale[q];
+          h = sh.tot[q] * (sq * sk);
           sh.h1[q] = h;
           sh.h2[q] = 0.0;
-          sh.hs[q] = (T)(h * sh.scale[q]);
+          sh.hs[q] = (T)(h * sq);
         }
-        const double proj = warp_sum(h * h);
-        const double ww = sh.tot[k + 1];
-        if (q == 0) sh.skip = ww - proj >= 0.5 * ww && ww > 0.0;
-      }
-      __syncthreads();
-      if (!sh.skip) {   // second projection: w -= V h1, h2 = V^T w
-        for (int r = threadIdx.x; r < nrow; r += nt) w[r] = gm_project(sh, w[r], V, vs, i0 + r, k);
-        gm_dots(sh, w, V, vs, i0, nrow, k);
-        gm_grid_sums(sh, k + 1, a, buf);
-        __syncthreads();
-        if ((int)threadIdx.x <= k) {
-          const double h = sh.tot[threadIdx.x] * sh.scale[threadIdx.x];
-          sh.h2[threadIdx.x] = h;
-          sh.hs[threadIdx.x] = (T)(h * sh.scale[threadIdx.x]);
+        const float hf = (float)h, wf = (float)ww, rest = wf - warp_sum(hf * hf);   // the test needs no more
+        if (q == 0) {
+          sh.ih = (T)sk;
+          sh.skip = rest >= 0.5f * wf && wf > 0.f;
         }
-        __syncthreads();
+      });
+      const bool skip = sh.skip;
+      if (!skip) {   // second projection: w = w - V h1, h2 = V^T w, ||w||^2
+        if (rows_warp) gm_reproject(sh, w, V, vs, ng, nt, k);
+        // a thread's dots read the groups it wrote
+        gm_dots(sh, w, V, vs, ng, nw, nt, k);
+        gm_exchange(sh, k + 2, nw, a, buf, [&]() {
+          const int q = threadIdx.x;
+          if (q <= k) {
+            const double sq = sh.scale[q], h = sh.tot[q] * sq;
+            sh.h2[q] = h;
+            sh.hs[q] = (T)(h * sq);
+          }
+          if (q == 0) {
+            sh.nrm2 = sh.tot[k + 1];
+            sh.ih = (T)1;
+          }
+        });
       }
-      // (2) v_{k+1} = w - V h, z = D^{-1} v_{k+1}, ||v_{k+1}||^2
-      nrm = 0;
-      T* vn = V + (size_t)(k + 1) * vs;
-#pragma unroll 2
-      for (int r = threadIdx.x; r < nrow; r += nt) {
-        const int64_t i = i0 + r;
-        const T wi = gm_project(sh, w[r], V, vs, i, k);
-        vn[i] = wi;
-        z[i] = dinv[i] * wi;
-        nrm = fma(wi, wi, nrm);
+      // (2) v_{k+1} = w - V h, z = D^{-1} v_{k+1}, ||v_{k+1}||^2; meanwhile the scalar warp
+      // rotates column k
+      if (rows_warp) {
+        gm_complete(sh, w, V, vs, ng, nt, k, dinv + i0, z + i0, nrow, skip);
+      } else {
+        gm_rotate(sh, k, !skip);
       }
-      gm_put(sh, nrm, 0);
-      gm_grid_sums(sh, 1, a, buf);
-      if (threadIdx.x == 0) gm_column(sh, k, a, *berr != 0);
-      __syncthreads();
-      ku = k + 1;
-      if (sh.done != 0 || sh.cycle_done != 0) break;
+      gm_exchange(sh, skip ? 1 : 0, nw, a, buf, [&]() {
+        if (skip && threadIdx.x == 0) sh.nrm2 = sh.tot[0];
+      });
     }
     if (sh.done != 0) break;
     // H y = g (columns from the last; lane c keeps g[c]), then x += D^{-1} sum_q y_q v_q / ||v_q||
@@ -783,41 +987,32 @@ __global__ void __launch_bounds__(kGmMaxBlock, 1) k_gm_fused(Offsets of, const T
       const int c = threadIdx.x;
       double gc = c < ku ? sh.g[c] : 0.0;
       const double inv = c < ku ? 1.0 / sh.H[c][c] : 0.0;
+#pragma unroll 1
       for (int q = ku - 1; q >= 0; --q) {
         const double yq = __shfl_sync(0xffffffffu, gc * inv, q);
         if (c == q) sh.y[q] = yq;
         if (c < q) gc = fma(-sh.H[c][q], yq, gc);
       }
       __syncwarp();
-      if (c < ku) sh.hs[c] = (T)(sh.y[c] * sh.scale[c]);
+      if (c < ku) sh.hs[c] = (T)(-sh.y[c] * sh.scale[c]);
     }
     __syncthreads();
-    for (int r = threadIdx.x; r < nrow; r += nt) {
-      const int64_t i = i0 + r;
-      T s = 0;
-      for (int q0 = 0; q0 < ku; q0 += 8) {
-        T v[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) v[j] = q0 + j < ku ? V[(size_t)(q0 + j) * vs + i] : (T)0;
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-          if (q0 + j < ku) s = fma(sh.hs[q0 + j], v[j], s);
-      }
-      const T d = dinv[i] * s;
-      x[i] = have_x ? x[i] + d : d;
+    if (rows_warp) {
+      gm_update(sh, w, V, vs, ng, nt, ku, dinv + i0, x + i0, nrow, have_x);
     }
     have_x = true;
-    grid_barrier(a.bar, a.wait_ns);   // the next residual gathers x
+    gm_exchange(sh, 0, nw, a, buf, [] {});   // a barrier: the next residual gathers x
   }
   // the solution, and the caller's update unless the solve broke down
   const bool upd = a.ep.u != nullptr && sh.done != 2;
-  for (int r = threadIdx.x; r < nrow; r += nt) {
+#pragma unroll 1
+  for (int r = threadIdx.x; r < nrow; r += blockDim.x) {
     const int64_t i = i0 + r;
     const double xi = have_x ? (double)x[i] : 0.0;
     a.xout[i] = xi;
     if (upd) krylov_update(a.ep, i, xi);
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
+  if (blockIdx.x == 0 && scalar) {
     double* sc = a.sc;
     sc[S_N0] = sh.n0;
     sc[S_TOL] = sh.tol;
@@ -845,11 +1040,23 @@ void krylov_free(afc_problem_s* p) {
 
 namespace {
 
+// The device must run cooperative launches (GB300 does); its SM count, asked once.
+int coop_device(afc_problem_s* p) {
+  KrylovWork& w = *p->kw;
+  if (w.nsm > 0) return AFC_OK;
+  int c = 0;
+  AFC_CUDA(cudaDeviceGetAttribute(&c, cudaDevAttrCooperativeLaunch, p->device));
+  if (!c) { set_error("the Krylov solvers need a device with cooperative launches"); return AFC_E_CUDA; }
+  AFC_CUDA(cudaDeviceGetAttribute(&w.nsm, cudaDevAttrMultiProcessorCount, p->device));
+  return AFC_OK;
+}
+
 int ensure_work(afc_problem_s* p, int nvec, bool fp32) {
   if (!p->kw) p->kw = new KrylovWork();
   KrylovWork& w = *p->kw;
   const size_t esz = fp32 ? sizeof(float) : sizeof(double);
-  const size_t vstride = (size_t)(p->N + 2 * p->pad + 32) & ~(size_t)31;
+  const size_t pad = ((size_t)p->pad + 31) & ~(size_t)31;   // vectors start on 16-byte boundaries
+  const size_t vstride = (((size_t)p->N + 31) & ~(size_t)31) + 2 * pad;
   const int64_t bytes = (int64_t)(nvec * vstride * esz);
   if (w.vec.base == nullptr || w.vec.n < bytes) {
     int st = w.vec.alloc(bytes);   // zero-filled
@@ -861,11 +1068,12 @@ int ensure_work(afc_problem_s* p, int nvec, bool fp32) {
   w.vstride = vstride;
   w.fp32 = fp32;
   w.N = p->N;
-  w.pad = p->pad;
+  w.pad = (int)pad;
   if (!w.sc.base) {
     int st = w.sc.alloc(S_END + 8);
     if (st) return st;
     if ((st = w.barrier.alloc(4))) return st;
+    if ((st = coop_device(p))) return st;
     if (cudaMallocHost((void**)&w.hsc, (S_END + 8) * sizeof(double)) != cudaSuccess) {
       set_error("cudaMallocHost failed");
       return AFC_E_OOM;
@@ -882,17 +1090,6 @@ int ensure_work(afc_problem_s* p, int nvec, bool fp32) {
 template <class T>
 T* vec_at(KrylovWork& w, int q) {
   return reinterpret_cast<T*>(w.vec.base) + q * w.vstride + w.pad;
-}
-
-// The device must run cooperative launches (GB300 does); its SM count, asked once.
-int coop_device(afc_problem_s* p) {
-  KrylovWork& w = *p->kw;
-  if (w.nsm > 0) return AFC_OK;
-  int c = 0;
-  AFC_CUDA(cudaDeviceGetAttribute(&c, cudaDevAttrCooperativeLaunch, p->device));
-  if (!c) { set_error("the Krylov solvers need a device with cooperative launches"); return AFC_E_CUDA; }
-  AFC_CUDA(cudaDeviceGetAttribute(&w.nsm, cudaDevAttrMultiProcessorCount, p->device));
-  return AFC_OK;
 }
 
 // The persistent BiCGStab launch on stream s (no synchronisation).
@@ -967,15 +1164,13 @@ int bicgstab_impl(afc_problem_s* p, const T* B, const T* dinv, const afc_opts* o
 }
 
 // The persistent GMRES launch on stream s (no synchronisation).  One block per SM at
-// most, of as many warps as its rows fill (64 to 1024 threads): small systems spread
-// over all SMs with few warps each, because a block's FP64 sums cost 16 cycles per warp,
-// and leave room for the launches of other streams.
+// most: small systems spread over all SMs with few warps each, because a block's FP64
+// sums cost 16 cycles per warp, and leave room for the launches of other streams.
 template <class T>
 int gmres_fused_launch(afc_problem_s* p, cudaStream_t s, const T* B, const T* dinv, const afc_opts* o,
                        const double* rhs, double* xout, const KrylovEpilogue* epi) {
   KrylovWork& w = *p->kw;
-  int st = coop_device(p);
-  if (st) return st;
+  int st = AFC_OK;
   const int64_t N = p->N;
   GmArgs a;
   a.N = N;
@@ -983,24 +1178,29 @@ int gmres_fused_launch(afc_problem_s* p, cudaStream_t s, const T* B, const T* di
   a.rhs = rhs;
   a.xout = xout;
   a.vstride = w.vstride;
-  a.part = w.part.p;
   a.bar = reinterpret_cast<GridBar*>(w.barrier.p);
+  a.part = w.part.p;
   a.atol = o->ksp_atol;
   a.rtol = o->ksp_rtol;
   a.maxit = o->ksp_maxit;
   a.m = o->gmres_restart;
   if (epi) a.ep = *epi;
   a.wait_ns = p->grid_wait_ns;
-  const int G = (int)std::max<int64_t>(1, std::min<int64_t>((N + 63) / 64, w.nsm));
-  const int64_t rows = (N + G - 1) / G;
-  const int block = (int)std::max<int64_t>(64, std::min<int64_t>(kGmMaxBlock, (rows + 31) / 32 * 32));
-  size_t smem = (size_t)rows * sizeof(T);
-  a.w_in_smem = smem <= kGmSmemW;
-  if (!a.w_in_smem) smem = 0;
+  const int64_t units = (N + kGmUnit - 1) / kGmUnit;
+  const int G = (int)std::max<int64_t>(1, std::min<int64_t>((units + 1) / 2, std::min(w.nsm, 160)));
+  const int64_t rows = (units + G - 1) / G * kGmUnit;   // most rows of a block
+  const size_t vec = (size_t)rows * sizeof(T);
+  const bool vs = (size_t)(a.m + 2) * vec <= kGmSmem;   // w and V_0 .. V_m
+  a.w_in_smem = vec <= kGmSmem;
+  a.rows = (int)rows;
+  const size_t smem = vs ? (a.m + 2) * vec : a.w_in_smem ? vec : 0;
+  const int most = (vs ? kGmBlockS : kGmBlock) - 32;
+  a.compute = (int)std::max<int64_t>(kGmMinCompute, std::min<int64_t>(most, (rows + 31) / 32 * 32));
+  const int block = a.compute + 32;
   with_K(p->K, [&](auto kc) {
     constexpr int KT = decltype(kc)::value;
-    auto kern = k_gm_fused<KT, T>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGmSmemW);
+    auto kern = vs ? k_gm_fused<KT, T, true> : k_gm_fused<KT, T, false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGmSmem);
     int nb = 0;
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, block, smem);
     if (e != cudaSuccess || nb < 1) {

@@ -129,7 +129,7 @@ struct afc_problem_s {
   afc::DBuf<double> d2_up;                        // Kup * N, MC: 2 |d_ij|
   afc::DBuf<float> pairf;                         // 3 * Kup * N, MC: 2|d_ij|, k_ij, k_ji rounded to single
   afc::DBuf<double> AG;                           // K * N, MC: unlimited operator K + eps S + c M_L
-  afc::DBuf<double> mL, f;                        // N
+  afc::DBuf<double> mL, imL, f;                   // N; imL = 1 / mL
   afc::DBuf<double> Bst;                          // K * N, stationary system (Dirichlet rows = identity)
   afc::DBuf<float> Bst32;
   afc::DBuf<double> dinv_st;
@@ -160,6 +160,7 @@ struct afc_problem_s {
   // mixed-precision explicit stage: m_ij, d_ij, r_ij (Kup * N) and u, udot^L (node vectors) in single
   afc::DBuf<float> m32_up, d32_up, r32, uf, udf;
   bool ssp32_ready = false;         // m32_up / d32_up match the assembled m_up / d_up
+  afc::DBuf<long long> range;       // k_range: running max and min keys, blocks done
   afc::DBuf<double> scal;           // small device scalars (norms, dt, ...)
   afc::DBuf<double> part;           // reduction partials
   double* host_scal = nullptr;      // pinned host mirror of scal
@@ -188,8 +189,11 @@ int build_cn_system(afc_problem_s* p, double dt);
 
 // ---- kernels of the hot path (fct.cu, mc.cu) ----
 // SSP forward-Euler stage: out = a * uA + b * FE(uin) (Eq. FE-SSP with Zalesak).
+// pdl: the stage's first pass follows another pass of the step (programmatic dependent launch)
 int fe_stage(afc_problem_s* p, const double* uin, double dt, int limiter, double a, const double* uA, double b,
-             double* out, bool mixed = false);
+             double* out, bool mixed = false, bool pdl = false);
+// the stages of one SSP2 / SSP3 step of the stored solution, in place
+int ssp_stages(afc_problem_s* p, const afc_opts* o);
 int ensure_ssp_mixed(afc_problem_s* p);   // single-precision copies of m_ij, d_ij for the mixed stage
 struct SspArrays;
 SspArrays ssp_arrays(afc_problem_s* p);
@@ -228,7 +232,12 @@ struct KrylovEpilogue {
   const double* uo = nullptr;
   double* a = nullptr;
   double* s = nullptr;
-  double* fp_sc = nullptr;   // graph form: the fixed-point scalars, where the solve counts itself
+  // graph form of the fixed point: its scalars, the residual's block partials and the loop's
+  // condition; the solve's launch decides whether the loop goes on, and counts itself
+  double* fp_sc = nullptr;
+  const double* part = nullptr;
+  int npart = 0;
+  cudaGraphConditionalHandle loop = 0;
 };
 // The updates of the fixed points: of a CN step, and of a stationary solve.
 inline KrylovEpilogue stationary_epilogue(afc_problem_s* p, const afc_opts* o) {
@@ -248,6 +257,7 @@ inline KrylovEpilogue step_epilogue(afc_problem_s* p, const afc_opts* o) {
 int krylov_solve(afc_problem_s* p, int system, const afc_opts* o, const double* rhs, double* x, int* its,
                  double* res, const KrylovEpilogue* epi = nullptr);
 int dia_spmv(afc_problem_s* p, const double* A, const double* x, double* y);
+int range_device(afc_problem_s* p, const double* x);   // min, max of x (and the scalars) into the host mirror
 int minmax_device(afc_problem_s* p, const double* x, double* mn, double* mx);
 void krylov_free(afc_problem_s* p);
 const void* krylov_key(afc_problem_s* p);   // changes when the solver workspace is reallocated

@@ -85,11 +85,13 @@ int create_common(afc_problem_s* p) {
                           &p->umin, &p->tmp, &p->cn_a, &p->cn_s, &p->bA, &p->bB, &p->Fold};
   for (auto* v : vecs)
     if ((st = v->alloc(N, p->pad))) return st;
-  if ((st = p->scal.alloc(64)) || (st = p->part.alloc(4 * std::max<int64_t>(kRedBlocks, grid_for(N))))) return st;
+  if ((st = p->range.alloc(4)) || (st = p->scal.alloc(64)) || (st = p->part.alloc(4 * std::max<int64_t>(kRedBlocks, grid_for(N))))) return st;
   if (cudaMallocHost((void**)&p->host_scal, 64 * sizeof(double)) != cudaSuccess) {
     set_error("cudaMallocHost failed");
     return AFC_E_OOM;
   }
+  const long long empty[4] = {INT64_MIN, INT64_MAX, 0, 0};   // k_range starts from and leaves this
+  AFC_CUDA(cudaMemcpyAsync(p->range.p, empty, sizeof(empty), cudaMemcpyHostToDevice, p->stream));
   cudaStream_t s = p->stream;
   AFC_CUDA(cudaMemcpyAsync(p->xyz.p, m.xyz.data(), 3 * N * sizeof(double), cudaMemcpyHostToDevice, s));
   AFC_CUDA(cudaMemcpyAsync(p->conn.p, m.conn.data(), m.conn.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
@@ -107,7 +109,7 @@ void destroy_all(afc_problem_s* p) {
   prof_free(p);
   krylov_free(p);
   DBuf<double>* dv[] = {&p->xyz, &p->bnod, &p->fnod, &p->udir, &p->Mfull, &p->Sfull, &p->Kfull, &p->Afull,
-                        &p->AA, &p->m_up, &p->d_up, &p->mL, &p->f, &p->Bst, &p->dinv_st, &p->Bcn, &p->dinv_cn,
+                        &p->AA, &p->m_up, &p->d_up, &p->mL, &p->imL, &p->f, &p->Bst, &p->dinv_st, &p->Bcn, &p->dinv_cn,
                         &p->u, &p->u0, &p->ustage, &p->udot, &p->ut, &p->Rp, &p->Rm, &p->Fs, &p->Qp, &p->Qm,
                         &p->b0, &p->res, &p->delta, &p->umax, &p->umin, &p->tmp, &p->cn_a, &p->cn_s,
                         &p->scal, &p->part, &p->r_up, &p->mdt_up, &p->mLdt, &p->kij_up, &p->kji_up,
@@ -115,7 +117,7 @@ void destroy_all(afc_problem_s* p) {
   for (auto* b : dv) b->free_();
   p->Bst32.free_(); p->dinv_st32.free_(); p->Bcn32.free_(); p->dinv_cn32.free_();
   p->conn.free_(); p->inc_ptr.free_(); p->inc.free_(); p->mask.free_(); p->dir.free_(); p->clip.free_();
-  p->pairf.free_(); p->nodef.free_();
+  p->pairf.free_(); p->nodef.free_();  p->range.free_();
   p->AGp.free_(); p->fp2.free_(); p->pk_hi.free_(); p->pk_lo.free_(); p->up2.free_(); p->yp2.free_(); p->abh2.free_(); p->abl2.free_();
   p->cp_up.free_(); p->mask32.free_(); p->clip32.free_(); p->mask16.free_(); p->clip16.free_();
   p->m32_up.free_(); p->d32_up.free_(); p->r32.free_(); p->uf.free_(); p->udf.free_();
@@ -464,7 +466,6 @@ int step_impl(afc_problem p, const afc_opts* o, afc_stats* stt) {
   }
   const int cn_family = lim == AFC_LIM_MC ? AFC_FAMILY_MC : AFC_FAMILY_FCT;
   cudaStream_t s = p->stream;
-  const bool mixed = o->precision == AFC_MIXED;
   const bool graph = o->graph != 0;   // captured on a private stream, launched on the problem's stream
   if (graph && (o->scheme == AFC_SSP2 || o->scheme == AFC_SSP3)) return ssp_step_graph(p, o, stt);
   // linear Zal+CN: one undamped correction from 2 u~ - u_old solves its linear system
@@ -481,23 +482,15 @@ int step_impl(afc_problem p, const afc_opts* o, afc_stats* stt) {
     if ((st = build_cn_system(p, o->dt))) return st;
     return cn_step_graph(p, o, stt);
   }
-  AFC_CUDA(cudaMemcpyAsync(p->u0.p, p->u.p, N * sizeof(double), cudaMemcpyDeviceToDevice, s));
-  if (o->scheme == AFC_SSP2) {
-    if ((st = fe_stage(p, p->u0.p, o->dt, lim, 0.0, nullptr, 1.0, p->ustage.p, mixed))) return st;
-    if ((st = fe_stage(p, p->ustage.p, o->dt, lim, 0.5, p->u0.p, 0.5, p->u.p, mixed))) return st;
-    if (stt) stt->stages = 2;
-    return finish_stats(p, stt, AFC_OK);
-  }
-  if (o->scheme == AFC_SSP3) {
-    if ((st = fe_stage(p, p->u0.p, o->dt, lim, 0.0, nullptr, 1.0, p->ustage.p, mixed))) return st;
-    if ((st = fe_stage(p, p->ustage.p, o->dt, lim, 0.75, p->u0.p, 0.25, p->tmp.p, mixed))) return st;
-    if ((st = fe_stage(p, p->tmp.p, o->dt, lim, 1.0 / 3.0, p->u0.p, 2.0 / 3.0, p->u.p, mixed))) return st;
-    if (stt) stt->stages = 3;
+  if (o->scheme == AFC_SSP2 || o->scheme == AFC_SSP3) {
+    if ((st = ssp_stages(p, o))) return st;
+    if (stt) stt->stages = o->scheme == AFC_SSP2 ? 2 : 3;
     return finish_stats(p, stt, AFC_OK);
   }
   if (!cn) { set_error("unknown scheme"); return AFC_E_INVALID; }
   if (p->family != cn_family) { set_error("CN FCT needs the FCT family"); return AFC_E_STATE; }
   if ((st = build_cn_system(p, o->dt))) return st;
+  AFC_CUDA(cudaMemcpyAsync(p->u0.p, p->u.p, N * sizeof(double), cudaMemcpyDeviceToDevice, s));
   if ((st = cn_predictor(p, p->u0.p, o->dt))) return st;
   if (lim == AFC_LIM_MC) {
     // CN with the MC limiter: F* = (F*(u) + F*(u_old)) / 2, plain damped updates

@@ -206,8 +206,8 @@ __global__ void k_assemble_rows(int64_t N, Offsets of, const double* __restrict_
 __global__ void k_lumped_and_A(int64_t N, Offsets of, int family, double eps, double c, const double* __restrict__ Mf,
                                const double* __restrict__ Sf, const double* __restrict__ Kf,
                                const double* __restrict__ Rf, const double* __restrict__ fn,
-                               double* __restrict__ mL, double* __restrict__ f, double* __restrict__ rl,
-                               double* __restrict__ Af) {
+                               double* __restrict__ mL, double* __restrict__ imL, double* __restrict__ f,
+                               double* __restrict__ rl, double* __restrict__ Af) {
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= N) return;
   double s = 0.0, sr = 0.0;
@@ -215,6 +215,7 @@ __global__ void k_lumped_and_A(int64_t N, Offsets of, int family, double eps, do
   if (Rf)
     for (int k = 0; k < of.K; ++k) sr += Rf[k * N + i];
   mL[i] = s;
+  imL[i] = 1.0 / s;
   f[i] = s * fn[i];
   rl[i] = Rf ? sr : c * s;
   for (int k = 0; k < of.K; ++k) {
@@ -327,7 +328,7 @@ int assemble_device(afc_problem_s* p, int family, int precision) {
   int st;
   if ((st = p->Mfull.alloc(K * N)) || (st = p->Sfull.alloc(K * N)) || (st = p->Kfull.alloc(K * N)) ||
       (st = p->Afull.alloc(K * N)) || (st = p->AA.alloc(K * N)) || (st = p->m_up.alloc(Kup * N)) ||
-      (st = p->d_up.alloc(Kup * N)) || (st = p->mL.alloc(N, p->pad)) || (st = p->f.alloc(N, p->pad)) ||
+      (st = p->d_up.alloc(Kup * N)) || (st = p->mL.alloc(N, p->pad)) || (st = p->imL.alloc(N)) || (st = p->f.alloc(N, p->pad)) ||
       (st = p->Bst.alloc(K * N)) || (st = p->dinv_st.alloc(N, p->pad)) || (st = p->r_up.alloc(Kup * N)) ||
       (st = p->rl.alloc(N, p->pad)))
     return st;
@@ -344,7 +345,7 @@ int assemble_device(afc_problem_s* p, int family, int precision) {
                                                          p->inc.p, p->Mfull.p, p->Sfull.p, p->Kfull.p, cn, Rf));
   AFC_CUDA(cudaGetLastError());
   AFC_LAUNCH(p, "k_lumped_and_A", k_lumped_and_A<<<g, kBlock, 0, s>>>(N, p->offs, family, p->eps, p->c, p->Mfull.p, p->Sfull.p, p->Kfull.p, Rf,
-                                      p->fnod.p, p->mL.p, p->f.p, p->rl.p, p->Afull.p));
+                                      p->fnod.p, p->mL.p, p->imL.p, p->f.p, p->rl.p, p->Afull.p));
   AFC_LAUNCH(p, "k_upwind_edges", k_upwind_edges<<<g, kBlock, 0, s>>>(N, p->offs, p->mask.p, p->Afull.p, p->d_up.p));
   AFC_LAUNCH(p, "k_low_order", k_low_order<<<g, kBlock, 0, s>>>(N, p->offs, family, p->eps, p->rl.p, p->mask.p, p->Afull.p, p->Sfull.p,
                                    p->d_up.p, p->AA.p));

@@ -8,7 +8,12 @@
 // small instances is one launch that fills the GPU instead of 256 launches that
 // each fill a few SMs.
 //
-// Launch shapes.  PER_PASS: one ordinary launch per pass, one tile per block.
+// Launch shapes.  PER_PASS (the default): one ordinary launch per pass, one tile per block,
+// each pass a kernel of its own: 32 registers for the rate and edge passes, 40 for the other
+// two with three neighbours' loads in flight.  As one kernel that held all passes and patterns
+// (64 registers, offsets and pointers searched per tile) 15 stages of 48 mixed Q1 instances (17 to
+// 49 nodes per side) took 12.4 ms, now 7.0 ms; at 64 registers and nine loads 7.9 ms, at 32
+// registers 6.9 ms but a small double-precision batch 7 % slower.
 // PER_STAGE / PER_STEP: one persistent cooperative launch per stage / per time
 // step; each block takes a contiguous range of tiles (neighbouring rows, few
 // instance switches) and the passes are separated by a grid-wide barrier.  The
@@ -54,7 +59,9 @@ struct StageArgs {
   double ca[3], cb[3];
 };
 
-template <int KT, bool MIXED>
+// S: neighbours whose loads a row issues together (the persistent kernel, which holds all
+// passes, takes them one by one to save registers)
+template <int KT, bool MIXED, int S>
 __device__ __forceinline__ void batch_row(const BInst& in, int phase, int st, const StageArgs& sa, int limiter,
                                           int64_t i) {
   const double dt = in.dt;
@@ -66,11 +73,11 @@ __device__ __forceinline__ void batch_row(const BInst& in, int phase, int st, co
       ssp_edges_row<KT, MIXED>(in.of, in.a, i, in.vec[sa.in[st]]);
       break;
     case 2:
-      ssp_factors_row<KT, MIXED>(in.of, in.a, i, dt);
+      ssp_factors_row<KT, MIXED, S>(in.of, in.a, i, dt);
       break;
     default: {
       const double* uA = sa.uA[st] >= 0 ? in.vec[sa.uA[st]] : nullptr;
-      ssp_correct_row<KT, MIXED>(in.of, in.a, i, limiter, dt, sa.ca[st], uA, sa.cb[st], in.vec[sa.out[st]]);
+      ssp_correct_row<KT, MIXED, S>(in.of, in.a, i, limiter, dt, sa.ca[st], uA, sa.cb[st], in.vec[sa.out[st]]);
     }
   }
 }
@@ -107,9 +114,9 @@ __device__ void batch_pass(const BInst* __restrict__ tab, int ninst, int64_t t0,
     const int64_t i = (t - sh_lo) * (int64_t)blockDim.x + threadIdx.x;
     if (i < sh.a.N) {
       const int K = sh.of.K;
-      if (K == 27) batch_row<27, MIXED>(sh, phase, st, sa, limiter, i);
-      else if (K == 15) batch_row<15, MIXED>(sh, phase, st, sa, limiter, i);
-      else batch_row<0, MIXED>(sh, phase, st, sa, limiter, i);
+      if (K == 27) batch_row<27, MIXED, 1>(sh, phase, st, sa, limiter, i);
+      else if (K == 15) batch_row<15, MIXED, 1>(sh, phase, st, sa, limiter, i);
+      else batch_row<0, MIXED, 1>(sh, phase, st, sa, limiter, i);
     }
   }
 }
@@ -120,9 +127,8 @@ __device__ __forceinline__ bool pass_needed(int phase, int limiter) {
   return true;
 }
 
-// Passes ph_lo..ph_hi of the stages in `sa`, over all tiles.  With a barrier
-// (persistent launches) block b takes the contiguous tile range b; without one
-// (ph_lo == ph_hi, one stage) the grid has a block per tile.
+// Passes ph_lo..ph_hi of the stages in `sa`, over all tiles: block b of the persistent
+// launch takes the contiguous tile range b.
 template <bool MIXED>
 __global__ void __launch_bounds__(512) k_batch_ssp(const BInst* __restrict__ tab, int ninst, int64_t ntiles,
                                                   StageArgs sa, int limiter, int ph_lo, int ph_hi, GridBar* bar) {
@@ -144,6 +150,24 @@ __global__ void __launch_bounds__(512) k_batch_ssp(const BInst* __restrict__ tab
       batch_pass<MIXED>(tab, ninst, t0, t1, ph, st, sa, limiter, sh, sh_lo, sh_hi);
     }
   }
+}
+
+// One pass (PH) over all tiles, a block per tile: map[tile] = (instance, tile of it).
+template <bool MIXED, int PH>
+__global__ void __launch_bounds__(512, PH < 2 ? 4 : 3) k_batch_pass(const BInst* __restrict__ tab, const int2* __restrict__ map,
+                                                    StageArgs sa, int limiter) {
+  __shared__ BInst sh;
+  const int2 at = map[blockIdx.x];
+  const unsigned int* src = reinterpret_cast<const unsigned int*>(tab + at.x);
+  unsigned int* dst = reinterpret_cast<unsigned int*>(&sh);
+  for (int w = threadIdx.x; w < (int)(sizeof(BInst) / 4); w += blockDim.x) dst[w] = src[w];
+  __syncthreads();
+  const int64_t i = (int64_t)at.y * blockDim.x + threadIdx.x;
+  if (i >= sh.a.N) return;
+  const int K = sh.of.K;
+  if (K == 27) batch_row<27, MIXED, 3>(sh, PH, 0, sa, limiter, i);
+  else if (K == 15) batch_row<15, MIXED, 3>(sh, PH, 0, sa, limiter, i);
+  else batch_row<0, MIXED, 1>(sh, PH, 0, sa, limiter, i);
 }
 
 // per instance: min and max of the stored solution
@@ -200,7 +224,9 @@ struct afc_batch_s {
   int64_t total_nodes = 0;
   afc::BInst* tab_h = nullptr;          // pinned
   afc::BInst* tab_d = nullptr;
+  int2* map_d = nullptr;                // tile -> (instance, tile of it), for the tiles of tab_block rows
   int tab_block = 0;                    // rows per tile the table was built for
+  int map_block = 0;                    // ... and the map
   std::vector<double> tab_dt;           // time steps in the table
   int64_t ntiles = 0;
   afc::GridBar* bar = nullptr;
@@ -258,8 +284,8 @@ afc_batch_tuning effective_tuning(afc_batch_s* b, const afc_opts* o) {
     if (it != g_tune_cache.end()) return it->second;
   }
   afc_batch_tuning t{};
-  t.mode = AFC_BATCH_PER_STAGE;
-  t.block = 256;
+  t.mode = AFC_BATCH_PER_PASS;
+  t.block = 128;
   t.blocks_per_sm = 0;
   return t;
 }
@@ -301,6 +327,15 @@ int build_table(afc_batch_s* b, int block, const double* dt, double dt_all, bool
   b->tab_block = block;
   b->tab_dt = dts;
   AFC_CUDA(cudaMemcpyAsync(b->tab_d, b->tab_h, b->list.size() * sizeof(BInst), cudaMemcpyHostToDevice, b->stream));
+  if (b->map_block != block) {
+    std::vector<int2> map((size_t)tile);
+    size_t t = 0;
+    for (size_t q = 0; q < b->list.size(); ++q)
+      for (int64_t u = 0; u < b->tab_h[q].ntiles; ++u) map[t++] = make_int2((int)q, (int)u);
+    AFC_CUDA(cudaMemcpyAsync(b->map_d, map.data(), map.size() * sizeof(int2), cudaMemcpyHostToDevice, b->stream));
+    AFC_CUDA(cudaStreamSynchronize(b->stream));   // `map` is pageable and goes
+    b->map_block = block;
+  }
   return AFC_OK;
 }
 
@@ -334,7 +369,7 @@ StageArgs step_args(int scheme) {
   return all;
 }
 
-int launch_batch(afc_batch_s* b, cudaStream_t s, bool mixed, bool coop, int grid, int block, StageArgs sa,
+int launch_batch(afc_batch_s* b, cudaStream_t s, bool mixed, int grid, int block, StageArgs sa,
                  int limiter, int lo, int hi) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
@@ -344,14 +379,32 @@ int launch_batch(afc_batch_s* b, cudaStream_t s, bool mixed, bool coop, int grid
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeCooperative;
   at[0].val.cooperative = 1;
-  cfg.attrs = coop ? at : nullptr;
-  cfg.numAttrs = coop ? 1 : 0;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
   const int ninst = (int)b->list.size();
   cudaError_t e = mixed ? cudaLaunchKernelEx(&cfg, k_batch_ssp<true>, (const BInst*)b->tab_d, ninst, b->ntiles, sa,
                                              limiter, lo, hi, b->bar)
                         : cudaLaunchKernelEx(&cfg, k_batch_ssp<false>, (const BInst*)b->tab_d, ninst, b->ntiles, sa,
                                              limiter, lo, hi, b->bar);
   if (e != cudaSuccess) return cuda_fail(e, "cudaLaunchKernelEx(k_batch_ssp)");
+  return AFC_OK;
+}
+
+// One pass over all instances.
+int launch_pass_of(afc_batch_s* b, cudaStream_t s, bool mixed, int block, const StageArgs& sa, int limiter,
+                   int ph) {
+  auto go = [&](auto kern) {
+    return launch_pass(false, kern, dim3((unsigned)b->ntiles), dim3((unsigned)block), s, (const BInst*)b->tab_d,
+                       (const int2*)b->map_d, sa, limiter);
+  };
+  cudaError_t e;
+  switch (ph) {
+    case 0: e = mixed ? go(k_batch_pass<true, 0>) : go(k_batch_pass<false, 0>); break;
+    case 1: e = mixed ? go(k_batch_pass<true, 1>) : go(k_batch_pass<false, 1>); break;
+    case 2: e = mixed ? go(k_batch_pass<true, 2>) : go(k_batch_pass<false, 2>); break;
+    default: e = mixed ? go(k_batch_pass<true, 3>) : go(k_batch_pass<false, 3>);
+  }
+  if (e != cudaSuccess) return cuda_fail(e, "cudaLaunchKernelEx(k_batch_pass)");
   return AFC_OK;
 }
 
@@ -379,7 +432,7 @@ int enqueue_step(afc_batch_s* b, cudaStream_t s, const afc_opts* o, const afc_ba
       for (int ph = 0; ph < 4; ++ph) {
         if (ph == 1 && o->limiter == AFC_LIM_NONE) continue;
         if (ph == 2 && o->limiter != AFC_LIM_ZALESAK) continue;
-        if ((st = launch_batch(b, s, mixed, false, (int)b->ntiles, t.block, sa, o->limiter, ph, ph))) return st;
+        if ((st = launch_pass_of(b, s, mixed, t.block, sa, o->limiter, ph))) return st;
         ++*nl;
       }
     }
@@ -387,12 +440,12 @@ int enqueue_step(afc_batch_s* b, cudaStream_t s, const afc_opts* o, const afc_ba
   }
   if (t.mode == AFC_BATCH_PER_STAGE) {
     for (int sidx = 0; sidx < ns; ++sidx) {
-      if ((st = launch_batch(b, s, mixed, true, grid, t.block, stage_args(o->scheme, sidx), o->limiter, 0, 3)))
+      if ((st = launch_batch(b, s, mixed, grid, t.block, stage_args(o->scheme, sidx), o->limiter, 0, 3)))
         return st;
       ++*nl;
     }
   } else {
-    if ((st = launch_batch(b, s, mixed, true, grid, t.block, step_args(o->scheme), o->limiter, 0, 3))) return st;
+    if ((st = launch_batch(b, s, mixed, grid, t.block, step_args(o->scheme), o->limiter, 0, 3))) return st;
     ++*nl;
   }
   return AFC_OK;
@@ -564,6 +617,7 @@ void batch_free(afc_batch_s* b) {
   if (b->tab_h) cudaFreeHost(b->tab_h);
   if (b->mm_h) cudaFreeHost(b->mm_h);
   if (b->tab_d) cudaFree(b->tab_d);
+  if (b->map_d) cudaFree(b->map_d);
   if (b->bar) cudaFree(b->bar);
   if (b->mm_d) cudaFree(b->mm_d);
   if (b->backup) cudaFree(b->backup);
@@ -621,7 +675,10 @@ int afc::batch_create_on_stream(const afc_problem* list, int count, cudaStream_t
   if ((e = cudaMallocHost((void**)&b->tab_h, count * sizeof(BInst))) != cudaSuccess ||
       (e = cudaMallocHost((void**)&b->mm_h, (2 * count + 1) * sizeof(double))) != cudaSuccess)
     return fail(cuda_fail(e, "cudaMallocHost"));
+  int64_t most_tiles = 0;   // at the smallest tile size
+  for (auto* p : b->list) most_tiles += (p->N + 127) / 128;
   if ((e = cudaMalloc((void**)&b->tab_d, count * sizeof(BInst))) != cudaSuccess ||
+      (e = cudaMalloc((void**)&b->map_d, most_tiles * sizeof(int2))) != cudaSuccess ||
       (e = cudaMalloc((void**)&b->bar, sizeof(GridBar))) != cudaSuccess ||
       (e = cudaMalloc((void**)&b->mm_d, 2 * count * sizeof(double))) != cudaSuccess) {
     cudaGetLastError();

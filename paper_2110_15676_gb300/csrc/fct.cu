@@ -20,30 +20,48 @@ namespace {
 
 // ---- explicit stage (per-row arithmetic in ssp_rows.cuh) ------------------------
 
+// On grids of at most kPdlRows rows consecutive passes of a step are launched with
+// programmatic dependent launch: a pass lets the next one launch once all its blocks run,
+// and waits for the one before it (which has waited for its own predecessor) before it
+// touches anything a pass writes.  On larger grids the waiting blocks take the place of
+// running ones (SSP3 step in double, us, with / without: P1 9^3 62 / 68, Q1 17^3 81 / 86, Q1 25^3
+// 84 / 86, Q1 33^3 113 / 90, Q1 41^3 179 / 117).
+constexpr int64_t kPdlRows = 16384;
+
 template <int KT, bool MIXED>
 __global__ void k_ssp_rate(Offsets of, SspArrays a, const double* __restrict__ u, double dt) {
+  pdl_trigger();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  pdl_wait();
   if (i < a.N) ssp_rate_row<KT, MIXED>(of, a, i, u, dt);
 }
 
 template <int KT, bool MIXED>
 __global__ void k_ssp_edges(Offsets of, SspArrays a, const double* __restrict__ u) {
+  pdl_trigger();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  pdl_wait();
   if (i < a.N) ssp_edges_row<KT, MIXED>(of, a, i, u);
 }
 
-template <int KT, bool MIXED>
+template <int KT, bool MIXED, bool SMALL>
 __global__ void k_ssp_factors(Offsets of, SspArrays a, double dt) {
+  pdl_trigger();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i < a.N) ssp_factors_row<KT, MIXED>(of, a, i, dt);
+  pdl_wait();
+  if (i < a.N) ssp_factors_row<KT, MIXED, kGroup<KT>, SMALL>(of, a, i, dt);
 }
 
-template <int KT, bool MIXED>
+template <int KT, bool MIXED, bool SMALL>
 __global__ void k_ssp_correct(Offsets of, SspArrays a, int limiter, double dt, double ca,
-                              const double* __restrict__ uA, double cb, double* __restrict__ out) {
+                              const double* uA, double cb, double* out) {
+  pdl_trigger();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i < a.N) ssp_correct_row<KT, MIXED>(of, a, i, limiter, dt, ca, uA, cb, out);
+  pdl_wait();
+  if (i < a.N) ssp_correct_row<KT, MIXED, kGroup<KT>, SMALL>(of, a, i, limiter, dt, ca, uA, cb, out);
 }
+// Below this many rows (about one resident wave) the passes take their SMALL form.
+constexpr int64_t kSmallRows = 300000;
 
 __global__ void k_to_float(int64_t n, const double* __restrict__ x, float* __restrict__ y) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -146,40 +164,51 @@ __global__ void k_cn_factors(int64_t N, Offsets of, const unsigned long long* __
   const double qp = mQp[i], qm = mQm[i];
   pdl_wait();
   if (isdir) { Rp[i] = 1.0; Rm[i] = 1.0; return; }
-  constexpr int KA = KT > 0 ? KT : kMaxOffsets;
-  SignedFixedSums acc;
+  SignedSums64 acc;
+  constexpr int S = kGroup<KT>;
 #pragma unroll
-  for (int k = 0; k < KA; ++k) {
-    if (k >= K || k == Kup || !((mk >> k) & 1ull)) continue;
-    acc.add((unsigned long long)__double_as_longlong(pair_flux(of, Kup, k, i, N, r_up)));
+  for (int k0 = 0; k0 < K; k0 += S) {
+    double r[S];
+#pragma unroll
+    for (int j = 0; j < S; ++j)
+      if (k0 + j != Kup) r[j] = r_up[pair_slot(of, Kup, k0 + j, i, N)];
+#pragma unroll
+    for (int j = 0; j < S; ++j) {
+      const int k = k0 + j;
+      if (k == Kup || !((mk >> k) & 1ull)) continue;
+      acc.add((unsigned long long)__double_as_longlong(r[j]) ^ (k > Kup ? 0ull : 0x8000000000000000ull));
+    }
   }
   double Pp, Pm;
-  acc.result(Pp, Pm);
+  acc.result<1023>(Pp, Pm);
   Rp[i] = zalesak_factor(qp, dt * Pp);
   Rm[i] = zalesak_factor(qm, dt * Pm);
 }
 
 // Zalesak step 4, F*, and the nonlinear residual of Eq. CNZal:
-// res = b0 + F* - (m/dt u + AA u / 2) on free rows, 0 on Dirichlet rows;
-// block partial sums of res^2 for the stopping test.
+// res = b0 + F* - (m/dt u + AA u / 2) on free rows, 0 on Dirichlet rows; block partial sums of
+// res^2 for the stopping test.  M_L/dt + AA/2 is the system matrix B of the solve that follows
+// (identity rows are Dirichlet rows, which are not formed): one matrix of 59 MB at Q1 65^3 in
+// the 129 MB L2 instead of AA beside it.
 template <int KT>
 __global__ void __launch_bounds__(256, 4) k_cn_residual(int64_t N, Offsets of, int limiter, const unsigned long long* __restrict__ mask,
-                              const double* __restrict__ r_up, const double* __restrict__ AA,
+                              const double* __restrict__ r_up, const double* __restrict__ B,
                               const double* __restrict__ un, const double* __restrict__ Rp,
-                              const double* __restrict__ Rm, const double* __restrict__ b0,
-                              const double* __restrict__ mLdt, const uint8_t* __restrict__ dir,
+                              const double* __restrict__ Rm,
+                              const double* __restrict__ b0,
+                              const uint8_t* __restrict__ dir,
                               double* __restrict__ res, double* __restrict__ Fout, double* __restrict__ part) {
   const int K = KT > 0 ? KT : of.K, Kup = K / 2;
   pdl_trigger();
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   double r2 = 0.0;
-  // y = AA u from the matrix and the state, before the wait for the factors pass: no pass
+  // y = B u from the matrix and the state, before the wait for the factors pass: no pass
   // of the limiter writes them (u is the solver's, complete before the edge pass started)
   const bool act = i < N && !dir[i];
   double y = 0.0;
   if (act) {
 #pragma unroll
-    for (int k = 0; k < K; ++k) y = fma(AA[k * N + i], un[i + of.o[k]], y);
+    for (int k = 0; k < K; ++k) y = fma(B[k * N + i], un[i + of.o[k]], y);
   }
   pdl_wait();
   if (i < N) {
@@ -188,20 +217,31 @@ __global__ void __launch_bounds__(256, 4) k_cn_residual(int64_t N, Offsets of, i
       const unsigned long long mk = mask[i];
       if (limiter != AFC_LIM_NONE) {
         const double rpi = Rp[i], rmi = Rm[i];
-      #pragma unroll
-  for (int k = 0; k < K; ++k) {
-          if (k == Kup || !((mk >> k) & 1ull)) continue;
-          const double r = pair_flux(of, Kup, k, i, N, r_up);
-          if (limiter == AFC_LIM_ZALESAK) {
-            const int64_t j = i + of.o[k];
-            const double alpha = gt0(r) ? imin_nn(rpi, Rm[j]) : imin_nn(rmi, Rp[j]);
-            F = fma(alpha, r, F);
-          } else {
-            F += r;
+        constexpr int S = kGroup<KT>;
+#pragma unroll
+        for (int k0 = 0; k0 < K; k0 += S) {
+          double r[S], Rj[S];
+#pragma unroll
+          for (int j = 0; j < S; ++j) {
+            if (k0 + j == Kup) continue;
+            r[j] = r_up[pair_slot(of, Kup, k0 + j, i, N)];
+            if (k0 + j < Kup) r[j] = neg_bits(r[j]);
+          }
+          if (limiter == AFC_LIM_ZALESAK) {   // R- of the neighbour for r > 0, R+ else: one load each
+#pragma unroll
+            for (int j = 0; j < S; ++j)
+              if (k0 + j != Kup) Rj[j] = (gt0(r[j]) ? Rm : Rp)[i + of.o[k0 + j]];
+          }
+#pragma unroll
+          for (int j = 0; j < S; ++j) {
+            const int k = k0 + j;
+            if (k == Kup || !((mk >> k) & 1ull)) continue;
+            if (limiter == AFC_LIM_ZALESAK) F = fma(imin_nn(gt0(r[j]) ? rpi : rmi, Rj[j]), r[j], F);
+            else F += r[j];
           }
         }
       }
-      rv = b0[i] + F - (mLdt[i] * un[i] + 0.5 * y);
+      rv = b0[i] + F - y;
     }
     res[i] = rv;
     if (Fout) Fout[i] = F;
@@ -221,6 +261,7 @@ SspArrays ssp_arrays(afc_problem_s* p) {
   a.m32 = p->m32_up.p;
   a.d32 = p->d32_up.p;
   a.mL = p->mL.p;
+  a.imL = p->imL.p;
   a.f = p->f.p;
   a.dir = p->dir.p;
   a.udir = p->udir.p;
@@ -252,24 +293,26 @@ int ensure_ssp_mixed(afc_problem_s* p) {
 }
 
 int fe_stage(afc_problem_s* p, const double* uin, double dt, int limiter, double a, const double* uA, double b,
-             double* out, bool mixed) {
+             double* out, bool mixed, bool pdl) {
   const int64_t N = p->N;
-  const int64_t g = grid_for(N);
+  const dim3 g((unsigned)grid_for(N)), blk(kBlock);
   cudaStream_t s = p->stream;
   if (mixed) {
     int st = ensure_ssp_mixed(p);
     if (st) return st;
   }
   const SspArrays arr = ssp_arrays(p);
+  const bool chain = N <= kPdlRows;
+  pdl = pdl && chain;
   if (limiter == AFC_LIM_MC) {
     // transient MC (Sec. 2.2): rate, clipped fluxes, then the unweighted sum of r*
     int st = AFC_OK;
     with_K(p->K, [&](auto kc) {
       constexpr int KT = decltype(kc)::value;
-      AFC_LAUNCH(p, "k_ssp_rate", k_ssp_rate<KT, false><<<g, kBlock, 0, s>>>(p->offs, arr, uin, dt));
+      AFC_LAUNCH(p, "k_ssp_rate", launch_pass(false, k_ssp_rate<KT, false>, g, blk, s, p->offs, arr, uin, dt));
       if ((st = mc_ssp_fluxes(p, uin))) return;
-      AFC_LAUNCH(p, "k_ssp_correct", k_ssp_correct<KT, false><<<g, kBlock, 0, s>>>(p->offs, arr, AFC_LIM_GALERKIN, dt,
-                                                                                  a, uA, b, out));
+      AFC_LAUNCH(p, "k_ssp_correct", launch_pass(false, k_ssp_correct<KT, false, false>, g, blk, s, p->offs, arr,
+                                                 (int)AFC_LIM_GALERKIN, dt, a, uA, b, out));
     });
     if (st) return st;
     AFC_CUDA(cudaGetLastError());
@@ -278,13 +321,15 @@ int fe_stage(afc_problem_s* p, const double* uin, double dt, int limiter, double
   auto run = [&](auto kc, auto mc) {
     constexpr int KT = decltype(kc)::value;
     constexpr bool MX = decltype(mc)::value;
-    AFC_LAUNCH(p, "k_ssp_rate", k_ssp_rate<KT, MX><<<g, kBlock, 0, s>>>(p->offs, arr, uin, dt));
+    AFC_LAUNCH(p, "k_ssp_rate", launch_pass(pdl, k_ssp_rate<KT, MX>, g, blk, s, p->offs, arr, uin, dt));
     if (limiter != AFC_LIM_NONE)
-      AFC_LAUNCH(p, "k_ssp_edges", k_ssp_edges<KT, MX><<<g, kBlock, 0, s>>>(p->offs, arr, uin));
+      AFC_LAUNCH(p, "k_ssp_edges", launch_pass(chain, k_ssp_edges<KT, MX>, g, blk, s, p->offs, arr, uin));
+    const bool small = N < kSmallRows;
+    auto factors = small ? k_ssp_factors<KT, MX, true> : k_ssp_factors<KT, MX, false>;
     if (limiter == AFC_LIM_ZALESAK)
-      AFC_LAUNCH(p, "k_ssp_factors", k_ssp_factors<KT, MX><<<g, kBlock, 0, s>>>(p->offs, arr, dt));
-    AFC_LAUNCH(p, "k_ssp_correct",
-               k_ssp_correct<KT, MX><<<g, kBlock, 0, s>>>(p->offs, arr, limiter, dt, a, uA, b, out));
+      AFC_LAUNCH(p, "k_ssp_factors", launch_pass(chain, factors, g, blk, s, p->offs, arr, dt));
+    auto correct = small ? k_ssp_correct<KT, MX, true> : k_ssp_correct<KT, MX, false>;
+    AFC_LAUNCH(p, "k_ssp_correct", launch_pass(chain, correct, g, blk, s, p->offs, arr, limiter, dt, a, uA, b, out));
   };
   with_K(p->K, [&](auto kc) {
     if (mixed) run(kc, std::true_type{});
@@ -292,6 +337,20 @@ int fe_stage(afc_problem_s* p, const double* uin, double dt, int limiter, double
   });
   AFC_CUDA(cudaGetLastError());
   return AFC_OK;
+}
+
+int ssp_stages(afc_problem_s* p, const afc_opts* o) {
+  const bool mixed = o->precision == AFC_MIXED;
+  const int lim = o->limiter;
+  const double dt = o->dt;
+  double *u = p->u.p, *v = p->ustage.p, *w = p->tmp.p;
+  // u^n stays in u until the last stage, whose passes read it at their own row only, in the
+  // pass that writes it
+  int st = fe_stage(p, u, dt, lim, 0.0, nullptr, 1.0, v, mixed);
+  if (st) return st;
+  if (o->scheme == AFC_SSP2) return fe_stage(p, v, dt, lim, 0.5, u, 0.5, u, mixed, true);
+  if ((st = fe_stage(p, v, dt, lim, 0.75, u, 0.25, w, mixed, true))) return st;
+  return fe_stage(p, w, dt, lim, 1.0 / 3.0, u, 2.0 / 3.0, u, mixed, true);
 }
 
 namespace {
@@ -442,14 +501,12 @@ int cn_limited_residual(afc_problem_s* p, const double* u_new, double dt, int li
       AFC_LAUNCH(p, "k_cn_factors", launch_pass(limiter != AFC_LIM_NONE, k_cn_factors<KT>, dim3((unsigned)g),
                                                 dim3(kBlock), s, N, p->offs, (const unsigned long long*)p->mask.p,
                                                 (const double*)p->r_up.p, (const double*)p->Qp.p,
-                                                (const double*)p->Qm.p, (const uint8_t*)p->dir.p, dt, p->Rp.p,
-                                                p->Rm.p));
+                                                (const double*)p->Qm.p, (const uint8_t*)p->dir.p, dt, p->Rp.p, p->Rm.p));
     AFC_LAUNCH(p, "k_cn_residual",
                launch_pass(limiter != AFC_LIM_NONE, k_cn_residual<KT>, dim3((unsigned)g), dim3(kBlock), s, N,
                            p->offs, limiter, (const unsigned long long*)p->mask.p, (const double*)p->r_up.p,
-                           (const double*)p->AA.p, u_new, (const double*)p->Rp.p, (const double*)p->Rm.p,
-                           (const double*)p->b0.p, (const double*)p->mLdt.p, (const uint8_t*)p->dir.p, res, p->Fs.p,
-                           p->part.p));
+                           (const double*)p->Bcn.p, u_new, (const double*)p->Rp.p, (const double*)p->Rm.p,
+                           (const double*)p->b0.p, (const uint8_t*)p->dir.p, res, p->Fs.p, p->part.p));
   });
   if (normsq_slot) finalize_sum(p, p->part.p, (int)g, normsq_slot);
   AFC_CUDA(cudaGetLastError());

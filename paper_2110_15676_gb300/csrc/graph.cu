@@ -1,10 +1,9 @@
 // One time step or one stationary solve as a single CUDA graph launch.
 //
 // The damped fixed point of Sec. 4 is a while node: its body evaluates the
-// limited residual and a one-thread control kernel decides on the device whether
-// to stop (Eq. tol_formula, the iteration limit, or a fixed count) and whether
-// the body's if node runs the linear solve (itself a while node over the Krylov
-// iterations) and the update.  The host launches the graph and synchronises once;
+// limited residual, and the persistent solver launch that follows first decides
+// whether to stop (Eq. tol_formula, the iteration limit, or a fixed count), then
+// solves and updates.  The host launches the graph and synchronises once;
 // no scalar travels to the host inside the step.  The explicit SSP step is a
 // plain captured graph.  Graphs are built on first use and rebuilt when the
 // options or the problem's buffers change.
@@ -32,36 +31,6 @@ __global__ void k_fp_init(double* sc, double thresh, int fixed, int maxit) {
   sc[F_TIMEOUT] = 0.0;
 }
 
-// After a residual evaluation: R = ||res||; stop or solve.  The residual pass leaves
-// its block partials of res^2 in part[0 .. npart); one block of 1024 threads sums them
-// (the order of finalize_sum) before the decision, so the sum needs no launch of its own.
-__global__ void k_fp_control(double* sc, const double* __restrict__ part, int npart,
-                             cudaGraphConditionalHandle h_loop, cudaGraphConditionalHandle h_solve) {
-  pdl_wait();   // the residual pass's partials (a no-op when launched without the attribute)
-  block_sum_to(strided_sum_1024(part, npart, threadIdx.x), sc + F_NORMSQ);   // one block of 1024
-  if (threadIdx.x != 0) return;
-  const double R = sqrt(sc[F_NORMSQ]);
-  const double it = sc[F_CORR];
-  if (sc[F_REVAL] == 0.0) sc[F_RES0] = R;
-  sc[F_RESF] = R;
-  sc[F_REVAL] += 1.0;
-  bool stop = false;
-  if (!isfinite(R) || sc[F_STATUS] == 2.0) {
-    stop = true;
-    sc[F_STATUS] = 2.0;
-  } else if (sc[F_FIXED] > 0.0) {
-    if (it >= sc[F_FIXED]) { stop = true; sc[F_STATUS] = 1.0; }
-  } else if (R < sc[F_THRESH]) {
-    stop = true;
-    sc[F_STATUS] = 1.0;
-  } else if (it >= sc[F_MAXIT]) {
-    stop = true;
-    sc[F_STATUS] = 3.0;
-  }
-  cudaGraphSetConditional(h_loop, stop ? 0u : 1u);
-  cudaGraphSetConditional(h_solve, stop ? 0u : 1u);
-}
-
 __global__ void k_copy(int64_t n, const double* __restrict__ x, double* __restrict__ y) {
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i < n) y[i] = x[i];
@@ -73,61 +42,6 @@ __global__ void k_apply_dirichlet_g(int64_t N, const uint8_t* __restrict__ dir, 
   if (i < N && dir[i]) u[i] = udir[i];
 }
 
-__global__ void k_minmax_g(int64_t N, const double* __restrict__ x, double* __restrict__ part) {
-  double mn = INFINITY, mx = -INFINITY;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
-    mn = fmin(mn, x[i]);
-    mx = fmax(mx, x[i]);
-  }
-  __shared__ double smn[kBlock], smx[kBlock];
-  smn[threadIdx.x] = mn;
-  smx[threadIdx.x] = mx;
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s) {
-      smn[threadIdx.x] = fmin(smn[threadIdx.x], smn[threadIdx.x + s]);
-      smx[threadIdx.x] = fmax(smx[threadIdx.x], smx[threadIdx.x + s]);
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    part[2 * blockIdx.x] = smn[0];
-    part[2 * blockIdx.x + 1] = smx[0];
-  }
-}
-
-__global__ void k_minmax_fin_g(const double* __restrict__ part, int n, double* __restrict__ out) {
-  __shared__ double smn[kBlock], smx[kBlock];
-  double mn = INFINITY, mx = -INFINITY;
-  for (int q = threadIdx.x; q < n; q += blockDim.x) {
-    mn = fmin(mn, part[2 * q]);
-    mx = fmax(mx, part[2 * q + 1]);
-  }
-  smn[threadIdx.x] = mn;
-  smx[threadIdx.x] = mx;
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s) {
-      smn[threadIdx.x] = fmin(smn[threadIdx.x], smn[threadIdx.x + s]);
-      smx[threadIdx.x] = fmax(smx[threadIdx.x], smx[threadIdx.x + s]);
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    out[0] = smn[0];
-    out[1] = smx[0];
-  }
-}
-
-// solution extremes into scal[60..61], then all scalars to the pinned host mirror
-int enqueue_stats(afc_problem_s* p) {
-  AFC_LAUNCH(p, "k_minmax", k_minmax_g<<<kRedBlocks, kBlock, 0, p->stream>>>(p->N, p->u.p, p->part.p));
-  AFC_LAUNCH(p, "k_minmax_fin", k_minmax_fin_g<<<1, kBlock, 0, p->stream>>>(p->part.p, kRedBlocks, p->scal.p + 60));
-  AFC_CUDA(cudaGetLastError());
-  AFC_CUDA(cudaMemcpyAsync(p->host_scal, p->scal.p, 64 * sizeof(double), cudaMemcpyDeviceToHost, p->stream));
-  return AFC_OK;
-}
-
 }  // namespace
 
 // Cached executable graph and the kernel count of each of its sections (for the
@@ -135,7 +49,7 @@ int enqueue_stats(afc_problem_s* p) {
 struct StepGraph {
   cudaGraphExec_t exec = nullptr;
   std::vector<unsigned char> key;
-  int64_t k_pro = 0, k_outer = 0, k_solve = 0, k_epi = 0;
+  int64_t k_pro = 0, k_outer = 0, k_epi = 0;
   int kind = 0;   // 1 fixed point, 2 explicit SSP
 };
 
@@ -171,8 +85,8 @@ struct ProfOff {   // no event records inside captured graphs; captured launches
   }
 };
 
-// Build the fixed-point graph: prologue, while(outer){ residual; control; if(solve){ Krylov } }, epilogue.  The
-// persistent solve applies the update `epi` and counts itself in the fixed-point scalars.  `system` 1: CN step, 0: stationary.
+// Build the fixed-point graph: prologue, while(outer){ residual; solve }, epilogue.  The
+// persistent solve decides first whether the loop goes on, and applies and counts the update.
 template <class Pro, class Res>
 int build_fixed_point(afc_problem_s* p, const afc_opts* o, int system, Pro prologue, Res residual, StepGraph& sg,
                       KrylovEpilogue epi) {
@@ -183,7 +97,7 @@ int build_fixed_point(afc_problem_s* p, const afc_opts* o, int system, Pro prolo
   AFC_CUDA(cudaGraphCreate(&g, 0));
   int st = AFC_OK;
   std::vector<cudaGraphNode_t> fr;
-  cudaGraphConditionalHandle h_loop, h_solve;
+  cudaGraphConditionalHandle h_loop;
   const double thresh = std::sqrt((double)p->N) * o->fp_tol;
   auto count = [&](auto&& f) {
     const int64_t l0 = p->launches;
@@ -207,39 +121,20 @@ int build_fixed_point(afc_problem_s* p, const afc_opts* o, int system, Pro prolo
     cudaGraph_t body;
     cudaGraphNode_t loop;
     if ((st = add_conditional(g, fr, h_loop, cudaGraphCondTypeWhile, &body, &loop))) break;
-    if (cudaGraphConditionalHandleCreate(&h_solve, body, 0, 0) != cudaSuccess) {
-      st = cuda_fail(cudaGetLastError(), "cudaGraphConditionalHandleCreate");
-      break;
-    }
     std::vector<cudaGraphNode_t> bf;
-    auto r2 = count([&]() -> int {
-      return capture_into(p, cs, body, {}, [&]() -> int {
-        int s = residual();
-        if (s) return s;
-        // programmatic dependency on the Zalesak CN residual pass, which ends the body's residual
-        // (the other residuals end with other work and keep a plain one)
-        const bool pdl = system == 1 && o->limiter == AFC_LIM_ZALESAK;
-        AFC_LAUNCH(p, "k_fp_control", launch_pass(pdl, k_fp_control, dim3(1), dim3(1024), p->stream,
-                                                  p->scal.p, (const double*)p->part.p, (int)grid_for(p->N), h_loop,
-                                                  h_solve));
-        AFC_CUDA(cudaGetLastError());
-        return AFC_OK;
-      }, bf);
-    });
+    auto r2 = count([&]() -> int { return capture_into(p, cs, body, {}, residual, bf); });
     if ((st = r2.first)) break;
-    sg.k_outer = r2.second;
-    cudaGraph_t sbody;
-    cudaGraphNode_t ifnode;
-    if ((st = add_conditional(body, bf, h_solve, cudaGraphCondTypeIf, &sbody, &ifnode))) break;
-    std::vector<cudaGraphNode_t> sf;
     epi.fp_sc = p->scal.p;
+    epi.part = p->part.p;
+    epi.npart = (int)grid_for(p->N);
+    epi.loop = h_loop;
     auto r3 = count([&]() -> int {
-      return krylov_graph(p, system, o, p->res.p, p->delta.p, cs, sbody, sf, &epi);
+      return krylov_graph(p, system, o, p->res.p, p->delta.p, cs, body, bf, &epi);
     });
     if ((st = r3.first)) break;
-    sg.k_solve = r3.second;
+    sg.k_outer = r2.second + r3.second;
     fr.assign(1, loop);
-    auto r4 = count([&]() -> int { return capture_into(p, cs, g, fr, [&]() -> int { return enqueue_stats(p); }, fr); });
+    auto r4 = count([&]() -> int { return capture_into(p, cs, g, fr, [&]() -> int { return range_device(p, p->u.p); }, fr); });
     if ((st = r4.first)) break;
     sg.k_epi = r4.second;
     cudaGraphExec_t ex = nullptr;
@@ -257,7 +152,7 @@ int run_fixed_point_graph(afc_problem_s* p, StepGraph& sg, afc_stats* stt) {
   AFC_CUDA(cudaStreamSynchronize(p->stream));
   const double* h = p->host_scal;
   const int64_t reval = (int64_t)h[F_REVAL], corr = (int64_t)h[F_CORR];
-  p->launches += sg.k_pro + reval * sg.k_outer + corr * sg.k_solve + sg.k_epi;
+  p->launches += sg.k_pro + reval * sg.k_outer + sg.k_epi;
   int status = h[F_STATUS] == 1.0 ? AFC_OK : h[F_STATUS] == 2.0 ? AFC_E_NAN : AFC_NOT_CONVERGED;
   if (h[F_TIMEOUT] != 0.0) {
     // the barrier counter is inconsistent after blocks skipped barriers: clear it so
@@ -377,21 +272,9 @@ int ssp_step_graph(afc_problem_s* p, const afc_opts* o, afc_stats* stt) {
     AFC_CUDA(cudaGraphCreate(&g, 0));
     std::vector<cudaGraphNode_t> fr;
     const int64_t l0 = p->launches;
-    const int lim = o->limiter;
-    const double dt = o->dt;
     int st = capture_into(p, p->cap_stream, g, fr, [&]() -> int {
-      const int64_t N = p->N;
-      AFC_LAUNCH(p, "k_copy", k_copy<<<grid_for(N), kBlock, 0, p->stream>>>(N, p->u.p, p->u0.p));
-      int s;
-      if (o->scheme == AFC_SSP2) {
-        if ((s = fe_stage(p, p->u0.p, dt, lim, 0.0, nullptr, 1.0, p->ustage.p, mixed))) return s;
-        if ((s = fe_stage(p, p->ustage.p, dt, lim, 0.5, p->u0.p, 0.5, p->u.p, mixed))) return s;
-      } else {
-        if ((s = fe_stage(p, p->u0.p, dt, lim, 0.0, nullptr, 1.0, p->ustage.p, mixed))) return s;
-        if ((s = fe_stage(p, p->ustage.p, dt, lim, 0.75, p->u0.p, 0.25, p->tmp.p, mixed))) return s;
-        if ((s = fe_stage(p, p->tmp.p, dt, lim, 1.0 / 3.0, p->u0.p, 2.0 / 3.0, p->u.p, mixed))) return s;
-      }
-      return enqueue_stats(p);
+      const int s = ssp_stages(p, o);
+      return s ? s : range_device(p, p->u.p);
     }, fr);
     if (!st) {
       cudaGraphExec_t ex = nullptr;

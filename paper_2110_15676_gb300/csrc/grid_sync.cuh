@@ -70,19 +70,20 @@ __device__ __forceinline__ unsigned int grid_arrive(GridBar* gb) {
 // once limit_ns of the global timer have passed (limit 0: at the first poll that finds
 // the barrier still closed), or when another block has.  The first polls look at the
 // counter alone: the error word and the global timer cost a trip each, so they are
-// read only on every 16th poll (a barrier opens within a few polls).
-__device__ __forceinline__ void grid_poll(GridBar* gb, unsigned int old, unsigned long long limit_ns) {
+// read only on every 16th poll (a barrier opens within a few polls).  False after an error.
+__device__ __forceinline__ bool grid_poll(GridBar* gb, unsigned int old, unsigned long long limit_ns) {
   unsigned long long t0 = 0;
   for (unsigned int n = 1; ((old ^ ld_acquire_gpu(&gb->arrive)) & 0x80000000u) == 0u; ++n) {
     if ((n & 15u) != 0u && limit_ns != 0ull) continue;
-    if (*(volatile int*)&gb->err != 0) break;
+    if (*(volatile int*)&gb->err != 0) return false;
     const unsigned long long now = global_ns();
     if (t0 == 0ull) t0 = now;
     if (now - t0 >= limit_ns) {
       atomicExch(&gb->err, 1);
-      break;
+      return false;
     }
   }
+  return true;
 }
 
 // The block waits (thread 0 passes what grid_arrive returned).

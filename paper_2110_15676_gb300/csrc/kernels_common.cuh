@@ -67,113 +67,71 @@ __device__ __forceinline__ double widen_exact(float x) {
   return __longlong_as_double((long long)(s | (de << 52) | ((unsigned long long)m << 29)));
 }
 
-// Sums of the positive and of the negative values of a row's pair fluxes, exact:
-// every mantissa is placed in a 128-bit fixed point scaled to the largest exponent
-// (its mantissa at bits 64..116, so up to 2^10 terms cannot overflow), the words are
-// added with carry on the integer pipe, and each total is rounded to double once.
-// Subnormal inputs count as zero.  On GB300 this replaces two FP64 adds per value (an
-// FP64 warp instruction occupies the pipe for 16 cycles) with about a dozen integer
-// instructions, and is more accurate.  The values are taken one at a time, so that
-// none has to be kept: the totals are held scaled to the largest exponent seen so
-// far, and a value with a larger exponent first shifts both totals right (the bits
-// that leave the 128-bit range are below 2^-64 of the new largest value's last
-// bit).  A row of 26 pair fluxes then needs no 52 registers to hold its bit
-// patterns until its largest exponent is known.
-struct SignedFixedSums {
+// Sums of the positive and of the negative values of a row's pair fluxes in 64-bit fixed point
+// (Zalesak's P+ and P-), on the integer pipe: the largest value's leading bit at bit 57 (up to 62
+// terms fit), every smaller term rounded to the last bit, each total rounded to double once.
+// A total carries an error of a few 2^-58 of the largest term, far below the rounding of the
+// result; a sum of FP64 adds carries one rounding per add.  Subnormal inputs count as zero.
+// On GB300 this replaces two FP64 adds per value (an FP64 warp instruction occupies the pipe
+// for 16 cycles) with about twenty integer instructions; 128-bit totals took half as many
+// again (k_cn_factors at Q1 65^3: 38 -> 29 us).  The values are taken one at a time, so that
+// none has to be kept until the largest exponent is known: the totals are held scaled to the
+// largest exponent seen so far, and a value with a larger one first shifts them right.
+struct SignedSums64 {
   unsigned emax = 0u;
-  unsigned long long ph = 0ull, pl = 0ull, nh = 0ull, nl = 0ull;
+  unsigned long long p = 0ull, n = 0ull;
 
-  __device__ static __forceinline__ void shr128(unsigned long long& h, unsigned long long& l, unsigned d) {
-    if (d >= 128u) {
-      h = 0ull;
-      l = 0ull;
-    } else if (d >= 64u) {
-      l = h >> (d - 64u);
-      h = 0ull;
-    } else {
-      l = (l >> d) | (h << (64u - d));
-      h >>= d;
-    }
+  __device__ __forceinline__ void raise(unsigned e) {   // scale the totals to a larger exponent
+    const unsigned d = e - emax;
+    p = d < 64u ? p >> d : 0ull;
+    n = d < 64u ? n >> d : 0ull;
+    emax = e;
   }
-  __device__ __forceinline__ void add(unsigned long long b) {
+  __device__ __forceinline__ void put(unsigned long long m, unsigned e, bool neg) {   // m: leading bit at bit 58
+    const unsigned sh = emax - e;
+    const unsigned long long v = ((sh < 64u ? m >> sh : 0ull) + 1ull) >> 1;
+    if (neg) n += v;
+    else p += v;
+  }
+  __device__ __forceinline__ void add(unsigned long long b) {   // a double
     const unsigned e = (unsigned)(b >> 52) & 0x7ffu;
     if (e == 0u) return;
-    if (e > emax) {
-      if (emax != 0u) {
-        shr128(ph, pl, e - emax);
-        shr128(nh, nl, e - emax);
-      }
-      emax = e;
-    }
-    const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
-    const int sh = (int)e - (int)emax + 64;   // <= 64
-    unsigned long long lo, hi;
-    if (sh >= 64) {
-      lo = 0ull;
-      hi = m;
-    } else if (sh > 0) {
-      lo = m << sh;
-      hi = m >> (64 - sh);
-    } else if (sh > -64) {
-      lo = m >> (-sh);
-      hi = 0ull;
-    } else {
-      lo = 0ull;
-      hi = 0ull;
-    }
-    if (b >> 63) {
-      nl += lo;
-      nh += hi + (nl < lo ? 1ull : 0ull);
-    } else {
-      pl += lo;
-      ph += hi + (pl < lo ? 1ull : 0ull);
-    }
+    if (e > emax) raise(e);
+    put(((b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << 6, e, b >> 63);
   }
-  // The totals rounded to double (nearest, ties to even) on the integer pipe; value
-  // = (h:l) * 2^(emax - 1139).  Totals whose double would be subnormal or overflow
-  // take the FP64 route in a separate function.
+  __device__ __forceinline__ void add(unsigned b) {   // a float
+    const unsigned e = (b >> 23) & 0xffu;
+    if (e == 0u) return;
+    if (e > emax) raise(e);
+    put((unsigned long long)((b & 0x7fffffu) | 0x800000u) << 35, e, b >> 31);
+  }
+  // totals of doubles (BIAS 1023) or floats (BIAS 127)
+  template <int BIAS>
   __device__ __forceinline__ void result(double& pos, double& neg) const {
-    if (emax == 0u) {
-      pos = 0.0;
-      neg = 0.0;
-      return;
-    }
-    const int ex = (int)emax - 1139;
-    pos = to_double(ph, pl, ex);
-    neg = neg_bits(to_double(nh, nl, ex));
+    pos = to_double(p, (int)emax - BIAS - 57);
+    neg = neg_bits(to_double(n, (int)emax - BIAS - 57));
   }
-  __device__ static __noinline__ double to_double_fp64(unsigned long long h, unsigned long long l, int ex) {
-    const double two64 = 18446744073709551616.0;
-    return scalbn(fma(__ull2double_rn(h), two64, __ull2double_rn(l)), ex);
+  __device__ static __noinline__ double to_double_edge(unsigned long long v, int ex) {
+    return scalbn(__ull2double_rn(v), ex);
   }
-  __device__ static __forceinline__ double to_double(unsigned long long h, unsigned long long l, int ex) {
-    if ((h | l) == 0ull) return 0.0;
-    const int lz = h != 0ull ? __clzll((long long)h) : 64 + __clzll((long long)l);
-    unsigned long long nh, nl;   // normalised: bit 127 set
-    if (lz >= 64) {
-      nh = l << (lz - 64);
-      nl = 0ull;
-    } else if (lz > 0) {
-      nh = (h << lz) | (l >> (64 - lz));
-      nl = l << lz;
-    } else {
-      nh = h;
-      nl = l;
-    }
-    unsigned long long m = nh >> 11;   // 53 bits, the leading one at bit 52
-    const bool half = (nh >> 10) & 1ull;
-    const bool sticky = ((nh & 0x3FFull) | nl) != 0ull;
-    if (half && (sticky || (m & 1ull))) ++m;
-    int e2 = 127 + ex - lz;            // exponent of the leading bit
-    if (m >> 53) {
-      m >>= 1;
-      ++e2;
-    }
-    const int be = e2 + 1023;
-    if (be <= 0 || be >= 2047) return to_double_fp64(h, l, ex);
-    return __longlong_as_double((long long)(((unsigned long long)be << 52) | (m & 0xFFFFFFFFFFFFFull)));
+  __device__ static __forceinline__ double to_double(unsigned long long v, int ex) {
+    if (v == 0ull) return 0.0;
+    const long long d = __double_as_longlong(__ull2double_rn(v));
+    const int be = (int)(d >> 52) + ex;
+    if (be <= 0 || be >= 2047) return to_double_edge(v, ex);
+    return __longlong_as_double(d + ((long long)ex << 52));
   }
 };
+
+// a / m for a divisor whose rounded reciprocal im is at hand (Markstein, IBM J. Res. Dev. 34
+// (1990) 111): q = a im, one residual, one correction, three FP64 operations where the inlined
+// division takes about ten; the correctly rounded quotient, as long as nothing in it
+// under- or overflows.  A product that is not finite is returned as it is.
+__device__ __forceinline__ double div_by(double a, double m, double im) {
+  const double q = a * im;
+  const double c = fma(fma(-q, m, a), im, q);
+  return (__double_as_longlong(q) & 0x7ff0000000000000ll) == 0x7ff0000000000000ll ? q : c;
+}
 
 // min / max of two values known to be >= 0 (correction factors, bounds): plain int compare
 __device__ __forceinline__ double imin_nn(double a, double b) {
@@ -222,6 +180,20 @@ __device__ __forceinline__ double pair_flux(const Offsets& of, int Kup, int k, i
   return neg_bits(r_up[(int64_t)(Kup - 1 - k) * N + i + of.o[k]]);   // -r_e, sign bit on the integer pipe
 }
 
+// Index of the pair (i, i + o_k) in pair data stored at the pair's lower row, for loads that
+// are issued whether or not the pair is in the pattern (the caller drops the value of an
+// absent one): always inside the array.  (A pair below the first row would start before it.)
+__device__ __forceinline__ int64_t pair_slot(const Offsets& of, int Kup, int k, int64_t i, int64_t N) {
+  if (k > Kup) return (int64_t)(k - Kup - 1) * N + i;
+  const int64_t q = (int64_t)(Kup - 1 - k) * N + i + of.o[k];
+  return q < 0 ? 0 : q;
+}
+// Neighbours whose loads a row issues together: a third of the structured patterns (a loop
+// that tests the pattern before each load waits for one load after the other, 12 us for a
+// pass over 729 rows; all at once take the registers of two rows).
+template <int KT>
+constexpr int kGroup = KT == 27 ? 9 : KT == 15 ? 5 : 1;
+
 template <class T>
 __device__ __forceinline__ T warp_sum(T v) {
 #pragma unroll
@@ -243,22 +215,30 @@ __device__ __forceinline__ double warp0_column_sum(const double* col) {
   return warp_sum(t);
 }
 
-// The final sums over a pass's block partials run as 1024 threads: thread t adds
-// part[t], part[t + 1024], part[t + 2048], ... (q < n) from left to right, then the
-// block sums the threads (block_sum_to).  This is thread t's sum; its loads go out
-// eight at a time instead of one round trip each.  A slot past n adds +0.0, which
-// leaves the sum unchanged (it starts at +0.0, so it is never -0.0).  The loads go
-// through L2 (partials of other blocks of the same grid are read this way too).
-__device__ __forceinline__ double strided_sum_1024(const double* part, int n, int t) {
-  double v = 0.0;
-  for (int q0 = t; q0 < n; q0 += 8 * 1024) {
-    double x[8];
+// The final sum over a pass's block partials, in an order that does not depend on the size of
+// the block that forms it (at least one full warp): eight strands, strand w adding partials
+// 32 w + lane, then + 256, ... four at a time and then its lanes, one warp per strand in turn;
+// the strands are added in pairs.  The fixed point's stop test in the solvers and the host-
+// driven loop (k_finalize_sum) so see the same bits.  The loads go through L2.  Every thread
+// of the block calls it and receives the total.
+__device__ __forceinline__ double final_sum(const double* part, int n) {
+  __shared__ double strand[8];
+  const int lane = threadIdx.x & 31;
+  for (int w = threadIdx.x >> 5; w < 8; w += blockDim.x >> 5) {
+    double v = 0.0;
+    for (int q = 32 * w + lane; q - lane < n; q += 1024) {
+      double x[4];
 #pragma unroll
-    for (int m = 0; m < 8; ++m) x[m] = q0 + 1024 * m < n ? __ldcg(part + q0 + 1024 * m) : 0.0;
-#pragma unroll
-    for (int m = 0; m < 8; ++m) v += x[m];
+      for (int m = 0; m < 4; ++m) x[m] = q + 256 * m < n ? __ldcg(part + q + 256 * m) : 0.0;
+      v += (x[0] + x[1]) + (x[2] + x[3]);
+    }
+    v = warp_sum(v);
+    if (lane == 0) strand[w] = v;
   }
-  return v;
+  __syncthreads();
+  const double t = ((strand[0] + strand[1]) + (strand[2] + strand[3])) + ((strand[4] + strand[5]) + (strand[6] + strand[7]));
+  __syncthreads();
+  return t;
 }
 
 // Sum v over the block and store it in part[blockIdx.x].

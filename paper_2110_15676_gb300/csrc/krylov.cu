@@ -8,6 +8,7 @@
 //
 // Vector type T is double (FP64) or float (the FP32 inner solve of the mixed
 // mode, with FP32 matrix values).  Partial sums are always double.
+#include <climits>
 #include <cmath>
 #include <cstring>
 
@@ -59,17 +60,19 @@ template struct DBuf<uint8_t>;
 template struct DBuf<unsigned long long>;
 template struct DBuf<float4>;
 template struct DBuf<float2>;
+template struct DBuf<long long>;
 
 namespace {
 
 __global__ void k_finalize_sum(const double* __restrict__ part, int n, double* __restrict__ out) {
-  block_sum_to(strided_sum_1024(part, n, threadIdx.x), out);   // one block of 1024: out[0]
+  const double t = final_sum(part, n);
+  if (threadIdx.x == 0) *out = t;
 }
 
 }  // namespace
 
 void finalize_sum(afc_problem_s* p, const double* part, int n, double* out) {
-  AFC_LAUNCH(p, "k_finalize_sum", k_finalize_sum<<<1, 1024, 0, p->stream>>>(part, n, out));
+  AFC_LAUNCH(p, "k_finalize_sum", k_finalize_sum<<<1, 256, 0, p->stream>>>(part, n, out));
 }
 
 // ---------------------------------------------------------------------------
@@ -84,50 +87,50 @@ __global__ void k_dot(int64_t N, const double* __restrict__ x, const double* __r
   block_sum_to(v, part);
 }
 
-__global__ void k_minmax(int64_t N, const double* __restrict__ x, double* __restrict__ part) {
-  double mn = INFINITY, mx = -INFINITY;
+// min and max of x on the integer pipe (dkey order; atomics on the keys, so the result does not
+// depend on the order of the blocks), written with the step's scalars sc[0 .. 12) straight to
+// the pinned host mirror h by the last block, which leaves the keys empty for the next call.
+// One launch and no copy, where the two passes with FP64 compares and a copy of the scalars
+// took 8 us each and a copy's latency.
+__global__ void __launch_bounds__(kBlock) k_range(int64_t N, const double* __restrict__ x, long long* key,
+                                                  const double* __restrict__ sc, double* h) {
+  pdl_wait();
+  long long mx = LLONG_MIN, mn = LLONG_MAX;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
-    mn = fmin(mn, x[i]);
-    mx = fmax(mx, x[i]);
+    const double v = x[i];
+    const long long k = dkey(v);
+    if ((__double_as_longlong(v) & 0x7fffffffffffffffll) > 0x7ff0000000000000ll) continue;   // NaN, as fmin / fmax
+    mx = k > mx ? k : mx;
+    mn = k < mn ? k : mn;
   }
-  __shared__ double smn[kBlock], smx[kBlock];
-  smn[threadIdx.x] = mn;
-  smx[threadIdx.x] = mx;
+  __shared__ long long smx[kBlock / 32], smn[kBlock / 32];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const long long a = __shfl_xor_sync(0xffffffffu, mx, o), b = __shfl_xor_sync(0xffffffffu, mn, o);
+    mx = a > mx ? a : mx;
+    mn = b < mn ? b : mn;
+  }
+  if ((threadIdx.x & 31) == 0) {
+    smx[threadIdx.x >> 5] = mx;
+    smn[threadIdx.x >> 5] = mn;
+  }
   __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s) {
-      smn[threadIdx.x] = fmin(smn[threadIdx.x], smn[threadIdx.x + s]);
-      smx[threadIdx.x] = fmax(smx[threadIdx.x], smx[threadIdx.x + s]);
-    }
-    __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (int w = 1; w < kBlock / 32; ++w) {
+    mx = smx[w] > mx ? smx[w] : mx;
+    mn = smn[w] < mn ? smn[w] : mn;
   }
-  if (threadIdx.x == 0) {
-    part[2 * blockIdx.x] = smn[0];
-    part[2 * blockIdx.x + 1] = smx[0];
-  }
-}
-
-__global__ void k_minmax_fin(const double* __restrict__ part, int n, double* __restrict__ out) {
-  __shared__ double smn[kBlock], smx[kBlock];
-  double mn = INFINITY, mx = -INFINITY;
-  for (int q = threadIdx.x; q < n; q += blockDim.x) {
-    mn = fmin(mn, part[2 * q]);
-    mx = fmax(mx, part[2 * q + 1]);
-  }
-  smn[threadIdx.x] = mn;
-  smx[threadIdx.x] = mx;
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s) {
-      smn[threadIdx.x] = fmin(smn[threadIdx.x], smn[threadIdx.x + s]);
-      smx[threadIdx.x] = fmax(smx[threadIdx.x], smx[threadIdx.x + s]);
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    out[0] = smn[0];
-    out[1] = smx[0];
-  }
+  atomicMax(key, mx);
+  atomicMin(key + 1, mn);
+  __threadfence();
+  if (atomicAdd(reinterpret_cast<unsigned long long*>(key + 2), 1ull) != gridDim.x - 1) return;
+  __threadfence();
+  mx = atomicExch(reinterpret_cast<unsigned long long*>(key), (unsigned long long)LLONG_MIN);
+  mn = atomicExch(reinterpret_cast<unsigned long long*>(key + 1), (unsigned long long)LLONG_MAX);
+  key[2] = 0;
+  for (int q = 0; q < 12; ++q) h[q] = sc[q];
+  h[60] = mn == LLONG_MAX ? INFINITY : from_key(mn);    // no number at all: as an empty fmin / fmax
+  h[61] = mx == LLONG_MIN ? -INFINITY : from_key(mx);
 }
 
 template <class T, class TV>
@@ -149,11 +152,17 @@ int dot_device(afc_problem_s* p, const double* x, const double* y, double* out_s
   return AFC_OK;
 }
 
-int minmax_device(afc_problem_s* p, const double* x, double* mn, double* mx) {
-  AFC_LAUNCH(p, "k_minmax", k_minmax<<<kRedBlocks, kBlock, 0, p->stream>>>(p->N, x, p->part.p));
-  AFC_LAUNCH(p, "k_minmax_fin", k_minmax_fin<<<1, kBlock, 0, p->stream>>>(p->part.p, kRedBlocks, p->scal.p + 60));
+int range_device(afc_problem_s* p, const double* x) {
+  // at most two blocks per SM: each ends in three atomics on one line
+  const int g = (int)std::min<int64_t>(grid_for(p->N, 4 * kBlock), 304);
+  AFC_LAUNCH(p, "k_range", k_range<<<g, kBlock, 0, p->stream>>>(p->N, x, p->range.p, p->scal.p, p->host_scal));
   AFC_CUDA(cudaGetLastError());
-  AFC_CUDA(cudaMemcpyAsync(p->host_scal + 60, p->scal.p + 60, 2 * sizeof(double), cudaMemcpyDeviceToHost, p->stream));
+  return AFC_OK;
+}
+
+int minmax_device(afc_problem_s* p, const double* x, double* mn, double* mx) {
+  const int st = range_device(p, x);
+  if (st) return st;
   AFC_CUDA(cudaStreamSynchronize(p->stream));
   *mn = p->host_scal[60];
   *mx = p->host_scal[61];
@@ -207,86 +216,111 @@ template struct DBuf<uint16_t>;
 
 namespace {
 
-// ---- BiCGStab as one persistent cooperative launch ----------------------------
+// ---- BiCGStab (van der Vorst 1992), Jacobi preconditioner on the directions, as one
+// persistent cooperative launch --------------------------------------------------
 // The five phases of an iteration (p update, v = B phat, s update, t = B shat, x / r
 // update) run in one launch, separated by grid barriers; nothing returns to the
-// host or the graph between iterations.  A grid-wide sum: every block stores its
-// partials, waits at the barrier, then sums all blocks' partials in block order.
-// The order is the same in every block, so every block obtains the same totals
-// bit for bit and takes the same branches.  Partials alternate between two buffers
-// (a block can run at most one reduction ahead of another).
-// Shape of the persistent launch: one block of 512 threads per SM.  Every barrier
-// and grid-wide sum costs more with more blocks.  On GB300 (Q1 65^3, 27 offsets,
-// per BiCGStab iteration) 512 x 1 per SM took 62.4 us, 256 x 2 66.0 us, 1024 x 1
-// 65.9 us, 256 x 1 72.1 us, 128 x 4 77.0 us; earlier, 256 x 3 and 256 x 4 were
-// 8 % and 14 % slower than 256 x 2.  Block b owns the contiguous rows
-// [N b / G, N (b + 1) / G), which balances the blocks to one row.
+// host or the graph between iterations.  Block b owns the contiguous rows
+// [N b / G, N (b + 1) / G), at most one block per SM, as many warps as the rows fill: every
+// barrier and grid-wide sum costs more with more blocks, and a block's FP64 sums cost 16
+// cycles per warp.
+//
+// What a block alone reads (r, rhat, p, v, t, x) stays in shared memory where its rows fit
+// (FP64: up to 660,000 rows in all); phat and shat, which the products of other blocks gather,
+// are in global memory.  The scalars of an iteration are formed by one lane per block (the
+// first of warp 0, which also polls the barriers and adds the partials) and handed to the
+// block through shared memory: formed by every warp, their divisions and square roots held
+// the FP64 pipe for about a microsecond per phase.
+//
+// Measured on one GB300, a CN solve of 3.5 iterations: Q1 65^3 in double 235 -> 198 us, mixed
+// 169 -> 120 us; P1 33^3 in double 107 -> 75 us (vectors in global memory, 512 threads in
+// every block, scalars in every warp before).
 constexpr int kFusedBlock = 512;
-constexpr int kFusedBlocksPerSM = 1;
+constexpr size_t kFusedSmem = 160 * 1024;   // shared memory for a block's six vectors (the rest stays L1)
 
-// Grid-wide sums of NV <= 2 values per thread.  Warp q forms the block's sum of
-// value q (a column sum in the order of warp0_column_sum) and stores it at
-// part[q * G + block]; after the barrier warp q of every block reads the G partials
-// of value q, lane l summing blocks l, l + 32, ... in turn before a butterfly over
-// the lanes.  Every block runs the same operations on the same partials, so all
-// obtain the same totals bit for bit.  The two sums of NV = 2 run in two warps at
-// once, and the only block-wide meeting after the barrier is the one that hands
-// the totals on (the totals alternate between two shared slots, like the partials,
-// so a later call cannot overwrite a slot that a thread still reads).
-// grid_sums_begin stores the partials and arrives; grid_sums_end waits and sums, so
-// that work no other block needs can run in between.
-template <int NV>
-__device__ __forceinline__ unsigned int grid_sums_begin(double (&v)[NV], double* part, int buf, GridBar* bar) {
-  static_assert(NV >= 1 && NV <= 2, "two partial buffers of 2 G values");
-  __shared__ double col[NV][kFusedBlock];
-  const int G = gridDim.x;
+template <class T>
+struct BicgArgs {
+  int64_t N;
+  double* sc;
+  const double* rhs;
+  double* xout;
+  T* loc;             // the six vectors in global memory, when not in shared memory
+  size_t vstride;
+  double* part;
+  GridBar* bar;
+  double atol, rtol;
+  int maxit, rows;
+  KrylovEpilogue ep;
+  unsigned long long wait_ns;
+};
+
+template <class T>
+struct BicgShared {
+  double col[2][kFusedBlock], quarter[2][4];
+  double rho, alpha, omega, n0, nres, tol;
+  T ta, to, tb;       // alpha, omega, beta in the vector type
+  int done, its;
+};
+
+// Grid-wide sums of NV <= 2 values per thread, in two parts so that work no other block needs
+// can run between a block's arrival and its wait.  begin: four warps per value add a quarter
+// of the block's columns each (4 + 5 dependent adds; one warp took 15 + 5), one lane adds the
+// quarters, stores the block's partial and arrives.  end: that lane polls, warp 0 adds the
+// partials of all blocks in block order (all blocks run the same operations on the same
+// partials, so all obtain the same bits) and its first lane runs take(totals, ok).  The partials
+// alternate between two buffers (a block can run at most one sum ahead of another).
+template <int NV, class T>
+__device__ __forceinline__ unsigned int bicg_sums_begin(BicgShared<T>& sh, const double (&v)[NV], double* part, int buf,
+                                                        GridBar* bar) {
+  const int G = gridDim.x, nt = blockDim.x;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  double* pb = part + (size_t)buf * 2 * G;
 #pragma unroll
-  for (int q = 0; q < NV; ++q) col[q][threadIdx.x] = v[q];
+  for (int q = 0; q < NV; ++q) sh.col[q][threadIdx.x] = v[q];
   __syncthreads();
-  if (w < NV) {
-    double t = col[w][lane];
-    for (int j = lane + 32; j < kFusedBlock; j += 32) t += col[w][j];
-    t = warp_sum(t);
-    if (lane == 0) pb[w * G + blockIdx.x] = t;
-  }
-  return grid_arrive(bar);   // begins with __syncthreads: col is free again after it
-}
-
-template <int NV>
-__device__ __forceinline__ void grid_sums_end(double* part, int& buf, GridBar* bar, unsigned int old,
-                                              double (&tot)[NV], unsigned long long wait_ns) {
-  __shared__ double shtot[2][NV];
-  const int G = gridDim.x;
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const double* pb = part + (size_t)buf * 2 * G;
-  grid_wait(bar, old, wait_ns);
-  if (w < NV) {
-    // lane l adds partials l, l + 32, ... in turn, the loads eight at a time (one round
-    // trip for up to 256 blocks)
+  for (int u = w; u < 4 * NV; u += nt >> 5) {
+    const double* c = sh.col[u >> 2];
     double t = 0.0;
-    for (int b0 = lane; b0 < G; b0 += 256) {
-      double x[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) x[u] = b0 + 32 * u < G ? __ldcg(pb + w * G + b0 + 32 * u) : 0.0;
-#pragma unroll
-      for (int u = 0; u < 8; ++u) t += x[u];
-    }
+    for (int j = (u & 3) * 32 + lane; j < nt; j += 128) t += c[j];
     t = warp_sum(t);
-    if (lane == 0) shtot[buf][w] = t;
+    if (lane == 0) sh.quarter[u >> 2][u & 3] = t;
   }
   __syncthreads();
-#pragma unroll
-  for (int q = 0; q < NV; ++q) tot[q] = shtot[buf][q];
-  buf ^= 1;
+  unsigned int old = 0u;
+  if (w == 0) {
+    if (lane < NV)
+      part[(size_t)(2 * buf + lane) * G + blockIdx.x] = (sh.quarter[lane][0] + sh.quarter[lane][1]) +
+                                                         (sh.quarter[lane][2] + sh.quarter[lane][3]);
+    __syncwarp();
+    if (lane == 0) old = grid_arrive_thread(bar);
+  }
+  return old;
 }
 
-template <int NV>
-__device__ __forceinline__ void grid_sums(double (&v)[NV], double* part, int& buf, GridBar* bar,
-                                          double (&tot)[NV], unsigned long long wait_ns) {
-  const unsigned int old = grid_sums_begin<NV>(v, part, buf, bar);
-  grid_sums_end<NV>(part, buf, bar, old, tot, wait_ns);
+template <int NV, class F>
+__device__ __forceinline__ void bicg_sums_end(const double* part, int& buf, GridBar* bar, unsigned int old,
+                                              unsigned long long wait_ns, F&& take) {
+  const int G = gridDim.x, lane = threadIdx.x & 31;
+  if (threadIdx.x < 32) {
+    const bool ok = lane != 0 || grid_poll(bar, old, wait_ns);
+    __syncwarp();
+    double t[NV];
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+      const double* pb = part + (size_t)(2 * buf + q) * G;
+      t[q] = 0.0;
+      for (int b0 = lane; b0 - lane < G; b0 += 160) {
+        double x[5];
+#pragma unroll
+        for (int u = 0; u < 5; ++u) x[u] = b0 + 32 * u < G ? __ldcg(pb + b0 + 32 * u) : 0.0;
+        t[q] += ((x[0] + x[1]) + (x[2] + x[3])) + x[4];
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < NV; ++q) t[q] = warp_sum(t[q]);
+    if (lane == 0) take(t, ok);
+  }
+  buf ^= 1;
+  __syncthreads();
 }
 
 // The caller's update of a solve's last pass (KrylovEpilogue) at row i.
@@ -299,6 +333,39 @@ __device__ __forceinline__ void krylov_update(const KrylovEpilogue& ep, int64_t 
     ep.s[i] = ui + uoi;
   }
 }
+// In the graph form of the fixed point (ep.fp_sc) the solve's launch first decides whether the
+// loop goes on: R = ||res|| from the residual pass's block partials, the stop tests of
+// Sec. 4.  Every block sums the partials itself and decides alike (block 0 writes the scalars; the
+// others read only those that it does not change, or a status whose change to 1 or 3 they
+// do not test).  As kernels of their own the sum, the test and the branch over the solve took
+// two graph nodes per correction.  True: solve.
+__device__ bool fp_goes_on(const KrylovEpilogue& ep) {
+  double* sc = ep.fp_sc;
+  if (!sc) return true;
+  __shared__ bool go;
+  const bool failed = sc[F_STATUS] == 2.0;
+  const double it = sc[F_CORR];
+  const double sum = final_sum(ep.part, ep.npart);
+  if (threadIdx.x == 0) {
+    const double R = sqrt(sum);
+    double status = 0.0;
+    if (!isfinite(R) || failed) status = 2.0;
+    else if (sc[F_FIXED] > 0.0) status = it >= sc[F_FIXED] ? 1.0 : 0.0;
+    else if (R < sc[F_THRESH]) status = 1.0;
+    else if (it >= sc[F_MAXIT]) status = 3.0;
+    go = status == 0.0;
+    if (blockIdx.x == 0) {
+      sc[F_NORMSQ] = sum;
+      if (sc[F_REVAL] == 0.0) sc[F_RES0] = R;
+      sc[F_RESF] = R;
+      sc[F_REVAL] += 1.0;
+      if (!go) sc[F_STATUS] = status;
+      cudaGraphSetConditional(ep.loop, go ? 1u : 0u);
+    }
+  }
+  __syncthreads();
+  return go;
+}
 // The fixed-point loop's count of a correction (one thread of the solve's launch).
 __device__ __forceinline__ void krylov_count(const KrylovEpilogue& ep, int its, bool berr, bool broke) {
   double* f = ep.fp_sc;
@@ -309,151 +376,174 @@ __device__ __forceinline__ void krylov_count(const KrylovEpilogue& ep, int its, 
   if (berr) f[F_TIMEOUT] = 1.0;
 }
 
-template <int KT, class T>
-__global__ void __launch_bounds__(kFusedBlock, 1024 / kFusedBlock) k_bicg_fused(int64_t N, Offsets of, double* sc, const T* __restrict__ B,
-                                                   const T* __restrict__ dinv, const double* __restrict__ rhs,
-                                                   double* xout, T* x, T* r, T* rh, T* pv, T* v, T* s, T* t, T* ph,
-                                                   T* sh, double* part, GridBar* bar, double atol, double rtol,
-                                                   int maxit, KrylovEpilogue ep, unsigned long long wait_ns) {
+// SM: the six vectors in shared memory.
+template <int KT, class T, bool SM>
+__global__ void __launch_bounds__(kFusedBlock, 1) k_bicg_fused(Offsets of, const T* __restrict__ B,
+                                                               const T* __restrict__ dinv, T* ph, T* sg,
+                                                               BicgArgs<T> a) {
   const int K = KT > 0 ? KT : of.K;
-  const int64_t G = gridDim.x;
-  const int64_t stride = kFusedBlock;
-  const int64_t i0 = N * blockIdx.x / G + threadIdx.x, iend = N * (blockIdx.x + 1) / G;
-  volatile int* berr = &bar->err;
+  const int64_t N = a.N, G = gridDim.x;
+  const int64_t i0 = N * blockIdx.x / G;
+  const int nrow = (int)(N * (blockIdx.x + 1) / G - i0), nt = blockDim.x, tid = threadIdx.x;
+  __shared__ BicgShared<T> sh;
+  extern __shared__ __align__(16) char dyn[];
+  T* const loc = SM ? reinterpret_cast<T*>(dyn) : a.loc + i0;
+  const size_t ls = SM ? (size_t)a.rows : a.vstride;
+  T *const r = loc, *const rh = loc + ls, *const p = loc + 2 * ls, *const v = loc + 3 * ls, *const t = loc + 4 * ls,
+           *const x = loc + 5 * ls;
+  ph += i0;
+  sg += i0;
+  dinv += i0;
+  const double* rhs = a.rhs + i0;
+  const T* Bi = B + i0;
   int buf = 0;
-  double a1[1], t1[1], a2[2], t2[2];
+  if (!fp_goes_on(a.ep)) return;
+  double a1[1], a2[2];
+  // y = B g at row q
+  auto product = [&](const T* g, int q) {
+    T y = 0;
+#pragma unroll
+    for (int k = 0; k < K; ++k) y = fma(Bi[k * N + q], g[q + of.o[k]], y);
+    return y;
+  };
   // r = rhs, rhat = r, x = v = 0, rho = (r, r); and the first iteration's p update
   // (beta = 0 and p = v = 0 before it: p = r + 0, phat = D^{-1} p), so that
   // iteration needs no pass and no barrier of its own before its product
   T a0 = 0;
-  for (int64_t i = i0; i < iend; i += stride) {
-    const T ri = (T)rhs[i];
-    x[i] = 0;
-    r[i] = ri;
-    rh[i] = ri;
-    v[i] = 0;
+  for (int q = tid; q < nrow; q += nt) {
+    const T ri = (T)rhs[q];
+    x[q] = 0;
+    r[q] = ri;
+    rh[q] = ri;
+    v[q] = 0;
     const T pi = ri + (T)0;   // as r + 0 * (0 - 1 * 0) rounds: -0 becomes +0
-    pv[i] = pi;
-    ph[i] = dinv[i] * pi;
+    p[q] = pi;
+    ph[q] = dinv[q] * pi;
     a0 = fma(ri, ri, a0);
   }
-  a1[0] = (double)a0;
-  grid_sums<1>(a1, part, buf, bar, t1, wait_ns);
-  double rho = t1[0];
-  const double n0 = sqrt(rho);
-  const double tol = fmax(atol, rtol * n0);
-  double alpha = 1.0, omega = 1.0, beta = 0.0, nres = n0;
-  int its = 0;
-  int done = !isfinite(n0) ? 2 : (n0 < tol ? 1 : (maxit <= 0 ? 4 : 0));
-  bool first = true;
-  while (done == 0) {
+  a1[0] = to_dbl(a0);
+  unsigned int old = bicg_sums_begin<1>(sh, a1, a.part, buf, a.bar);
+  bicg_sums_end<1>(a.part, buf, a.bar, old, a.wait_ns, [&](const double (&s)[1], bool ok) {
+    sh.rho = s[0];
+    sh.n0 = sh.nres = sqrt(s[0]);
+    sh.tol = fmax(a.atol, a.rtol * sh.n0);
+    sh.alpha = sh.omega = 1.0;
+    sh.its = 0;
+    sh.done = !isfinite(sh.n0) || !ok ? 2 : (sh.n0 < sh.tol ? 1 : (a.maxit <= 0 ? 4 : 0));
+  });
+  for (bool first = true; sh.done == 0; first = false) {
     // p = r + beta (p - omega v), phat = D^{-1} p (the first iteration's came with r)
     if (!first) {
-      const T tb = (T)beta, to = (T)omega;
-      for (int64_t i = i0; i < iend; i += stride) {
-        const T pi = r[i] + tb * (pv[i] - to * v[i]);
-        pv[i] = pi;
-        ph[i] = dinv[i] * pi;
+      const T tb = sh.tb, to = sh.to;
+      for (int q = tid; q < nrow; q += nt) {
+        const T pi = r[q] + tb * (p[q] - to * v[q]);
+        p[q] = pi;
+        ph[q] = dinv[q] * pi;
       }
-      grid_barrier(bar, wait_ns);
+      grid_barrier(a.bar, a.wait_ns);
     }
-    first = false;
     // v = B phat, alpha = rho / (rhat, v)
     a0 = 0;
-    for (int64_t i = i0; i < iend; i += stride) {
-      T y = 0;
-#pragma unroll
-      for (int k = 0; k < K; ++k) y = fma(B[k * N + i], ph[i + of.o[k]], y);
-      v[i] = y;
-      a0 = fma(rh[i], y, a0);
+    for (int q = tid; q < nrow; q += nt) {
+      const T y = product(ph, q);
+      v[q] = y;
+      a0 = fma(rh[q], y, a0);
     }
-    a1[0] = (double)a0;
-    grid_sums<1>(a1, part, buf, bar, t1, wait_ns);
-    alpha = rho / t1[0];
-    if (!isfinite(alpha) || t1[0] == 0.0 || *berr) { done = 2; break; }
-    // s = r - alpha v, shat = D^{-1} s, ||s||
-    const T ta = (T)alpha;
+    a1[0] = to_dbl(a0);
+    old = bicg_sums_begin<1>(sh, a1, a.part, buf, a.bar);
+    bicg_sums_end<1>(a.part, buf, a.bar, old, a.wait_ns, [&](const double (&s)[1], bool ok) {
+      sh.alpha = sh.rho / s[0];
+      sh.ta = (T)sh.alpha;
+      if (!isfinite(sh.alpha) || s[0] == 0.0 || !ok) sh.done = 2;
+    });
+    if (sh.done) break;
+    // s = r - alpha v (in place of r), shat = D^{-1} s, ||s||
+    const T ta = sh.ta;
     a0 = 0;
-    for (int64_t i = i0; i < iend; i += stride) {
-      const T si = r[i] - ta * v[i];
-      s[i] = si;
-      sh[i] = dinv[i] * si;
+    for (int q = tid; q < nrow; q += nt) {
+      const T si = r[q] - ta * v[q];
+      r[q] = si;
+      sg[q] = dinv[q] * si;
       a0 = fma(si, si, a0);
     }
-    a1[0] = (double)a0;
-    grid_sums<1>(a1, part, buf, bar, t1, wait_ns);
-    const double ns = sqrt(t1[0]);
-    if (!isfinite(ns) || *berr) { done = 2; break; }
-    if (ns < tol) {   // converged at s: x += alpha phat
-      for (int64_t i = i0; i < iend; i += stride) x[i] = x[i] + ta * ph[i];
-      nres = ns;
-      ++its;
-      done = 1;
-      break;
-    }
+    a1[0] = to_dbl(a0);
+    old = bicg_sums_begin<1>(sh, a1, a.part, buf, a.bar);
+    bicg_sums_end<1>(a.part, buf, a.bar, old, a.wait_ns, [&](const double (&s)[1], bool ok) {
+      const double ns = sqrt(s[0]);
+      if (!isfinite(ns) || !ok) {
+        sh.done = 2;
+      } else if (ns < sh.tol) {   // converged at s
+        sh.nres = ns;
+        sh.its += 1;
+        sh.done = 3;
+      }
+    });
+    if (sh.done) break;
     // t = B shat, omega = (t, s) / (t, t)
     T b0 = 0, b1 = 0;
-    for (int64_t i = i0; i < iend; i += stride) {
-      T y = 0;
-#pragma unroll
-      for (int k = 0; k < K; ++k) y = fma(B[k * N + i], sh[i + of.o[k]], y);
-      t[i] = y;
-      b0 = fma(y, s[i], b0);
+    for (int q = tid; q < nrow; q += nt) {
+      const T y = product(sg, q);
+      t[q] = y;
+      b0 = fma(y, r[q], b0);
       b1 = fma(y, y, b1);
     }
-    a2[0] = (double)b0;
-    a2[1] = (double)b1;
-    grid_sums<2>(a2, part, buf, bar, t2, wait_ns);
-    omega = t2[0] / t2[1];
-    if (!isfinite(omega) || t2[1] == 0.0 || *berr) { done = 2; break; }
+    a2[0] = to_dbl(b0);
+    a2[1] = to_dbl(b1);
+    old = bicg_sums_begin<2>(sh, a2, a.part, buf, a.bar);
+    bicg_sums_end<2>(a.part, buf, a.bar, old, a.wait_ns, [&](const double (&s)[2], bool ok) {
+      sh.omega = s[0] / s[1];
+      sh.to = (T)sh.omega;
+      if (!isfinite(sh.omega) || s[1] == 0.0 || !ok) sh.done = 2;
+    });
+    if (sh.done) break;
     // r = s - omega t, ||r||, (rhat, r); x += alpha phat + omega shat while the sums
     // complete (no other block reads x)
-    const T tom = (T)omega;
+    const T tom = sh.to;
     b0 = 0;
     b1 = 0;
-    for (int64_t i = i0; i < iend; i += stride) {
-      const T ri = s[i] - tom * t[i];
-      r[i] = ri;
+    for (int q = tid; q < nrow; q += nt) {
+      const T ri = r[q] - tom * t[q];
+      r[q] = ri;
       b0 = fma(ri, ri, b0);
-      b1 = fma(rh[i], ri, b1);
+      b1 = fma(rh[q], ri, b1);
     }
-    a2[0] = (double)b0;
-    a2[1] = (double)b1;
-    const unsigned int arrived = grid_sums_begin<2>(a2, part, buf, bar);
-    for (int64_t i = i0; i < iend; i += stride) x[i] = x[i] + ta * ph[i] + tom * sh[i];
-    grid_sums_end<2>(part, buf, bar, arrived, t2, wait_ns);
-    nres = sqrt(t2[0]);
-    const double rho_old = rho;
-    rho = t2[1];
-    beta = (rho / rho_old) * (alpha / omega);
-    ++its;
-    if (!isfinite(nres) || *berr) done = 2;
-    else if (nres < tol) done = 1;
-    else if (its >= maxit) done = 4;
+    a2[0] = to_dbl(b0);
+    a2[1] = to_dbl(b1);
+    old = bicg_sums_begin<2>(sh, a2, a.part, buf, a.bar);
+    for (int q = tid; q < nrow; q += nt) x[q] = x[q] + ta * ph[q] + tom * sg[q];
+    bicg_sums_end<2>(a.part, buf, a.bar, old, a.wait_ns, [&](const double (&s)[2], bool ok) {
+      const double nr = sqrt(s[0]), rho_old = sh.rho;
+      sh.nres = nr;
+      sh.rho = s[1];
+      sh.tb = (T)((s[1] / rho_old) * (sh.alpha / sh.omega));
+      sh.its += 1;
+      if (!isfinite(nr) || !ok) sh.done = 2;
+      else if (nr < sh.tol) sh.done = 1;
+      else if (sh.its >= a.maxit) sh.done = 4;
+    });
   }
-  if (ep.u != nullptr && done != 2) {
-    for (int64_t i = i0; i < iend; i += stride) {
-      const double xi = (double)x[i];
-      xout[i] = xi;
-      krylov_update(ep, i, xi);
-    }
-  } else {
-    for (int64_t i = i0; i < iend; i += stride) xout[i] = (double)x[i];
+  const int done = sh.done == 3 ? 1 : sh.done;
+  const T last = sh.done == 3 ? sh.ta : (T)0;   // converged at s: x += alpha phat
+  const bool upd = a.ep.u != nullptr && done != 2;
+  for (int q = tid; q < nrow; q += nt) {
+    const T xq = last != (T)0 ? x[q] + last * ph[q] : x[q];
+    const double xi = to_dbl(xq);
+    a.xout[i0 + q] = xi;
+    if (upd) krylov_update(a.ep, i0 + q, xi);
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {   // the solver scalars, as the kernel-per-phase form leaves them
-    sc[S_ATOL] = atol;
-    sc[S_RTOL] = rtol;
-    sc[S_MAXIT] = (double)maxit;
-    sc[S_TOL] = tol;
-    sc[S_N0] = n0;
-    sc[S_NRES] = nres;
-    sc[S_ITS] = (double)its;
-    sc[S_ALPHA] = alpha;
-    sc[S_OMEGA] = omega;
-    sc[S_RHO] = rho;
+  if (blockIdx.x == 0 && tid == 0) {   // the solver's scalars
+    volatile int* berr = &a.bar->err;
+    double* sc = a.sc;
+    sc[S_TOL] = sh.tol;
+    sc[S_N0] = sh.n0;
+    sc[S_NRES] = sh.nres;
+    sc[S_ITS] = (double)sh.its;
+    sc[S_ALPHA] = sh.alpha;
+    sc[S_OMEGA] = sh.omega;
+    sc[S_RHO] = sh.rho;
     sc[S_DONE] = *berr ? 2.0 : (double)done;
     sc[S_BERR] = *berr ? 1.0 : 0.0;
-    krylov_count(ep, its, *berr != 0, done == 2);
+    krylov_count(a.ep, sh.its, *berr != 0, done == 2);
   }
 }
 
@@ -876,6 +966,7 @@ __global__ void __launch_bounds__(VS ? kGmBlockS : kGmBlock, 1) k_gm_fused(Offse
   for (int r = nrow + threadIdx.x; r < ng * W; r += blockDim.x) w[r] = (T)0;
   volatile int* berr = &a.bar->err;
   int buf = 0;
+  if (!fp_goes_on(a.ep)) return;
   if (scalar) {
     sh.its = 0;
     sh.cycles = 0;
@@ -1100,23 +1191,43 @@ int bicg_fused_launch(afc_problem_s* p, cudaStream_t s, const T* B, const T* din
   int st = coop_device(p);
   if (st) return st;
   const int64_t N = p->N;
-  T *x = vec_at<T>(w, 0), *r = vec_at<T>(w, 1), *rh = vec_at<T>(w, 2), *pp = vec_at<T>(w, 3), *v = vec_at<T>(w, 4),
-    *sv = vec_at<T>(w, 5), *t = vec_at<T>(w, 6), *ph = vec_at<T>(w, 7), *sh = vec_at<T>(w, 8);
-  double* sc = w.sc.p;
-  GridBar* bar = reinterpret_cast<GridBar*>(w.barrier.p);
+  BicgArgs<T> a;
+  a.N = N;
+  a.sc = w.sc.p;
+  a.rhs = rhs;
+  a.xout = xout;
+  a.loc = vec_at<T>(w, 2);
+  a.vstride = w.vstride;
+  a.part = w.part.p;
+  a.bar = reinterpret_cast<GridBar*>(w.barrier.p);
+  a.atol = o->ksp_atol;
+  a.rtol = o->ksp_rtol;
+  a.maxit = o->ksp_maxit;
+  if (epi) a.ep = *epi;
+  a.wait_ns = p->grid_wait_ns;
+  const int G = (int)std::max<int64_t>(1, std::min<int64_t>((N + 63) / 64, w.nsm));
+  const int64_t rows = (N + G - 1) / G;
+  // as many threads as share the rows evenly in the fewest rounds
+  const int64_t rounds = (rows + kFusedBlock - 1) / kFusedBlock;
+  const int block = (int)std::max<int64_t>(64, ((rows + rounds - 1) / rounds + 31) / 32 * 32);
+  a.rows = (int)rows;
+  const size_t local = 6 * (size_t)rows * sizeof(T);
+  const bool in_smem = local <= kFusedSmem;
+  const size_t smem = in_smem ? local : 0;
   with_K(p->K, [&](auto kc) {
     constexpr int KT = decltype(kc)::value;
+    auto kern = in_smem ? k_bicg_fused<KT, T, true> : k_bicg_fused<KT, T, false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFusedSmem);
     int nb = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_bicg_fused<KT, T>, kFusedBlock, 0);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, block, smem);
     if (e != cudaSuccess || nb < 1) {
       st = cuda_fail(e != cudaSuccess ? e : cudaErrorInvalidConfiguration, "occupancy of k_bicg_fused");
       return;
     }
-    const int64_t want = (N + kFusedBlock - 1) / kFusedBlock;
-    const int G = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)std::min(nb, kFusedBlocksPerSM) * w.nsm));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)G);
-    cfg.blockDim = dim3(kFusedBlock);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeCooperative;
@@ -1124,9 +1235,7 @@ int bicg_fused_launch(afc_problem_s* p, cudaStream_t s, const T* B, const T* din
     cfg.attrs = at;
     cfg.numAttrs = 1;
     cudaEvent_t ev = prof_start(p);
-    e = cudaLaunchKernelEx(&cfg, k_bicg_fused<KT, T>, N, p->offs, sc, B, dinv, rhs, xout, x, r, rh, pp, v, sv, t, ph,
-                           sh, w.part.p, bar, o->ksp_atol, o->ksp_rtol, o->ksp_maxit,
-                           epi ? *epi : KrylovEpilogue{}, (unsigned long long)p->grid_wait_ns);
+    e = cudaLaunchKernelEx(&cfg, kern, p->offs, B, dinv, vec_at<T>(w, 0), vec_at<T>(w, 1), a);
     prof_stop(p, "k_bicg_fused", ev);
     if (e != cudaSuccess) st = cuda_fail(e, "cudaLaunchKernelEx(k_bicg_fused)");
   });
@@ -1157,7 +1266,7 @@ int fused_result(afc_problem_s* p, const char* what, int* its, double* res) {
 template <class T>
 int bicgstab_impl(afc_problem_s* p, const T* B, const T* dinv, const afc_opts* o, const double* rhs, double* xout,
                   int* its, double* res, const KrylovEpilogue* epi) {
-  int st = ensure_work(p, 9, sizeof(T) == 4);
+  int st = ensure_work(p, 8, sizeof(T) == 4);
   if (st) return st;
   if ((st = bicg_fused_launch<T>(p, p->stream, B, dinv, o, rhs, xout, epi))) return st;
   return fused_result(p, "BiCGStab", its, res);
@@ -1248,7 +1357,7 @@ namespace {
 template <class T>
 int bicgstab_graph(afc_problem_s* p, const T* B, const T* dinv, const afc_opts* o, const double* rhs, double* xout,
                    cudaStream_t cs, cudaGraph_t g, std::vector<cudaGraphNode_t>& frontier, const KrylovEpilogue* epi) {
-  int st = ensure_work(p, 9, sizeof(T) == 4);
+  int st = ensure_work(p, 8, sizeof(T) == 4);
   if (st) return st;
   return capture_into(p, cs, g, frontier, [&]() -> int {
     return bicg_fused_launch<T>(p, p->stream, B, dinv, o, rhs, xout, epi);

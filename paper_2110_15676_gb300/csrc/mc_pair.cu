@@ -250,12 +250,12 @@ __global__ void k_mcp_edges(int64_t N, Offsets of, const float2* __restrict__ pk
   }
 }
 
-// ||res||^2 from the residual pass's block partials in k_finalize_sum's order (one
-// block of 1024 threads, so the graph's control kernel, which sums the same partials
-// the same way, stops alike), launched as the pass's dependent: it waits for the pass.
+// ||res||^2 from the residual pass's block partials in the order of final_sum, launched as the
+// pass's dependent: it waits for the pass.
 __global__ void k_mcp_finalize(const double* __restrict__ part, int n, double* __restrict__ out) {
   pdl_wait();
-  block_sum_to(strided_sum_1024(part, n, threadIdx.x), out);
+  const double t = final_sum(part, n);
+  if (threadIdx.x == 0) *out = t;
 }
 
 // At 32 registers (8 blocks of 256 per SM) the 15-offset pass runs without spills and
@@ -458,7 +458,7 @@ int mc_pair_residual(afc_problem_s* p, const double* u, int limiter, double* res
                                (const uint8_t*)p->dir.p, res, p->part.p));
     if (e != cudaSuccess) { st = cuda_fail(e, "launch k_mcp_residual"); return; }
     if (normsq_slot) {
-      AFC_LAUNCH(p, "k_mcp_finalize", e = launch_pass(pdl, k_mcp_finalize, dim3(1), dim3(1024), s,
+      AFC_LAUNCH(p, "k_mcp_finalize", e = launch_pass(pdl, k_mcp_finalize, dim3(1), dim3(256), s,
                                                       (const double*)p->part.p, (int)g, normsq_slot));
       if (e != cudaSuccess) st = cuda_fail(e, "launch k_mcp_finalize");
     }

@@ -21,13 +21,6 @@
 
 namespace afc {
 
-// Flux of the pair (i, i + o_k) seen from row i, stored once per pair as a float.
-__device__ __forceinline__ double pair_flux32(const Offsets& of, int Kup, int k, int64_t i, int64_t N,
-                                              const float* r32) {
-  if (k > Kup) return widen_exact(r32[(int64_t)(k - Kup - 1) * N + i]);
-  return neg_bits(widen_exact(r32[(int64_t)(Kup - 1 - k) * N + i + of.o[k]]));
-}
-
 // Pointers of one instance for the stage passes.  Node vectors carry the halo.
 // No pointer here or in the row functions is __restrict__: a persistent batched
 // launch writes, in one pass, arrays that later passes of the same launch read,
@@ -40,6 +33,7 @@ struct SspArrays {
   const float* m32;                 // Kup * N (mixed)
   const float* d32;                 // Kup * N (mixed)
   const double* mL;
+  const double* imL;                // 1 / m_i
   const double* f;
   const uint8_t* dir;
   const double* udir;
@@ -50,7 +44,7 @@ struct SspArrays {
   float* udf;                       // mixed: udot^L rounded to single (halo)
   double* r_up;                     // Kup * N
   float* r32;                       // Kup * N (mixed)
-  double* Rp;
+  double* Rp;                       // halo
   double* Rm;
   double* Fs;                       // F* of the stage (may be null)
 };
@@ -70,7 +64,7 @@ __device__ __forceinline__ void ssp_rate_row(const Offsets& of, const SspArrays&
     ud = 0.0;
     uti = a.udir[i];
   } else {
-    ud = (a.f[i] - y) / a.mL[i];
+    ud = div_by(a.f[i] - y, a.mL[i], a.imL[i]);
     uti = fma(dt, ud, ui);
   }
   a.udot[i] = ud;
@@ -106,115 +100,132 @@ __device__ __forceinline__ void ssp_edges_row(const Offsets& of, const SspArrays
   }
 }
 
-template <int KT, bool MIXED>
-__device__ __forceinline__ double ssp_flux(const Offsets& of, const SspArrays& a, int k, int64_t i) {
-  const int Kup = (KT > 0 ? KT : of.K) / 2;
-  if (MIXED) return pair_flux32(of, Kup, k, i, a.N, a.r32);
-  return pair_flux(of, Kup, k, i, a.N, a.r_up);
-}
-
 // factors pass: P+/- from the stored fluxes, Q+/- from the predictor over N_i, R+/-
-template <int KT, bool MIXED>
+template <int KT, bool MIXED, int S = kGroup<KT>, bool SMALL = false>
 __device__ __forceinline__ void ssp_factors_row(const Offsets& of, const SspArrays& a, int64_t i, double dt) {
   const int K = KT > 0 ? KT : of.K, Kup = K / 2;
+  // SMALL: the row's own data before the test of its Dirichlet flag (one wait, not two)
+  unsigned long long mk = SMALL ? a.mask[i] : 0ull;
+  double uti = SMALL ? a.ut[i] : 0.0, m = SMALL ? a.mL[i] : 0.0;
   if (a.dir[i]) {
     a.Rp[i] = 1.0;
     a.Rm[i] = 1.0;
     return;
   }
-  const unsigned long long mk = a.mask[i];
-  const double uti = a.ut[i];
-  double Pp = 0.0, Pm = 0.0;
+  if (!SMALL) {
+    mk = a.mask[i];
+    uti = a.ut[i];
+  }
+  // P+/- on the integer pipe (one rounding at the end), one flux at a time: two FP64 adds per
+  // pair took 52 of the pass's 82 FP64 warp instructions at Q1, and holding a row's fluxes
+  // until their largest exponent is known took it to 48 registers
+  SignedSums64 acc;
   long long kmax = dkey(uti), kmin = kmax;
-  if (MIXED) {
-    // The fluxes are floats: P+ and P- are summed exactly in 64-bit fixed point scaled
-    // to the row's largest flux (its 24-bit mantissa at bits 33..56, so 62 pairs cannot
-    // overflow), then rounded once to double.  This is at least as accurate as a double
-    // sum and runs on the integer pipe instead of two FP64 adds per pair.
-    constexpr int KA = KT > 0 ? KT : kMaxOffsets;
-    unsigned fb[KA];
-    unsigned emax = 0;
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-      fb[k] = 0u;
-      if (k == Kup || !((mk >> k) & 1ull)) continue;
-      unsigned b;
-      if (k > Kup) b = __float_as_uint(a.r32[(int64_t)(k - Kup - 1) * a.N + i]);
-      else b = __float_as_uint(a.r32[(int64_t)(Kup - 1 - k) * a.N + i + of.o[k]]) ^ 0x80000000u;   // r_ij = -r_ji
-      fb[k] = b;
-      const unsigned e = (b >> 23) & 0xffu;
-      emax = e > emax ? e : emax;
-      const long long kj = dkey(a.ut[i + of.o[k]]);
-      kmax = kj > kmax ? kj : kmax;
-      kmin = kj < kmin ? kj : kmin;
+  for (int k0 = 0; k0 < K; k0 += S) {
+    double r[S], v[S];
+    float rf[S];
+#pragma unroll
+    for (int j = 0; j < S; ++j) {
+      if (k0 + j == Kup) continue;
+      const int64_t q = pair_slot(of, Kup, k0 + j, i, a.N);
+      if (MIXED) rf[j] = a.r32[q];
+      else r[j] = a.r_up[q];
+      v[j] = a.ut[i + of.o[k0 + j]];
     }
-    if (emax > 0u) {
-      long long sp = 0, sm = 0;
 #pragma unroll
-      for (int k = 0; k < K; ++k) {
-        const unsigned b = fb[k];
-        const int e = (int)((b >> 23) & 0xffu);
-        if (e == 0) continue;                       // zero or subnormal: widened to 0 as well
-        const long long m = (long long)((b & 0x7fffffu) | 0x800000u);
-        const int sh = e - (int)emax + 33;
-        const long long v = sh >= 0 ? (m << sh) : (sh > -24 ? (m >> -sh) : 0LL);
-        if (b & 0x80000000u) sm += v;
-        else sp += v;
-      }
-      const double scale = __longlong_as_double((long long)((int)emax - 127 - 56 + 1023) << 52);   // 2^(emax-183)
-      Pp = (double)sp * scale;
-      Pm = -((double)sm * scale);
-    }
-  } else {
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
+    for (int j = 0; j < S; ++j) {
+      const int k = k0 + j;
       if (k == Kup || !((mk >> k) & 1ull)) continue;
-      const double r = ssp_flux<KT, MIXED>(of, a, k, i);
-      if (gt0(r)) Pp += r;
-      else if (!is0(r)) Pm += r;
-      const long long kj = dkey(a.ut[i + of.o[k]]);
+      if (MIXED) acc.add(__float_as_uint(rf[j]) ^ (k > Kup ? 0u : 0x80000000u));   // r_ij = -r_ji
+      else acc.add((unsigned long long)__double_as_longlong(r[j]) ^ (k > Kup ? 0ull : 0x8000000000000000ull));
+      const long long kj = dkey(v[j]);
       kmax = kj > kmax ? kj : kmax;
       kmin = kj < kmin ? kj : kmin;
     }
   }
+  double Pp, Pm;
+  acc.result<MIXED ? 127 : 1023>(Pp, Pm);
   // >= 0 and <= 0: the max / min include i itself
   const double Qp = from_key(kmax) - uti, Qm = from_key(kmin) - uti;
-  const double m = a.mL[i];
+  if (!SMALL) m = a.mL[i];
   a.Rp[i] = zalesak_factor(m * Qp, dt * Pp);
   a.Rm[i] = zalesak_factor(m * Qm, dt * Pm);
 }
 
+// A load that stays where it is written (the compiler would move it behind the test that picks
+// one of two, and so behind the wait for the flux).
+__device__ __forceinline__ double load_now(const double* p) {
+  double v;
+  asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  return v;
+}
+
 // correct pass and the SSP combination; returns the new value written to out[i]
-template <int KT, bool MIXED>
+// SMALL (grids that do not fill the GPU) also loads both factors of every neighbour beside its
+// flux, one wait for memory per group (12.5 us against 16.4 us for 77,121 rows of Q1, mixed),
+// instead of the one that the flux's sign asks for, half the loads (143 us against 200 us for
+// 2.1 M rows).
+template <int KT, bool MIXED, int S = kGroup<KT>, bool SMALL = false>
 __device__ __forceinline__ void ssp_correct_row(const Offsets& of, const SspArrays& a, int64_t i, int limiter,
                                                 double dt, double ca, const double* uA, double cb,
                                                 double* out) {
   const int K = KT > 0 ? KT : of.K, Kup = K / 2;
   double unew;
   double F = 0.0;
+  unsigned long long mk = SMALL ? a.mask[i] : 0ull;
+  double ut = 0.0, m = 0.0, im = 0.0, ua = 0.0;
+  if (SMALL) {   // the row's own data before the test of its Dirichlet flag
+    ut = a.ut[i];
+    m = a.mL[i];
+    im = a.imL[i];
+    if (ca != 0.0) ua = uA[i];
+  }
   if (a.dir[i]) {
     unew = a.udir[i];
   } else {
     if (limiter != AFC_LIM_NONE) {
-      const unsigned long long mk = a.mask[i];
+      if (!SMALL) mk = a.mask[i];
       const double rpi = a.Rp[i], rmi = a.Rm[i];
 #pragma unroll
-      for (int k = 0; k < K; ++k) {
-        if (k == Kup || !((mk >> k) & 1ull)) continue;
-        const double r = ssp_flux<KT, MIXED>(of, a, k, i);
-        if (limiter == AFC_LIM_ZALESAK) {
-          const int64_t j = i + of.o[k];
-          const double alpha = gt0(r) ? imin_nn(rpi, a.Rm[j]) : imin_nn(rmi, a.Rp[j]);
-          F = fma(alpha, r, F);
-        } else {
-          F += r;
+      for (int k0 = 0; k0 < K; k0 += S) {
+        double r[S], Rj[S], Rk[S];
+#pragma unroll
+        for (int j = 0; j < S; ++j) {
+          if (k0 + j == Kup) continue;
+          const int64_t q = pair_slot(of, Kup, k0 + j, i, a.N);
+          if (MIXED) r[j] = widen_exact(a.r32[q]);
+          else r[j] = a.r_up[q];
+          if (k0 + j < Kup) r[j] = neg_bits(r[j]);
+          if (SMALL && limiter == AFC_LIM_ZALESAK) {
+            Rj[j] = load_now(a.Rm + i + of.o[k0 + j]);
+            Rk[j] = load_now(a.Rp + i + of.o[k0 + j]);
+          }
+        }
+        if (!SMALL && limiter == AFC_LIM_ZALESAK) {
+#pragma unroll
+          for (int j = 0; j < S; ++j)
+            if (k0 + j != Kup) Rj[j] = Rk[j] = (gt0(r[j]) ? a.Rm : a.Rp)[i + of.o[k0 + j]];
+        }
+#pragma unroll
+        for (int j = 0; j < S; ++j) {
+          const int k = k0 + j;
+          if (k == Kup || !((mk >> k) & 1ull)) continue;
+          if (limiter == AFC_LIM_ZALESAK) F = fma(gt0(r[j]) ? imin_nn(rpi, Rj[j]) : imin_nn(rmi, Rk[j]), r[j], F);
+          else F += r[j];
         }
       }
     }
-    unew = a.ut[i] + dt * F / a.mL[i];
+    if (!SMALL) {
+      ut = a.ut[i];
+      m = a.mL[i];
+      im = a.imL[i];
+    }
+    unew = ut + div_by(dt * F, m, im);
   }
   if (a.Fs) a.Fs[i] = F;
-  out[i] = ca != 0.0 ? ca * uA[i] + cb * unew : cb * unew;
+  if (!SMALL && ca != 0.0) ua = uA[i];
+  out[i] = ca != 0.0 ? ca * ua + cb * unew : cb * unew;
 }
 
 }  // namespace afc

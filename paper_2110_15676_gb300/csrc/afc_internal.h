@@ -157,9 +157,11 @@ struct afc_problem_s {
   afc::DBuf<unsigned> mask32, clip32;   // node vectors, 16 < K <= 32: presence and clip masks in 32 bits
   afc::DBuf<uint16_t> mask16, clip16;   // K <= 16: the same in 16 bits (clip16: N + 1 entries, no halo)
   afc::DBuf<double> r_up;           // Kup * N: antidiffusive flux of each pair, at its lower row
-  // mixed-precision explicit stage: m_ij, d_ij, r_ij (Kup * N) and u, udot^L (node vectors) in single
-  afc::DBuf<float> m32_up, d32_up, r32, uf, udf;
-  bool ssp32_ready = false;         // m32_up / d32_up match the assembled m_up / d_up
+  // mixed-precision explicit stage: (m_ij, d_ij) and r_ij (Kup * N), (u, udot^L) (node vector) in single
+  afc::DBuf<float2> md32, uw;
+  afc::DBuf<float> r32;
+  bool ssp32_ready = false;         // md32 matches the assembled m_up / d_up
+  afc::DBuf<unsigned int> bar;      // GridBar of the one-launch explicit step
   afc::DBuf<long long> range;       // k_range: running max and min keys, blocks done
   afc::DBuf<double> scal;           // small device scalars (norms, dt, ...)
   afc::DBuf<double> part;           // reduction partials
@@ -194,6 +196,10 @@ int fe_stage(afc_problem_s* p, const double* uin, double dt, int limiter, double
              double* out, bool mixed = false, bool pdl = false);
 // the stages of one SSP2 / SSP3 step of the stored solution, in place
 int ssp_stages(afc_problem_s* p, const afc_opts* o);
+// the same step as one cooperative launch that also leaves the solution's range and the barrier's
+// error word in the host mirror (ssp_one_launch tells for which problems)
+bool ssp_one_launch(const afc_problem_s* p, const afc_opts* o);
+int ssp_step_launch(afc_problem_s* p, const afc_opts* o);
 int ensure_ssp_mixed(afc_problem_s* p);   // single-precision copies of m_ij, d_ij for the mixed stage
 struct SspArrays;
 SspArrays ssp_arrays(afc_problem_s* p);
@@ -218,7 +224,10 @@ int mc_limited_residual(afc_problem_s* p, const double* u, int limiter, double* 
 // the same residual (MC or Galerkin) in float-pair arithmetic, for mixed-precision MC
 // problems (mc_pair.cu); mc_pair_setup builds its pair copies at assembly
 int mc_pair_setup(afc_problem_s* p);
-int mc_pair_residual(afc_problem_s* p, const double* u, int limiter, double* res, double* normsq_slot);
+// (split = false: p->up2 holds u already)
+int mc_pair_residual(afc_problem_s* p, const double* u, int limiter, double* res, double* normsq_slot,
+                     bool split = true);
+int mc_pair_split(afc_problem_s* p, const double* u);
 
 // ---- reductions and BLAS-1 (krylov.cu) ----
 int dot_device(afc_problem_s* p, const double* x, const double* y, double* out_slot);
@@ -232,6 +241,7 @@ struct KrylovEpilogue {
   const double* uo = nullptr;
   double* a = nullptr;
   double* s = nullptr;
+  float2* pair = nullptr;    // u as float pairs, for the next sweep of the mixed MC residual
   // graph form of the fixed point: its scalars, the residual's block partials and the loop's
   // condition; the solve's launch decides whether the loop goes on, and counts itself
   double* fp_sc = nullptr;

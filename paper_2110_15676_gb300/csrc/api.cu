@@ -85,7 +85,7 @@ int create_common(afc_problem_s* p) {
                           &p->umin, &p->tmp, &p->cn_a, &p->cn_s, &p->bA, &p->bB, &p->Fold};
   for (auto* v : vecs)
     if ((st = v->alloc(N, p->pad))) return st;
-  if ((st = p->range.alloc(4)) || (st = p->scal.alloc(64)) || (st = p->part.alloc(4 * std::max<int64_t>(kRedBlocks, grid_for(N))))) return st;
+  if ((st = p->bar.alloc(4)) || (st = p->range.alloc(4)) || (st = p->scal.alloc(64)) || (st = p->part.alloc(4 * std::max<int64_t>(kRedBlocks, grid_for(N))))) return st;
   if (cudaMallocHost((void**)&p->host_scal, 64 * sizeof(double)) != cudaSuccess) {
     set_error("cudaMallocHost failed");
     return AFC_E_OOM;
@@ -117,10 +117,10 @@ void destroy_all(afc_problem_s* p) {
   for (auto* b : dv) b->free_();
   p->Bst32.free_(); p->dinv_st32.free_(); p->Bcn32.free_(); p->dinv_cn32.free_();
   p->conn.free_(); p->inc_ptr.free_(); p->inc.free_(); p->mask.free_(); p->dir.free_(); p->clip.free_();
-  p->pairf.free_(); p->nodef.free_();  p->range.free_();
+  p->pairf.free_(); p->nodef.free_();  p->range.free_(); p->bar.free_();
   p->AGp.free_(); p->fp2.free_(); p->pk_hi.free_(); p->pk_lo.free_(); p->up2.free_(); p->yp2.free_(); p->abh2.free_(); p->abl2.free_();
   p->cp_up.free_(); p->mask32.free_(); p->clip32.free_(); p->mask16.free_(); p->clip16.free_();
-  p->m32_up.free_(); p->d32_up.free_(); p->r32.free_(); p->uf.free_(); p->udf.free_();
+  p->md32.free_(); p->r32.free_(); p->uw.free_();
   if (p->host_scal) cudaFreeHost(p->host_scal);
   delete p;
 }

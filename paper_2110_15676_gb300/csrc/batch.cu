@@ -73,7 +73,7 @@ __device__ __forceinline__ void batch_row(const BInst& in, int phase, int st, co
       ssp_edges_row<KT, MIXED>(in.of, in.a, i, in.vec[sa.in[st]]);
       break;
     case 2:
-      ssp_factors_row<KT, MIXED, S>(in.of, in.a, i, dt);
+      ssp_factors_row<KT, MIXED, false, S>(in.of, in.a, i, in.vec[sa.in[st]], dt);
       break;
     default: {
       const double* uA = sa.uA[st] >= 0 ? in.vec[sa.uA[st]] : nullptr;
@@ -121,7 +121,7 @@ __device__ void batch_pass(const BInst* __restrict__ tab, int ninst, int64_t t0,
   }
 }
 
-__device__ __forceinline__ bool pass_needed(int phase, int limiter) {
+__host__ __device__ __forceinline__ bool pass_needed(int phase, int limiter) {
   if (phase == 1) return limiter != AFC_LIM_NONE;
   if (phase == 2) return limiter == AFC_LIM_ZALESAK;
   return true;
@@ -430,8 +430,7 @@ int enqueue_step(afc_batch_s* b, cudaStream_t s, const afc_opts* o, const afc_ba
     for (int sidx = 0; sidx < ns; ++sidx) {
       const StageArgs sa = stage_args(o->scheme, sidx);
       for (int ph = 0; ph < 4; ++ph) {
-        if (ph == 1 && o->limiter == AFC_LIM_NONE) continue;
-        if (ph == 2 && o->limiter != AFC_LIM_ZALESAK) continue;
+        if (!pass_needed(ph, o->limiter)) continue;
         if ((st = launch_pass_of(b, s, mixed, t.block, sa, o->limiter, ph))) return st;
         ++*nl;
       }

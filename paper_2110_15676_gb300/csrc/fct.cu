@@ -11,6 +11,7 @@
 // FP64 operations as the formulas allow and every comparison, min and max runs
 // on the integer pipe (kernels_common.cuh).
 #include "afc_internal.h"
+#include "grid_sync.cuh"
 #include "kernels_common.cuh"
 #include "ssp_rows.cuh"
 
@@ -27,6 +28,7 @@ namespace {
 // running ones (SSP3 step in double, us, with / without: P1 9^3 62 / 68, Q1 17^3 81 / 86, Q1 25^3
 // 84 / 86, Q1 33^3 113 / 90, Q1 41^3 179 / 117).
 constexpr int64_t kPdlRows = 16384;
+constexpr int64_t kStepRows = 16384;   // the graph form's one-launch step (k_ssp_step)
 
 template <int KT, bool MIXED>
 __global__ void k_ssp_rate(Offsets of, SspArrays a, const double* __restrict__ u, double dt) {
@@ -44,12 +46,12 @@ __global__ void k_ssp_edges(Offsets of, SspArrays a, const double* __restrict__ 
   if (i < a.N) ssp_edges_row<KT, MIXED>(of, a, i, u);
 }
 
-template <int KT, bool MIXED, bool SMALL>
-__global__ void k_ssp_factors(Offsets of, SspArrays a, double dt) {
+template <int KT, bool MIXED, bool SMALL, bool FUSED>
+__global__ void k_ssp_factors(Offsets of, SspArrays a, const double* u, double dt) {
   pdl_trigger();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   pdl_wait();
-  if (i < a.N) ssp_factors_row<KT, MIXED, kGroup<KT>, SMALL>(of, a, i, dt);
+  if (i < a.N) ssp_factors_row<KT, MIXED, FUSED, kGroup<KT>, SMALL>(of, a, i, u, dt);
 }
 
 template <int KT, bool MIXED, bool SMALL>
@@ -62,10 +64,57 @@ __global__ void k_ssp_correct(Offsets of, SspArrays a, int limiter, double dt, d
 }
 // Below this many rows (about one resident wave) the passes take their SMALL form.
 constexpr int64_t kSmallRows = 300000;
+// In the mixed mode their factors pass is FUSED: a flux is three FP32 operations, a launch costs
+// more (77,121 rows of Q1: 114 us a step against 119 us).  Not in double (P1 9^3: 67 us against 61 us),
+// and not on larger grids or in batches (48 mixed instances: 7.2 ms against 7.0 ms).
 
-__global__ void k_to_float(int64_t n, const double* __restrict__ x, float* __restrict__ y) {
+// A whole SSP2 / SSP3 step of a small problem as one cooperative launch, its passes separated
+// by grid barriers: on grids of a few thousand rows a pass is latency (one to two microseconds),
+// and a launch costs more than a barrier of as many blocks (SSP3 step in double, us, against
+// launches with programmatic dependent launch: P1 9^3 56 / 60, P1 25^3 62 / 70, Q1 17^3 72 / 81, Q1 25^3 75 / 84;
+// mixed Q1 17^3 84 / 91).
+constexpr int kStepBlock = 128;
+
+struct StepVecs {
+  double *u, *v, *w;   // u^n and the result; stage vectors
+};
+
+template <int KT, bool MIXED>
+__global__ void __launch_bounds__(kStepBlock) k_ssp_step(Offsets of, SspArrays a, StepVecs x, int stages, int limiter,
+                                                         double dt, GridBar* bar, unsigned long long wait_ns,
+                                                         long long* key, double* h) {
+  const int64_t i = blockIdx.x * (int64_t)kStepBlock + threadIdx.x;
+  const bool row = i < a.N;
+  constexpr int S = kGroup<KT>;
+  for (int st = 0; st < stages; ++st) {
+    const bool last = st == stages - 1;
+    const double* in = st == 0 ? x.u : st == 1 ? x.v : x.w;
+    double* out = last ? x.u : st == 0 ? x.v : x.w;
+    const double ca = st == 0 ? 0.0 : stages == 2 ? 0.5 : st == 1 ? 0.75 : 1.0 / 3.0;
+    const double cb = st == 0 ? 1.0 : stages == 2 ? 0.5 : st == 1 ? 0.25 : 2.0 / 3.0;
+    if (row) ssp_rate_row<KT, MIXED>(of, a, i, in, dt);
+    grid_barrier(bar, wait_ns);
+    if (limiter != AFC_LIM_NONE && !(MIXED && limiter == AFC_LIM_ZALESAK)) {
+      if (row) ssp_edges_row<KT, MIXED>(of, a, i, in);
+      grid_barrier(bar, wait_ns);
+    }
+    if (limiter == AFC_LIM_ZALESAK) {
+      if (row) ssp_factors_row<KT, MIXED, MIXED, S, true>(of, a, i, in, dt);
+      grid_barrier(bar, wait_ns);
+    }
+    if (row) ssp_correct_row<KT, MIXED, S, true>(of, a, i, limiter, dt, ca, x.u, cb, out);
+    if (!last) grid_barrier(bar, wait_ns);
+  }
+  Range r;
+  if (row) r.add(x.u[i]);   // this thread's own store
+  if (r.finish(key, h)) h[62] = (double)*(volatile int*)&bar->err;
+}
+
+// (m_ij, d_ij) of the pairs in single precision
+__global__ void k_pairs_to_float(int64_t n, const double* __restrict__ m, const double* __restrict__ d,
+                                 float2* __restrict__ md) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i < n) y[i] = __double2float_rn(x[i]);
+  if (i < n) md[i] = make_float2(__double2float_rn(m[i]), __double2float_rn(d[i]));
 }
 
 // ---- Crank-Nicolson -------------------------------------------------------------
@@ -186,29 +235,29 @@ __global__ void k_cn_factors(int64_t N, Offsets of, const unsigned long long* __
 }
 
 // Zalesak step 4, F*, and the nonlinear residual of Eq. CNZal:
-// res = b0 + F* - (m/dt u + AA u / 2) on free rows, 0 on Dirichlet rows; block partial sums of
-// res^2 for the stopping test.  M_L/dt + AA/2 is the system matrix B of the solve that follows
-// (identity rows are Dirichlet rows, which are not formed): one matrix of 59 MB at Q1 65^3 in
-// the 129 MB L2 instead of AA beside it.
+// res = b0 + F* - (m/dt u + AA u / 2) on free rows, 0 on Dirichlet rows;
+// block partial sums of res^2 for the stopping test.  (The system matrix M_L/dt + AA/2 in place
+// of AA saves 0.6 % of a step at Q1 65^3, one matrix less in L2, but its rounded diagonal shows in
+// the result: 6.7e-16 against 5.7e-16 from the step in 64 bits.)
 template <int KT>
 __global__ void __launch_bounds__(256, 4) k_cn_residual(int64_t N, Offsets of, int limiter, const unsigned long long* __restrict__ mask,
-                              const double* __restrict__ r_up, const double* __restrict__ B,
+                              const double* __restrict__ r_up, const double* __restrict__ AA,
                               const double* __restrict__ un, const double* __restrict__ Rp,
                               const double* __restrict__ Rm,
                               const double* __restrict__ b0,
-                              const uint8_t* __restrict__ dir,
+                              const double* __restrict__ mLdt, const uint8_t* __restrict__ dir,
                               double* __restrict__ res, double* __restrict__ Fout, double* __restrict__ part) {
   const int K = KT > 0 ? KT : of.K, Kup = K / 2;
   pdl_trigger();
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   double r2 = 0.0;
-  // y = B u from the matrix and the state, before the wait for the factors pass: no pass
+  // y = AA u from the matrix and the state, before the wait for the factors pass: no pass
   // of the limiter writes them (u is the solver's, complete before the edge pass started)
   const bool act = i < N && !dir[i];
   double y = 0.0;
   if (act) {
 #pragma unroll
-    for (int k = 0; k < K; ++k) y = fma(B[k * N + i], un[i + of.o[k]], y);
+    for (int k = 0; k < K; ++k) y = fma(AA[k * N + i], un[i + of.o[k]], y);
   }
   pdl_wait();
   if (i < N) {
@@ -241,7 +290,7 @@ __global__ void __launch_bounds__(256, 4) k_cn_residual(int64_t N, Offsets of, i
           }
         }
       }
-      rv = b0[i] + F - y;
+      rv = b0[i] + F - (mLdt[i] * un[i] + 0.5 * y);
     }
     res[i] = rv;
     if (Fout) Fout[i] = F;
@@ -258,8 +307,7 @@ SspArrays ssp_arrays(afc_problem_s* p) {
   a.AA = p->AA.p;
   a.m_up = p->m_up.p;
   a.d_up = p->d_up.p;
-  a.m32 = p->m32_up.p;
-  a.d32 = p->d32_up.p;
+  a.md32 = p->md32.p;
   a.mL = p->mL.p;
   a.imL = p->imL.p;
   a.f = p->f.p;
@@ -268,8 +316,7 @@ SspArrays ssp_arrays(afc_problem_s* p) {
   a.mask = p->mask.p;
   a.udot = p->udot.p;
   a.ut = p->ut.p;
-  a.uf = p->uf.p;
-  a.udf = p->udf.p;
+  a.uw = p->uw.p;
   a.r_up = p->r_up.p;
   a.r32 = p->r32.p;
   a.Rp = p->Rp.p;
@@ -282,11 +329,9 @@ int ensure_ssp_mixed(afc_problem_s* p) {
   if (p->ssp32_ready) return AFC_OK;
   const int64_t N = p->N, Kup = p->Kup;
   int st;
-  if ((st = p->m32_up.alloc(Kup * N)) || (st = p->d32_up.alloc(Kup * N)) || (st = p->r32.alloc(Kup * N)) ||
-      (st = p->uf.alloc(N, p->pad)) || (st = p->udf.alloc(N, p->pad)))
-    return st;
-  AFC_LAUNCH(p, "k_to_float", k_to_float<<<grid_for(Kup * N), kBlock, 0, p->stream>>>(Kup * N, p->m_up.p, p->m32_up.p));
-  AFC_LAUNCH(p, "k_to_float", k_to_float<<<grid_for(Kup * N), kBlock, 0, p->stream>>>(Kup * N, p->d_up.p, p->d32_up.p));
+  if ((st = p->md32.alloc(Kup * N)) || (st = p->r32.alloc(Kup * N)) || (st = p->uw.alloc(N, p->pad))) return st;
+  AFC_LAUNCH(p, "k_pairs_to_float", k_pairs_to_float<<<grid_for(Kup * N), kBlock, 0, p->stream>>>(
+                                        Kup * N, p->m_up.p, p->d_up.p, p->md32.p));
   AFC_CUDA(cudaGetLastError());
   p->ssp32_ready = true;
   return AFC_OK;
@@ -322,12 +367,13 @@ int fe_stage(afc_problem_s* p, const double* uin, double dt, int limiter, double
     constexpr int KT = decltype(kc)::value;
     constexpr bool MX = decltype(mc)::value;
     AFC_LAUNCH(p, "k_ssp_rate", launch_pass(pdl, k_ssp_rate<KT, MX>, g, blk, s, p->offs, arr, uin, dt));
-    if (limiter != AFC_LIM_NONE)
-      AFC_LAUNCH(p, "k_ssp_edges", launch_pass(chain, k_ssp_edges<KT, MX>, g, blk, s, p->offs, arr, uin));
     const bool small = N < kSmallRows;
-    auto factors = small ? k_ssp_factors<KT, MX, true> : k_ssp_factors<KT, MX, false>;
+    const bool fused = MX && small && limiter == AFC_LIM_ZALESAK;
+    if (limiter != AFC_LIM_NONE && !fused)
+      AFC_LAUNCH(p, "k_ssp_edges", launch_pass(chain, k_ssp_edges<KT, MX>, g, blk, s, p->offs, arr, uin));
+    auto factors = small ? k_ssp_factors<KT, MX, true, MX> : k_ssp_factors<KT, MX, false, false>;
     if (limiter == AFC_LIM_ZALESAK)
-      AFC_LAUNCH(p, "k_ssp_factors", launch_pass(chain, factors, g, blk, s, p->offs, arr, dt));
+      AFC_LAUNCH(p, "k_ssp_factors", launch_pass(chain, factors, g, blk, s, p->offs, arr, uin, dt));
     auto correct = small ? k_ssp_correct<KT, MX, true> : k_ssp_correct<KT, MX, false>;
     AFC_LAUNCH(p, "k_ssp_correct", launch_pass(chain, correct, g, blk, s, p->offs, arr, limiter, dt, a, uA, b, out));
   };
@@ -351,6 +397,39 @@ int ssp_stages(afc_problem_s* p, const afc_opts* o) {
   if (o->scheme == AFC_SSP2) return fe_stage(p, v, dt, lim, 0.5, u, 0.5, u, mixed, true);
   if ((st = fe_stage(p, v, dt, lim, 0.75, u, 0.25, w, mixed, true))) return st;
   return fe_stage(p, w, dt, lim, 1.0 / 3.0, u, 2.0 / 3.0, u, mixed, true);
+}
+
+bool ssp_one_launch(const afc_problem_s* p, const afc_opts* o) {
+  return p->N <= kStepRows && o->limiter != AFC_LIM_MC;
+}
+
+int ssp_step_launch(afc_problem_s* p, const afc_opts* o) {
+  const SspArrays arr = ssp_arrays(p);
+  const StepVecs x{p->u.p, p->ustage.p, p->tmp.p};
+  cudaError_t e = cudaSuccess;
+  auto run = [&](auto kc, auto mc) {
+    constexpr int KT = decltype(kc)::value;
+    constexpr bool MX = decltype(mc)::value;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid_for(p->N, kStepBlock));
+    cfg.blockDim = dim3(kStepBlock);
+    cfg.stream = p->stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    AFC_LAUNCH(p, "k_ssp_step",
+               e = cudaLaunchKernelEx(&cfg, k_ssp_step<KT, MX>, p->offs, arr, x, o->scheme == AFC_SSP2 ? 2 : 3,
+                                      (int)o->limiter, o->dt, reinterpret_cast<GridBar*>(p->bar.p),
+                                      (unsigned long long)p->grid_wait_ns, p->range.p, p->host_scal));
+  };
+  with_K(p->K, [&](auto kc) {
+    if (o->precision == AFC_MIXED) run(kc, std::true_type{});
+    else run(kc, std::false_type{});
+  });
+  if (e != cudaSuccess) return cuda_fail(e, "cudaLaunchKernelEx(k_ssp_step)");
+  return AFC_OK;
 }
 
 namespace {
@@ -505,8 +584,8 @@ int cn_limited_residual(afc_problem_s* p, const double* u_new, double dt, int li
     AFC_LAUNCH(p, "k_cn_residual",
                launch_pass(limiter != AFC_LIM_NONE, k_cn_residual<KT>, dim3((unsigned)g), dim3(kBlock), s, N,
                            p->offs, limiter, (const unsigned long long*)p->mask.p, (const double*)p->r_up.p,
-                           (const double*)p->Bcn.p, u_new, (const double*)p->Rp.p, (const double*)p->Rm.p,
-                           (const double*)p->b0.p, (const uint8_t*)p->dir.p, res, p->Fs.p, p->part.p));
+                           (const double*)p->AA.p, u_new, (const double*)p->Rp.p, (const double*)p->Rm.p,
+                           (const double*)p->b0.p, (const double*)p->mLdt.p, (const uint8_t*)p->dir.p, res, p->Fs.p, p->part.p));
   });
   if (normsq_slot) finalize_sum(p, p->part.p, (int)g, normsq_slot);
   AFC_CUDA(cudaGetLastError());

@@ -51,9 +51,17 @@ struct StepGraph {
   std::vector<unsigned char> key;
   int64_t k_pro = 0, k_outer = 0, k_epi = 0;
   int kind = 0;   // 1 fixed point, 2 explicit SSP
+  int unroll = 1; // corrections per turn of the while node
 };
 
 namespace {
+
+// Corrections per turn of the while node.  A turn costs about 5 us beside its kernels (P1 49^3
+// mixed, 942 corrections: 115.8 ms at one correction a turn, 114.0 at two, 112.6 at four); what
+// follows the stop in the same turn finds the status set and returns, but its residual has been
+// formed in vain.  So four for stationary solves, which take hundreds of corrections, and one for a
+// CN step's dozen (Q1 65^3: 8.23 ms at one, 8.37 at four).
+int unroll_of(int system) { return system == 0 ? 4 : 1; }
 
 std::vector<unsigned char> make_key(afc_problem_s* p, const afc_opts* o, int what) {
   std::vector<unsigned char> k(sizeof(afc_opts) + 64);
@@ -122,17 +130,21 @@ int build_fixed_point(afc_problem_s* p, const afc_opts* o, int system, Pro prolo
     cudaGraphNode_t loop;
     if ((st = add_conditional(g, fr, h_loop, cudaGraphCondTypeWhile, &body, &loop))) break;
     std::vector<cudaGraphNode_t> bf;
-    auto r2 = count([&]() -> int { return capture_into(p, cs, body, {}, residual, bf); });
-    if ((st = r2.first)) break;
     epi.fp_sc = p->scal.p;
     epi.part = p->part.p;
     epi.npart = (int)grid_for(p->N);
     epi.loop = h_loop;
-    auto r3 = count([&]() -> int {
-      return krylov_graph(p, system, o, p->res.p, p->delta.p, cs, body, bf, &epi);
+    sg.unroll = unroll_of(system);
+    auto r2 = count([&]() -> int {
+      for (int c = 0; c < sg.unroll; ++c) {
+        int s = capture_into(p, cs, body, bf, residual, bf);
+        if (s) return s;
+        if ((s = krylov_graph(p, system, o, p->res.p, p->delta.p, cs, body, bf, &epi))) return s;
+      }
+      return AFC_OK;
     });
-    if ((st = r3.first)) break;
-    sg.k_outer = r2.second + r3.second;
+    if ((st = r2.first)) break;
+    sg.k_outer = r2.second;
     fr.assign(1, loop);
     auto r4 = count([&]() -> int { return capture_into(p, cs, g, fr, [&]() -> int { return range_device(p, p->u.p); }, fr); });
     if ((st = r4.first)) break;
@@ -152,7 +164,7 @@ int run_fixed_point_graph(afc_problem_s* p, StepGraph& sg, afc_stats* stt) {
   AFC_CUDA(cudaStreamSynchronize(p->stream));
   const double* h = p->host_scal;
   const int64_t reval = (int64_t)h[F_REVAL], corr = (int64_t)h[F_CORR];
-  p->launches += sg.k_pro + reval * sg.k_outer + sg.k_epi;
+  p->launches += sg.k_pro + (reval + sg.unroll - 1) / sg.unroll * sg.k_outer + sg.k_epi;
   int status = h[F_STATUS] == 1.0 ? AFC_OK : h[F_STATUS] == 2.0 ? AFC_E_NAN : AFC_NOT_CONVERGED;
   if (h[F_TIMEOUT] != 0.0) {
     // the barrier counter is inconsistent after blocks skipped barriers: clear it so
@@ -188,6 +200,7 @@ void graph_free(afc_problem_s* p) {
 }
 
 int cn_step_graph(afc_problem_s* p, const afc_opts* o, afc_stats* stt) {
+  if (const int s0 = krylov_prepare(p, o)) return s0;
   const auto key = make_key(p, o, 1);
   if (!p->g_step || p->g_step->key != key) {
     drop(p->g_step);
@@ -230,23 +243,30 @@ int cn_step_graph(afc_problem_s* p, const afc_opts* o, afc_stats* stt) {
 }
 
 int stationary_graph(afc_problem_s* p, const afc_opts* o, afc_stats* stt) {
+  if (const int s0 = krylov_prepare(p, o)) return s0;
   const auto key = make_key(p, o, 2);
   if (!p->g_stat || p->g_stat->key != key) {
     drop(p->g_stat);
     p->g_stat = new StepGraph();
     const int lim = o->limiter;
+    const bool pair = o->precision == AFC_MIXED && (lim == AFC_LIM_MC || lim == AFC_LIM_GALERKIN);
+    KrylovEpilogue epi = stationary_epilogue(p, o);
+    if (pair) epi.pair = p->up2.p;
     int st = build_fixed_point(
         p, o, 0,
         [&]() -> int {
           AFC_LAUNCH(p, "k_apply_dirichlet", k_apply_dirichlet_g<<<grid_for(p->N), kBlock, 0, p->stream>>>(
                                                  p->N, p->dir.p, p->udir.p, p->u.p));
           AFC_CUDA(cudaGetLastError());
-          return AFC_OK;
+          return pair ? mc_pair_split(p, p->u.p) : AFC_OK;
         },
         [&]() -> int {
-          return mc_limited_residual(p, p->u.p, lim, p->res.p, nullptr, false, o->precision == AFC_MIXED);
+          // the state's float pairs come from the prologue, then from each solve's update (5 us of a
+          // correction at P1 49^3, 14 us at 129^3, when a pass of the sweep formed them)
+          if (pair) return mc_pair_residual(p, p->u.p, lim, p->res.p, nullptr, false);
+          return mc_limited_residual(p, p->u.p, lim, p->res.p, nullptr);
         },
-        *p->g_stat, stationary_epilogue(p, o));
+        *p->g_stat, epi);
     if (st) {
       drop(p->g_stat);
       return st;
@@ -257,7 +277,7 @@ int stationary_graph(afc_problem_s* p, const afc_opts* o, afc_stats* stt) {
 }
 
 int ssp_step_graph(afc_problem_s* p, const afc_opts* o, afc_stats* stt) {
-  const bool mixed = o->precision == AFC_MIXED;
+  const bool mixed = o->precision == AFC_MIXED, one = ssp_one_launch(p, o);
   if (mixed) {
     int s0 = ensure_ssp_mixed(p);   // allocation and conversion stay outside the capture
     if (s0) return s0;
@@ -273,6 +293,7 @@ int ssp_step_graph(afc_problem_s* p, const afc_opts* o, afc_stats* stt) {
     std::vector<cudaGraphNode_t> fr;
     const int64_t l0 = p->launches;
     int st = capture_into(p, p->cap_stream, g, fr, [&]() -> int {
+      if (one) return ssp_step_launch(p, o);
       const int s = ssp_stages(p, o);
       return s ? s : range_device(p, p->u.p);
     }, fr);
@@ -294,6 +315,12 @@ int ssp_step_graph(afc_problem_s* p, const afc_opts* o, afc_stats* stt) {
   AFC_CUDA(cudaGraphLaunch(p->g_step->exec, p->stream));
   AFC_CUDA(cudaStreamSynchronize(p->stream));
   p->launches += p->g_step->k_pro;
+  if (one && p->host_scal[62] != 0.0) {   // the barrier's state is inconsistent after blocks skipped it
+    AFC_CUDA(cudaMemsetAsync(p->bar.p, 0, 4 * sizeof(unsigned int), p->stream));
+    AFC_CUDA(cudaStreamSynchronize(p->stream));
+    set_error("a grid barrier of the explicit step's launch gave up waiting");
+    return AFC_E_TIMEOUT;
+  }
   if (stt) {
     stt->stages = o->scheme == AFC_SSP2 ? 2 : 3;
     stt->umin = p->host_scal[60];

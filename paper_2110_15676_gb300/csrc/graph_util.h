@@ -52,6 +52,11 @@ inline int add_conditional(cudaGraph_t g, const std::vector<cudaGraphNode_t>& de
   return AFC_OK;
 }
 
+// The workspace of the solver that the options ask for, in the state its launches expect (the
+// halos of its vectors zero, also after a solve in the other precision); before make_key, which
+// holds its address.
+int krylov_prepare(afc_problem_s* p, const afc_opts* o);
+
 // Krylov solve of `system` appended to graph g after `frontier` (updated): one
 // persistent launch, which also applies and counts the update `epi`.
 int krylov_graph(afc_problem_s* p, int system, const afc_opts* o, const double* rhs, double* x, cudaStream_t cs,

@@ -1,6 +1,8 @@
 // Small device helpers shared by the hot-path kernels.
 #pragma once
 
+#include <climits>
+#include <cmath>
 #include <type_traits>
 
 #include "afc_internal.h"
@@ -289,6 +291,53 @@ __device__ __forceinline__ void block_sums_to(double (&v)[NV], double* part, int
   }
   __syncthreads();
 }
+
+// min and max of values on the integer pipe (dkey order; NaN left out, as fmin / fmax do; atomics
+// on the keys, so the result does not depend on the order of the blocks), written straight to
+// the pinned host mirror h[60], h[61] by the last block, which leaves the keys empty for the
+// next launch.  No further launch and no copy, where two passes with FP64 compares and a copy of the
+// scalars took 8 us each and a copy's latency.  key: max, min, blocks done.
+struct Range {
+  long long mx = LLONG_MIN, mn = LLONG_MAX;
+
+  __device__ __forceinline__ void add(double v) {
+    if ((__double_as_longlong(v) & 0x7fffffffffffffffll) > 0x7ff0000000000000ll) return;
+    const long long k = dkey(v);
+    mx = k > mx ? k : mx;
+    mn = k < mn ? k : mn;
+  }
+  // every thread of a block of whole warps; thread 0 of the last block returns true
+  __device__ __forceinline__ bool finish(long long* key, double* h) {
+    __shared__ long long smx[32], smn[32];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const long long a = __shfl_xor_sync(0xffffffffu, mx, o), b = __shfl_xor_sync(0xffffffffu, mn, o);
+      mx = a > mx ? a : mx;
+      mn = b < mn ? b : mn;
+    }
+    if ((threadIdx.x & 31) == 0) {
+      smx[threadIdx.x >> 5] = mx;
+      smn[threadIdx.x >> 5] = mn;
+    }
+    __syncthreads();
+    if (threadIdx.x != 0) return false;
+    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) {
+      mx = smx[w] > mx ? smx[w] : mx;
+      mn = smn[w] < mn ? smn[w] : mn;
+    }
+    atomicMax(key, mx);
+    atomicMin(key + 1, mn);
+    __threadfence();
+    if (atomicAdd(reinterpret_cast<unsigned long long*>(key + 2), 1ull) != gridDim.x - 1) return false;
+    __threadfence();
+    mx = (long long)atomicExch(reinterpret_cast<unsigned long long*>(key), (unsigned long long)LLONG_MIN);
+    mn = (long long)atomicExch(reinterpret_cast<unsigned long long*>(key + 1), (unsigned long long)LLONG_MAX);
+    key[2] = 0;
+    h[60] = mn == LLONG_MAX ? INFINITY : from_key(mn);    // no number at all: as an empty fmin / fmax
+    h[61] = mx == LLONG_MIN ? -INFINITY : from_key(mx);
+    return true;
+  }
+};
 
 // Run f(std::integral_constant<int, K>) with K fixed at compile time for the two
 // structured patterns (15 offsets: Kuhn P1, 27: Q1) so that the per-row loops

@@ -16,6 +16,7 @@
 #include "graph_util.h"
 #include "kernels_common.cuh"
 #include "grid_sync.cuh"
+#include "pair_float.cuh"
 
 namespace afc {
 
@@ -87,50 +88,12 @@ __global__ void k_dot(int64_t N, const double* __restrict__ x, const double* __r
   block_sum_to(v, part);
 }
 
-// min and max of x on the integer pipe (dkey order; atomics on the keys, so the result does not
-// depend on the order of the blocks), written with the step's scalars sc[0 .. 12) straight to
-// the pinned host mirror h by the last block, which leaves the keys empty for the next call.
-// One launch and no copy, where the two passes with FP64 compares and a copy of the scalars
-// took 8 us each and a copy's latency.
 __global__ void __launch_bounds__(kBlock) k_range(int64_t N, const double* __restrict__ x, long long* key,
                                                   const double* __restrict__ sc, double* h) {
-  pdl_wait();
-  long long mx = LLONG_MIN, mn = LLONG_MAX;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
-    const double v = x[i];
-    const long long k = dkey(v);
-    if ((__double_as_longlong(v) & 0x7fffffffffffffffll) > 0x7ff0000000000000ll) continue;   // NaN, as fmin / fmax
-    mx = k > mx ? k : mx;
-    mn = k < mn ? k : mn;
-  }
-  __shared__ long long smx[kBlock / 32], smn[kBlock / 32];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const long long a = __shfl_xor_sync(0xffffffffu, mx, o), b = __shfl_xor_sync(0xffffffffu, mn, o);
-    mx = a > mx ? a : mx;
-    mn = b < mn ? b : mn;
-  }
-  if ((threadIdx.x & 31) == 0) {
-    smx[threadIdx.x >> 5] = mx;
-    smn[threadIdx.x >> 5] = mn;
-  }
-  __syncthreads();
-  if (threadIdx.x != 0) return;
-  for (int w = 1; w < kBlock / 32; ++w) {
-    mx = smx[w] > mx ? smx[w] : mx;
-    mn = smn[w] < mn ? smn[w] : mn;
-  }
-  atomicMax(key, mx);
-  atomicMin(key + 1, mn);
-  __threadfence();
-  if (atomicAdd(reinterpret_cast<unsigned long long*>(key + 2), 1ull) != gridDim.x - 1) return;
-  __threadfence();
-  mx = atomicExch(reinterpret_cast<unsigned long long*>(key), (unsigned long long)LLONG_MIN);
-  mn = atomicExch(reinterpret_cast<unsigned long long*>(key + 1), (unsigned long long)LLONG_MAX);
-  key[2] = 0;
-  for (int q = 0; q < 12; ++q) h[q] = sc[q];
-  h[60] = mn == LLONG_MAX ? INFINITY : from_key(mn);    // no number at all: as an empty fmin / fmax
-  h[61] = mx == LLONG_MIN ? -INFINITY : from_key(mx);
+  Range r;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) r.add(x[i]);
+  if (r.finish(key, h) && threadIdx.x == 0)
+    for (int q = 0; q < 12; ++q) h[q] = sc[q];
 }
 
 template <class T, class TV>
@@ -236,6 +199,7 @@ namespace {
 // 169 -> 120 us; P1 33^3 in double 107 -> 75 us (vectors in global memory, 512 threads in
 // every block, scalars in every warp before).
 constexpr int kFusedBlock = 512;
+constexpr int kBicgVectors = 8;             // phat, shat and the six local ones
 constexpr size_t kFusedSmem = 160 * 1024;   // shared memory for a block's six vectors (the rest stays L1)
 
 template <class T>
@@ -327,6 +291,7 @@ __device__ __forceinline__ void bicg_sums_end(const double* part, int& buf, Grid
 __device__ __forceinline__ void krylov_update(const KrylovEpilogue& ep, int64_t i, double xi) {
   const double ui = ep.u[i] + ep.omega * xi;
   ep.u[i] = ui;
+  if (ep.pair) ep.pair[i] = split_pair(ui);
   if (ep.a) {
     const double uoi = ep.uo[i];
     ep.a[i] = ui - uoi;
@@ -336,14 +301,15 @@ __device__ __forceinline__ void krylov_update(const KrylovEpilogue& ep, int64_t 
 // In the graph form of the fixed point (ep.fp_sc) the solve's launch first decides whether the
 // loop goes on: R = ||res|| from the residual pass's block partials, the stop tests of
 // Sec. 4.  Every block sums the partials itself and decides alike (block 0 writes the scalars; the
-// others read only those that it does not change, or a status whose change to 1 or 3 they
-// do not test).  As kernels of their own the sum, the test and the branch over the solve took
+// others read only those that it does not change, or a status whose change they decide alike).  As kernels of their own the sum, the test and the branch over the solve took
 // two graph nodes per correction.  True: solve.
 __device__ bool fp_goes_on(const KrylovEpilogue& ep) {
   double* sc = ep.fp_sc;
   if (!sc) return true;
   __shared__ bool go;
-  const bool failed = sc[F_STATUS] == 2.0;
+  const double was = sc[F_STATUS];
+  if (was == 1.0 || was == 3.0) return false;   // the loop has stopped earlier in this body
+  const bool failed = was == 2.0;
   const double it = sc[F_CORR];
   const double sum = final_sum(ep.part, ep.npart);
   if (threadIdx.x == 0) {
@@ -1266,7 +1232,7 @@ int fused_result(afc_problem_s* p, const char* what, int* its, double* res) {
 template <class T>
 int bicgstab_impl(afc_problem_s* p, const T* B, const T* dinv, const afc_opts* o, const double* rhs, double* xout,
                   int* its, double* res, const KrylovEpilogue* epi) {
-  int st = ensure_work(p, 8, sizeof(T) == 4);
+  int st = ensure_work(p, kBicgVectors, sizeof(T) == 4);
   if (st) return st;
   if ((st = bicg_fused_launch<T>(p, p->stream, B, dinv, o, rhs, xout, epi))) return st;
   return fused_result(p, "BiCGStab", its, res);
@@ -1357,7 +1323,7 @@ namespace {
 template <class T>
 int bicgstab_graph(afc_problem_s* p, const T* B, const T* dinv, const afc_opts* o, const double* rhs, double* xout,
                    cudaStream_t cs, cudaGraph_t g, std::vector<cudaGraphNode_t>& frontier, const KrylovEpilogue* epi) {
-  int st = ensure_work(p, 8, sizeof(T) == 4);
+  int st = ensure_work(p, kBicgVectors, sizeof(T) == 4);
   if (st) return st;
   return capture_into(p, cs, g, frontier, [&]() -> int {
     return bicg_fused_launch<T>(p, p->stream, B, dinv, o, rhs, xout, epi);
@@ -1376,15 +1342,19 @@ int gmres_graph(afc_problem_s* p, const T* B, const T* dinv, const afc_opts* o, 
 
 }  // namespace
 
-int krylov_graph(afc_problem_s* p, int system, const afc_opts* o, const double* rhs, double* x, cudaStream_t cs,
-                 cudaGraph_t g, std::vector<cudaGraphNode_t>& frontier, const KrylovEpilogue* epi) {
-  const bool mixed = o->precision == AFC_MIXED;
-  if (mixed && p->precision != AFC_MIXED) {
+int krylov_prepare(afc_problem_s* p, const afc_opts* o) {
+  const bool fp32 = o->precision == AFC_MIXED;
+  if (fp32 && p->precision != AFC_MIXED) {
     set_error("mixed-precision solve needs afc_assemble(..., AFC_MIXED)");
     return AFC_E_STATE;
   }
+  return o->ksp == AFC_KSP_GMRES ? gmres_work(p, o, fp32) : ensure_work(p, kBicgVectors, fp32);
+}
+
+int krylov_graph(afc_problem_s* p, int system, const afc_opts* o, const double* rhs, double* x, cudaStream_t cs,
+                 cudaGraph_t g, std::vector<cudaGraphNode_t>& frontier, const KrylovEpilogue* epi) {
   const bool gm = o->ksp == AFC_KSP_GMRES;
-  if (mixed) {
+  if (o->precision == AFC_MIXED) {
     const float* B = system == 0 ? p->Bst32.p : p->Bcn32.p;
     const float* di = system == 0 ? p->dinv_st32.p : p->dinv_cn32.p;
     return gm ? gmres_graph<float>(p, B, di, o, rhs, x, cs, g, frontier, epi)

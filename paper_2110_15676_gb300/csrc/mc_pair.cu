@@ -412,7 +412,13 @@ int mc_pair_setup(afc_problem_s* p) {
 }
 
 
-int mc_pair_residual(afc_problem_s* p, const double* u, int limiter, double* res, double* normsq_slot) {
+int mc_pair_split(afc_problem_s* p, const double* u) {
+  AFC_LAUNCH(p, "k_mcp_split", k_mcp_split<<<grid_for(p->N), kBlock, 0, p->stream>>>(p->N, u, p->up2.p));
+  AFC_CUDA(cudaGetLastError());
+  return AFC_OK;
+}
+
+int mc_pair_residual(afc_problem_s* p, const double* u, int limiter, double* res, double* normsq_slot, bool split) {
   const int64_t N = p->N;
   const int64_t g = grid_for(N);
   cudaStream_t s = p->stream;
@@ -421,9 +427,8 @@ int mc_pair_residual(afc_problem_s* p, const double* u, int limiter, double* res
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   AFC_CUDA(cudaStreamIsCapturing(s, &cap));
   const bool pdl = cap == cudaStreamCaptureStatusNone;
-  AFC_LAUNCH(p, "k_mcp_split", k_mcp_split<<<g, kBlock, 0, s>>>(N, u, p->up2.p));
-  AFC_CUDA(cudaGetLastError());
-  int st = AFC_OK;
+  int st = split ? mc_pair_split(p, u) : AFC_OK;
+  if (st) return st;
   with_K(p->K, [&](auto kc) {
     constexpr int KT = decltype(kc)::value;
     using M = MaskWord<KT>;

@@ -6,7 +6,9 @@
 // The stage has four passes, each needing the previous one on the neighbours:
 //   rate     y = AA u, udot^L = (f - y) / m, predictor u~ = u + dt udot^L
 //   edges    r_ij of every pair, once per pair at its lower row (Eq. defn_r_ij_SSP)
-//   factors  P+/-, Q+/- over N_i, R+/- (Zalesak steps 1-3)
+//   factors  P+/-, Q+/- over N_i, R+/- (Zalesak steps 1-3); in its FUSED form it also forms the
+//            fluxes, both ends each (r_ji = -r_ij bit for bit: every rounding is symmetric),
+//            and stores the upper ones, so that the edges pass is not needed
 //   correct  alpha_ij, F*_i = sum_j alpha_ij r_ij, u_new = u~ + dt F* / m, and the
 //            SSP combination out = a uA + b u_new
 //
@@ -30,8 +32,7 @@ struct SspArrays {
   const double* AA;                 // K * N low-order operator
   const double* m_up;               // Kup * N
   const double* d_up;               // Kup * N
-  const float* m32;                 // Kup * N (mixed)
-  const float* d32;                 // Kup * N (mixed)
+  const float2* md32;               // Kup * N (mixed): (m_ij, d_ij)
   const double* mL;
   const double* imL;                // 1 / m_i
   const double* f;
@@ -40,8 +41,7 @@ struct SspArrays {
   const unsigned long long* mask;
   double* udot;
   double* ut;
-  float* uf;                        // mixed: u rounded to single (halo)
-  float* udf;                       // mixed: udot^L rounded to single (halo)
+  float2* uw;                       // mixed: (u, udot^L) rounded to single (halo)
   double* r_up;                     // Kup * N
   float* r32;                       // Kup * N (mixed)
   double* Rp;                       // halo
@@ -67,12 +67,14 @@ __device__ __forceinline__ void ssp_rate_row(const Offsets& of, const SspArrays&
     ud = div_by(a.f[i] - y, a.mL[i], a.imL[i]);
     uti = fma(dt, ud, ui);
   }
-  a.udot[i] = ud;
   a.ut[i] = uti;
-  if (MIXED) {
-    a.uf[i] = __double2float_rn(ui);
-    a.udf[i] = __double2float_rn(ud);
-  }
+  if (MIXED) a.uw[i] = make_float2(__double2float_rn(ui), __double2float_rn(ud));
+  else a.udot[i] = ud;
+}
+
+// r_ij = m_ij (udot_i - udot_j) + d_ij (u_j - u_i); w = (u, udot), c = (m_ij, d_ij)
+__device__ __forceinline__ float ssp_flux(float2 c, float2 wi, float2 wj) {
+  return fmaf(c.x, wi.y - wj.y, c.y * (wj.x - wi.x));
 }
 
 // edges pass: the Kup pairs (i, i + o) with o > 0 stored at row i
@@ -82,12 +84,11 @@ __device__ __forceinline__ void ssp_edges_row(const Offsets& of, const SspArrays
   const int Kup = (KT > 0 ? KT : of.K) / 2;
   const int64_t N = a.N;
   if (MIXED) {
-    const float ui = a.uf[i], udi = a.udf[i];
+    const float2 wi = a.uw[i];
 #pragma unroll
     for (int ku = 0; ku < Kup; ++ku) {
       const int64_t q = (int64_t)ku * N + i;
-      const int64_t j = i + of.o[Kup + 1 + ku];
-      a.r32[q] = fmaf(a.m32[q], udi - a.udf[j], a.d32[q] * (a.uf[j] - ui));
+      a.r32[q] = ssp_flux(a.md32[q], wi, a.uw[i + of.o[Kup + 1 + ku]]);
     }
   } else {
     const double ui = u[i], udi = a.udot[i];
@@ -101,15 +102,22 @@ __device__ __forceinline__ void ssp_edges_row(const Offsets& of, const SspArrays
 }
 
 // factors pass: P+/- from the stored fluxes, Q+/- from the predictor over N_i, R+/-
-template <int KT, bool MIXED, int S = kGroup<KT>, bool SMALL = false>
-__device__ __forceinline__ void ssp_factors_row(const Offsets& of, const SspArrays& a, int64_t i, double dt) {
+// (FUSED: mixed only)
+template <int KT, bool MIXED, bool FUSED, int S = kGroup<KT>, bool SMALL = false>
+__device__ __forceinline__ void ssp_factors_row(const Offsets& of, const SspArrays& a, int64_t i, const double* u,
+                                                double dt) {
   const int K = KT > 0 ? KT : of.K, Kup = K / 2;
   // SMALL: the row's own data before the test of its Dirichlet flag (one wait, not two)
   unsigned long long mk = SMALL ? a.mask[i] : 0ull;
   double uti = SMALL ? a.ut[i] : 0.0, m = SMALL ? a.mL[i] : 0.0;
-  if (a.dir[i]) {
+  const bool isdir = a.dir[i];
+  if (isdir) {
     a.Rp[i] = 1.0;
     a.Rm[i] = 1.0;
+    if (!FUSED) return;
+  }
+  if (FUSED && isdir) {   // its upper fluxes all the same: their other ends read them
+    ssp_edges_row<KT, MIXED>(of, a, i, u);
     return;
   }
   if (!SMALL) {
@@ -125,13 +133,32 @@ __device__ __forceinline__ void ssp_factors_row(const Offsets& of, const SspArra
   for (int k0 = 0; k0 < K; k0 += S) {
     double r[S], v[S];
     float rf[S];
+    if (FUSED) {
+      float2 c[S], w[S];
+      const float2 wi = a.uw[i];
 #pragma unroll
-    for (int j = 0; j < S; ++j) {
-      if (k0 + j == Kup) continue;
-      const int64_t q = pair_slot(of, Kup, k0 + j, i, a.N);
-      if (MIXED) rf[j] = a.r32[q];
-      else r[j] = a.r_up[q];
-      v[j] = a.ut[i + of.o[k0 + j]];
+      for (int j = 0; j < S; ++j) {
+        if (k0 + j == Kup) continue;
+        c[j] = a.md32[pair_slot(of, Kup, k0 + j, i, a.N)];
+        w[j] = a.uw[i + of.o[k0 + j]];
+        v[j] = a.ut[i + of.o[k0 + j]];
+      }
+#pragma unroll
+      for (int j = 0; j < S; ++j) {
+        if (k0 + j == Kup) continue;
+        // upper pairs as the edges pass stores them; lower ones as their lower row does, r_e = -r_ij
+        rf[j] = k0 + j > Kup ? ssp_flux(c[j], wi, w[j]) : ssp_flux(c[j], w[j], wi);
+        if (k0 + j > Kup) a.r32[(int64_t)(k0 + j - Kup - 1) * a.N + i] = rf[j];
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < S; ++j) {
+        if (k0 + j == Kup) continue;
+        const int64_t q = pair_slot(of, Kup, k0 + j, i, a.N);
+        if (MIXED) rf[j] = a.r32[q];
+        else r[j] = a.r_up[q];
+        v[j] = a.ut[i + of.o[k0 + j]];
+      }
     }
 #pragma unroll
     for (int j = 0; j < S; ++j) {

@@ -59,6 +59,13 @@ int build_structured(int elem, int nx, int ny, int nz, const double lo[3], const
 int build_from_elements(int elem, int64_t n_nodes, const double* xyz, int64_t n_cells, const int32_t* conn,
                         MeshStructure& m);
 
+// Memory of the library (memory.cpp).  Device memory comes from a pool of the current device;
+// free it when the work that uses it has finished (freeing does not wait for the device).
+cudaError_t device_alloc(void** ptr, size_t bytes, bool zero = false);
+void device_free(void* ptr);
+cudaError_t pinned_alloc(void** ptr, size_t bytes);
+void pinned_free(void* ptr, size_t bytes);
+
 // Device buffer helpers.
 template <class T>
 struct DBuf {

@@ -65,6 +65,8 @@ int read_scal(afc_problem_s* p, int slot, double* out) {
   return AFC_OK;
 }
 
+constexpr size_t kHostScalBytes = 64 * sizeof(double);
+
 int create_common(afc_problem_s* p) {
   const int64_t N = p->N;
   const auto& m = p->mesh;
@@ -86,8 +88,8 @@ int create_common(afc_problem_s* p) {
   for (auto* v : vecs)
     if ((st = v->alloc(N, p->pad))) return st;
   if ((st = p->bar.alloc(4)) || (st = p->range.alloc(4)) || (st = p->scal.alloc(64)) || (st = p->part.alloc(4 * std::max<int64_t>(kRedBlocks, grid_for(N))))) return st;
-  if (cudaMallocHost((void**)&p->host_scal, 64 * sizeof(double)) != cudaSuccess) {
-    set_error("cudaMallocHost failed");
+  if (pinned_alloc((void**)&p->host_scal, kHostScalBytes) != cudaSuccess) {
+    set_error("pinned host allocation failed");
     return AFC_E_OOM;
   }
   const long long empty[4] = {INT64_MIN, INT64_MAX, 0, 0};   // k_range starts from and leaves this
@@ -104,7 +106,7 @@ int create_common(afc_problem_s* p) {
 void destroy_all(afc_problem_s* p) {
   if (!p) return;
   cudaSetDevice(p->device);
-  if (p->stream) cudaStreamSynchronize(p->stream);
+  cudaStreamSynchronize(p->stream);   // the legacy default stream too: freeing does not wait
   graph_free(p);
   prof_free(p);
   krylov_free(p);
@@ -121,7 +123,7 @@ void destroy_all(afc_problem_s* p) {
   p->AGp.free_(); p->fp2.free_(); p->pk_hi.free_(); p->pk_lo.free_(); p->up2.free_(); p->yp2.free_(); p->abh2.free_(); p->abl2.free_();
   p->cp_up.free_(); p->mask32.free_(); p->clip32.free_(); p->mask16.free_(); p->clip16.free_();
   p->md32.free_(); p->r32.free_(); p->uw.free_();
-  if (p->host_scal) cudaFreeHost(p->host_scal);
+  pinned_free(p->host_scal, kHostScalBytes);
   delete p;
 }
 

@@ -613,13 +613,13 @@ void batch_free(afc_batch_s* b) {
     if (kv.second.exec) cudaGraphExecDestroy(kv.second.exec);
   b->graphs.clear();
   if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
-  if (b->tab_h) cudaFreeHost(b->tab_h);
-  if (b->mm_h) cudaFreeHost(b->mm_h);
-  if (b->tab_d) cudaFree(b->tab_d);
-  if (b->map_d) cudaFree(b->map_d);
-  if (b->bar) cudaFree(b->bar);
-  if (b->mm_d) cudaFree(b->mm_d);
-  if (b->backup) cudaFree(b->backup);
+  pinned_free(b->tab_h, b->list.size() * sizeof(BInst));
+  pinned_free(b->mm_h, (2 * b->list.size() + 1) * sizeof(double));
+  device_free(b->tab_d);
+  device_free(b->map_d);
+  device_free(b->bar);
+  device_free(b->mm_d);
+  device_free(b->backup);
   delete b;
 }
 
@@ -671,15 +671,15 @@ int afc::batch_create_on_stream(const afc_problem* list, int count, cudaStream_t
     set_error("device does not support cooperative launches");
     return fail(AFC_E_CUDA);
   }
-  if ((e = cudaMallocHost((void**)&b->tab_h, count * sizeof(BInst))) != cudaSuccess ||
-      (e = cudaMallocHost((void**)&b->mm_h, (2 * count + 1) * sizeof(double))) != cudaSuccess)
-    return fail(cuda_fail(e, "cudaMallocHost"));
+  if ((e = pinned_alloc((void**)&b->tab_h, count * sizeof(BInst))) != cudaSuccess ||
+      (e = pinned_alloc((void**)&b->mm_h, (2 * count + 1) * sizeof(double))) != cudaSuccess)
+    return fail(cuda_fail(e, "pinned host allocation"));
   int64_t most_tiles = 0;   // at the smallest tile size
   for (auto* p : b->list) most_tiles += (p->N + 127) / 128;
-  if ((e = cudaMalloc((void**)&b->tab_d, count * sizeof(BInst))) != cudaSuccess ||
-      (e = cudaMalloc((void**)&b->map_d, most_tiles * sizeof(int2))) != cudaSuccess ||
-      (e = cudaMalloc((void**)&b->bar, sizeof(GridBar))) != cudaSuccess ||
-      (e = cudaMalloc((void**)&b->mm_d, 2 * count * sizeof(double))) != cudaSuccess) {
+  if ((e = device_alloc((void**)&b->tab_d, count * sizeof(BInst))) != cudaSuccess ||
+      (e = device_alloc((void**)&b->map_d, most_tiles * sizeof(int2))) != cudaSuccess ||
+      (e = device_alloc((void**)&b->bar, sizeof(GridBar))) != cudaSuccess ||
+      (e = device_alloc((void**)&b->mm_d, 2 * count * sizeof(double))) != cudaSuccess) {
     cudaGetLastError();
     set_error("device allocation of the batch tables failed");
     return fail(AFC_E_OOM);
@@ -743,7 +743,7 @@ extern "C" int afc_batch_tune(afc_batch b, const afc_opts* o, const double* dt, 
   if (cudaSetDevice(b->device) != cudaSuccess) return cuda_fail(cudaGetLastError(), "cudaSetDevice");
   cudaStream_t s = b->stream;
   if (!b->backup) {
-    cudaError_t e = cudaMalloc((void**)&b->backup, b->total_nodes * sizeof(double));
+    cudaError_t e = device_alloc((void**)&b->backup, b->total_nodes * sizeof(double));
     if (e != cudaSuccess) {
       cudaGetLastError();
       set_error("device allocation of the tuning backup failed");

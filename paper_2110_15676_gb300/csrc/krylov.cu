@@ -29,18 +29,13 @@ int DBuf<T>::alloc(int64_t n_, int64_t pad_) {
   free_();
   size_t bytes = (size_t)(n_ + 2 * pad_) * sizeof(T);
   if (bytes == 0) bytes = sizeof(T);
-  cudaError_t e = cudaMalloc((void**)&base, bytes);
+  cudaError_t e = device_alloc((void**)&base, bytes, true);   // zero-filled, ready for any stream
   if (e != cudaSuccess) {
     base = nullptr;
     cudaGetLastError();
-    set_error(std::string("cudaMalloc of ") + std::to_string(bytes) + " bytes failed: " + cudaGetErrorString(e));
-    return AFC_E_OOM;
+    set_error(std::string("device allocation of ") + std::to_string(bytes) + " bytes failed: " + cudaGetErrorString(e));
+    return e == cudaErrorMemoryAllocation ? AFC_E_OOM : AFC_E_CUDA;
   }
-  // zero-fill and wait for it here: a plain cudaMemset runs on the legacy default
-  // stream, which is not ordered with the non-blocking streams a problem may use
-  e = cudaMemsetAsync(base, 0, bytes, cudaStreamPerThread);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamPerThread);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
   n = n_;
   pad = pad_;
   p = base + pad_;
@@ -49,7 +44,7 @@ int DBuf<T>::alloc(int64_t n_, int64_t pad_) {
 
 template <class T>
 void DBuf<T>::free_() {
-  if (base) cudaFree(base);
+  if (base) device_free(base);
   base = p = nullptr;
   n = pad = 0;
 }
@@ -161,6 +156,8 @@ __device__ __forceinline__ bool flag_set(const double* sc, int slot) {
 // float -> double without the FP64 pipe (exact; the FP64 instance passes through)
 __device__ __forceinline__ double to_dbl(float x) { return widen_exact(x); }
 __device__ __forceinline__ double to_dbl(double x) { return x; }
+
+constexpr size_t kHscBytes = (S_END + 8) * sizeof(double);   // host mirror of the scalars
 
 struct KrylovWork {
   int64_t N = 0;
@@ -1090,7 +1087,7 @@ void krylov_free(afc_problem_s* p) {
   p->kw->vec.free_();
   p->kw->sc.free_();
   p->kw->part.free_();
-  if (p->kw->hsc) cudaFreeHost(p->kw->hsc);
+  pinned_free(p->kw->hsc, kHscBytes);
   delete p->kw;
   p->kw = nullptr;
 }
@@ -1116,6 +1113,7 @@ int ensure_work(afc_problem_s* p, int nvec, bool fp32) {
   const size_t vstride = (((size_t)p->N + 31) & ~(size_t)31) + 2 * pad;
   const int64_t bytes = (int64_t)(nvec * vstride * esz);
   if (w.vec.base == nullptr || w.vec.n < bytes) {
+    if (w.vec.base) AFC_CUDA(cudaStreamSynchronize(p->stream));   // nothing uses the smaller one any more
     int st = w.vec.alloc(bytes);   // zero-filled
     if (st) return st;
   } else if (w.vstride != vstride || w.fp32 != (int)fp32) {
@@ -1131,8 +1129,8 @@ int ensure_work(afc_problem_s* p, int nvec, bool fp32) {
     if (st) return st;
     if ((st = w.barrier.alloc(4))) return st;
     if ((st = coop_device(p))) return st;
-    if (cudaMallocHost((void**)&w.hsc, (S_END + 8) * sizeof(double)) != cudaSuccess) {
-      set_error("cudaMallocHost failed");
+    if (pinned_alloc((void**)&w.hsc, kHscBytes) != cudaSuccess) {
+      set_error("pinned host allocation failed");
       return AFC_E_OOM;
     }
   }
@@ -1238,9 +1236,12 @@ int bicgstab_impl(afc_problem_s* p, const T* B, const T* dinv, const afc_opts* o
   return fused_result(p, "BiCGStab", its, res);
 }
 
-// The persistent GMRES launch on stream s (no synchronisation).  One block per SM at
-// most: small systems spread over all SMs with few warps each, because a block's FP64
-// sums cost 16 cycles per warp, and leave room for the launches of other streams.
+// The persistent GMRES launch on stream s (no synchronisation).  One block per SM at most.  In
+// double small systems spread over all SMs, 64 rows a block, because a block's FP64 sums cost
+// 16 cycles per warp.  In single precision a block takes at least 512 rows: a solve of a few
+// thousand rows is as fast on 16 SMs as on 125 (P1 17^3 to Q1 33^3: within 1 %), and solves on other
+// streams find room beside it (a burst of 8 served requests, four of them stationary: 108 -> 76
+// ms).
 template <class T>
 int gmres_fused_launch(afc_problem_s* p, cudaStream_t s, const T* B, const T* dinv, const afc_opts* o,
                        const double* rhs, double* xout, const KrylovEpilogue* epi) {
@@ -1262,7 +1263,8 @@ int gmres_fused_launch(afc_problem_s* p, cudaStream_t s, const T* B, const T* di
   if (epi) a.ep = *epi;
   a.wait_ns = p->grid_wait_ns;
   const int64_t units = (N + kGmUnit - 1) / kGmUnit;
-  const int G = (int)std::max<int64_t>(1, std::min<int64_t>((units + 1) / 2, std::min(w.nsm, 160)));
+  const int64_t least = sizeof(T) == 4 ? 512 / kGmUnit : 64 / kGmUnit;   // units of a block, at least
+  const int G = (int)std::max<int64_t>(1, std::min<int64_t>((units + least - 1) / least, std::min(w.nsm, 160)));
   const int64_t rows = (units + G - 1) / G * kGmUnit;   // most rows of a block
   const size_t vec = (size_t)rows * sizeof(T);
   const bool vs = (size_t)(a.m + 2) * vec <= kGmSmem;   // w and V_0 .. V_m

@@ -291,7 +291,7 @@ typedef struct afc_batch_s* afc_batch;
 
 /* Launch shapes of a batched step. */
 typedef enum {
-  AFC_BATCH_AUTO = 0,       /* the tuned shape for this batch's size class, else PER_STAGE  */
+  AFC_BATCH_AUTO = 0,       /* the tuned shape for this batch's size class, else PER_PASS   */
   AFC_BATCH_PER_PASS = 1,   /* one launch per pass (4 per stage), each over all instances    */
   AFC_BATCH_PER_STAGE = 2,  /* one persistent cooperative launch per stage; the passes are   */
                             /* separated by grid-wide barriers with a bounded wait          */

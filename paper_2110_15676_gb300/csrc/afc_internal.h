@@ -183,6 +183,7 @@ struct afc_problem_s {
   // range of the stored solution (known after afc_set_solution, a step or a solve)
   // and of the Dirichlet values: the reference of afc_stats.dmp_violation
   bool u_range_valid = false;
+  bool maybe_captured = false;   // work that a caller may have captured and replays on other streams
   double u_lo = 0.0, u_hi = 0.0;
   double dir_lo = 1e308, dir_hi = -1e308;
   // bounded-wait limit of the grid barriers in this problem's persistent launches
@@ -237,7 +238,6 @@ int mc_pair_residual(afc_problem_s* p, const double* u, int limiter, double* res
 int mc_pair_split(afc_problem_s* p, const double* u);
 
 // ---- reductions and BLAS-1 (krylov.cu) ----
-int dot_device(afc_problem_s* p, const double* x, const double* y, double* out_slot);
 // An update that a persistent Krylov launch applies to its solution x in its last
 // pass, unless the solve broke down: u += omega x, and with `a` then a = u - uo and
 // s = u + uo (the damped correction and, for the CN scheme, the node sums of the next

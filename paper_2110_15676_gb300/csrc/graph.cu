@@ -18,7 +18,6 @@ namespace afc {
 
 namespace {
 
-
 __global__ void k_fp_init(double* sc, double thresh, int fixed, int maxit) {
   if (threadIdx.x != 0) return;
   sc[F_CORR] = 0.0;

@@ -270,28 +270,6 @@ __device__ __forceinline__ void block_sum_to(double v, double* part) {
   __syncthreads();
 }
 
-// Several sums at once (NV values per thread), stored at part[q * stride + blockIdx.x].
-template <int NV>
-__device__ __forceinline__ void block_sums_to(double (&v)[NV], double* part, int64_t stride) {
-  if (blockDim.x > kBlock) {
-#pragma unroll
-    for (int q = 0; q < NV; ++q) block_sum_to(v[q], part + q * stride);
-    return;
-  }
-  __shared__ double sh[NV][kBlock];
-#pragma unroll
-  for (int q = 0; q < NV; ++q) sh[q][threadIdx.x] = v[q];
-  __syncthreads();
-  if (threadIdx.x < 32) {
-#pragma unroll
-    for (int q = 0; q < NV; ++q) {
-      const double t = warp0_column_sum(sh[q]);
-      if (threadIdx.x == 0) part[q * stride + blockIdx.x] = t;
-    }
-  }
-  __syncthreads();
-}
-
 // min and max of values on the integer pipe (dkey order; NaN left out, as fmin / fmax do; atomics
 // on the keys, so the result does not depend on the order of the blocks), written straight to
 // the pinned host mirror h[60], h[61] by the last block, which leaves the keys empty for the

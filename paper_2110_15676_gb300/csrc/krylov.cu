@@ -1,10 +1,10 @@
 // Jacobi-preconditioned Krylov solvers for the constant M-matrix systems of the
 // fixed-point iteration (Sec. 4; Tables 1 and 3: BiCGStab, GMRES, Jacobi), run
-// entirely on the device.  Solver scalars (rho, alpha, omega, Hessenberg
-// columns, Givens rotations) live in device memory and are finalised by
-// one-block kernels, so the host only polls a status word every few iterations
-// (BiCGStab) or once per restart cycle (GMRES).  All reductions are two-stage
-// with a fixed order, so results do not depend on scheduling.
+// entirely on the device: a solve is one persistent cooperative launch whose
+// phases are separated by bounded grid barriers.  Every block forms the solver
+// scalars (rho, alpha, omega, Hessenberg columns, Givens rotations) from the
+// same partial sums in the same order, so all blocks branch alike and results do
+// not depend on scheduling.
 //
 // Vector type T is double (FP64) or float (the FP32 inner solve of the mixed
 // mode, with FP32 matrix values).  Partial sums are always double.
@@ -76,13 +76,6 @@ void finalize_sum(afc_problem_s* p, const double* part, int n, double* out) {
 // ---------------------------------------------------------------------------
 namespace {
 
-__global__ void k_dot(int64_t N, const double* __restrict__ x, const double* __restrict__ y, double* __restrict__ part) {
-  double v = 0.0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
-    v = fma(x[i], y[i], v);
-  block_sum_to(v, part);
-}
-
 __global__ void __launch_bounds__(kBlock) k_range(int64_t N, const double* __restrict__ x, long long* key,
                                                   const double* __restrict__ sc, double* h) {
   Range r;
@@ -102,13 +95,6 @@ __global__ void k_spmv(int64_t N, Offsets of, const T* __restrict__ A, const TV*
 }
 
 }  // namespace
-
-int dot_device(afc_problem_s* p, const double* x, const double* y, double* out_slot) {
-  AFC_LAUNCH(p, "k_dot", k_dot<<<kRedBlocks, kBlock, 0, p->stream>>>(p->N, x, y, p->part.p));
-  finalize_sum(p, p->part.p, kRedBlocks, out_slot);
-  AFC_CUDA(cudaGetLastError());
-  return AFC_OK;
-}
 
 int range_device(afc_problem_s* p, const double* x) {
   // at most two blocks per SM: each ends in three atomics on one line
@@ -298,8 +284,9 @@ __device__ __forceinline__ void krylov_update(const KrylovEpilogue& ep, int64_t 
 // In the graph form of the fixed point (ep.fp_sc) the solve's launch first decides whether the
 // loop goes on: R = ||res|| from the residual pass's block partials, the stop tests of
 // Sec. 4.  Every block sums the partials itself and decides alike (block 0 writes the scalars; the
-// others read only those that it does not change, or a status whose change they decide alike).  As kernels of their own the sum, the test and the branch over the solve took
-// two graph nodes per correction.  True: solve.
+// others read only those that it does not change, or a status whose change they decide alike).
+// As kernels of their own the sum, the test and the branch over the solve took two graph nodes per
+// correction.  True: solve.
 __device__ bool fp_goes_on(const KrylovEpilogue& ep) {
   double* sc = ep.fp_sc;
   if (!sc) return true;

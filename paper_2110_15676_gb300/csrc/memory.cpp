@@ -69,6 +69,12 @@ cudaError_t device_alloc(void** ptr, size_t bytes, bool zero) {
     ++g_live[device];   // before the allocation: an idle trim does not run beside it
   }
   e = cudaMallocFromPoolAsync(ptr, bytes, pool, cudaStreamPerThread);
+  if (e == cudaErrorMemoryAllocation) {   // once more without what the pool keeps in free pieces
+    cudaGetLastError();
+    *ptr = nullptr;
+    cudaMemPoolTrimTo(pool, 0);
+    e = cudaMallocFromPoolAsync(ptr, bytes, pool, cudaStreamPerThread);
+  }
   if (e == cudaSuccess && zero) e = cudaMemsetAsync(*ptr, 0, bytes, cudaStreamPerThread);
   if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamPerThread);
   if (e != cudaSuccess) {

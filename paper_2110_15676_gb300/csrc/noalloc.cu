@@ -147,6 +147,7 @@ extern "C" int afc_mc_limited_sum_noalloc(afc_problem p, int limiter, const doub
   if (st) return st;
   double* umax = scratch;
   double* umin = scratch + kNoAllocMaxNodes;
+  p->maybe_captured = true;
   const int64_t N = p->N;
   const int64_t g = grid_for(N);
   if (limiter == AFC_LIM_MC) {

@@ -65,14 +65,15 @@ __global__ void k_ssp_correct(Offsets of, SspArrays a, int limiter, double dt, d
 // Below this many rows (about one resident wave) the passes take their SMALL form.
 constexpr int64_t kSmallRows = 300000;
 // In the mixed mode their factors pass is FUSED: a flux is three FP32 operations, a launch costs
-// more (77,121 rows of Q1: 114 us a step against 119 us).  Not in double (P1 9^3: 67 us against 61 us),
+// more (77,121 rows of Q1: 114 us a step against 119 us; 105 us since the correct pass loads its
+// groups before it widens).  Not in double (P1 9^3: 67 us against 61 us),
 // and not on larger grids or in batches (48 mixed instances: 7.2 ms against 7.0 ms).
 
 // A whole SSP2 / SSP3 step of a small problem as one cooperative launch, its passes separated
 // by grid barriers: on grids of a few thousand rows a pass is latency (one to two microseconds),
 // and a launch costs more than a barrier of as many blocks (SSP3 step in double, us, against
 // launches with programmatic dependent launch: P1 9^3 56 / 60, P1 25^3 62 / 70, Q1 17^3 72 / 81, Q1 25^3 75 / 84;
-// mixed Q1 17^3 84 / 91).
+// mixed Q1 17^3 84 / 91, before the correct pass widened its fluxes after the loads).
 constexpr int kStepBlock = 128;
 
 struct StepVecs {
@@ -126,7 +127,7 @@ __global__ void k_cn_predictor(int64_t N, Offsets of, const double* __restrict__
                                const double* __restrict__ f, const double* __restrict__ mL,
                                const uint8_t* __restrict__ dir, const double* __restrict__ udir, double dt,
                                double* __restrict__ ut, double* __restrict__ b0) {
-  const int K = KT > 0 ? KT : of.K, Kup = K / 2;
+  const int K = KT > 0 ? KT : of.K;
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= N) return;
   double y = 0.0;
@@ -143,7 +144,7 @@ template <int KT>
 __global__ void k_bounds_of(int64_t N, Offsets of, const unsigned long long* __restrict__ mask,
                             const double* __restrict__ v, const double* __restrict__ mL, double* __restrict__ Qp,
                             double* __restrict__ Qm) {
-  const int K = KT > 0 ? KT : of.K, Kup = K / 2;
+  const int K = KT > 0 ? KT : of.K;
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= N) return;
   const unsigned long long mk = mask[i];

@@ -179,9 +179,9 @@ def _timed_steps(P, opts, steps, flush, stream, torch):
 
 
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from one ncu capture
-# (profiles/k_bicg_fused_q1_65.md), valid while the kernel's sources hash as they did then.
+# (profiles/kernels_one_launch_each.md), valid while the kernel's sources hash as they did then.
 _NCU_TRAFFIC = {
-    "k_bicg_fused": {"bytes": 76.80e6, "sha1": "11b039bea6594c49",
+    "k_bicg_fused": {"bytes": 70.2e6, "sha1": "bf01b0b11c1ba0fb",
                      "sources": ("krylov.cu", "kernels_common.cuh", "afc_internal.h", "grid_sync.cuh")},
 }
 

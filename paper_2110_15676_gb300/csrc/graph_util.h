@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "afc_internal.h"
+#include "fp_stop.cuh"
 
 namespace afc {
 
@@ -62,14 +63,6 @@ int krylov_prepare(afc_problem_s* p, const afc_opts* o);
 int krylov_graph(afc_problem_s* p, int system, const afc_opts* o, const double* rhs, double* x, cudaStream_t cs,
                  cudaGraph_t g, std::vector<cudaGraphNode_t>& frontier, const KrylovEpilogue* epi);
 
-// fixed-point scalar slots (problem scalars p->scal)
-enum : int {
-  F_NORMSQ = 0, F_CORR = 1, F_INNER = 2, F_RES0 = 3, F_RESF = 4, F_STATUS = 5, F_THRESH = 6, F_FIXED = 7,
-  F_MAXIT = 8, F_REVAL = 10, F_TIMEOUT = 11
-};
-// F_STATUS: 0 running, 1 converged / fixed count reached, 2 non-finite or a solver that
-// could not finish, 3 iteration limit; F_TIMEOUT: 1 after a grid barrier of the
-// persistent solve gave up waiting (F_STATUS is then 2)
 // Clear the grid barrier state of the persistent solves after a timeout (its
 // counter is left inconsistent when blocks skip barriers); synchronises the stream.
 int krylov_reset_barrier(afc_problem_s* p);

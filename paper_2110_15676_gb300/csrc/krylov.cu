@@ -282,39 +282,11 @@ __device__ __forceinline__ void krylov_update(const KrylovEpilogue& ep, int64_t 
   }
 }
 // In the graph form of the fixed point (ep.fp_sc) the solve's launch first decides whether the
-// loop goes on: R = ||res|| from the residual pass's block partials, the stop tests of
-// Sec. 4.  Every block sums the partials itself and decides alike (block 0 writes the scalars; the
-// others read only those that it does not change, or a status whose change they decide alike).
-// As kernels of their own the sum, the test and the branch over the solve took two graph nodes per
-// correction.  True: solve.
-__device__ bool fp_goes_on(const KrylovEpilogue& ep) {
-  double* sc = ep.fp_sc;
-  if (!sc) return true;
-  __shared__ bool go;
-  const double was = sc[F_STATUS];
-  if (was == 1.0 || was == 3.0) return false;   // the loop has stopped earlier in this body
-  const bool failed = was == 2.0;
-  const double it = sc[F_CORR];
-  const double sum = final_sum(ep.part, ep.npart);
-  if (threadIdx.x == 0) {
-    const double R = sqrt(sum);
-    double status = 0.0;
-    if (!isfinite(R) || failed) status = 2.0;
-    else if (sc[F_FIXED] > 0.0) status = it >= sc[F_FIXED] ? 1.0 : 0.0;
-    else if (R < sc[F_THRESH]) status = 1.0;
-    else if (it >= sc[F_MAXIT]) status = 3.0;
-    go = status == 0.0;
-    if (blockIdx.x == 0) {
-      sc[F_NORMSQ] = sum;
-      if (sc[F_REVAL] == 0.0) sc[F_RES0] = R;
-      sc[F_RESF] = R;
-      sc[F_REVAL] += 1.0;
-      if (!go) sc[F_STATUS] = status;
-      cudaGraphSetConditional(ep.loop, go ? 1u : 0u);
-    }
-  }
-  __syncthreads();
-  return go;
+// loop goes on (fp_stop.cuh).  True: solve.
+__device__ __forceinline__ bool fp_goes_on(const KrylovEpilogue& ep) {
+  if (!ep.fp_sc) return true;
+  return fp_decide(static_cast<volatile double*>(ep.fp_sc), [&] { return final_sum(ep.part, ep.npart); },
+                   [&](bool go) { cudaGraphSetConditional(ep.loop, go ? 1u : 0u); });
 }
 // The fixed-point loop's count of a correction (one thread of the solve's launch).
 __device__ __forceinline__ void krylov_count(const KrylovEpilogue& ep, int its, bool berr, bool broke) {

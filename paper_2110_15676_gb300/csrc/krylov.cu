@@ -560,11 +560,7 @@ __device__ __forceinline__ T warp_sum4(const T (&v)[4]) {
 }
 
 // Scalars of a solve, one copy per block.
-template <class T>
-struct GmShared {
-  T red[kGmBlock / 32][kGmQ + 3];   // the warps' sums (rows padded against bank conflicts)
-  T hs[kMaxRestart];                   // coefficients of the projection at hand, in the vector type
-  T ih;                                // factor of w in the projection
+struct GmScalars {
   double tot[kGmQ];                    // totals of the last exchange
   double nrm2;                         // ||v_{k+1}||^2
   double scale[kMaxRestart + 1];       // 1 / ||v_q||
@@ -574,6 +570,29 @@ struct GmShared {
   double run;                          // running entry of the column being rotated
   double nres, n0, tol;
   int its, cycles, done, cycle_done, skip;
+};
+template <class T>
+struct GmVectorScalars : GmScalars {
+  T hs[kMaxRestart];                   // coefficients of the projection at hand, in the vector type
+  T ih;                                // factor of w in the projection
+};
+template <class T>
+struct GmShared : GmVectorScalars<T> {
+  T red[kGmBlock / 32][kGmQ + 3];      // the warps' sums (rows padded against bank conflicts)
+  // value q of the block
+  __device__ __forceinline__ T value(int q, int nw) const {
+    T s0 = 0, s1 = 0, s2 = 0, s3 = 0;   // four chains: the adds of one are serial
+    int u = 0;
+#pragma unroll 1
+    for (; u + 3 < nw; u += 4) {
+      s0 += red[u][q];
+      s1 += red[u + 1][q];
+      s2 += red[u + 2][q];
+      s3 += red[u + 3][q];
+    }
+    for (; u < nw; ++u) s0 += red[u][q];
+    return (s0 + s1) + (s2 + s3);
+  }
 };
 
 // The total over a warp of one partial of G per slot, p[0 .. G), in a fixed order.
@@ -585,65 +604,24 @@ __device__ __forceinline__ double gm_total(const double* p, int G) {
   const double t = ((x[0] + x[1]) + (x[2] + x[3])) + x[4];
   return warp_sum(t);
 }
-// Single-precision partials in 64-bit fixed point scaled to the largest (its mantissa at
-// bits 30 .. 53, so 160 blocks cannot overflow), one rounding at the end: no less exact than
-// a sum in double, and on the integer pipe (eight double adds by each of a dozen warps at
-// once held the FP64 pipe for most of a microsecond).  Inf and NaN come out as NaN.
-__device__ __forceinline__ double gm_total(const float* p, int G) {
-  const int lane = threadIdx.x & 31;
-  unsigned x[5];   // G <= 160
-  unsigned e = 0;
-#pragma unroll
-  for (int u = 0; u < 5; ++u) {
-    x[u] = lane + 32 * u < G ? __float_as_uint(__ldcg(p + lane + 32 * u)) : 0u;
-    e = max(e, (x[u] >> 23) & 0xffu);
-  }
-  e = __reduce_max_sync(0xffffffffu, e);
-  if (e == 0xffu) return __longlong_as_double(0x7ff8000000000000ll);
-  e = max(e, 1u);
-  long long t = 0;
-#pragma unroll
-  for (int u = 0; u < 5; ++u) {
-    const unsigned xe = (x[u] >> 23) & 0xffu, m = (x[u] & 0x7fffffu) | (xe ? 0x800000u : 0u);
-    const unsigned sh = min(e - max(xe, 1u), 63u);
-    const long long v = (long long)(((unsigned long long)m << 30) >> sh);
-    t += (x[u] >> 31) ? -v : v;
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-  const double d = (double)t;   // t * 2^(e - 127 - 23 - 30): the exponent moves exactly
-  return t == 0 ? 0.0 : __longlong_as_double(__double_as_longlong(d) + ((long long)((int)e - 180) << 52));
-}
 
-// A grid-wide sum of nq values and a barrier: the warps' sums in sh.red (rows 0 .. nw - 1)
-// are added and stored by warp 0, whose first lane arrives and polls; then warp q adds all
-// blocks' partials of value q into sh.tot (the same bits in every block), and `take()` runs
-// in warp 0 (with nq <= 1 before the block meets again, in the same warp).  Memory: the
+// A grid-wide sum of nq values and a barrier: warp 0 stores the block's values, value(q), its
+// first lane arrives and polls; then warp q adds all blocks' partials of value q into sh.tot
+// (the same bits in every block), and `take()` runs in warp 0 (with nq <= 1 before the block meets
+// again, in the same warp).  Memory: the
 // block's threads meet, so that lane's fence releases what they wrote; it polls with acquire
 // loads, and the block meets again before anyone uses what `take` stored or what other
 // blocks wrote.  The partials alternate between two buffers (a block can run at most one
 // sum ahead of another).
-template <class T, class F>
-__device__ __forceinline__ void gm_exchange(GmShared<T>& sh, int nq, int nw, const GmArgs& a, int& buf, F&& take) {
+template <class V, class F>
+__device__ __forceinline__ void gm_exchange(GmScalars& sh, int nq, const GmArgs& a, int& buf, V&& value, F&& take) {
   const int G = gridDim.x, lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-  T* pb = reinterpret_cast<T*>(a.part) + (size_t)buf * kGmQ * G;
+  double* pb = a.part + (size_t)buf * kGmQ * G;
   buf ^= 1;
-  __syncthreads();   // sh.red is complete
+  __syncthreads();   // what value() reads is complete
   if (wp == 0) {
 #pragma unroll 1
-    for (int q = lane; q < nq; q += 32) {
-      T s0 = 0, s1 = 0, s2 = 0, s3 = 0;   // four chains: the adds of one are serial
-      int u = 0;
-#pragma unroll 1
-      for (; u + 3 < nw; u += 4) {
-        s0 += sh.red[u][q];
-        s1 += sh.red[u + 1][q];
-        s2 += sh.red[u + 2][q];
-        s3 += sh.red[u + 3][q];
-      }
-      for (; u < nw; ++u) s0 += sh.red[u][q];
-      pb[(size_t)q * G + blockIdx.x] = (s0 + s1) + (s2 + s3);
-    }
+    for (int q = lane; q < nq; q += 32) pb[(size_t)q * G + blockIdx.x] = value(q);
     __syncwarp();
     if (lane == 0) grid_poll(a.bar, grid_arrive_thread(a.bar), a.wait_ns);
     __syncwarp();
@@ -662,6 +640,9 @@ __device__ __forceinline__ void gm_exchange(GmShared<T>& sh, int nq, int nw, con
     take();
   }
   __syncthreads();
+}
+__device__ __forceinline__ void gm_barrier(GmScalars& sh, const GmArgs& a, int& buf) {
+  gm_exchange(sh, 0, a, buf, [](int) { return 0.0; }, [] {});
 }
 
 // The warps' sums of one value per thread, as value q of sh.red.
@@ -722,7 +703,7 @@ __device__ __forceinline__ void gm_dots(GmShared<T>& sh, const T* w, const T* V,
 
 // ih w - sum_q hs[q] v_q (q <= k) of group g.
 template <class T>
-__device__ __forceinline__ Pack<T> gm_project(const GmShared<T>& sh, T ih, const T* w, const T* V, size_t vs, int g,
+__device__ __forceinline__ Pack<T> gm_project(const GmVectorScalars<T>& sh, T ih, const T* w, const T* V, size_t vs, int g,
                                               int k) {
   constexpr int W = Pack<T>::W;
   Pack<T> wi = *reinterpret_cast<const Pack<T>*>(w + g * W);
@@ -794,8 +775,7 @@ __device__ __forceinline__ void gm_update(const GmShared<T>& sh, const T* w, con
 // Column k of the Hessenberg matrix, in the scalar warp: the earlier rotations (while the
 // other warps complete v_{k+1}).  The running entry c <- -sn_q c + cs_q b_q is one dependent
 // multiply-add per rotation; lane q forms the products and its entry of the column.
-template <class T>
-__device__ __forceinline__ void gm_rotate(GmShared<T>& sh, int k, bool twice) {
+__device__ __forceinline__ void gm_rotate(GmScalars& sh, int k, bool twice) {
   const int q = threadIdx.x & 31;
   double cb = 0.0, sb = 0.0, cs = 0.0, sn = 0.0, mine = 0.0;
   if (q < k) {
@@ -822,8 +802,7 @@ __device__ __forceinline__ void gm_rotate(GmShared<T>& sh, int k, bool twice) {
 }
 // ... then, from ||v_{k+1}||^2, the new rotation, the residual estimate and the
 // end-of-cycle test (while they form the next product).
-template <class T>
-__device__ __forceinline__ void gm_column(GmShared<T>& sh, int k, const GmArgs& a, bool berr) {
+__device__ __forceinline__ void gm_column(GmScalars& sh, int k, const GmArgs& a, bool berr) {
   const double n2 = sh.nrm2, c = sh.run, den2 = fma(c, c, n2);
   const double inv = rsqrt(n2), hk1 = n2 > 0.0 ? n2 * inv : sqrt(n2);
   const double rden = rsqrt(den2), den = den2 > 0.0 ? den2 * rden : sqrt(den2);
@@ -839,6 +818,20 @@ __device__ __forceinline__ void gm_column(GmShared<T>& sh, int k, const GmArgs& 
   sh.scale[k + 1] = inv;
   if (!isfinite(den) || den == 0.0 || berr) sh.done = 2;
   else if (fabs(gn) < sh.tol || sh.its >= a.maxit || k + 1 == a.m || hk1 == 0.0) sh.cycle_done = 1;
+}
+
+// H y = g for the leading ku columns (from the last; lane c keeps g[c]), in one warp.
+__device__ __forceinline__ void gm_triangle(GmScalars& sh, int ku) {
+  const int c = threadIdx.x & 31;
+  double gc = c < ku ? sh.g[c] : 0.0;
+  const double inv = c < ku ? 1.0 / sh.H[c][c] : 0.0;
+#pragma unroll 1
+  for (int q = ku - 1; q >= 0; --q) {
+    const double yq = __shfl_sync(0xffffffffu, gc * inv, q);
+    if (c == q) sh.y[q] = yq;
+    if (c < q) gc = fma(-sh.H[c][q], yq, gc);
+  }
+  __syncwarp();
 }
 
 // w = B z over a block's rows (B, z, w at the block's first row).  The row's addresses are
@@ -861,6 +854,20 @@ __device__ __forceinline__ void gm_product(const Offsets& of, int64_t N, const T
     for (int q = 0; q < K; ++q) s = fma(STREAM ? __ldcs(br + q * n) : br[q * n], zr[of.o[q]], s);
     w[r] = s;
   }
+}
+
+// The solver's scalars at the end of a solve.
+__device__ __forceinline__ void gm_report(const GmScalars& sh, const GmArgs& a, bool berr) {
+  double* sc = a.sc;
+  sc[S_N0] = sh.n0;
+  sc[S_TOL] = sh.tol;
+  sc[S_NRES] = sh.nres;
+  sc[S_BETA] = sh.nres;
+  sc[S_ITS] = (double)sh.its;
+  sc[S_CYCLES] = (double)sh.cycles;
+  sc[S_DONE] = berr ? 2.0 : (double)sh.done;
+  sc[S_BERR] = berr ? 1.0 : 0.0;
+  krylov_count(a.ep, sh.its, berr, sh.done == 2);
 }
 
 // VS: the basis in shared memory.
@@ -888,6 +895,7 @@ __global__ void __launch_bounds__(VS ? kGmBlockS : kGmBlock, 1) k_gm_fused(Offse
   for (int r = nrow + threadIdx.x; r < ng * W; r += blockDim.x) w[r] = (T)0;
   volatile int* berr = &a.bar->err;
   int buf = 0;
+  auto value = [&](int q) { return sh.value(q, nw); };
   if (!fp_goes_on(a.ep)) return;
   if (scalar) {
     sh.its = 0;
@@ -918,7 +926,7 @@ __global__ void __launch_bounds__(VS ? kGmBlockS : kGmBlock, 1) k_gm_fused(Offse
       }
       gm_put(sh, nrm, 0);
     }
-    gm_exchange(sh, 1, nw, a, buf, [&]() {
+    gm_exchange(sh, 1, a, buf, value, [&]() {
       if (threadIdx.x != 0) return;
       const double beta = sqrt(sh.tot[0]);
       if (!have_x) {
@@ -948,7 +956,7 @@ __global__ void __launch_bounds__(VS ? kGmBlockS : kGmBlock, 1) k_gm_fused(Offse
       if (sh.done != 0 || (k > 0 && sh.cycle_done != 0)) break;
       gm_dots(sh, w, V, vs, ng, nw, nt, k);
       // h1 and the projection's coefficients: w stands for w / ||v_k||, v_q for v_q / ||v_q||
-      gm_exchange(sh, k + 2, nw, a, buf, [&]() {
+      gm_exchange(sh, k + 2, a, buf, value, [&]() {
         const int q = threadIdx.x;
         const double sk = sh.scale[k], ww = sh.tot[k + 1] * (sk * sk);
         double h = 0.0;
@@ -970,7 +978,7 @@ __global__ void __launch_bounds__(VS ? kGmBlockS : kGmBlock, 1) k_gm_fused(Offse
         if (rows_warp) gm_reproject(sh, w, V, vs, ng, nt, k);
         // a thread's dots read the groups it wrote
         gm_dots(sh, w, V, vs, ng, nw, nt, k);
-        gm_exchange(sh, k + 2, nw, a, buf, [&]() {
+        gm_exchange(sh, k + 2, a, buf, value, [&]() {
           const int q = threadIdx.x;
           if (q <= k) {
             const double sq = sh.scale[q], h = sh.tot[q] * sq;
@@ -990,23 +998,15 @@ __global__ void __launch_bounds__(VS ? kGmBlockS : kGmBlock, 1) k_gm_fused(Offse
       } else {
         gm_rotate(sh, k, !skip);
       }
-      gm_exchange(sh, skip ? 1 : 0, nw, a, buf, [&]() {
+      gm_exchange(sh, skip ? 1 : 0, a, buf, value, [&]() {
         if (skip && threadIdx.x == 0) sh.nrm2 = sh.tot[0];
       });
     }
     if (sh.done != 0) break;
-    // H y = g (columns from the last; lane c keeps g[c]), then x += D^{-1} sum_q y_q v_q / ||v_q||
+    // x += D^{-1} sum_q y_q v_q / ||v_q||
     if (threadIdx.x < 32) {
+      gm_triangle(sh, ku);
       const int c = threadIdx.x;
-      double gc = c < ku ? sh.g[c] : 0.0;
-      const double inv = c < ku ? 1.0 / sh.H[c][c] : 0.0;
-#pragma unroll 1
-      for (int q = ku - 1; q >= 0; --q) {
-        const double yq = __shfl_sync(0xffffffffu, gc * inv, q);
-        if (c == q) sh.y[q] = yq;
-        if (c < q) gc = fma(-sh.H[c][q], yq, gc);
-      }
-      __syncwarp();
       if (c < ku) sh.hs[c] = (T)(-sh.y[c] * sh.scale[c]);
     }
     __syncthreads();
@@ -1014,7 +1014,7 @@ __global__ void __launch_bounds__(VS ? kGmBlockS : kGmBlock, 1) k_gm_fused(Offse
       gm_update(sh, w, V, vs, ng, nt, ku, dinv + i0, x + i0, nrow, have_x);
     }
     have_x = true;
-    gm_exchange(sh, 0, nw, a, buf, [] {});   // a barrier: the next residual gathers x
+    gm_barrier(sh, a, buf);   // the next residual gathers x
   }
   // the solution, and the caller's update unless the solve broke down
   const bool upd = a.ep.u != nullptr && sh.done != 2;
@@ -1025,18 +1025,380 @@ __global__ void __launch_bounds__(VS ? kGmBlockS : kGmBlock, 1) k_gm_fused(Offse
     a.xout[i] = xi;
     if (upd) krylov_update(a.ep, i, xi);
   }
-  if (blockIdx.x == 0 && scalar) {
-    double* sc = a.sc;
-    sc[S_N0] = sh.n0;
-    sc[S_TOL] = sh.tol;
-    sc[S_NRES] = sh.nres;
-    sc[S_BETA] = sh.nres;
-    sc[S_ITS] = (double)sh.its;
-    sc[S_CYCLES] = (double)sh.cycles;
-    sc[S_DONE] = *berr ? 2.0 : (double)sh.done;
-    sc[S_BERR] = *berr ? 1.0 : 0.0;
-    krylov_count(a.ep, sh.its, *berr != 0, sh.done == 2);
+  if (blockIdx.x == 0 && scalar) gm_report(sh, a, *berr != 0);
+}
+
+// ---- GMRES(m) on single-precision vectors -----------------------------------------
+//
+// The same method and launch, but with every single-precision rounding in a fixed place.  The
+// damped iteration around a mixed solve amplifies the rounding of its inner solver at isolated
+// nodes: with the dots added in another order and the basis unnormalised, whole stationary solves
+// moved by up to 2e-8 (P1 129^3, the same number of corrections and the same residual).  So here
+//  * the basis vectors are normalised and rounded once, v_k = w (1 / ||w||), z = D^{-1} v_k;
+//  * a dot is formed by single-precision strands: rows come in chunks of 256, chunk c adds to strand
+//    set c mod (gm_strand_sets * SMs), each of whose 256 strands takes its rows in ascending order by
+//    multiply-adds; 32 strands are added by a butterfly, the eight results of a set in turn, and the
+//    sets' sums in double.  The order of the double-precision additions is free: their rounding is
+//    far below the last bit of the single-precision coefficients they give;
+//  * the squares of a new vector's entries are added in single precision along a strand and in
+//    double across strands, those of the true residual in double from the first addition.
+// gm_strand_sets (per SM) is part of that definition: a result depends on it, and on the device's
+// SM count, but not on scheduling or on where the vectors are kept.
+//
+// Block b owns chunks b, b + G, b + 2 G, ... (G blocks; G = SMs, or fewer when each has at most two
+// chunks): the chunks of a strand set are then all in one block, for every number of sets, so that
+// w and the basis stay local to it.  In a block of chunks s = 0 .. S - 1 the sets are s mod R, and
+// a row's local index is 256 s + its place in the chunk.
+constexpr int kGsChunk = 256;
+// strand sets per SM of a step with n basis vectors (n <= kMaxRestart)
+__host__ __device__ __forceinline__ constexpr int gm_strand_sets(int n) {
+  return n <= 4 ? 6 : n <= 12 ? 5 : n <= 16 ? 4 : n <= 20 ? 3 : 2;
+}
+// values times sets of one exchange, at most
+constexpr int gs_most_sums() {
+  int most = 0;
+  for (int k = 0; k < kMaxRestart; ++k) most = (k + 2) * gm_strand_sets(k + 1) > most ? (k + 2) * gm_strand_sets(k + 1) : most;
+  return most;
+}
+constexpr int kGsSums = gs_most_sums();
+constexpr int kGsWarpRows = 128;           // rows of a chunk that a warp takes at once, 16 bytes a lane
+constexpr int kGsParts = kGsChunk / 32;    // butterflies of a strand set
+
+struct GsShared : GmVectorScalars<float> {
+  float red[kGsSums][kGsParts + 1];      // [q R + r]: the butterflies of value q, set r
+  double fold[kGsSums];                  // ... added in turn
+  double col[kGmBlock], quarter[4];              // one double per thread, and their sums
+};
+
+// A block's rows.
+struct GsRows {
+  int b, G, nrow;   // nrow: local rows in use
+  int64_t N;
+  // place in a vector of all rows
+  __device__ __forceinline__ int64_t at(int l) const { return l + ((int64_t)b + (int64_t)(G - 1) * (l / kGsChunk)) * kGsChunk; }
+};
+// Where the local rows of w and of the basis are kept: in shared memory (at their local index), or in
+// global memory (at their place among all rows).
+__device__ __forceinline__ int64_t gs_at(const GsRows& rw, bool smem, int l) { return smem ? l : rw.at(l); }
+
+// w = B z over the block's rows (see gm_product).
+template <int KT, bool STREAM>
+__device__ __forceinline__ void gs_product(const Offsets& of, const GsRows& rw, const float* __restrict__ B, const float* z,
+                                           float* w, bool ws, int nt) {
+  const int K = KT > 0 ? KT : of.K;
+#pragma unroll 1
+  for (int l = threadIdx.x; l < rw.nrow; l += nt) {
+    const int64_t i = rw.at(l);
+    int64_t n = rw.N;
+    const float* zr = z + i;
+    asm volatile("" : "+l"(n), "+l"(zr));
+    const float* br = B + i;
+    float s = 0.f;
+#pragma unroll
+    for (int q = 0; q < K; ++q) s = fma(STREAM ? __ldcs(br + q * n) : br[q * n], zr[of.o[q]], s);
+    w[ws ? l : i] = s;
   }
+}
+
+// The strands of NQ vectors v_0, v_vs, ... with w for 128 rows of strand set r (half h of its
+// chunks), four adjacent strands per lane; then the butterflies of 32 strands each: partners at
+// distance 16, 8 and 4 are lanes at distance 4, 2 and 1, those at distance 2 and 1 are entries of a
+// lane (halving the entries with the lanes, six shuffles instead of twenty).  Every sum has the
+// operands of a butterfly over 32 lanes.
+template <int NQ>
+__device__ __forceinline__ void gs_strands(GsShared& sh, const float* w, int64_t wstep, const float* V, int64_t vstep,
+                                           size_t vs, int r, int h, int R, int S, int nrow, int q0) {
+  const int lane = threadIdx.x & 31;
+  float acc[NQ][4] = {};
+  auto add = [&](const float* wp, const float* vp) {
+    const Pack<float> wi = *reinterpret_cast<const Pack<float>*>(wp);
+    Pack<float> v[NQ];
+#pragma unroll
+    for (int j = 0; j < NQ; ++j) v[j] = *reinterpret_cast<const Pack<float>*>(vp + j * vs);
+#pragma unroll
+    for (int j = 0; j < NQ; ++j)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[j][e] = fma(wi.e[e], v[j].e[e], acc[j][e]);
+  };
+  int s = r;
+#pragma unroll 2
+  for (; s < S - 1; s += R, w += wstep, V += vstep) add(w, V);
+  if (s == S - 1 && s * kGsChunk + h * kGsWarpRows + 4 * lane < nrow) add(w, V);   // the last chunk may end early
+  const bool b2 = lane & 4, b1 = lane & 2;
+#pragma unroll
+  for (int j = 0; j < NQ; ++j) {
+    float a[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {   // distance 16: entries e (lanes without bit 2) or e + 2
+      const float send = b2 ? acc[j][e] : acc[j][e + 2], keep = b2 ? acc[j][e + 2] : acc[j][e];
+      a[e] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
+    }
+    const float send = b1 ? a[0] : a[1], keep = b1 ? a[1] : a[0];
+    float t = keep + __shfl_xor_sync(0xffffffffu, send, 2);   // 8: entry (b2, b1)
+    t += __shfl_xor_sync(0xffffffffu, t, 1);                  // 4
+    t += __shfl_xor_sync(0xffffffffu, t, 4);                  // 2: entries 0 and 2, 1 and 3
+    t += __shfl_xor_sync(0xffffffffu, t, 2);                  // 1
+    if ((lane & 7) == 0) sh.red[(q0 + j) * R + r][4 * h + (lane >> 3)] = t;
+  }
+}
+
+// The strand sums of (w, v_q), q <= k, as values 0 .. k, and with `norm` of (w, w) as value k + 1.
+// Items: 128 rows of a strand set (both halves of R sets) times a few of the vectors, as many as
+// leave an item for every warp.  Every warp with rows calls it.
+__device__ __forceinline__ void gs_dots(GsShared& sh, const GsRows& rw, const float* w, bool ws, const float* V, bool vsm,
+                                        size_t vs, int R, int S, int nwarp, int k, bool norm) {
+  const int units = 2 * R, most = max(1, nwarp / units);
+  const int per = min(4, (k + most) / most);                  // ceil((k + 1) / most)
+  const int groups = (k + per) / per;                         // ceil((k + 1) / per)
+  const int items = units * (groups + (norm ? 1 : 0));
+  const int64_t step = (int64_t)R * kGsChunk;
+  const int64_t vstep = vsm ? step : step * rw.G, wstep = ws ? step : step * rw.G;
+  const int lane = threadIdx.x & 31;
+#pragma unroll 1
+  for (int it = threadIdx.x >> 5; it < items; it += nwarp) {
+    const int u = it % units, gq = it / units, r = u >> 1, h = u & 1;
+    const int l = r * kGsChunk + h * kGsWarpRows + 4 * lane;
+    const float* wl = w + gs_at(rw, ws, l);
+    if (gq == groups) {
+      gs_strands<1>(sh, wl, wstep, wl, wstep, 0, r, h, R, S, rw.nrow, k + 1);
+      continue;
+    }
+    const int q0 = gq * per;
+    const float* vl = V + (size_t)q0 * vs + gs_at(rw, vsm, l);
+    switch (min(per, k + 1 - q0)) {
+      case 4: gs_strands<4>(sh, wl, wstep, vl, vstep, vs, r, h, R, S, rw.nrow, q0); break;
+      case 3: gs_strands<3>(sh, wl, wstep, vl, vstep, vs, r, h, R, S, rw.nrow, q0); break;
+      case 2: gs_strands<2>(sh, wl, wstep, vl, vstep, vs, r, h, R, S, rw.nrow, q0); break;
+      default: gs_strands<1>(sh, wl, wstep, vl, vstep, vs, r, h, R, S, rw.nrow, q0);
+    }
+  }
+}
+// ... a set's butterflies added in turn (the block).
+__device__ __forceinline__ void gs_fold(GsShared& sh, int n) {
+  __syncthreads();
+  for (int x = threadIdx.x; x < n; x += blockDim.x) {
+    float s = 0.f;
+#pragma unroll
+    for (int u = 0; u < kGsParts; ++u) s += sh.red[x][u];
+    sh.fold[x] = widen_exact(s);
+  }
+}
+
+// The sum of one double per thread with rows, in four warps, as sh.quarter (the block).
+__device__ __forceinline__ void gs_column(GsShared& sh, int nt) {
+  const int wp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  __syncthreads();
+  if (wp >= 4) return;
+  double t = 0.0;
+  for (int j = wp * 32 + lane; j < nt; j += 128) t += sh.col[j];
+  t = warp_sum(t);
+  if (lane == 0) sh.quarter[wp] = t;
+}
+// This thread's part of ||w||^2, a single-precision sum per strand: a warp takes 32 strands.
+__device__ __forceinline__ double gs_norm(const GsRows& rw, const float* w, bool ws, int R, int S, int nwarp) {
+  const int lane = threadIdx.x & 31;
+  const int64_t step = (int64_t)R * kGsChunk * (ws ? 1 : rw.G);
+  double sum = 0.0;
+#pragma unroll 1
+  for (int u = threadIdx.x >> 5; u < R * kGsParts; u += nwarp) {
+    const int r = u / kGsParts, l = r * kGsChunk + 32 * (u % kGsParts) + lane;
+    const float* p = w + gs_at(rw, ws, l);
+    float nrm = 0.f;
+    int s = r;
+#pragma unroll 4
+    for (; s < S - 1; s += R, p += step) nrm = fma(*p, *p, nrm);
+    if (s == S - 1 && l + (s - r) * kGsChunk < rw.nrow) nrm = fma(*p, *p, nrm);
+    sum += widen_exact(nrm);
+  }
+  return sum;
+}
+
+// VS: the basis in shared memory (then w too).
+template <int KT, bool VS>
+__global__ void __launch_bounds__(VS ? kGmBlockS : kGmBlock, 1) k_gm_single(Offsets of, const float* __restrict__ B,
+                                                                const float* __restrict__ dinv, float* x, float* z,
+                                                                float* wg, float* Vg, GmArgs a) {
+  constexpr int W = Pack<float>::W;
+  const int64_t chunks = (a.N + kGsChunk - 1) / kGsChunk;
+  GsRows rw;
+  rw.b = blockIdx.x;
+  rw.G = gridDim.x;
+  rw.N = a.N;
+  const int S = (int)((chunks - rw.b + rw.G - 1) / rw.G);
+  rw.nrow = S * kGsChunk;
+  if ((chunks - 1) % rw.G == rw.b) rw.nrow -= (int)(chunks * kGsChunk - a.N);   // it owns the last chunk
+  const int nt = a.compute, nwarp = nt >> 5;      // threads with rows; the last warp has the scalars
+  const bool rows_warp = (int)threadIdx.x < nt, scalar = (int)threadIdx.x == nt;   // scalar: its first lane
+  const int ng = (rw.nrow + W - 1) / W;           // 16-byte groups; the last one may reach past N
+  __shared__ GsShared sh;
+  extern __shared__ __align__(16) char dyn[];
+  const bool ws = VS || a.w_in_smem;
+  float* const w = ws ? reinterpret_cast<float*>(dyn) : wg;
+  float* const V = VS ? reinterpret_cast<float*>(dyn) + a.rows : Vg;
+  const size_t vs = VS ? (size_t)a.rows : a.vstride;
+  for (int l = rw.nrow + threadIdx.x; l < ng * W; l += blockDim.x) w[gs_at(rw, ws, l)] = 0.f;   // and stays so
+  volatile int* berr = &a.bar->err;
+  int buf = 0;
+  if (!fp_goes_on(a.ep)) return;
+  if (scalar) {
+    sh.its = 0;
+    sh.cycles = 0;
+    sh.done = 0;
+  }
+  // w -= sum_q hs[q] v_q, q <= k
+  auto project = [&](int k) {
+#pragma unroll 1
+    for (int g = threadIdx.x; g < ng; g += nt) {
+      float* wl = w + gs_at(rw, ws, g * W);
+      *reinterpret_cast<Pack<float>*>(wl) = gm_project(sh, 1.f, wl, V + gs_at(rw, VS, g * W), vs, 0, k);
+    }
+  };
+  // v_q = ih w, z = D^{-1} v_q
+  auto normalise = [&](int q) {
+    const float ih = sh.ih;
+    float* vq = V + (size_t)q * vs;
+#pragma unroll 1
+    for (int g = threadIdx.x; g < ng; g += nt) {
+      const int l = g * W;
+      const int64_t i = rw.at(l);
+      Pack<float> v = *reinterpret_cast<const Pack<float>*>(w + (ws ? l : i));
+#pragma unroll
+      for (int e = 0; e < W; ++e) {
+        v.e[e] *= ih;
+        if (l + e < rw.nrow) z[i + e] = dinv[i + e] * v.e[e];
+      }
+      *reinterpret_cast<Pack<float>*>(vq + (VS ? l : i)) = v;
+    }
+  };
+  auto norm_value = [&](int) { return (sh.quarter[0] + sh.quarter[1]) + (sh.quarter[2] + sh.quarter[3]); };
+  bool have_x = false;   // x = 0 until the first cycle's update
+  for (;;) {
+    // true residual w = rhs - B x and its norm, v_0 = w / ||w||
+    if (have_x && rows_warp) gs_product<KT, !VS>(of, rw, B, x, w, ws, nt);
+    if (rows_warp) {   // a thread's own rows
+      double nrm = 0.0;
+#pragma unroll 1
+      for (int l = threadIdx.x; l < rw.nrow; l += nt) {
+        const int64_t i = rw.at(l);
+        float* wl = w + (ws ? l : i);
+        const float v = have_x ? (float)a.rhs[i] - *wl : (float)a.rhs[i];
+        *wl = v;
+        nrm += widen_exact(v * v);
+      }
+      sh.col[threadIdx.x] = nrm;
+    }
+    gs_column(sh, nt);
+    gm_exchange(sh, 1, a, buf, norm_value, [&]() {
+      if (threadIdx.x != 0) return;
+      const double beta = sqrt(sh.tot[0]);
+      if (!have_x) {
+        sh.n0 = beta;
+        sh.tol = fmax(a.atol, a.rtol * beta);
+      }
+      sh.cycles += 1;
+      sh.nres = beta;
+      sh.cycle_done = 0;
+      if (!isfinite(beta) || *berr) sh.done = 2;
+      else if (beta < sh.tol) sh.done = 1;
+      else if (sh.its >= a.maxit) sh.done = 4;
+      sh.g[0] = beta;
+      sh.ih = (float)(1.0 / beta);
+    });
+    if (sh.done != 0) break;
+    if (rows_warp) normalise(0);
+    gm_barrier(sh, a, buf);   // the product gathers z
+    int ku = 0;   // columns of this cycle
+    for (int k = 0;; ++k) {
+      // (1) w = B z and its dots; meanwhile the scalar warp ends column k - 1
+      if (rows_warp) {
+        gs_product<KT, !VS>(of, rw, B, z, w, ws, nt);
+      } else if (scalar && k > 0) {
+        gm_column(sh, k - 1, a, *berr != 0);
+      }
+      __syncthreads();
+      ku = k;
+      if (sh.done != 0 || (k > 0 && sh.cycle_done != 0)) break;
+      const int R = min(gm_strand_sets(k + 1), S);
+      auto value = [&](int q) {
+        double t = 0.0;
+        for (int r = 0; r < R; ++r) t += sh.fold[q * R + r];
+        return t;
+      };
+      if (rows_warp) gs_dots(sh, rw, w, ws, V, VS, vs, R, S, nwarp, k, true);
+      gs_fold(sh, (k + 2) * R);
+      // h1 and the DGKS test
+      gm_exchange(sh, k + 2, a, buf, value, [&]() {
+        const int q = threadIdx.x;
+        double h = 0.0;
+        if (q <= k) {
+          h = sh.tot[q];
+          sh.h1[q] = h;
+          sh.h2[q] = 0.0;
+          sh.hs[q] = (float)h;
+        }
+        const double ww = sh.tot[k + 1], rest = ww - warp_sum(h * h);
+        if (q == 0) sh.skip = rest >= 0.5 * ww && ww > 0.0;
+      });
+      if (!sh.skip) {   // second projection: w = w - V h1, h2 = V^T w
+        if (rows_warp) project(k);
+        __syncthreads();
+        if (rows_warp) gs_dots(sh, rw, w, ws, V, VS, vs, R, S, nwarp, k, false);
+        gs_fold(sh, (k + 1) * R);
+        gm_exchange(sh, k + 1, a, buf, value, [&]() {
+          const int q = threadIdx.x;
+          if (q <= k) {
+            const double h = sh.tot[q];
+            sh.h2[q] = h;
+            sh.hs[q] = (float)h;
+          }
+        });
+      }
+      // (2) w -= V h and its norm (meanwhile the scalar warp rotates column k), v_{k+1} = w / ||w||
+      if (rows_warp) project(k);
+      else gm_rotate(sh, k, false);
+      __syncthreads();
+      if (rows_warp) sh.col[threadIdx.x] = gs_norm(rw, w, ws, R, S, nwarp);
+      gs_column(sh, nt);
+      gm_exchange(sh, 1, a, buf, norm_value, [&]() {
+        if (threadIdx.x != 0) return;
+        sh.nrm2 = sh.tot[0];
+        sh.ih = sh.tot[0] == 0.0 ? 0.f : (float)(1.0 / sqrt(sh.tot[0]));   // 0: the cycle ends with this column
+      });
+      if (rows_warp) normalise(k + 1);
+      gm_barrier(sh, a, buf);
+    }
+    if (sh.done != 0) break;
+    // x += D^{-1} sum_q y_q v_q
+    if (threadIdx.x < 32) {
+      gm_triangle(sh, ku);
+      const int c = threadIdx.x;
+      if (c < ku) sh.hs[c] = (float)-sh.y[c];   // the projection's sign
+    }
+    __syncthreads();
+    if (rows_warp) {
+#pragma unroll 1
+      for (int g = threadIdx.x; g < ng; g += nt) {
+        const int l = g * W;
+        const int64_t i = rw.at(l);
+        const Pack<float> v = gm_project(sh, 0.f, w + (ws ? l : i), V + (VS ? l : i), vs, 0, ku - 1);
+#pragma unroll
+        for (int e = 0; e < W; ++e)
+          if (l + e < rw.nrow) x[i + e] = fma(dinv[i + e], v.e[e], have_x ? x[i + e] : 0.f);
+      }
+    }
+    have_x = true;
+    gm_barrier(sh, a, buf);   // the next residual gathers x
+  }
+  // the solution, and the caller's update unless the solve broke down
+  const bool upd = a.ep.u != nullptr && sh.done != 2;
+#pragma unroll 1
+  for (int l = threadIdx.x; l < rw.nrow; l += blockDim.x) {
+    const int64_t i = rw.at(l);
+    const double xi = have_x ? (double)x[i] : 0.0;
+    a.xout[i] = xi;
+    if (upd) krylov_update(a.ep, i, xi);
+  }
+  if (blockIdx.x == 0 && scalar) gm_report(sh, a, *berr != 0);
 }
 
 }  // namespace
@@ -1221,10 +1583,11 @@ int gmres_fused_launch(afc_problem_s* p, cudaStream_t s, const T* B, const T* di
   a.m = o->gmres_restart;
   if (epi) a.ep = *epi;
   a.wait_ns = p->grid_wait_ns;
-  const int64_t units = (N + kGmUnit - 1) / kGmUnit;
-  const int64_t least = sizeof(T) == 4 ? 512 / kGmUnit : 64 / kGmUnit;   // units of a block, at least
+  constexpr bool kSingle = sizeof(T) == 4;
+  const int64_t unit = kSingle ? kGsChunk : kGmUnit, units = (N + unit - 1) / unit;
+  const int64_t least = kSingle ? 2 : 64 / kGmUnit;   // units of a block, at least
   const int G = (int)std::max<int64_t>(1, std::min<int64_t>((units + least - 1) / least, std::min(w.nsm, 160)));
-  const int64_t rows = (units + G - 1) / G * kGmUnit;   // most rows of a block
+  const int64_t rows = (units + G - 1) / G * unit;   // most rows of a block
   const size_t vec = (size_t)rows * sizeof(T);
   const bool vs = (size_t)(a.m + 2) * vec <= kGmSmem;   // w and V_0 .. V_m
   a.w_in_smem = vec <= kGmSmem;
@@ -1235,12 +1598,15 @@ int gmres_fused_launch(afc_problem_s* p, cudaStream_t s, const T* B, const T* di
   const int block = a.compute + 32;
   with_K(p->K, [&](auto kc) {
     constexpr int KT = decltype(kc)::value;
-    auto kern = vs ? k_gm_fused<KT, T, true> : k_gm_fused<KT, T, false>;
+    auto kern = [&] {
+      if constexpr (kSingle) return vs ? k_gm_single<KT, true> : k_gm_single<KT, false>;
+      else return vs ? k_gm_fused<KT, T, true> : k_gm_fused<KT, T, false>;
+    }();
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGmSmem);
     int nb = 0;
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, block, smem);
     if (e != cudaSuccess || nb < 1) {
-      st = cuda_fail(e != cudaSuccess ? e : cudaErrorInvalidConfiguration, "occupancy of k_gm_fused");
+      st = cuda_fail(e != cudaSuccess ? e : cudaErrorInvalidConfiguration, "occupancy of the GMRES launch");
       return;
     }
     cudaLaunchConfig_t cfg = {};
@@ -1256,8 +1622,8 @@ int gmres_fused_launch(afc_problem_s* p, cudaStream_t s, const T* B, const T* di
     cudaEvent_t ev = prof_start(p);
     e = cudaLaunchKernelEx(&cfg, kern, p->offs, B, dinv, vec_at<T>(w, 0), vec_at<T>(w, 1), vec_at<T>(w, 2),
                            vec_at<T>(w, 3), a);
-    prof_stop(p, "k_gm_fused", ev);
-    if (e != cudaSuccess) st = cuda_fail(e, "cudaLaunchKernelEx(k_gm_fused)");
+    prof_stop(p, kSingle ? "k_gm_single" : "k_gm_fused", ev);
+    if (e != cudaSuccess) st = cuda_fail(e, "cudaLaunchKernelEx(GMRES)");
   });
   return st;
 }

@@ -227,6 +227,7 @@ struct afc_batch_s {
   afc::BInst* tab_d = nullptr;
   int2* map_d = nullptr;                // tile -> (instance, tile of it), for the tiles of tab_block rows
   int tab_block = 0;                    // rows per tile the table was built for
+  bool tab_mixed = false;               // ... with the single-precision arrays of every instance
   int map_block = 0;                    // ... and the map
   std::vector<double> tab_dt;           // time steps in the table
   int64_t ntiles = 0;
@@ -305,7 +306,9 @@ int build_table(afc_batch_s* b, int block, const double* dt, double dt_all, bool
       if (st) return st;
       if (!ready && p->stream != b->stream) AFC_CUDA(cudaStreamSynchronize(p->stream));
     }
-  if (b->tab_block == block && b->tab_dt == dts) return AFC_OK;
+  // (a table built for steps in double may hold null single-precision arrays: they are made by the
+  // first mixed call)
+  if (b->tab_block == block && b->tab_dt == dts && (b->tab_mixed || !mixed)) return AFC_OK;
   // the previous upload may still be reading the pinned table
   AFC_CUDA(cudaStreamSynchronize(b->stream));
   int64_t tile = 0;
@@ -326,6 +329,7 @@ int build_table(afc_batch_s* b, int block, const double* dt, double dt_all, bool
   }
   b->ntiles = tile;
   b->tab_block = block;
+  b->tab_mixed = mixed;
   b->tab_dt = dts;
   AFC_CUDA(cudaMemcpyAsync(b->tab_d, b->tab_h, b->list.size() * sizeof(BInst), cudaMemcpyHostToDevice, b->stream));
   if (b->map_block != block) {

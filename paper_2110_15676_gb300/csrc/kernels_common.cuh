@@ -70,48 +70,54 @@ __device__ __forceinline__ double widen_exact(float x) {
 }
 
 // Sums of the positive and of the negative values of a row's pair fluxes in 64-bit fixed point
-// (Zalesak's P+ and P-), on the integer pipe: the largest value's leading bit at bit 57 (up to 62
-// terms fit), every smaller term rounded to the last bit, each total rounded to double once.
-// A total carries an error of a few 2^-58 of the largest term, far below the rounding of the
-// result; a sum of FP64 adds carries one rounding per add.  Subnormal inputs count as zero.
-// On GB300 this replaces two FP64 adds per value (an FP64 warp instruction occupies the pipe
-// for 16 cycles) with about twenty integer instructions; 128-bit totals took half as many
-// again (k_cn_factors at Q1 65^3: 38 -> 29 us).  The values are taken one at a time, so that
-// none has to be kept until the largest exponent is known: the totals are held scaled to the
-// largest exponent seen so far, and a value with a larger one first shifts them right.
+// (Zalesak's P+ and P-), on the integer pipe.  Each of the two has a scale of its own: its largest
+// value's leading bit at bit 57 (up to 62 terms fit), every other term, and the total when a larger
+// one rescales it, rounded to the last bit; the totals are rounded to double once.  A total of n
+// terms so carries at most 2 n 2^-58 of its own largest term and one rounding, where a sum of FP64
+// adds carries n - 1 roundings.  (With one scale for both, a P- below 2^-58 of P+ came out as 0,
+// and R- as 1.)  Subnormal values keep their bits.
+// On GB300 this replaces two FP64 adds per value (an FP64 warp instruction occupies the pipe for
+// 16 cycles).  The values are taken one at a time, so that none has to be kept until the largest
+// exponent is known.
 struct SignedSums64 {
-  unsigned emax = 0u;
+  unsigned ep = 0u, en = 0u;
   unsigned long long p = 0ull, n = 0ull;
 
-  __device__ __forceinline__ void raise(unsigned e) {   // scale the totals to a larger exponent
-    const unsigned d = e - emax;
-    p = d < 64u ? p >> d : 0ull;
-    n = d < 64u ? n >> d : 0ull;
-    emax = e;
-  }
-  __device__ __forceinline__ void put(unsigned long long m, unsigned e, bool neg) {   // m: leading bit at bit 58
-    const unsigned sh = emax - e;
-    const unsigned long long v = ((sh < 64u ? m >> sh : 0ull) + 1ull) >> 1;
-    if (neg) n += v;
-    else p += v;
+  // m: the significand, a normal value's leading bit at bit 58; e >= 1
+  __device__ __forceinline__ void put(unsigned long long m, unsigned e, bool neg) {
+    unsigned at = neg ? en : ep;
+    unsigned long long t = neg ? n : p;
+    if (e > at) {   // scale the total to the larger exponent
+      const unsigned d = e - at;
+      t = d < 64u ? ((t >> (d - 1u)) + 1ull) >> 1 : 0ull;
+      at = e;
+    }
+    const unsigned sh = at - e;
+    t += ((sh < 64u ? m >> sh : 0ull) + 1ull) >> 1;
+    if (neg) {
+      en = at;
+      n = t;
+    } else {
+      ep = at;
+      p = t;
+    }
   }
   __device__ __forceinline__ void add(unsigned long long b) {   // a double
+    if ((b << 1) == 0ull) return;
     const unsigned e = (unsigned)(b >> 52) & 0x7ffu;
-    if (e == 0u) return;
-    if (e > emax) raise(e);
-    put(((b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << 6, e, b >> 63);
+    const unsigned long long f = b & 0xFFFFFFFFFFFFFull;
+    put((e ? f | 0x10000000000000ull : f) << 6, e ? e : 1u, b >> 63);
   }
   __device__ __forceinline__ void add(unsigned b) {   // a float
-    const unsigned e = (b >> 23) & 0xffu;
-    if (e == 0u) return;
-    if (e > emax) raise(e);
-    put((unsigned long long)((b & 0x7fffffu) | 0x800000u) << 35, e, b >> 31);
+    if ((b << 1) == 0u) return;
+    const unsigned e = (b >> 23) & 0xffu, f = b & 0x7fffffu;
+    put((unsigned long long)(e ? f | 0x800000u : f) << 35, e ? e : 1u, b >> 31);
   }
   // totals of doubles (BIAS 1023) or floats (BIAS 127)
   template <int BIAS>
   __device__ __forceinline__ void result(double& pos, double& neg) const {
-    pos = to_double(p, (int)emax - BIAS - 57);
-    neg = neg_bits(to_double(n, (int)emax - BIAS - 57));
+    pos = to_double(p, (int)ep - BIAS - 57);
+    neg = neg_bits(to_double(n, (int)en - BIAS - 57));
   }
   __device__ static __noinline__ double to_double_edge(unsigned long long v, int ex) {
     return scalbn(__ull2double_rn(v), ex);

@@ -1121,7 +1121,7 @@ __device__ __forceinline__ void gs_strands(GsShared& sh, const float* w, int64_t
       for (int e = 0; e < 4; ++e) acc[j][e] = fma(wi.e[e], v[j].e[e], acc[j][e]);
   };
   int s = r;
-#pragma unroll 2
+#pragma unroll 1
   for (; s < S - 1; s += R, w += wstep, V += vstep) add(w, V);
   if (s == S - 1 && s * kGsChunk + h * kGsWarpRows + 4 * lane < nrow) add(w, V);   // the last chunk may end early
   const bool b2 = lane & 4, b1 = lane & 2;

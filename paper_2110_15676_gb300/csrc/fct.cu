@@ -214,7 +214,7 @@ __global__ void k_cn_factors(int64_t N, Offsets of, const unsigned long long* __
   const double qp = mQp[i], qm = mQm[i];
   pdl_wait();
   if (isdir) { Rp[i] = 1.0; Rm[i] = 1.0; return; }
-  SignedSums64 acc;
+  SignedSums128 acc;
   constexpr int S = kGroup<KT>;
 #pragma unroll
   for (int k0 = 0; k0 < K; k0 += S) {
@@ -230,7 +230,7 @@ __global__ void k_cn_factors(int64_t N, Offsets of, const unsigned long long* __
     }
   }
   double Pp, Pm;
-  acc.result<1023>(Pp, Pm);
+  acc.result(Pp, Pm);
   Rp[i] = zalesak_factor(qp, dt * Pp);
   Rm[i] = zalesak_factor(qm, dt * Pm);
 }

@@ -131,6 +131,60 @@ struct SignedSums64 {
   }
 };
 
+// The same sums with 64 bits more (the CN scheme's, whose factors enter every correction of a
+// step's fixed point): what falls off the end is below 2^-120 of a sum's largest term, and each
+// total is rounded to double once.
+struct SignedSums128 {
+  unsigned ep = 0u, en = 0u;
+  unsigned long long ph = 0ull, pl = 0ull, nh = 0ull, nl = 0ull;   // largest term's leading bit: bit 57 of the high word
+
+  __device__ __forceinline__ void add(unsigned long long b) {   // a double
+    if ((b << 1) == 0ull) return;
+    unsigned e = (unsigned)(b >> 52) & 0x7ffu;
+    unsigned long long m = b & 0xFFFFFFFFFFFFFull;
+    if (e) m |= 0x10000000000000ull;
+    else e = 1u;
+    m <<= 5;
+    const bool neg = b >> 63;
+    unsigned at = neg ? en : ep;
+    unsigned long long h = neg ? nh : ph, l = neg ? nl : pl;
+    if (e > at) {   // scale the total to the larger exponent
+      shift(h, l, e - at);
+      at = e;
+    }
+    unsigned long long vl = 0ull;
+    shift(m, vl, at - e);
+    l += vl;
+    h += m + (l < vl ? 1ull : 0ull);
+    if (neg) {
+      en = at;
+      nh = h;
+      nl = l;
+    } else {
+      ep = at;
+      ph = h;
+      pl = l;
+    }
+  }
+  __device__ static __forceinline__ void shift(unsigned long long& h, unsigned long long& l, unsigned d) {   // right
+    if (d == 0u) return;
+    if (d < 64u) {
+      l = (l >> d) | (h << (64u - d));
+      h >>= d;
+    } else {
+      l = d < 128u ? h >> (d - 64u) : 0ull;
+      h = 0ull;
+    }
+  }
+  // A total whose largest term is normal has its leading bit at bit 57 of the high word or above, so
+  // that the low word matters to the rounding only by being zero or not; one of subnormal terms is
+  // exact in the high word.
+  __device__ __forceinline__ void result(double& pos, double& neg) const {
+    pos = SignedSums64::to_double(ph | (pl != 0ull ? 1ull : 0ull), (int)ep - 1023 - 57);
+    neg = neg_bits(SignedSums64::to_double(nh | (nl != 0ull ? 1ull : 0ull), (int)en - 1023 - 57));
+  }
+};
+
 // a / m for a divisor whose rounded reciprocal im is at hand (Markstein, IBM J. Res. Dev. 34
 // (1990) 111): q = a im, one residual, one correction, three FP64 operations where the inlined
 // division takes about ten; the correctly rounded quotient, as long as nothing in it

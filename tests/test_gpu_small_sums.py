@@ -62,3 +62,50 @@ def test_explicit_factors(afc, elem, small, tol, sign):
     got = _problem(afc, elem, n, b, mask, u).fe_stage(dt)
     for k, sel in rows.items():
         assert np.all(np.abs(got[k] - want[k])[sel] <= tol), k
+
+
+def _cn(prob, u, dt):
+    """Fluxes, predictor and limiter of the CN residual at u_new = u_old = u."""
+    ut = u - 0.5 * dt * (prob.AA @ u - prob.f) / prob.mL
+    ut[prob.dir_mask] = 0.0
+    return O.zalesak_limiter(prob, O.cn_fluxes(prob, u, u, dt, False), ut, dt)[1]
+
+
+@pytest.mark.parametrize("elem", ["p1", "q1"])
+@pytest.mark.parametrize("small", [1e-19, 1e-25])
+@pytest.mark.parametrize("sign", [1.0, -1.0])
+def test_cn_factors(afc, elem, small, sign):
+    n, b, mask, u, prob = _field(elem, small, sign)
+    dt = 3.0 * O.cfl_timestep(prob, 1.0)
+    want = _cn(prob, u, dt)
+    rows = _rows(want, 2.0 ** -58)
+    assert rows["Rp"].any() or rows["Rm"].any()
+    got = _problem(afc, elem, n, b, mask, u).cn_limited_sum(dt, u, u, prelimit=0)
+    for k, sel in rows.items():
+        assert np.all(np.abs(got[k] - want[k])[sel] <= 1e-12), k
+
+
+@pytest.mark.parametrize("elem", ["p1", "q1"])
+def test_cn_sums_are_rounded_once(afc, elem):
+    """R+/- of the CN scheme bit for bit from correctly rounded P+/- (u_new = u_old, no
+    prelimiting: r_ij = d_ij (u_j - u_i), with the library's own d_ij, predictor and masses)."""
+    import math
+    n, b, mask, _, prob = _field(elem, 1.0, 1.0)
+    N = len(mask)
+    u = np.where(mask != 0, 0.0, np.random.default_rng(3).uniform(-1.0, 1.0, N))
+    g = _problem(afc, elem, n, b, mask, u)
+    dt = 4.0 * g.cfl_timestep(1.0)
+    got = g.cn_limited_sum(dt, u, u, prelimit=0)
+    rowptr, col, d = g.export_csr(afc.AFC_MAT_D)
+    m, ut = g.lumped_mass(), got["u_tilde"]
+    decided = 0
+    for i in np.flatnonzero(mask == 0):
+        at = slice(rowptr[i], rowptr[i + 1])
+        j = col[at]
+        r = np.where(j == i, 0.0, d[at] * (2.0 * u[j] - 2.0 * u[i])) / 2.0
+        for k, P, Q in (("Rp", math.fsum(r[r > 0]), ut[j].max() - ut[i]), ("Rm", math.fsum(r[r < 0]), ut[j].min() - ut[i])):
+            num, den = m[i] * Q, dt * P
+            want = 1.0 if den == 0.0 or abs(num) >= abs(den) else num / den
+            assert got[k][i] == want, (i, k)
+            decided += want < 1.0
+    assert decided > N // 4

@@ -569,7 +569,7 @@ struct GmScalars {
   double H[kMaxRestart][kMaxRestart];  // H[row][col], upper triangle after the rotations
   double run;                          // running entry of the column being rotated
   double nres, n0, tol;
-  int its, cycles, done, cycle_done, skip;
+  int its, cycles, done, cycle_done, skip, sum_norm;
 };
 template <class T>
 struct GmVectorScalars : GmScalars {
@@ -731,11 +731,11 @@ __device__ __forceinline__ void gm_reproject(const GmShared<T>& sh, T* w, const 
   for (int g = threadIdx.x; g < ng; g += nt)
     *reinterpret_cast<Pack<T>*>(w + g * Pack<T>::W) = gm_project(sh, ih, w, V, vs, g, k);
 }
-// v_{k+1} = ih w - V h, z = D^{-1} v_{k+1} at the block's rows, and with `norm` the warps' sums
-// of ||v_{k+1}||^2.
+// v_{k+1} = ih w - V h, z = D^{-1} v_{k+1} at the block's rows, and the warps' sums of
+// ||v_{k+1}||^2.
 template <class T>
 __device__ __forceinline__ void gm_complete(GmShared<T>& sh, const T* w, T* V, size_t vs, int ng, int nt, int k,
-                                         const T* __restrict__ dinv, T* z, int nrow, bool norm) {
+                                         const T* __restrict__ dinv, T* z, int nrow) {
   constexpr int W = Pack<T>::W;
   const T ih = sh.ih;
   T* vn = V + (size_t)(k + 1) * vs;
@@ -751,7 +751,7 @@ __device__ __forceinline__ void gm_complete(GmShared<T>& sh, const T* w, T* V, s
       nrm = fma(v.e[e], v.e[e], nrm);
     }
   }
-  if (norm) gm_put(sh, nrm, 0);
+  gm_put(sh, nrm, 0);
 }
 // x (+)= D^{-1} sum_q hs[q] v_q, q < ku (sh.ih = 0 and hs negated: the projection's form).
 template <class T>
@@ -775,7 +775,7 @@ __device__ __forceinline__ void gm_update(const GmShared<T>& sh, const T* w, con
 // Column k of the Hessenberg matrix, in the scalar warp: the earlier rotations (while the
 // other warps complete v_{k+1}).  The running entry c <- -sn_q c + cs_q b_q is one dependent
 // multiply-add per rotation; lane q forms the products and its entry of the column.
-__device__ __forceinline__ void gm_rotate(GmScalars& sh, int k, bool twice) {
+__device__ __forceinline__ void gm_rotate(GmScalars& sh, int k) {
   const int q = threadIdx.x & 31;
   double cb = 0.0, sb = 0.0, cs = 0.0, sn = 0.0, mine = 0.0;
   if (q < k) {
@@ -793,12 +793,16 @@ __device__ __forceinline__ void gm_rotate(GmScalars& sh, int k, bool twice) {
   }
   if (q < k) sh.H[q][k] = fma(cs, mine, sb);
   if (q == 0) sh.run = c;
-  // after a second projection w was almost orthogonal: ||w - V h2||^2 = ||w||^2 - ||h2||^2 loses
-  // nothing, and the norm needs no sum of its own
-  if (twice) {
-    const double h = q <= k ? sh.h2[q] : 0.0, p = warp_sum(h * h);
-    if (q == 0) sh.nrm2 = fmax(sh.nrm2 - p, 0.0);
-  }
+}
+// ||v_{k+1}||^2 after a second projection, in the same warp: w was almost orthogonal to the basis, so
+// that ||w - V h2||^2 = ||w||^2 - ||h2||^2 needs no sum of its own (3 us of a step of 18).  Only where
+// less than 2^-10 of ||w||^2 is taken away: the difference is then as exact as the sum ||w||^2.
+__device__ __forceinline__ void gm_second_norm(GmScalars& sh, int k) {
+  const int q = threadIdx.x & 31;
+  const double h = !sh.skip && q <= k ? sh.h2[q] : 0.0, p = warp_sum(h * h);
+  if (q != 0) return;
+  sh.sum_norm = sh.skip || !(p <= 0x1p-10 * sh.nrm2);
+  if (!sh.sum_norm) sh.nrm2 -= p;
 }
 // ... then, from ||v_{k+1}||^2, the new rotation, the residual estimate and the
 // end-of-cycle test (while they form the next product).
@@ -967,14 +971,13 @@ __global__ void __launch_bounds__(VS ? kGmBlockS : kGmBlock, 1) k_gm_fused(Offse
           sh.h2[q] = 0.0;
           sh.hs[q] = (T)(h * sq);
         }
-        const float hf = (float)h, wf = (float)ww, rest = wf - warp_sum(hf * hf);   // the test needs no more
+        const double rest = ww - warp_sum(h * h);
         if (q == 0) {
           sh.ih = (T)sk;
-          sh.skip = rest >= 0.5f * wf && wf > 0.f;
+          sh.skip = rest >= 0.5 * ww && ww > 0.0;
         }
       });
-      const bool skip = sh.skip;
-      if (!skip) {   // second projection: w = w - V h1, h2 = V^T w, ||w||^2
+      if (!sh.skip) {   // second projection: w = w - V h1, h2 = V^T w, ||w||^2
         if (rows_warp) gm_reproject(sh, w, V, vs, ng, nt, k);
         // a thread's dots read the groups it wrote
         gm_dots(sh, w, V, vs, ng, nw, nt, k);
@@ -994,12 +997,15 @@ __global__ void __launch_bounds__(VS ? kGmBlockS : kGmBlock, 1) k_gm_fused(Offse
       // (2) v_{k+1} = w - V h, z = D^{-1} v_{k+1}, ||v_{k+1}||^2; meanwhile the scalar warp
       // rotates column k
       if (rows_warp) {
-        gm_complete(sh, w, V, vs, ng, nt, k, dinv + i0, z + i0, nrow, skip);
+        gm_complete(sh, w, V, vs, ng, nt, k, dinv + i0, z + i0, nrow);
       } else {
-        gm_rotate(sh, k, !skip);
+        gm_rotate(sh, k);
+        gm_second_norm(sh, k);
       }
-      gm_exchange(sh, skip ? 1 : 0, a, buf, value, [&]() {
-        if (skip && threadIdx.x == 0) sh.nrm2 = sh.tot[0];
+      __syncthreads();
+      const bool sum = sh.sum_norm;
+      gm_exchange(sh, sum ? 1 : 0, a, buf, value, [&]() {
+        if (sum && threadIdx.x == 0) sh.nrm2 = sh.tot[0];
       });
     }
     if (sh.done != 0) break;
@@ -1355,7 +1361,7 @@ __global__ void __launch_bounds__(VS ? kGmBlockS : kGmBlock, 1) k_gm_single(Offs
       }
       // (2) w -= V h and its norm (meanwhile the scalar warp rotates column k), v_{k+1} = w / ||w||
       if (rows_warp) project(k);
-      else gm_rotate(sh, k, false);
+      else gm_rotate(sh, k);
       __syncthreads();
       if (rows_warp) sh.col[threadIdx.x] = gs_norm(rw, w, ws, R, S, nwarp);
       gs_column(sh, nt);

@@ -48,7 +48,7 @@ __global__ void k_apply_dirichlet_g(int64_t N, const uint8_t* __restrict__ dir, 
 struct StepGraph {
   cudaGraphExec_t exec = nullptr;
   std::vector<unsigned char> key;
-  int64_t k_pro = 0, k_outer = 0, k_epi = 0;
+  int64_t k_pro = 0, k_first = 0, k_outer = 0, k_epi = 0;
   int kind = 0;   // 1 fixed point, 2 explicit SSP
   int unroll = 1; // corrections per turn of the while node
 };
@@ -59,7 +59,8 @@ namespace {
 // mixed, 942 corrections: 115.8 ms at one correction a turn, 114.0 at two, 112.6 at four); what
 // follows the stop in the same turn finds the status set and returns, but its residual has been
 // formed in vain.  So four for stationary solves, which take hundreds of corrections, and one for a
-// CN step's dozen (Q1 65^3: 8.23 ms at one, 8.37 at four).
+// CN step's dozen (Q1 65^3: 8.23 ms at one, 8.37 at four).  A loop of several begins with a residual
+// and a solve of its own: a solve that starts converged stops there (P1 129^3, mixed: 0.28 ms, 0.90 with four residuals).
 int unroll_of(int system) { return system == 0 ? 4 : 1; }
 
 std::vector<unsigned char> make_key(afc_problem_s* p, const afc_opts* o, int what) {
@@ -92,8 +93,9 @@ struct ProfOff {   // no event records inside captured graphs; captured launches
   }
 };
 
-// Build the fixed-point graph: prologue, while(outer){ residual; solve }, epilogue.  The
-// persistent solve decides first whether the loop goes on, and applies and counts the update.
+// Build the fixed-point graph: prologue, while(outer){ residual; solve }, epilogue (with several
+// corrections per turn, the first residual and solve before the loop).  The persistent solve decides
+// first whether the loop goes on, and applies and counts the update.
 template <class Pro, class Res>
 int build_fixed_point(afc_problem_s* p, const afc_opts* o, int system, Pro prologue, Res residual, StepGraph& sg,
                       KrylovEpilogue epi) {
@@ -125,23 +127,31 @@ int build_fixed_point(afc_problem_s* p, const afc_opts* o, int system, Pro prolo
       st = cuda_fail(cudaGetLastError(), "cudaGraphConditionalHandleCreate");
       break;
     }
-    cudaGraph_t body;
-    cudaGraphNode_t loop;
-    if ((st = add_conditional(g, fr, h_loop, cudaGraphCondTypeWhile, &body, &loop))) break;
-    std::vector<cudaGraphNode_t> bf;
     epi.fp_sc = p->scal.p;
     epi.part = p->part.p;
     epi.npart = (int)grid_for(p->N);
     epi.loop = h_loop;
     sg.unroll = unroll_of(system);
-    auto r2 = count([&]() -> int {
-      for (int c = 0; c < sg.unroll; ++c) {
-        int s = capture_into(p, cs, body, bf, residual, bf);
-        if (s) return s;
-        if ((s = krylov_graph(p, system, o, p->res.p, p->delta.p, cs, body, bf, &epi))) return s;
-      }
-      return AFC_OK;
-    });
+    auto corrections = [&](int n, cudaGraph_t into, std::vector<cudaGraphNode_t>& at) {
+      return count([&]() -> int {
+        for (int c = 0; c < n; ++c) {
+          int s = capture_into(p, cs, into, at, residual, at);
+          if (s) return s;
+          if ((s = krylov_graph(p, system, o, p->res.p, p->delta.p, cs, into, at, &epi))) return s;
+        }
+        return AFC_OK;
+      });
+    };
+    if (sg.unroll > 1) {
+      auto rf = corrections(1, g, fr);
+      if ((st = rf.first)) break;
+      sg.k_first = rf.second;
+    }
+    cudaGraph_t body;
+    cudaGraphNode_t loop;
+    if ((st = add_conditional(g, fr, h_loop, cudaGraphCondTypeWhile, &body, &loop))) break;
+    std::vector<cudaGraphNode_t> bf;
+    auto r2 = corrections(sg.unroll, body, bf);
     if ((st = r2.first)) break;
     sg.k_outer = r2.second;
     fr.assign(1, loop);
@@ -163,7 +173,8 @@ int run_fixed_point_graph(afc_problem_s* p, StepGraph& sg, afc_stats* stt) {
   AFC_CUDA(cudaStreamSynchronize(p->stream));
   const double* h = p->host_scal;
   const int64_t reval = (int64_t)h[F_REVAL], corr = (int64_t)h[F_CORR];
-  p->launches += sg.k_pro + (reval + sg.unroll - 1) / sg.unroll * sg.k_outer + sg.k_epi;
+  const int64_t looped = sg.k_first ? reval - 1 : reval;   // residuals of the loop
+  p->launches += sg.k_pro + sg.k_first + (looped + sg.unroll - 1) / sg.unroll * sg.k_outer + sg.k_epi;
   int status = h[F_STATUS] == 1.0 ? AFC_OK : h[F_STATUS] == 2.0 ? AFC_E_NAN : AFC_NOT_CONVERGED;
   if (h[F_TIMEOUT] != 0.0) {
     // the barrier counter is inconsistent after blocks skipped barriers: clear it so

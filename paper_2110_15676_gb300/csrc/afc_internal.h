@@ -186,7 +186,7 @@ struct afc_problem_s {
   bool maybe_captured = false;   // work that a caller may have captured and replays on other streams
   double u_lo = 0.0, u_hi = 0.0;
   double dir_lo = 1e308, dir_hi = -1e308;
-  // bounded-wait limit of the grid barriers in this problem's persistent launches
+  // bounded-wait limit of the grid barriers in this problem's persistent BiCGStab launches (the others: kBarrierWaitNs)
   unsigned long long grid_wait_ns = 4000000000ull;
   int64_t device_bytes = 0;
 };

@@ -423,7 +423,7 @@ int ssp_step_launch(afc_problem_s* p, const afc_opts* o) {
     AFC_LAUNCH(p, "k_ssp_step",
                e = cudaLaunchKernelEx(&cfg, k_ssp_step<KT, MX>, p->offs, arr, x, o->scheme == AFC_SSP2 ? 2 : 3,
                                       (int)o->limiter, o->dt, reinterpret_cast<GridBar*>(p->bar.p),
-                                      (unsigned long long)p->grid_wait_ns, p->range.p, p->host_scal));
+                                      kBarrierWaitNs, p->range.p, p->host_scal));
   };
   with_K(p->K, [&](auto kc) {
     if (o->precision == AFC_MIXED) run(kc, std::true_type{});

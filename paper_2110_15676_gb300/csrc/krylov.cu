@@ -1588,7 +1588,7 @@ int gmres_fused_launch(afc_problem_s* p, cudaStream_t s, const T* B, const T* di
   a.maxit = o->ksp_maxit;
   a.m = o->gmres_restart;
   if (epi) a.ep = *epi;
-  a.wait_ns = p->grid_wait_ns;
+  a.wait_ns = kBarrierWaitNs;   // afc_set_grid_wait_limit is of the BiCGStab launches
   constexpr bool kSingle = sizeof(T) == 4;
   const int64_t unit = kSingle ? kGsChunk : kGmUnit, units = (N + unit - 1) / unit;
   const int64_t least = kSingle ? 2 : 64 / kGmUnit;   // units of a block, at least

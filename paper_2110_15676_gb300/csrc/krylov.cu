@@ -1414,6 +1414,7 @@ void krylov_free(afc_problem_s* p) {
   p->kw->vec.free_();
   p->kw->sc.free_();
   p->kw->part.free_();
+  p->kw->barrier.free_();
   pinned_free(p->kw->hsc, kHscBytes);
   delete p->kw;
   p->kw = nullptr;

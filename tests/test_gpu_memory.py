@@ -1,0 +1,56 @@
+"""Device memory that the library gives back, in a process of its own (no other problem lives)."""
+import os
+import subprocess
+import sys
+
+import pytest
+
+pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+SCRIPT = """
+import sys
+import numpy as np
+import torch
+from paper_2110_15676_gb300 import afc, workloads as W
+
+ksp = afc.AFC_KSP_GMRES if sys.argv[1] == "gmres" else afc.AFC_KSP_BICGSTAB
+
+
+def solved(n):
+    ix, iy, iz = W.grid_index(n)
+    N = len(ix)
+    mask = ((ix == 0) | (iy == n[1] - 1) | (iz == 0)).astype(np.uint8)
+    g = afc.Problem.structured("q1", n)
+    g.set_coefficients(1e-3, np.array([1.0, -0.5, 0.25]), 1.0, np.ones(N))
+    g.set_dirichlet(mask, np.zeros(N))
+    g.assemble(afc.AFC_FAMILY_MC, afc.AFC_MIXED)
+    g.set_solution(np.zeros(N))
+    g.solve_stationary(afc.default_opts(limiter=afc.AFC_LIM_MC, fp_fixed_its=2, ksp=ksp, ksp_atol=0.0, ksp_rtol=1e-2,
+                                        precision=afc.AFC_MIXED))
+    return g
+
+
+def free():
+    torch.cuda.synchronize()
+    return torch.cuda.mem_get_info()[0]
+
+
+solved((5, 4, 4)).close()   # what the process and its modules take for good
+before = free()
+g = solved((81, 81, 81))
+held = before - free()
+g.close()
+print(held, before - free())
+"""
+
+
+@pytest.mark.parametrize("ksp", ["gmres", "bicgstab"])
+def test_memory_after_the_last_problem(ksp):
+    """A problem of more than 1 GiB, solved and freed: at most 1 GiB stays (nothing of it is still
+    allocated, its solver's workspace included)."""
+    r = subprocess.run([sys.executable, "-c", SCRIPT, ksp], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
+    held, kept = map(int, r.stdout.split())
+    assert held > (5 << 28)
+    assert kept <= (1 << 30)

@@ -144,6 +144,13 @@ int afc_create_from_elements(int elem, int64_t n_nodes, const double* xyz, int64
 
 int afc_destroy(afc_problem p);
 
+/* Device memory comes from a pool of the library's own on each device.  Of what problems and
+ * batches free, the pool keeps up to 2 GiB for the next ones while any problem, batch or server
+ * lives, and nothing once none does.  afc_trim_memory gives what it keeps on `device` back to the
+ * device now (to other allocators of the process, for example); the memory of problems and
+ * batches that live is not touched.  AFC_E_CUDA if the device does not exist. */
+int afc_trim_memory(int device);
+
 /* ---- data --------------------------------------------------------------------- */
 
 /* Coefficients of Eq. tcdr / Eq. cdr (host arrays):

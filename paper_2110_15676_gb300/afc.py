@@ -99,6 +99,7 @@ _SIGS = {
     "afc_create_structured": (C.c_int, [C.c_int, C.c_int, C.c_int, C.c_int, _D, _D, C.c_int, _P, C.POINTER(_P)]),
     "afc_create_from_elements": (C.c_int, [C.c_int, C.c_int64, _D, C.c_int64, _I32, C.c_int, _P, C.POINTER(_P)]),
     "afc_destroy": (C.c_int, [_P]),
+    "afc_trim_memory": (C.c_int, [C.c_int]),
     "afc_set_coefficients": (C.c_int, [_P, C.c_double, _D, _D, _D, C.c_double, _D]),
     "afc_set_dirichlet": (C.c_int, [_P, _U8, _D]),
     "afc_assemble": (C.c_int, [_P, C.c_int, C.c_int]),
@@ -212,6 +213,11 @@ def selftest_split(x, device: int = 0):
     _check(_lib.afc_selftest_split(int(device), _dp(a), n, hi.ctypes.data_as(fp), lo.ctypes.data_as(fp), _dp(back)),
            "afc_selftest_split")
     return hi, lo, back
+
+
+def trim_memory(device: int = 0) -> None:
+    """Give the free memory that the library's pool keeps on a device back to the device."""
+    _check(_lib.afc_trim_memory(int(device)), "afc_trim_memory")
 
 
 def selftest_grid_wait(limit_ms: float = 50.0, device: int = 0) -> tuple[int, float]:

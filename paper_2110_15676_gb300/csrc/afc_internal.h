@@ -63,6 +63,8 @@ int build_from_elements(int elem, int64_t n_nodes, const double* xyz, int64_t n_
 // free it when the work that uses it has finished (freeing does not wait for the device).
 cudaError_t device_alloc(void** ptr, size_t bytes, bool zero = false);
 void device_free(void* ptr);
+void device_hold(int device, bool on);   // a server lives: its requests reuse each other's memory
+cudaError_t device_trim(int device);   // give the pool's free memory back
 cudaError_t pinned_alloc(void** ptr, size_t bytes);
 void pinned_free(void* ptr, size_t bytes);
 

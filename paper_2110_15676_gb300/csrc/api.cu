@@ -271,6 +271,16 @@ int afc_destroy(afc_problem p) {
   return AFC_OK;
 }
 
+int afc_trim_memory(int device) {
+  int now = 0;
+  AFC_CUDA(cudaGetDevice(&now));
+  if (now != device) AFC_CUDA(cudaSetDevice(device));
+  const cudaError_t e = device_trim(device);
+  if (now != device) cudaSetDevice(now);
+  if (e != cudaSuccess) return cuda_fail(e, "afc_trim_memory");
+  return AFC_OK;
+}
+
 int afc_set_coefficients(afc_problem p, double eps, const double* b_nodal, const double b_const[3],
                          const double* c_nodal, double c_const, const double* f_nodal) {
   int st = check(p, false);

@@ -11,8 +11,9 @@
 // caller frees memory only when the work that uses it has finished (it has synchronised the
 // streams that it was used on).  The runtime orders a reuse on another thread's stream after the
 // free.
-// Bounds.  The pool keeps at most kKeepBytes of free memory while problems live, and kIdleBytes
-// once none does; the pinned lists keep at most kKeepBlocks blocks each.
+// Bounds.  The pool keeps at most kKeepBytes of free memory while problems, batches or servers live (a
+// burst of eight served requests of 17 to 33 nodes a side holds 0.75 GB) and none once none does;
+// afc_trim_memory gives it back at any time.  The pinned lists keep at most kKeepBlocks blocks each.
 #include <cstdint>
 #include <mutex>
 #include <vector>
@@ -24,14 +25,13 @@ namespace afc {
 namespace {
 
 constexpr int kMaxDevices = 64;
-constexpr uint64_t kKeepBytes = (uint64_t)8 << 30;
-constexpr size_t kIdleBytes = (size_t)1 << 30;
+constexpr uint64_t kKeepBytes = (uint64_t)2 << 30;
 constexpr size_t kBlockBytes[2] = {4096, 65536};   // scalars of a problem; tables of a batch
 constexpr size_t kKeepBlocks[2] = {256, 32};
 
 std::mutex g_mu;
 cudaMemPool_t g_pool[kMaxDevices] = {};
-int64_t g_live[kMaxDevices] = {};        // allocations not freed
+int64_t g_live[kMaxDevices] = {};        // allocations not freed, and holders
 std::vector<void*> g_blocks[2];          // free pinned blocks
 
 cudaError_t pool_of(int device, cudaMemPool_t* out) {   // with g_mu held
@@ -86,15 +86,10 @@ cudaError_t device_alloc(void** ptr, size_t bytes, bool zero) {
   return e;
 }
 
-void device_free(void* ptr) {
-  if (!ptr) return;
-  cudaPointerAttributes at = {};
-  int device = 0, now = 0;
-  if (cudaPointerGetAttributes(&at, ptr) == cudaSuccess) device = at.device;
-  else cudaGetDevice(&device);
-  cudaGetDevice(&now);
-  if (now != device) cudaSetDevice(device);
-  cudaFreeAsync(ptr, cudaStreamPerThread);
+namespace {
+
+// One allocation or holder less on `device`, which is current; the last one trims the pool.
+void drop(int device) {
   bool idle = false;
   cudaMemPool_t pool = nullptr;
   {
@@ -106,9 +101,50 @@ void device_free(void* ptr) {
   }
   if (idle && pool) {
     cudaStreamSynchronize(cudaStreamPerThread);
-    cudaMemPoolTrimTo(pool, kIdleBytes);
+    cudaMemPoolTrimTo(pool, 0);
   }
+}
+
+}  // namespace
+
+void device_free(void* ptr) {
+  if (!ptr) return;
+  cudaPointerAttributes at = {};
+  int device = 0, now = 0;
+  if (cudaPointerGetAttributes(&at, ptr) == cudaSuccess) device = at.device;
+  else cudaGetDevice(&device);
+  cudaGetDevice(&now);
+  if (now != device) cudaSetDevice(device);
+  cudaFreeAsync(ptr, cudaStreamPerThread);
+  drop(device);
   if (now != device) cudaSetDevice(now);
+}
+
+void device_hold(int device, bool on) {
+  if (device < 0 || device >= kMaxDevices) return;
+  if (on) {
+    std::lock_guard<std::mutex> lk(g_mu);
+    ++g_live[device];
+    return;
+  }
+  int now = 0;
+  cudaGetDevice(&now);
+  if (now != device) cudaSetDevice(device);
+  drop(device);
+  if (now != device) cudaSetDevice(now);
+}
+
+cudaError_t device_trim(int device) {
+  cudaMemPool_t pool = nullptr;
+  {
+    std::lock_guard<std::mutex> lk(g_mu);
+    if (device < 0 || device >= kMaxDevices) return cudaErrorInvalidDevice;
+    pool = g_pool[device];
+  }
+  if (!pool) return cudaSuccess;   // nothing was allocated there yet
+  // what other threads freed is free once their frees have run: wait for this thread's alone
+  const cudaError_t e = cudaStreamSynchronize(cudaStreamPerThread);
+  return e != cudaSuccess ? e : cudaMemPoolTrimTo(pool, 0);
 }
 
 // Pinned host memory in blocks of two sizes from the lists (larger: from the runtime).

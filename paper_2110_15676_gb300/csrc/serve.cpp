@@ -460,6 +460,7 @@ extern "C" int afc_serve_create(int device, const afc_serve_config* cfg, afc_ser
   s->cfg = c;
   s->device = device;
   s->t0 = Clock::now();
+  device_hold(device, true);
   if (c.mode == AFC_SERVE_SERIAL) {
     s->threads.emplace_back(serial_loop, s);
   } else {
@@ -602,6 +603,7 @@ extern "C" int afc_serve_destroy(afc_server s) {
   // admitted requests the threads did not reach
   for (auto& r : s->arrivals) finish(s, r, AFC_REQ_CANCELLED, AFC_OK);
   for (auto& r : s->stat_queue) finish(s, r, AFC_REQ_CANCELLED, AFC_OK);
+  device_hold(s->device, false);
   delete s;
   return AFC_OK;
 }

@@ -710,9 +710,11 @@ extern "C" int afc_batch_step(afc_batch b, const afc_opts* o, const double* dt, 
   if (nsteps < 0) { set_error("nsteps must be >= 0"); return AFC_E_INVALID; }
   if (cudaSetDevice(b->device) != cudaSuccess) return cuda_fail(cudaGetLastError(), "cudaSetDevice");
   const afc_batch_tuning t = effective_tuning(b, o);
-  if ((st = batch_input_ranges(b, t.block, dt, o))) return st;
-  if ((st = run_steps(b, o, dt, nsteps, t))) return st;
-  return batch_status(b, stats, nsteps * (o->scheme == AFC_SSP2 ? 2 : 3));
+  if (!(st = batch_input_ranges(b, t.block, dt, o)) && !(st = run_steps(b, o, dt, nsteps, t)))
+    st = batch_status(b, stats, nsteps * (o->scheme == AFC_SSP2 ? 2 : 3));
+  // after an error steps may still be under way, on instances that the caller may free now
+  if (st) cudaStreamSynchronize(b->stream);
+  return st;
 }
 
 extern "C" int afc_batch_set_tuning(afc_batch b, const afc_batch_tuning* t) {
@@ -799,8 +801,10 @@ extern "C" int afc_batch_tune(afc_batch b, const afc_opts* o, const double* dt, 
   cudaEventDestroy(e1);
   int st2 = copy_all(false);
   for (auto* p : b->list) p->u_range_valid = false;   // the trials' ranges are not the restored states'
-  if (st) return st;
-  if (st2) return st2;
+  if (st || st2) {   // as in afc_batch_step
+    cudaStreamSynchronize(s);
+    return st ? st : st2;
+  }
   AFC_CUDA(cudaStreamSynchronize(s));
   b->tuning = win;
   b->fixed = true;

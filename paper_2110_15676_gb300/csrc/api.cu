@@ -107,11 +107,7 @@ void destroy_all(afc_problem_s* p) {
   if (!p) return;
   cudaSetDevice(p->device);
   cudaStreamSynchronize(p->stream);   // the legacy default stream too: freeing does not wait
-  if (p->maybe_captured) {   // a caller's graph may run on any stream: cudaFree waits for all
-    void* w = nullptr;
-    if (cudaMalloc(&w, 1) == cudaSuccess) cudaFree(w);
-    else cudaGetLastError();
-  }
+  if (p->maybe_captured) cudaDeviceSynchronize();   // a caller's graph may run on any stream
   graph_free(p);
   prof_free(p);
   krylov_free(p);

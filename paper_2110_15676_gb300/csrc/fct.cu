@@ -26,7 +26,8 @@ namespace {
 // and waits for the one before it (which has waited for its own predecessor) before it
 // touches anything a pass writes.  On larger grids the waiting blocks take the place of
 // running ones (SSP3 step in double, us, with / without: P1 9^3 62 / 68, Q1 17^3 81 / 86, Q1 25^3
-// 84 / 86, Q1 33^3 113 / 90, Q1 41^3 179 / 117).
+// 84 / 86, Q1 33^3 113 / 90, Q1 41^3 179 / 117).  With graph = 1 these sizes take the one-launch step
+// (k_ssp_step) instead, so that this serves host-driven steps.
 constexpr int64_t kPdlRows = 16384;
 constexpr int64_t kStepRows = 16384;   // the graph form's one-launch step (k_ssp_step)
 

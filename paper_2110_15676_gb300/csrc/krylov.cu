@@ -7,7 +7,9 @@
 // not depend on scheduling.
 //
 // Vector type T is double (FP64) or float (the FP32 inner solve of the mixed
-// mode, with FP32 matrix values).  Partial sums are always double.
+// mode, with FP32 matrix values).  What a thread adds over its rows is in T; everything from there on
+// is in double, but for the dots of single-precision GMRES, which are added in single precision in
+// a defined order up to 256 values (k_gm_single).
 #include <climits>
 #include <cmath>
 #include <cstring>
@@ -476,17 +478,17 @@ __global__ void __launch_bounds__(kFusedBlock, 1) k_bicg_fused(Offsets of, const
 // was bound by launches: five per Arnoldi step (7 to 21 us each on P1 49^3 to 129^3
 // for 1 to 10 us of traffic), and a captured cycle ran all m = 20 steps although the
 // stationary solves stop after 5 to 10 of them (the rest returned at once, but were
-// launched).  Here a step is two grid-wide sums (barriers), and a solve stops where it
-// stops.  Measured on one GB300, whole stationary MC solves (omega = 0.5, inner rtol 1e-2),
-// against the launches per pass: Q1 27x21x33 in double 301 -> 63 ms, P1 49^3 mixed 470 ->
-// 111 ms, P1 129^3 mixed 1.70 -> 0.95 s; the same iteration counts.  Per Arnoldi step (P1 49^3 /
-// 129^3): product 1.7 / 25 us, dots 0.8 / 10, sums 2.9 / 5, second projection 3.7 / 20 (when
-// taken), completion 1.3 / 13, barrier 1.5 / 3.
+// launched).  Here a step is two or three grid-wide sums, and a solve stops where it stops.
+// Measured on one GB300 against the launches per pass, a stationary MC solve (omega = 0.5, inner
+// rtol 1e-2) of Q1 27x21x33 in double: 289 -> 59 ms, the same iteration counts.  The second
+// projection is taken in nearly all steps (3431 of 3441 there): with the Jacobi preconditioner
+// B D^{-1} has a unit diagonal, so that w is mostly v_k.  The single-precision solve has a kernel of
+// its own below (k_gm_single).
 //
 // Layout.  Block b owns a contiguous range of rows (a multiple of 32) for every pass, so
 // everything but the product's gather of z is local to a block:
 //  * w (the new direction) stays in shared memory between the passes of a step, and so
-//    do the basis vectors where all m + 1 of a block fit (P1 65^3 in single precision);
+//    do the basis vectors where all m + 1 of a block fit (up to 928 rows a block at m = 20);
 //    otherwise they are in global memory, read 16 bytes per load, four vectors at a
 //    time, each once per pass;
 //  * the basis vectors are stored unnormalised with their scale 1 / ||v_q|| beside them
@@ -505,7 +507,8 @@ __global__ void __launch_bounds__(kFusedBlock, 1) k_bicg_fused(Offsets of, const
 //      DGKS test: if ||w - V h1||^2 = ||w||^2 - ||h1||^2 >= ||w||^2 / 2 little of w lay in
 //      the basis and a second projection would change nothing worth keeping;
 //      otherwise w -= V h1, h2 = V^T w, ||w||^2                      -> grid sums
-//  (2) v_{k+1} = w - V h, z = D^{-1} v_{k+1}, ||v_{k+1}||^2          -> grid sum (or barrier)
+//  (2) v_{k+1} = w - V h, z = D^{-1} v_{k+1}, ||v_{k+1}||^2          -> grid sum, or a barrier
+//      (gm_second_norm)
 //      Hessenberg column, rotations, |g[k+1]|, the end-of-cycle test.
 // Threads of a block, at most: with the basis in shared memory (few rows: 96 registers keep
 // more of a row's loads in flight), and in global memory (64 registers).
@@ -841,8 +844,9 @@ __device__ __forceinline__ void gm_triangle(GmScalars& sh, int ku) {
 // w = B z over a block's rows (B, z, w at the block's first row).  The row's addresses are
 // formed inside the loop, from a stride and a base the compiler cannot see through: hoisted
 // out of it they took 4 K registers, and the row's 2 K loads went out a few at a time.
-// STREAM: the matrix goes past L2 (evict first), which the basis vectors then keep (P1 129^3 in
-// single precision: product 26.8 -> 24.9 us, dots 13.9 -> 10.4 us).
+// STREAM: the matrix goes past L2 (evict first), which the basis vectors then keep (measured at
+// P1 129^3 in single precision with the rows of a block in one range: product 26.8 -> 24.9 us, dots
+// 13.9 -> 10.4 us).
 template <int KT, bool STREAM, class T>
 __device__ __forceinline__ void gm_product(const Offsets& of, int64_t N, const T* __restrict__ B, const T* z, T* w,
                                            int nrow, int nt) {
@@ -1039,7 +1043,8 @@ __global__ void __launch_bounds__(VS ? kGmBlockS : kGmBlock, 1) k_gm_fused(Offse
 // The same method and launch, but with every single-precision rounding in a fixed place.  The
 // damped iteration around a mixed solve amplifies the rounding of its inner solver at isolated
 // nodes: with the dots added in another order and the basis unnormalised, whole stationary solves
-// moved by up to 2e-8 (P1 129^3, the same number of corrections and the same residual).  So here
+// moved by 2e-12 to 2e-8 (P1 49^3 and 129^3, the same number of corrections and the same residual).
+// So here
 //  * the basis vectors are normalised and rounded once, v_k = w (1 / ||w||), z = D^{-1} v_k;
 //  * a dot is formed by single-precision strands: rows come in chunks of 256, chunk c adds to strand
 //    set c mod (gm_strand_sets * SMs), each of whose 256 strands takes its rows in ascending order by
@@ -1050,6 +1055,10 @@ __global__ void __launch_bounds__(VS ? kGmBlockS : kGmBlock, 1) k_gm_fused(Offse
 //    double across strands, those of the true residual in double from the first addition.
 // gm_strand_sets (per SM) is part of that definition: a result depends on it, and on the device's
 // SM count, but not on scheduling or on where the vectors are kept.
+// The norm needs a grid-wide sum of its own and z a barrier after it: a step is three sums and a
+// barrier where the kernel above takes two and a barrier.  Measured on one GB300 (a kernel per pass ->
+// unnormalised in this kernel's place -> this kernel): stationary P1 49^3 511 -> 101 -> 152 ms, 129^3
+// 1.75 -> 0.82 -> 1.01 s, a burst of 8 served requests 911 -> 74 -> 98 ms.
 //
 // Block b owns chunks b, b + G, b + 2 G, ... (G blocks; G = SMs, or fewer when each has at most two
 // chunks): the chunks of a strand set are then all in one block, for every number of sets, so that
@@ -1566,10 +1575,10 @@ int bicgstab_impl(afc_problem_s* p, const T* B, const T* dinv, const afc_opts* o
 
 // The persistent GMRES launch on stream s (no synchronisation).  One block per SM at most.  In
 // double small systems spread over all SMs, 64 rows a block, because a block's FP64 sums cost
-// 16 cycles per warp.  In single precision a block takes at least 512 rows: a solve of a few
-// thousand rows is as fast on 16 SMs as on 125 (P1 17^3 to Q1 33^3: within 1 %), and solves on other
-// streams find room beside it (a burst of 8 served requests, four of them stationary: 108 -> 76
-// ms).
+// 16 cycles per warp.  In single precision a block takes two chunks (512 rows) where there are SMs
+// enough: solves on other streams find room beside it, at no cost to a solve alone (measured with
+// at least 512 rows a block against 64: a burst of 8 served requests 108 -> 76 ms, P1 17^3 to Q1 33^3
+// within 1 %).
 template <class T>
 int gmres_fused_launch(afc_problem_s* p, cudaStream_t s, const T* B, const T* dinv, const afc_opts* o,
                        const double* rhs, double* xout, const KrylovEpilogue* epi) {

@@ -109,3 +109,22 @@ def test_cn_sums_are_rounded_once(afc, elem):
             assert got[k][i] == want, (i, k)
             decided += want < 1.0
     assert decided > N // 4
+
+
+@pytest.mark.parametrize("elem", ["p1", "q1"])
+def test_explicit_factors_of_a_nan_flux(afc, elem):
+    """One node is NaN.  Its neighbours' rates and predictors are NaN; a free row that is no neighbour
+    of it but has one of a lower index has a finite predictor, a finite Q- (NaN sorts as a maximum) and
+    a NaN flux with the sign bit set (the negative of the pair's): its P- and so its R- are NaN."""
+    n, b, mask, u, prob = _field(elem, 1.0, 1.0)
+    centre = np.ravel_multi_index((5, 5, 5), (n[2], n[1], n[0]))
+    u[centre] = np.nan
+    g = _problem(afc, elem, n, b, mask, u)
+    got = g.fe_stage(0.5 * O.cfl_timestep(prob, 1.0))
+    rowptr, col, _ = g.export_csr(afc.AFC_MAT_MC)
+    near = [set(col[rowptr[i]:rowptr[i + 1]]) for i in range(len(mask))]
+    ring = {j for j in near[centre] if mask[j] == 0}
+    rows = [i for i in range(len(mask)) if mask[i] == 0 and i not in near[centre] and any(j < i for j in near[i] & ring)]
+    assert len(rows) >= 20
+    assert np.isfinite(got["u_tilde"][rows]).all()
+    assert np.isnan(got["Rm"][rows]).all()

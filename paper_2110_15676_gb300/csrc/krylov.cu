@@ -217,8 +217,9 @@ struct BicgShared {
 // quarters, stores the block's partial and arrives.  end: that lane polls, warp 0 adds the
 // partials of all blocks in block order (all blocks run the same operations on the same
 // partials, so all obtain the same bits) and its first lane runs take(totals, ok).  The partials
-// alternate between two buffers (a block can run at most one sum ahead of another).
-template <int NV, class T>
+// alternate between two buffers (a block can run at most one sum ahead of another).  TURN: one warp
+// adds a block's columns, and a lane its partials, one after the other.
+template <int NV, bool TURN, class T>
 __device__ __forceinline__ unsigned int bicg_sums_begin(BicgShared<T>& sh, const double (&v)[NV], double* part, int buf,
                                                         GridBar* bar) {
   const int G = gridDim.x, nt = blockDim.x;
@@ -229,7 +230,10 @@ __device__ __forceinline__ unsigned int bicg_sums_begin(BicgShared<T>& sh, const
   for (int u = w; u < 4 * NV; u += nt >> 5) {
     const double* c = sh.col[u >> 2];
     double t = 0.0;
-    for (int j = (u & 3) * 32 + lane; j < nt; j += 128) t += c[j];
+    if (!TURN)
+      for (int j = (u & 3) * 32 + lane; j < nt; j += 128) t += c[j];
+    else if ((u & 3) == 0)   // the other quarters are 0
+      for (int j = lane; j < nt; j += 32) t += c[j];
     t = warp_sum(t);
     if (lane == 0) sh.quarter[u >> 2][u & 3] = t;
   }
@@ -245,7 +249,7 @@ __device__ __forceinline__ unsigned int bicg_sums_begin(BicgShared<T>& sh, const
   return old;
 }
 
-template <int NV, class F>
+template <int NV, bool TURN, class F>
 __device__ __forceinline__ void bicg_sums_end(const double* part, int& buf, GridBar* bar, unsigned int old,
                                               unsigned long long wait_ns, F&& take) {
   const int G = gridDim.x, lane = threadIdx.x & 31;
@@ -261,7 +265,7 @@ __device__ __forceinline__ void bicg_sums_end(const double* part, int& buf, Grid
         double x[5];
 #pragma unroll
         for (int u = 0; u < 5; ++u) x[u] = b0 + 32 * u < G ? __ldcg(pb + b0 + 32 * u) : 0.0;
-        t[q] += ((x[0] + x[1]) + (x[2] + x[3])) + x[4];
+        t[q] = TURN ? ((((t[q] + x[0]) + x[1]) + x[2]) + x[3]) + x[4] : t[q] + (((x[0] + x[1]) + (x[2] + x[3])) + x[4]);
       }
     }
 #pragma unroll
@@ -300,8 +304,8 @@ __device__ __forceinline__ void krylov_count(const KrylovEpilogue& ep, int its, 
   if (berr) f[F_TIMEOUT] = 1.0;
 }
 
-// SM: the six vectors in shared memory.
-template <int KT, class T, bool SM>
+// SM: the six vectors in shared memory.  TURN: the sums in one order (bicg_fused_launch).
+template <int KT, class T, bool SM, bool TURN>
 __global__ void __launch_bounds__(kFusedBlock, 1) k_bicg_fused(Offsets of, const T* __restrict__ B,
                                                                const T* __restrict__ dinv, T* ph, T* sg,
                                                                BicgArgs<T> a) {
@@ -346,8 +350,8 @@ __global__ void __launch_bounds__(kFusedBlock, 1) k_bicg_fused(Offsets of, const
     a0 = fma(ri, ri, a0);
   }
   a1[0] = to_dbl(a0);
-  unsigned int old = bicg_sums_begin<1>(sh, a1, a.part, buf, a.bar);
-  bicg_sums_end<1>(a.part, buf, a.bar, old, a.wait_ns, [&](const double (&s)[1], bool ok) {
+  unsigned int old = bicg_sums_begin<1, TURN>(sh, a1, a.part, buf, a.bar);
+  bicg_sums_end<1, TURN>(a.part, buf, a.bar, old, a.wait_ns, [&](const double (&s)[1], bool ok) {
     sh.rho = s[0];
     sh.n0 = sh.nres = sqrt(s[0]);
     sh.tol = fmax(a.atol, a.rtol * sh.n0);
@@ -374,8 +378,8 @@ __global__ void __launch_bounds__(kFusedBlock, 1) k_bicg_fused(Offsets of, const
       a0 = fma(rh[q], y, a0);
     }
     a1[0] = to_dbl(a0);
-    old = bicg_sums_begin<1>(sh, a1, a.part, buf, a.bar);
-    bicg_sums_end<1>(a.part, buf, a.bar, old, a.wait_ns, [&](const double (&s)[1], bool ok) {
+    old = bicg_sums_begin<1, TURN>(sh, a1, a.part, buf, a.bar);
+    bicg_sums_end<1, TURN>(a.part, buf, a.bar, old, a.wait_ns, [&](const double (&s)[1], bool ok) {
       sh.alpha = sh.rho / s[0];
       sh.ta = (T)sh.alpha;
       if (!isfinite(sh.alpha) || s[0] == 0.0 || !ok) sh.done = 2;
@@ -391,8 +395,8 @@ __global__ void __launch_bounds__(kFusedBlock, 1) k_bicg_fused(Offsets of, const
       a0 = fma(si, si, a0);
     }
     a1[0] = to_dbl(a0);
-    old = bicg_sums_begin<1>(sh, a1, a.part, buf, a.bar);
-    bicg_sums_end<1>(a.part, buf, a.bar, old, a.wait_ns, [&](const double (&s)[1], bool ok) {
+    old = bicg_sums_begin<1, TURN>(sh, a1, a.part, buf, a.bar);
+    bicg_sums_end<1, TURN>(a.part, buf, a.bar, old, a.wait_ns, [&](const double (&s)[1], bool ok) {
       const double ns = sqrt(s[0]);
       if (!isfinite(ns) || !ok) {
         sh.done = 2;
@@ -413,8 +417,8 @@ __global__ void __launch_bounds__(kFusedBlock, 1) k_bicg_fused(Offsets of, const
     }
     a2[0] = to_dbl(b0);
     a2[1] = to_dbl(b1);
-    old = bicg_sums_begin<2>(sh, a2, a.part, buf, a.bar);
-    bicg_sums_end<2>(a.part, buf, a.bar, old, a.wait_ns, [&](const double (&s)[2], bool ok) {
+    old = bicg_sums_begin<2, TURN>(sh, a2, a.part, buf, a.bar);
+    bicg_sums_end<2, TURN>(a.part, buf, a.bar, old, a.wait_ns, [&](const double (&s)[2], bool ok) {
       sh.omega = s[0] / s[1];
       sh.to = (T)sh.omega;
       if (!isfinite(sh.omega) || s[1] == 0.0 || !ok) sh.done = 2;
@@ -433,9 +437,9 @@ __global__ void __launch_bounds__(kFusedBlock, 1) k_bicg_fused(Offsets of, const
     }
     a2[0] = to_dbl(b0);
     a2[1] = to_dbl(b1);
-    old = bicg_sums_begin<2>(sh, a2, a.part, buf, a.bar);
+    old = bicg_sums_begin<2, TURN>(sh, a2, a.part, buf, a.bar);
     for (int q = tid; q < nrow; q += nt) x[q] = x[q] + ta * ph[q] + tom * sg[q];
-    bicg_sums_end<2>(a.part, buf, a.bar, old, a.wait_ns, [&](const double (&s)[2], bool ok) {
+    bicg_sums_end<2, TURN>(a.part, buf, a.bar, old, a.wait_ns, [&](const double (&s)[2], bool ok) {
       const double nr = sqrt(s[0]), rho_old = sh.rho;
       sh.nres = nr;
       sh.rho = s[1];
@@ -1486,7 +1490,7 @@ T* vec_at(KrylovWork& w, int q) {
 
 // The persistent BiCGStab launch on stream s (no synchronisation).
 template <class T>
-int bicg_fused_launch(afc_problem_s* p, cudaStream_t s, const T* B, const T* dinv, const afc_opts* o,
+int bicg_fused_launch(afc_problem_s* p, cudaStream_t s, int system, const T* B, const T* dinv, const afc_opts* o,
                       const double* rhs, double* xout, const KrylovEpilogue* epi) {
   KrylovWork& w = *p->kw;
   int st = coop_device(p);
@@ -1508,16 +1512,23 @@ int bicg_fused_launch(afc_problem_s* p, cudaStream_t s, const T* B, const T* din
   a.wait_ns = p->grid_wait_ns;
   const int G = (int)std::max<int64_t>(1, std::min<int64_t>((N + 63) / 64, w.nsm));
   const int64_t rows = (N + G - 1) / G;
-  // as many threads as share the rows evenly in the fewest rounds
   const int64_t rounds = (rows + kFusedBlock - 1) / kFusedBlock;
-  const int block = (int)std::max<int64_t>(64, ((rows + rounds - 1) / rounds + 31) / 32 * 32);
+  // A mixed stationary solve amplifies the rounding of its inner solver at isolated nodes (with other
+  // sums P1 57^3 moved by up to 6e-10): from several rows a thread on, the sums of its solver have
+  // one order, every 512th row of a block to a thread and the partials in turn.  Elsewhere as many
+  // threads as share the rows evenly in the fewest rounds, and quarters of the columns (a CN step of
+  // Q1 65^3 with single-precision solves is 3 % faster for it).
+  const bool turn = sizeof(T) == 4 && system == 0 && rounds > 1;
+  const int block = turn ? kFusedBlock : (int)std::max<int64_t>(64, ((rows + rounds - 1) / rounds + 31) / 32 * 32);
   a.rows = (int)rows;
   const size_t local = 6 * (size_t)rows * sizeof(T);
   const bool in_smem = local <= kFusedSmem;
   const size_t smem = in_smem ? local : 0;
   with_K(p->K, [&](auto kc) {
     constexpr int KT = decltype(kc)::value;
-    auto kern = in_smem ? k_bicg_fused<KT, T, true> : k_bicg_fused<KT, T, false>;
+    auto kern = in_smem ? k_bicg_fused<KT, T, true, false> : k_bicg_fused<KT, T, false, false>;
+    if constexpr (sizeof(T) == 4)
+      if (turn) kern = in_smem ? k_bicg_fused<KT, T, true, true> : k_bicg_fused<KT, T, false, true>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFusedSmem);
     int nb = 0;
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, block, smem);
@@ -1565,11 +1576,11 @@ int fused_result(afc_problem_s* p, const char* what, int* its, double* res) {
 }
 
 template <class T>
-int bicgstab_impl(afc_problem_s* p, const T* B, const T* dinv, const afc_opts* o, const double* rhs, double* xout,
+int bicgstab_impl(afc_problem_s* p, int system, const T* B, const T* dinv, const afc_opts* o, const double* rhs, double* xout,
                   int* its, double* res, const KrylovEpilogue* epi) {
   int st = ensure_work(p, kBicgVectors, sizeof(T) == 4);
   if (st) return st;
-  if ((st = bicg_fused_launch<T>(p, p->stream, B, dinv, o, rhs, xout, epi))) return st;
+  if ((st = bicg_fused_launch<T>(p, p->stream, system, B, dinv, o, rhs, xout, epi))) return st;
   return fused_result(p, "BiCGStab", its, res);
 }
 
@@ -1664,12 +1675,12 @@ int gmres_impl(afc_problem_s* p, const T* B, const T* dinv, const afc_opts* o, c
 namespace {
 
 template <class T>
-int bicgstab_graph(afc_problem_s* p, const T* B, const T* dinv, const afc_opts* o, const double* rhs, double* xout,
+int bicgstab_graph(afc_problem_s* p, int system, const T* B, const T* dinv, const afc_opts* o, const double* rhs, double* xout,
                    cudaStream_t cs, cudaGraph_t g, std::vector<cudaGraphNode_t>& frontier, const KrylovEpilogue* epi) {
   int st = ensure_work(p, kBicgVectors, sizeof(T) == 4);
   if (st) return st;
   return capture_into(p, cs, g, frontier, [&]() -> int {
-    return bicg_fused_launch<T>(p, p->stream, B, dinv, o, rhs, xout, epi);
+    return bicg_fused_launch<T>(p, p->stream, system, B, dinv, o, rhs, xout, epi);
   }, frontier);
 }
 
@@ -1701,12 +1712,12 @@ int krylov_graph(afc_problem_s* p, int system, const afc_opts* o, const double* 
     const float* B = system == 0 ? p->Bst32.p : p->Bcn32.p;
     const float* di = system == 0 ? p->dinv_st32.p : p->dinv_cn32.p;
     return gm ? gmres_graph<float>(p, B, di, o, rhs, x, cs, g, frontier, epi)
-              : bicgstab_graph<float>(p, B, di, o, rhs, x, cs, g, frontier, epi);
+              : bicgstab_graph<float>(p, system, B, di, o, rhs, x, cs, g, frontier, epi);
   }
   const double* B = system == 0 ? p->Bst.p : p->Bcn.p;
   const double* di = system == 0 ? p->dinv_st.p : p->dinv_cn.p;
   return gm ? gmres_graph<double>(p, B, di, o, rhs, x, cs, g, frontier, epi)
-            : bicgstab_graph<double>(p, B, di, o, rhs, x, cs, g, frontier, epi);
+            : bicgstab_graph<double>(p, system, B, di, o, rhs, x, cs, g, frontier, epi);
 }
 
 int krylov_reset_barrier(afc_problem_s* p) {
@@ -1730,12 +1741,12 @@ int krylov_solve(afc_problem_s* p, int system, const afc_opts* o, const double* 
     const float* B = system == 0 ? p->Bst32.p : p->Bcn32.p;
     const float* di = system == 0 ? p->dinv_st32.p : p->dinv_cn32.p;
     return gm ? gmres_impl<float>(p, B, di, o, rhs, x, its, res, epi)
-              : bicgstab_impl<float>(p, B, di, o, rhs, x, its, res, epi);
+              : bicgstab_impl<float>(p, system, B, di, o, rhs, x, its, res, epi);
   }
   const double* B = system == 0 ? p->Bst.p : p->Bcn.p;
   const double* di = system == 0 ? p->dinv_st.p : p->dinv_cn.p;
   return gm ? gmres_impl<double>(p, B, di, o, rhs, x, its, res, epi)
-            : bicgstab_impl<double>(p, B, di, o, rhs, x, its, res, epi);
+            : bicgstab_impl<double>(p, system, B, di, o, rhs, x, its, res, epi);
 }
 
 }  // namespace afc

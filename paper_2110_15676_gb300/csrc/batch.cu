@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(512, PH < 2 ? 4 : 3) k_batch_pass(const BInst*
   const int K = sh.of.K;
   if (K == 27) batch_row<27, MIXED, 3>(sh, PH, 0, sa, limiter, i);
   else if (K == 15) batch_row<15, MIXED, 3>(sh, PH, 0, sa, limiter, i);
-  else batch_row<0, MIXED, 1>(sh, PH, 0, sa, limiter, i);
+  else batch_row<0, MIXED, 3>(sh, PH, 0, sa, limiter, i);
 }
 
 // per instance: min and max of the stored solution

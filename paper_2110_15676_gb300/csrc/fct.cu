@@ -222,7 +222,7 @@ __global__ void k_cn_factors(int64_t N, Offsets of, const unsigned long long* __
     double r[S];
 #pragma unroll
     for (int j = 0; j < S; ++j)
-      if (k0 + j != Kup) r[j] = r_up[pair_slot(of, Kup, k0 + j, i, N)];
+      if (k0 + j != Kup) r[j] = r_up[pair_slot(of, Kup, group_at<KT>(k0 + j, K), i, N)];
 #pragma unroll
     for (int j = 0; j < S; ++j) {
       const int k = k0 + j;
@@ -275,13 +275,13 @@ __global__ void __launch_bounds__(256, 4) k_cn_residual(int64_t N, Offsets of, i
 #pragma unroll
           for (int j = 0; j < S; ++j) {
             if (k0 + j == Kup) continue;
-            r[j] = r_up[pair_slot(of, Kup, k0 + j, i, N)];
+            r[j] = r_up[pair_slot(of, Kup, group_at<KT>(k0 + j, K), i, N)];
             if (k0 + j < Kup) r[j] = neg_bits(r[j]);
           }
           if (limiter == AFC_LIM_ZALESAK) {   // R- of the neighbour for r > 0, R+ else: one load each
 #pragma unroll
             for (int j = 0; j < S; ++j)
-              if (k0 + j != Kup) Rj[j] = (gt0(r[j]) ? Rm : Rp)[i + of.o[k0 + j]];
+              if (k0 + j != Kup) Rj[j] = (gt0(r[j]) ? Rm : Rp)[i + of.o[group_at<KT>(k0 + j, K)]];
           }
 #pragma unroll
           for (int j = 0; j < S; ++j) {

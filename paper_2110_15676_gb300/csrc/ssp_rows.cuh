@@ -139,25 +139,27 @@ __device__ __forceinline__ void ssp_factors_row(const Offsets& of, const SspArra
 #pragma unroll
       for (int j = 0; j < S; ++j) {
         if (k0 + j == Kup) continue;
-        c[j] = a.md32[pair_slot(of, Kup, k0 + j, i, a.N)];
-        w[j] = a.uw[i + of.o[k0 + j]];
-        v[j] = a.ut[i + of.o[k0 + j]];
+        const int k = group_at<KT>(k0 + j, K);
+        c[j] = a.md32[pair_slot(of, Kup, k, i, a.N)];
+        w[j] = a.uw[i + of.o[k]];
+        v[j] = a.ut[i + of.o[k]];
       }
 #pragma unroll
       for (int j = 0; j < S; ++j) {
         if (k0 + j == Kup) continue;
         // upper pairs as the edges pass stores them; lower ones as their lower row does, r_e = -r_ij
         rf[j] = k0 + j > Kup ? ssp_flux(c[j], wi, w[j]) : ssp_flux(c[j], w[j], wi);
-        if (k0 + j > Kup) a.r32[(int64_t)(k0 + j - Kup - 1) * a.N + i] = rf[j];
+        if (k0 + j > Kup) a.r32[(int64_t)(group_at<KT>(k0 + j, K) - Kup - 1) * a.N + i] = rf[j];
       }
     } else {
 #pragma unroll
       for (int j = 0; j < S; ++j) {
         if (k0 + j == Kup) continue;
-        const int64_t q = pair_slot(of, Kup, k0 + j, i, a.N);
+        const int k = group_at<KT>(k0 + j, K);
+        const int64_t q = pair_slot(of, Kup, k, i, a.N);
         if (MIXED) rf[j] = a.r32[q];
         else r[j] = a.r_up[q];
-        v[j] = a.ut[i + of.o[k0 + j]];
+        v[j] = a.ut[i + of.o[k]];
       }
     }
 #pragma unroll
@@ -233,12 +235,13 @@ __device__ __forceinline__ void ssp_correct_row(const Offsets& of, const SspArra
 #pragma unroll
         for (int j = 0; j < S; ++j) {
           if (k0 + j == Kup) continue;
-          const int64_t q = pair_slot(of, Kup, k0 + j, i, a.N);
+          const int k = group_at<KT>(k0 + j, K);
+          const int64_t q = pair_slot(of, Kup, k, i, a.N);
           if (MIXED) rf[j] = a.r32[q];
           else r[j] = a.r_up[q];
           if (SMALL && limiter == AFC_LIM_ZALESAK) {
-            Rj[j] = load_now(a.Rm + i + of.o[k0 + j]);
-            Rk[j] = load_now(a.Rp + i + of.o[k0 + j]);
+            Rj[j] = load_now(a.Rm + i + of.o[k]);
+            Rk[j] = load_now(a.Rp + i + of.o[k]);
           }
         }
 #pragma unroll
@@ -250,7 +253,7 @@ __device__ __forceinline__ void ssp_correct_row(const Offsets& of, const SspArra
         if (!SMALL && limiter == AFC_LIM_ZALESAK) {
 #pragma unroll
           for (int j = 0; j < S; ++j)
-            if (k0 + j != Kup) Rj[j] = Rk[j] = (gt0(r[j]) ? a.Rm : a.Rp)[i + of.o[k0 + j]];
+            if (k0 + j != Kup) Rj[j] = Rk[j] = (gt0(r[j]) ? a.Rm : a.Rp)[i + of.o[group_at<KT>(k0 + j, K)]];
         }
 #pragma unroll
         for (int j = 0; j < S; ++j) {

@@ -228,6 +228,10 @@ __device__ __forceinline__ unsigned int bicg_sums_begin(BicgShared<T>& sh, const
   for (int q = 0; q < NV; ++q) sh.col[q][threadIdx.x] = v[q];
   __syncthreads();
   for (int u = w; u < 4 * NV; u += nt >> 5) {
+    if ((u & 3) * 32 >= nt) {   // blocks of fewer than 128 threads: no columns in this quarter
+      if (lane == 0) sh.quarter[u >> 2][u & 3] = 0.0;
+      continue;
+    }
     const double* c = sh.col[u >> 2];
     double t = 0.0;
     if (!TURN)

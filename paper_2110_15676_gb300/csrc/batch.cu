@@ -12,8 +12,7 @@
 // each pass a kernel of its own: 32 registers for the rate and edge passes, 40 for the other
 // two with three neighbours' loads in flight.  As one kernel that held all passes and patterns
 // (64 registers, offsets and pointers searched per tile) 15 stages of 48 mixed Q1 instances (17 to
-// 49 nodes per side) took 12.4 ms, now 7.0 ms (and 5 % less since the correct pass widens its fluxes after the
-// loads); at 64 registers and nine loads 7.9 ms, at 32
+// 49 nodes per side) took 12.4 ms against 7.0 ms; at 64 registers and nine loads 7.9 ms, at 32
 // registers 6.9 ms but a small double-precision batch 7 % slower.
 // PER_STAGE / PER_STEP: one persistent cooperative launch per stage / per time
 // step; each block takes a contiguous range of tiles (neighbouring rows, few

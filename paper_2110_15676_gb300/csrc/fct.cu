@@ -63,18 +63,22 @@ __global__ void k_ssp_correct(Offsets of, SspArrays a, int limiter, double dt, d
   pdl_wait();
   if (i < a.N) ssp_correct_row<KT, MIXED, kGroup<KT>, SMALL>(of, a, i, limiter, dt, ca, uA, cb, out);
 }
-// Below this many rows (about one resident wave) the passes take their SMALL form.
-constexpr int64_t kSmallRows = 300000;
+// Below this many rows the passes take their SMALL form: one resident wave of it (Q1 at 89 to 96
+// registers: two blocks of 256 on each of 152 SMs); beyond that its registers cost more than its
+// loads in flight gain.  SSP3 step, us, large / small form: Q1 mixed 68,921 rows 115 / 105, 91,125 130 / 133,
+// 274,625 249 / 303; Q1 in double 35,937 rows 95.2 / 94.7, 91,125 154 / 160; P1 in double 1 % of each
+// other up to 117,649.  The mixed form takes 56 to 72 registers for the other patterns: P1 117,649 rows
+// 108 / 101, 274,625 166 / 165, 389,017 223 / 229.
+constexpr int64_t kSmallRows = 2 * 152 * kBlock, kSmallRowsMixed = 300000;
 // In the mixed mode their factors pass is FUSED: a flux is three FP32 operations, a launch costs
-// more (77,121 rows of Q1: 114 us a step against 119 us; 105 us since the correct pass loads its
-// groups before it widens).  Not in double (P1 9^3: 67 us against 61 us),
+// more (77,121 rows of Q1: 114 us a step against 119 us).  Not in double (P1 9^3: 67 us against 61 us),
 // and not on larger grids or in batches (48 mixed instances: 7.2 ms against 7.0 ms).
 
 // A whole SSP2 / SSP3 step of a small problem as one cooperative launch, its passes separated
 // by grid barriers: on grids of a few thousand rows a pass is latency (one to two microseconds),
 // and a launch costs more than a barrier of as many blocks (SSP3 step in double, us, against
 // launches with programmatic dependent launch: P1 9^3 56 / 60, P1 25^3 62 / 70, Q1 17^3 72 / 81, Q1 25^3 75 / 84;
-// mixed Q1 17^3 84 / 91, before the correct pass widened its fluxes after the loads).
+// mixed Q1 17^3 84 / 91).
 constexpr int kStepBlock = 128;
 
 struct StepVecs {
@@ -369,7 +373,7 @@ int fe_stage(afc_problem_s* p, const double* uin, double dt, int limiter, double
     constexpr int KT = decltype(kc)::value;
     constexpr bool MX = decltype(mc)::value;
     AFC_LAUNCH(p, "k_ssp_rate", launch_pass(pdl, k_ssp_rate<KT, MX>, g, blk, s, p->offs, arr, uin, dt));
-    const bool small = N < kSmallRows;
+    const bool small = N < (MX && KT != 27 ? kSmallRowsMixed : kSmallRows);
     const bool fused = MX && small && limiter == AFC_LIM_ZALESAK;
     if (limiter != AFC_LIM_NONE && !fused)
       AFC_LAUNCH(p, "k_ssp_edges", launch_pass(chain, k_ssp_edges<KT, MX>, g, blk, s, p->offs, arr, uin));

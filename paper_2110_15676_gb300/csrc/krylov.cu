@@ -124,7 +124,7 @@ int dia_spmv(afc_problem_s* p, const double* A, const double* x, double* y) {
 // ---------------------------------------------------------------------------
 // Solver workspace
 // ---------------------------------------------------------------------------
-constexpr int kMaxRestart = 32;   // GMRES(m), m <= 32: the Gram-Schmidt kernel keeps m dots in registers
+constexpr int kMaxRestart = 32;   // GMRES(m), m <= 32: a Hessenberg column has an entry per lane of a warp
 
 // device scalar slots
 enum : int {
